@@ -32,6 +32,12 @@ __device__ __forceinline__ ff ff_quick_two_sum(float a, float b) {   // |a| >= |
   return ff_make(s, e);
 }
 
+__device__ __forceinline__ ff ff_two_sum(float a, float b) {   // exact a + b
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  return ff_make(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
+
 __device__ __forceinline__ ff ff_add(ff a, ff b) {
   const float s = __fadd_rn(a.hi, b.hi);
   const float bb = __fsub_rn(s, a.hi);

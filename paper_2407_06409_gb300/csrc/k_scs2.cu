@@ -11,14 +11,15 @@
 //    with their frequency-independent geometry and damping F, dF/dr (k_scs_count/k_scs_fill);
 //  * erf and exp of r/sigma_ij are evaluated once per atom pair and frequency (k_pair_radial,
 //    FP64), not once per local system holding the pair; the local systems read the table;
-//  * B_K is factorised in FP32 (Cholesky, packed lower triangle in shared memory) and the
-//    FP64 solution is recovered by iterative refinement: the residual d - B X is formed in
-//    FP64 from the sparse pair list, corrections come from the FP32 factor (classical mixed-
-//    precision refinement, Wilkinson/Moler; converges when cond(B) * eps_fp32 << 1);
-//  * the adjoint solve B lambda = dL/dX reuses the stored FP32 factor with the same refinement,
-//    and contracts dB/dr, dd/dr pair by pair from the stored radial terms.
-#include "lmbd_internal.cuh"
+//  * a system is solved by conjugate gradients in FP32 and the FP64 solution recovered by
+//    iterative refinement: the residual d - B X is formed in float-float from the sparse pair
+//    list, corrections come from further FP32 solves (mixed-precision refinement, Wilkinson/Moler);
+//  * the adjoint solve B lambda = dL/dX is the same kernel; the contraction with dB/dr, dd/dr
+//    runs pair by pair over all frequencies from the stored radial terms (k_scs_contract).
+#include <algorithm>
+
 #include "ff.cuh"
+#include "lmbd_internal.cuh"
 
 // pair predicate shared by the counting and filling kernels (identical FP64 arithmetic)
 __device__ __forceinline__ bool scs_pair_in(const double* xs, int ld, int i, int j, double rc2, double& rx,
@@ -42,8 +43,6 @@ __device__ __forceinline__ bool scs_pair_in_screened(const float* xf, const doub
   double rx, ry, rz, r2;
   return scs_pair_in(xs, ld, i, j, rc2, rx, ry, rz, r2);
 }
-
-__device__ __forceinline__ long long packed_idx(int i, int k) { return (long long)i * (i + 1) / 2 + k; }
 
 // ---------------------------------------------------------------------------------------
 // pair lists: count (before the workspace is sized) and fill
@@ -92,17 +91,19 @@ __global__ void __launch_bounds__(256) k_scs_count(Work w, DevParams p, int max_
   }
 }
 
-// One block per central atom.  Pairs are ordered by owner row i: first the K1 partners
-// j < i (ascending), then the K2 partners (ascending); adjacency rows list every K1
-// partner j != i (ascending) with the index of the shared pair.
+// One block per central atom.  The K1 pairs of all rows come first (row i: its partners j < i,
+// ascending), then the K2 pairs of all rows (partners ascending), so that kernels take one kind
+// with whole warps; adjacency rows list every K1 partner j != i (ascending) with the index of the
+// shared pair.
 __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, int max_n12, int max_n1) {
   extern __shared__ double smem_d[];
   double* xs = smem_d;                             // 3 x max_n12
   int* pid = (int*)(xs + 3 * max_n12);             // max_n1 x max_n1 (pair index, -1 = none)
   int* rowk1 = pid + max_n1 * max_n1;              // max_n1
   int* rowcnt = rowk1 + max_n1;                    // max_n1
-  int* rowstart = rowcnt + max_n1;                 // max_n1 + 1
-  int* adjcnt = rowstart + max_n1 + 1;             // max_n1
+  int* k1start = rowcnt + max_n1;                  // max_n1 + 1: first K1 pair of each row
+  int* k2start = k1start + max_n1 + 1;             // max_n1 + 1: first K2 pair of each row
+  int* adjcnt = k2start + max_n1 + 1;              // max_n1
   int* adjstart = adjcnt + max_n1;                 // max_n1 + 1
   int* k2cnt = adjstart + max_n1 + 1;              // max_n12
   int* klist = k2cnt + max_n12;                    // per warp max_n1: atoms of one K1 list
@@ -137,19 +138,20 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
       bool in = j < n12 && scs_pair_in_screened(xf, xs, max_n12, i, j, lo2, hi2, rc2);
       k2 += __popc(__ballot_sync(0xffffffffu, in));
     }
-    if (lane == 0) { rowk1[i] = k1; rowcnt[i] = k1 + k2; }
+    if (lane == 0) { rowk1[i] = k1; rowcnt[i] = k2; }
   }
   __syncthreads();
   if (tid == 0) {
     int run = 0;
-    for (int i = 0; i < n1; ++i) { rowstart[i] = run; run += rowcnt[i]; }
-    rowstart[n1] = run;
+    for (int i = 0; i < n1; ++i) { k1start[i] = run; run += rowk1[i]; }
+    k1start[n1] = run;
+    for (int i = 0; i < n1; ++i) { k2start[i] = run; run += rowcnt[i]; }
+    k2start[n1] = run;
   }
   __syncthreads();
   // phase 2a: pairs in order (row, partner) and their entry in the atom-pair radial table
   int* lst = klist + warp * max_n1;
   for (int i = warp; i < n1; i += nw) {
-    int pos = rowstart[i];
     // atoms of the K1 list of site i's atom, for the radial-table lookup below
     const int ai = w.site_atom[sbase + i];
     const int na = w.counts[ai].n1;
@@ -159,6 +161,7 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     __syncwarp();
     for (int pass = 0; pass < 2; ++pass) {
       int jb = pass == 0 ? 0 : n1, je = pass == 0 ? i : n12;
+      int pos = pass == 0 ? k1start[i] : k2start[i];
       for (int j0 = jb; j0 < je; j0 += 32) {
         int j = j0 + lane;
         bool in = j < je && scs_pair_in_screened(xf, xs, max_n12, i, j, lo2, hi2, rc2);
@@ -184,21 +187,24 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
               break;
             }
           }
-          w.pr_g[q] = gi;
+          w.pr_ga[q] = make_int2(gi, aj);
           if (pass == 0) pid[i * max_n1 + j] = slot;
         }
         pos += __popc(m);
       }
     }
     if (lane == 0) {
-      w.prow[rbase + i] = rowstart[i];
-      w.prow_k2[rbase + i] = rowstart[i] + rowk1[i];
+      w.prow[rbase + i] = k1start[i];
+      w.prow_k2[rbase + i] = k2start[i];
     }
   }
-  if (tid == 0) w.prow[rbase + n1] = rowstart[n1];
+  if (tid == 0) {
+    w.prow[rbase + n1] = k1start[n1];
+    w.prow_k2[rbase + n1] = k2start[n1];
+  }
   __syncthreads();
   // phase 2b: FP64 geometry and damping of every pair, one thread per pair
-  for (int t = tid; t < rowstart[n1]; t += blockDim.x) {
+  for (int t = tid; t < k2start[n1]; t += blockDim.x) {
     const long long q = offp + t;
     const int i = w.pr_ij[2 * q], j = w.pr_ij[2 * q + 1];
     double rx, ry, rz, r2;
@@ -266,7 +272,7 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     for (int j = n1 + lane; j < n12; j += 32) k2cnt[j] = 0;
     __syncwarp();
     for (int i = 0; i < n1; ++i) {
-      const int b = rowstart[i] + rowk1[i], e = rowstart[i + 1];
+      const int b = k2start[i], e = k2start[i + 1];
       for (int t = b + lane; t < e; t += 32) ++k2cnt[w.pr_ij[2 * (offp + t) + 1]];
       __syncwarp();
     }
@@ -282,7 +288,7 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     }
     __syncwarp();
     for (int i = 0; i < n1; ++i) {
-      const int b = rowstart[i] + rowk1[i], e = rowstart[i + 1];
+      const int b = k2start[i], e = k2start[i + 1];
       for (int t = b + lane; t < e; t += 32) {
         const int j = w.pr_ij[2 * (offp + t) + 1];
         w.k2rev[offp + k2cnt[j]] = t;
@@ -291,388 +297,6 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
       __syncwarp();
     }
   }
-}
-
-// ---------------------------------------------------------------------------------------
-// FP32 Cholesky and triangular solves on a packed lower triangle in shared memory
-// (whole thread block of 256 threads; 16-wide blocks; 3 right-hand sides)
-// ---------------------------------------------------------------------------------------
-#define CB 16
-#define CBP (CB * (CB + 1) / 2)   // packed lower triangle of one diagonal-block inverse
-__device__ __forceinline__ int pidx16(int i, int j) { return i * (i + 1) / 2 + j; }
-
-// The 16 x 16 diagonal block at k0, one warp: right-looking Cholesky in registers (one row per
-// lane, rows beyond the block hold the identity; one reciprocal square root per pivot, so
-// sinv[i] = 1/L_ii is that reciprocal), then the inverse of the factor block, one column per
-// lane, into binv (packed lower triangle).  A non-positive pivot sets *bad.
-__device__ void chol32_diag(float* A, int n, int k0, int* bad, float* sinv, float* binv) {
-  const int lane = threadIdx.x & 31;
-  const int kb = min(CB, n - k0);
-  const bool act = lane < kb;
-  float a[CB];
-#pragma unroll
-  for (int u = 0; u < CB; ++u)
-    a[u] = act ? (u <= lane ? A[packed_idx(k0 + lane, k0 + u)] : 0.f) : (u == lane ? 1.f : 0.f);
-  bool fail = false;
-  float il_own = 1.f;
-#pragma unroll
-  for (int t = 0; t < CB; ++t) {
-    float d = __shfl_sync(0xffffffffu, a[t], t);
-    if (t < kb && !(d > 0.f)) {
-      fail = true;
-      d = 1.f;
-    }
-    const float il = rsqrtf(d), l = d * il;
-    if (lane == t) {
-      a[t] = l;
-      il_own = il;
-    } else if (lane > t) {
-      a[t] *= il;
-    }
-#pragma unroll
-    for (int j = 1; j < CB; ++j) {
-      if (j > t) {
-        const float ljt = __shfl_sync(0xffffffffu, a[t], j);
-        if (lane >= j) a[j] -= a[t] * ljt;
-      }
-    }
-  }
-  if (fail && lane == 0) *bad = 1;
-#pragma unroll
-  for (int u = 0; u < CB; ++u)
-    if (act && u <= lane) A[packed_idx(k0 + lane, k0 + u)] = a[u];
-  if (act) sinv[k0 + lane] = il_own;
-  __syncwarp();
-  // inverse of the factor block: lane c solves L x = e_c, reading L from shared memory
-  // (every lane reads the same element: broadcast)
-  float* inv = binv + (k0 / CB) * CBP;
-  float x[CB];
-#pragma unroll
-  for (int i = 0; i < CB; ++i) {
-    float v = 0.f;
-    if (i < kb) {
-      const float* Li = A + packed_idx(k0 + i, k0);
-      float s = (i == lane) ? 1.f : 0.f;
-#pragma unroll
-      for (int u = 0; u < i; ++u) s -= Li[u] * x[u];
-      v = (i >= lane && act) ? s * sinv[k0 + i] : 0.f;
-    }
-    x[i] = v;
-    if (lane < CB && i >= lane) inv[pidx16(i, lane)] = v;
-  }
-  __syncwarp();
-}
-
-// named barrier 1 between warp 0 (waits) and warp 1 (arrives): 64 threads
-__device__ __forceinline__ void nbar_sync_w01() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
-__device__ __forceinline__ void nbar_arrive_w01() { asm volatile("bar.arrive 1, 64;" ::: "memory"); }
-
-// Right-looking blocked Cholesky of the packed lower triangle (16-wide blocks, 256 threads),
-// with lookahead.  Per block column k: all threads form the panel rows below the diagonal block
-// from the inverse diagonal block (L_ik = A_ik L_kk^-T, independent dot products); then warp 1
-// updates the next diagonal block first and hands it to warp 0 through a named barrier, warp 0
-// factors and inverts it while warps 1..7 update the trailing rows below it, two rows per warp
-// at a time (each panel value a lane loads serves both rows).  Two block barriers per block
-// column; the factor of the next diagonal block is off the path of the trailing update.
-// sinv[i] = 1/L_ii; binv holds the inverses of the diagonal blocks (solve32_warp).
-__device__ __noinline__ void chol32_packed(float* A, int n, int* bad, float* sinv, float* binv) {
-  constexpr int RB = 2;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  if (warp == 0) chol32_diag(A, n, 0, bad, sinv, binv);
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += CB) {
-    const int kb = min(CB, n - k0), r0 = k0 + kb;
-    if (r0 >= n) break;
-    const float* inv = binv + (k0 / CB) * CBP;
-    for (int i = r0 + tid; i < n; i += blockDim.x) {
-      float* row = A + packed_idx(i, k0);
-      float v[CB], o[CB];
-#pragma unroll
-      for (int t = 0; t < CB; ++t) v[t] = t < kb ? row[t] : 0.f;
-#pragma unroll
-      for (int t = 0; t < CB; ++t) {
-        float sum = 0.f;
-#pragma unroll
-        for (int u = 0; u <= t; ++u) sum += v[u] * inv[pidx16(t, u)];
-        o[t] = sum;
-      }
-#pragma unroll
-      for (int t = 0; t < CB; ++t)
-        if (t < kb) row[t] = o[t];
-    }
-    __syncthreads();
-    const int k1 = r0, kb1 = min(CB, n - k1), r1 = k1 + kb1;
-    if (warp == 0) {
-      nbar_sync_w01();
-      chol32_diag(A, n, k1, bad, sinv, binv);
-    } else {
-      if (warp == 1) {
-        // the next diagonal block: lane l takes row l % 16, the columns of parity l / 16
-        const int i = lane & 15;
-        if (i < kb1) {
-          const float* li = A + packed_idx(k1 + i, k0);
-          float a[CB];
-#pragma unroll
-          for (int t = 0; t < CB; ++t) a[t] = t < kb ? li[t] : 0.f;
-          for (int j = lane >> 4; j <= i; j += 2) {
-            const float* lj = A + packed_idx(k1 + j, k0);
-            float sum = 0.f;
-#pragma unroll
-            for (int t = 0; t < CB; ++t)
-              if (t < kb) sum += a[t] * lj[t];
-            A[packed_idx(k1 + i, k1 + j)] -= sum;
-          }
-        }
-        __threadfence_block();
-        nbar_arrive_w01();
-      }
-      for (int i0 = r1 + RB * (warp - 1); i0 < n; i0 += RB * (nw - 1)) {
-        float a[RB][CB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-          const float* li = A + packed_idx(min(i0 + r, n - 1), k0);
-#pragma unroll
-          for (int t = 0; t < CB; ++t) a[r][t] = t < kb ? li[t] : 0.f;
-        }
-        const int ilast = min(i0 + RB - 1, n - 1);
-        for (int j = k1 + lane; j <= ilast; j += 32) {
-          const float* lj = A + packed_idx(j, k0);
-          float sum[RB];
-#pragma unroll
-          for (int r = 0; r < RB; ++r) sum[r] = 0.f;
-#pragma unroll
-          for (int t = 0; t < CB; ++t) {
-            const float v = t < kb ? lj[t] : 0.f;
-#pragma unroll
-            for (int r = 0; r < RB; ++r) sum[r] += a[r][t] * v;
-          }
-#pragma unroll
-          for (int r = 0; r < RB; ++r)
-            if (j <= i0 + r && i0 + r < n) A[packed_idx(i0 + r, j)] -= sum[r];
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// y (n x 3, FP32, shared) <- (L L^T)^-1 y with binv the inverses of the 16 x 16 diagonal blocks,
-// a blocked substitution with one warp per right-hand side column: warps 0..2 each solve their
-// column with warp-level
-// synchronisation only (a block row: half-warp partial sums of its 16 rows over the solved part,
-// combined across the halves with a shuffle, then the product with the inverse diagonal block by
-// shuffles), so the substitution needs no block barrier; z (n x 3) is scratch.  The caller's
-// writes to y must be visible (a block barrier before); the result is visible after the final one.
-__device__ void solve32_warp(const float* L, int n, const float* binv, float* y, float* z) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < 3) {
-    const int c = warp, r = lane & 15, h = lane >> 4;
-    // forward: z = L^-1 y
-    for (int b0 = 0; b0 < n; b0 += CB) {
-      const int bb = min(CB, n - b0);
-      const float* inv = binv + (b0 / CB) * CBP;
-      float t = 0.f;
-      if (r < bb) {
-        const float* row = L + packed_idx(b0 + r, 0);
-        for (int k = h; k < b0; k += 2) t += row[k] * z[3 * k + c];
-      }
-      t += __shfl_xor_sync(0xffffffffu, t, 16);
-      const float v = r < bb ? y[3 * (b0 + r) + c] - t : 0.f;
-      float acc = 0.f;
-#pragma unroll
-      for (int u = 0; u < CB; ++u) {
-        const float vu = __shfl_sync(0xffffffffu, v, u);
-        if (u <= r && r < bb) acc += inv[pidx16(r, u)] * vu;
-      }
-      if (h == 0 && r < bb) z[3 * (b0 + r) + c] = acc;
-      __syncwarp();
-    }
-    // backward: y = L^-T z
-    const int nblk = (n + CB - 1) / CB;
-    for (int blk = nblk - 1; blk >= 0; --blk) {
-      const int b0 = blk * CB, bb = min(CB, n - b0), b1 = b0 + bb;
-      const float* inv = binv + blk * CBP;
-      float t = 0.f;
-      if (r < bb)
-        for (int k = b1 + h; k < n; k += 2) t += L[packed_idx(k, b0 + r)] * y[3 * k + c];
-      t += __shfl_xor_sync(0xffffffffu, t, 16);
-      const float v = r < bb ? z[3 * (b0 + r) + c] - t : 0.f;
-      float acc = 0.f;
-#pragma unroll
-      for (int u = 0; u < CB; ++u) {
-        const float vu = __shfl_sync(0xffffffffu, v, u);
-        if (u >= r && u < bb) acc += inv[pidx16(u, r)] * vu;
-      }
-      if (h == 0 && r < bb) y[3 * (b0 + r) + c] = acc;
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-}
-
-// ---------------------------------------------------------------------------------------
-// shared memory of the per-(atom, frequency) kernels
-// ---------------------------------------------------------------------------------------
-struct Scs2Smem {
-  float* A;       // packed lower factor, N1 (N1 + 1) / 2
-  float* sinv;    // N1
-  float* binv;    // ceil(N1/16) x 136: inverses of the diagonal blocks (packed lower)
-  float* y;       // N1 x 3 (FP32 right-hand side / correction)
-  float* z;       // N1 x 3 (FP32 scratch of the triangular solves)
-  double* rhs;    // N1 x 3 (FP64 right-hand side d or dL/dX)
-  double* x;      // N1 x 3 (FP64 solution X or lambda)
-  double* xs;     // N1 x 3 (adjoint: X of the forward solve)
-  ff* abf;        // n12 (alpha_bar at this frequency, float-float)
-  double* iab;    // n1 (1 / alpha_bar of the coupled sites)
-  double* red;    // 64
-};
-
-__host__ __device__ inline size_t scs2_smem_bytes(int max_n1, int max_n12, bool adjoint) {
-  size_t N1 = 3 * (size_t)max_n1;
-  size_t fl = N1 * (N1 + 1) / 2 + N1 + 6 * N1 + (N1 + 15) / 16 * CBP;
-  fl = (fl + 1) & ~size_t(1);
-  size_t dd = 2 * 3 * N1 + (size_t)max_n12 + (size_t)max_n1 + 64;
-  if (adjoint) dd += 3 * N1;
-  return fl * sizeof(float) + dd * sizeof(double);
-}
-
-__device__ inline Scs2Smem scs2_carve(unsigned char* base, int max_n1, int max_n12, bool adjoint) {
-  Scs2Smem s;
-  size_t N1 = 3 * (size_t)max_n1;
-  s.A = (float*)base;
-  s.sinv = s.A + N1 * (N1 + 1) / 2;
-  s.y = s.sinv + N1;
-  s.z = s.y + 3 * N1;
-  s.binv = s.z + 3 * N1;
-  size_t fl = N1 * (N1 + 1) / 2 + N1 + 6 * N1 + (N1 + 15) / 16 * CBP;
-  fl = (fl + 1) & ~size_t(1);
-  double* d = (double*)(base + fl * sizeof(float));
-  s.rhs = d;
-  s.x = s.rhs + 3 * N1;
-  s.abf = reinterpret_cast<ff*>(s.x + 3 * N1);      // one ff per site: 8 bytes, as a double
-  s.iab = reinterpret_cast<double*>(s.abf + max_n12);
-  s.red = s.iab + max_n1;
-  s.xs = adjoint ? s.red + 64 : nullptr;
-  return s;
-}
-
-// rhs <- rhs - B y for the FP32 vector y, in float-float arithmetic on the FP32 pipe (B from the
-// float-float tables: 1/alpha_bar on the diagonal, F A0 delta + F B0 r r^T per K1 pair).  Called
-// with the FP32 solution x0 = y it forms the residual d - B x0 (error ~2^-46 |B| |x0|, so the
-// refined solution carries a relative error ~cond(B) 2^-46); called with a correction delta
-// (~1e-7 of x) it updates the residual of x + delta to FP64 rounding.
-__device__ void scs2_residual_update(const Work& w, const DevParams& p, int n1, long long offp, long long offa,
-                                     long long rbase, int q, Scs2Smem& sm) {
-  // two threads per (coupled site i, right-hand side c), neighbouring lanes, each summing half of
-  // the adjacency row; the halves are combined with a shuffle in a fixed order
-  const int items = 6 * n1;
-  for (int base = 0; base < items; base += blockDim.x) {
-    const int e = base + threadIdx.x;
-    const bool act = e < items;
-    const int i = act ? e / 6 : 0, c = act ? (e >> 1) % 3 : 0, half = e & 1;
-    ff a0 = ff_make(0.f, 0.f), a1 = a0, a2 = a0;
-    if (act) {
-      if (half == 0) {
-        const ff ia = ff_from_double(sm.iab[i]);
-        a0 = ff_scale(ia, sm.y[9 * i + c]);
-        a1 = ff_scale(ia, sm.y[9 * i + 3 + c]);
-        a2 = ff_scale(ia, sm.y[9 * i + 6 + c]);
-      }
-      const int b0 = w.arow[rbase + i], en0 = w.arow[rbase + i + 1];
-      const int mid = b0 + (en0 - b0 + 1) / 2;
-      const int b = half == 0 ? b0 : mid, en = half == 0 ? mid : en0;
-      for (int t = b; t < en; ++t) {
-        const int j = w.adj[2 * (offa + t)];
-        const long long pq = offp + w.adj[2 * (offa + t) + 1];
-        const float2* gf = w.pr_gff + 6 * pq;
-        const float2* rf = w.pr_rad_ff + 2 * (pq * p.nqs + q);
-        const ff rx = ff_make(gf[0].x, gf[0].y), ry = ff_make(gf[1].x, gf[1].y), rz = ff_make(gf[2].x, gf[2].y);
-        const ff fa = ff_make(rf[0].x, rf[0].y), fb = ff_make(rf[1].x, rf[1].y);
-        const float d0 = sm.y[9 * j + c], d1 = sm.y[9 * j + 3 + c], d2 = sm.y[9 * j + 6 + c];
-        const ff bu = ff_mul(fb, ff_add(ff_add(ff_scale(rx, d0), ff_scale(ry, d1)), ff_scale(rz, d2)));
-        a0 = ff_add(a0, ff_add(ff_scale(fa, d0), ff_mul(bu, rx)));
-        a1 = ff_add(a1, ff_add(ff_scale(fa, d1), ff_mul(bu, ry)));
-        a2 = ff_add(a2, ff_add(ff_scale(fa, d2), ff_mul(bu, rz)));
-      }
-    }
-    const ff o0 = ff_make(__shfl_xor_sync(0xffffffffu, a0.hi, 1), __shfl_xor_sync(0xffffffffu, a0.lo, 1));
-    const ff o1 = ff_make(__shfl_xor_sync(0xffffffffu, a1.hi, 1), __shfl_xor_sync(0xffffffffu, a1.lo, 1));
-    const ff o2 = ff_make(__shfl_xor_sync(0xffffffffu, a2.hi, 1), __shfl_xor_sync(0xffffffffu, a2.lo, 1));
-    if (act && half == 0) {
-      sm.rhs[9 * i + c] -= ff_to_double(ff_add(a0, o0));
-      sm.rhs[9 * i + 3 + c] -= ff_to_double(ff_add(a1, o1));
-      sm.rhs[9 * i + 6 + c] -= ff_to_double(ff_add(a2, o2));
-    }
-  }
-}
-
-// x = B^-1 rhs: FP32 solve, then FP64 refinement until the predicted error is below
-// rel_tol |x|: the residual is formed once in FP64 and then updated by the corrections (rhs is
-// overwritten).  Returns the number of corrections; *fail set if it does not converge.
-// rel_tol = 2^-52 for the forward solve (alpha_K and alpha_I to FP64 accuracy); the adjoint
-// solve, whose lambda only feeds the forces (1e-8 eV/A tolerance; a relative error of 1e-9 in
-// lambda moves them by ~1e-11 eV/A), stops at 2^-30 and may stop after the first correction on
-// an a-priori contraction estimate (below).
-__device__ int scs2_refine(const Work& w, const DevParams& p, int n1, long long offp, long long offa,
-                           long long rbase, int q, Scs2Smem& sm, int* fail, double rel_tol) {
-  const int N1 = 3 * n1, tid = threadIdx.x;
-  for (int e = tid; e < 3 * N1; e += blockDim.x) sm.y[e] = (float)sm.rhs[e];
-  __syncthreads();
-  solve32_warp(sm.A, N1, sm.binv, sm.y, sm.z);
-  for (int e = tid; e < 3 * N1; e += blockDim.x) sm.x[e] = (double)sm.y[e];
-  __syncthreads();
-  // the residual d - B x0 of the FP32 solution x0 = y, in float-float arithmetic on the FP32
-  // pipe (kept in rhs), then updated by -B delta per correction the same way
-  scs2_residual_update(w, p, n1, offp, offa, rbase, q, sm);
-  __syncthreads();
-  for (int e = tid; e < 3 * N1; e += blockDim.x) sm.y[e] = (float)sm.rhs[e];
-  __syncthreads();
-  double prev = 0.0;
-  int it = 0;
-  for (; it < 12; ++it) {
-    solve32_warp(sm.A, N1, sm.binv, sm.y, sm.z);
-    double dmax = 0.0, xmax = 0.0;
-    for (int e = tid; e < 3 * N1; e += blockDim.x) {
-      double dlt = (double)sm.y[e];
-      double xn = sm.x[e] + dlt;
-      sm.x[e] = xn;
-      dmax = fmax(dmax, fabs(dlt));
-      xmax = fmax(xmax, fabs(xn));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      xmax = fmax(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
-    }
-    if ((tid & 31) == 0) { sm.red[tid >> 5] = dmax; sm.red[32 + (tid >> 5)] = xmax; }
-    __syncthreads();
-    dmax = 0.0;
-    xmax = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-      dmax = fmax(dmax, sm.red[k]);
-      xmax = fmax(xmax, sm.red[32 + k]);
-    }
-    __syncthreads();
-    // contraction estimate rho = |delta_k| / |delta_{k-1}|; stop when rho |delta_k| is negligible.
-    // With the looser adjoint tolerance the first correction already gives an estimate: the
-    // FP32 solution's relative error, i.e. |delta_0| / |x|, is the contraction factor of the
-    // iteration (error_0 = (M^-1 - B^-1) d with M = L L^T), so the error left after it is about
-    // (|delta_0| / |x|) |delta_0|; a margin of 10 on that
-    const double tol = rel_tol * xmax;
-    if (dmax <= tol) { ++it; break; }
-    if (it == 0 && rel_tol > 1e-15 && 10.0 * (dmax / xmax) * dmax <= tol) { ++it; break; }
-    if (it >= 1) {
-      double rho = prev > 0.0 ? dmax / prev : 1.0;
-      if (rho < 0.5 && rho * dmax <= tol) { ++it; break; }
-    }
-    prev = dmax;
-    if (it == 11 && tid == 0) *fail = 1;
-    scs2_residual_update(w, p, n1, offp, offa, rbase, q, sm);
-    __syncthreads();
-    for (int e = tid; e < 3 * N1; e += blockDim.x) sm.y[e] = (float)sm.rhs[e];
-    __syncthreads();
-  }
-  return it;
 }
 
 // Radial terms of T_SR (see lmbd_internal.cuh): A0 = g/r^3, B0 = (h~ - 3g)/r^5 and their
@@ -704,6 +328,13 @@ __global__ void __launch_bounds__(128) k_pair_radial(Work w, DevParams p) {
   if (a >= w.n_atoms) return;
   const int n1 = w.counts[a].n1;
   const long long ab = (long long)a * w.site_cap, base = w.off_k1[a];
+  // alpha_bar and 1/alpha_bar as float-float, for the solves
+  for (int q = threadIdx.x; q < p.nqs; q += blockDim.x) {
+    const double v = w.abar[(long long)a * p.nqs + q];
+    const ff f = ff_from_double(v), g = ff_from_double(1.0 / v);
+    w.abff[(long long)a * p.nqs + q] = make_float2(f.hi, f.lo);
+    w.iabff[(long long)a * p.nqs + q] = make_float2(g.hi, g.lo);
+  }
   for (int e = threadIdx.x; e < n1 * p.nqs; e += blockDim.x) {
     const int s = e / p.nqs, q = e % p.nqs;
     if (s == 0) continue;
@@ -726,60 +357,12 @@ __global__ void __launch_bounds__(128) k_pair_radial(Work w, DevParams p) {
   }
 }
 
-// ---------------------------------------------------------------------------------------
-// pieces shared by the Cholesky kernels and the LU fallback
-// ---------------------------------------------------------------------------------------
-// alpha_bar of every site at SCS frequency q, and 1/alpha_bar of the coupled sites
-__device__ __forceinline__ void scs2_load_abar(const Work& w, const DevParams& p, int c, int q, int n1, int n12, Scs2Smem& sm) {
-  const long long sbase = (long long)c * w.site_cap;
-  for (int s = threadIdx.x; s < n12; s += blockDim.x) {
-    int a = w.site_atom[sbase + s];
-    const double ab = w.abar[(long long)a * p.nqs + q];
-    sm.abf[s] = ff_from_double(ab);
-    if (s < n1) sm.iab[s] = 1.0 / ab;
-  }
-}
-
-// right-hand side d_i = 1 - sum_{j in K2} T_SR,ij alpha_bar_j (Eq. local_pol) in float-float
-// arithmetic on the FP32 pipe (fixed order, ~2^-46 relative), rounded to FP64; one thread per
-// (coupled site i, column c): column c of T_SR,ij is F A0 e_c + F B0 r r_c.  rhs is N1 x 3
-// row-major (row 3 i + alpha).  Needs the float-float radial terms of this frequency.
-__device__ __forceinline__ void scs2_build_rhs(const Work& w, const DevParams& p, int n1, long long offp,
-                                               long long rbase, int q, const ff* abf, double* rhs) {
-  for (int e = threadIdx.x; e < 3 * n1; e += blockDim.x) {
-    const int i = e / 3, c = e % 3;
-    ff a0 = ff_make(0.f, 0.f), a1 = a0, a2 = a0, ad = a0;
-    const int b = w.prow_k2[rbase + i], en = w.prow[rbase + i + 1];
-    for (int t = b; t < en; ++t) {
-      const long long pq = offp + t;
-      const int j = w.pr_ij[2 * pq + 1];
-      const float2* gf = w.pr_gff + 6 * pq;
-      const float2* rf = w.pr_rad_ff + 2 * (pq * p.nqs + q);
-      const ff rx = ff_make(gf[0].x, gf[0].y), ry = ff_make(gf[1].x, gf[1].y), rz = ff_make(gf[2].x, gf[2].y);
-      const ff rc = c == 0 ? rx : (c == 1 ? ry : rz);
-      const ff abj = abf[j];
-      ad = ff_fma(abj, ff_make(rf[0].x, rf[0].y), ad);
-      const ff wb = ff_mul(ff_mul(abj, ff_make(rf[1].x, rf[1].y)), rc);
-      a0 = ff_fma(wb, rx, a0);
-      a1 = ff_fma(wb, ry, a1);
-      a2 = ff_fma(wb, rz, a2);
-    }
-    if (c == 0) a0 = ff_add(a0, ad);
-    if (c == 1) a1 = ff_add(a1, ad);
-    if (c == 2) a2 = ff_add(a2, ad);
-    double* y = rhs + 9 * i;
-    y[c] = (c == 0 ? 1.0 : 0.0) - ff_to_double(a0);
-    y[3 + c] = (c == 1 ? 1.0 : 0.0) - ff_to_double(a1);
-    y[6 + c] = (c == 2 ? 1.0 : 0.0) - ff_to_double(a2);
-  }
-}
-
 // FP64 damped radial terms F A0, F B0 of pair pq at SCS frequency q (LU fallback): from the
 // atom-pair table, or evaluated when the pair has no table entry
 __device__ __forceinline__ void pair_rad64(const Work& w, const DevParams& p, int c, int q, long long pq, double& fa,
                                            double& fb) {
   const double* g = w.pr_geo + 8 * pq;
-  const int gi = w.pr_g[pq];
+  const int gi = w.pr_ga[pq].x;
   double A0, B0;
   if (gi >= 0) {
     const double* ra = w.rad_ab + 2 * ((long long)gi * p.nqs + q);
@@ -803,7 +386,7 @@ __device__ void scs2_build_rhs64(const Work& w, const DevParams& p, int c, int n
   for (int e = threadIdx.x; e < 3 * n1; e += blockDim.x) {
     const int i = e / 3, cc = e % 3;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, ad = 0.0;
-    const int b = w.prow_k2[rbase + i], en = w.prow[rbase + i + 1];
+    const int b = w.prow_k2[rbase + i], en = w.prow_k2[rbase + i + 1];
     for (int t = b; t < en; ++t) {
       const long long pq = offp + t;
       const int j = w.pr_ij[2 * pq + 1];
@@ -824,293 +407,876 @@ __device__ void scs2_build_rhs64(const Work& w, const DevParams& p, int c, int n
   }
 }
 
-// X (N1 x 3), alpha_K,i = Tr(X_i)/3 and alpha_I,c = alpha_K,0 of one (centre, frequency)
-__device__ __forceinline__ void scs2_store_solution(const Work& w, const DevParams& p, int c, int q, int n1, const double* x) {
-  const int N1 = 3 * n1;
-  const long long offk1 = w.off_k1[c];
-  double* X = w.xsol + offk1 * p.nqs * 9 + (long long)q * N1 * 3;
-  for (int e = threadIdx.x; e < N1 * 3; e += blockDim.x) X[e] = x[e];
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) {
-    double a = (x[9 * i + 0] + x[9 * i + 4] + x[9 * i + 8]) / 3.0;
-    w.alphaK[(offk1 + i) * p.nqs + q] = a;
-    if (i == 0) w.alphaI[(long long)c * p.nqs + q] = a;
+// ---------------------------------------------------------------------------------------
+// local screening solves: conjugate gradients in FP32 inside a float-float refinement
+// ---------------------------------------------------------------------------------------
+// The scaled matrix A^(1/2) B A^(1/2), A = diag(alpha_bar), is I plus the damped dipole coupling:
+// its eigenvalues lie in about [0.3, 1.9] at the benchmark density (and tend to 1 at high
+// frequency), so conjugate gradients gain a digit in two to three steps: 13 steps to 2e-6 at
+// omega = 0, 2 at the highest node.
+//
+// A thread owns one site: a system is S = 1..3 warps (NC = 3: all three right-hand sides per thread), or three such
+// groups (NC = 1: a right-hand side each, independent until the end).  The only large array is the
+// packed triangle of pair couplings (11 KB at |K1| = 52 where a packed factor took 49 KB): twelve
+// or more systems per SM instead of two or three.
+//
+// The product B p is dense over the sites: for each partner j its position and p_j are broadcast
+// from shared memory (three 16-byte loads, one wavefront each) and a thread reads the scalar
+// couplings of its own site from the triangle without bank conflicts (triangular numbers run
+// through all residues).  The sparse form (a gather of p_j by adjacency) needs half the FMAs but
+// about thirty shared-memory wavefronts per entry.
+//
+// An FP32 Cholesky factor per system (block-wide, 16-wide blocks, in shared memory) took 32.5 ms
+// forward and 22.8 ms for the adjoint solves and their contraction per 4096-atom step, at 40 % of
+// the issue slots (two block barriers per block column, serial substitutions, two or three
+// systems per SM); this kernel takes 14.0 + 7.7 ms and k_scs_contract 4.1 ms.  It is bound by the
+// FP32 issue rate and the latency of the pair loads in the float-float residuals (60 % of the
+// issue slots).  A warp per system with packed FP32 pairs (fma.rn.f32x2) measured 17.4 + 10.5 ms:
+// the pairs cost as many moves as they save, with half the warps.  A system whose condition number
+// is above about 10^3 needs more steps than a factor would cost; beyond CG_MAXIT it goes to LU.
+#define CG_MAXIT 250          // steps of one inner solve; systems that need more go to LU
+#define CG_OUTER 12           // refinement steps
+
+// What every thread reads of a partner site: position (bohr) and the search direction or correction
+// p of the three columns.
+struct CgSite {
+  float4 a;   // x, y, z, p[2][2]
+  float4 b;   // p[0][0..2], p[1][0]
+  float4 c;   // p[1][1..2], p[2][0..1]
+};
+struct CgSmem {
+  CgSite* site;
+  float2* F;      // packed lower triangle with diagonal: scaled F A0, F B0 of the pair (1, 0 on it)
+  float* s;       // sqrt(alpha_bar)
+  float* part;    // 4 x 3 x 3 partial sums of the warps of a group
+};
+__host__ __device__ inline size_t cg_smem_bytes(int ld) {
+  return (size_t)ld * (sizeof(CgSite) + sizeof(float)) + (size_t)ld * (ld + 1) / 2 * sizeof(float2) + 36 * sizeof(float);
+}
+__device__ inline CgSmem cg_carve(unsigned char* base, int ld) {
+  CgSmem s;
+  s.site = reinterpret_cast<CgSite*>(base);
+  s.F = reinterpret_cast<float2*>(s.site + ld);
+  s.s = reinterpret_cast<float*>(s.F + ld * (ld + 1) / 2);
+  s.part = s.s + ld;
+  return s;
+}
+// component a of column c in a site record, and the same as an address (c, a may be run-time)
+__device__ __forceinline__ float* cg_slot(CgSite& t, int c, int a) {
+  return reinterpret_cast<float*>(&t) + (3 * c + a == 8 ? 3 : 4 + 3 * c + a);
+}
+
+// The S warps that share a system's columns: synchronisation, sums and maxima over them.
+template <int S>
+struct CgGroup {
+  int id, warp;   // group (NC = 1: the column), warp within it
+  __device__ __forceinline__ void sync() const {
+    if (S == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + id), "n"(32 * S) : "memory");
+  }
+  // slot: one of four partial-sum areas; the same one may be used again after one more sync()
+  template <int NC>
+  __device__ __forceinline__ void sum(float (&v)[NC], const CgSmem& sm, int slot) const {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+    if (S == 1) return;
+    float* part = sm.part + 9 * slot;
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) part[3 * (id + c) + warp] = v[c];
+    sync();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      v[c] = part[3 * (id + c)];
+#pragma unroll
+      for (int k = 1; k < S; ++k) v[c] += part[3 * (id + c) + k];
+    }
+  }
+  template <int NC>
+  __device__ __forceinline__ void max(float (&v)[NC], const CgSmem& sm, int slot) const {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[c] = fmaxf(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
+    if (S == 1) return;
+    float* part = sm.part + 9 * slot;
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) part[3 * (id + c) + warp] = v[c];
+    sync();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int k = 0; k < S; ++k) v[c] = fmaxf(v[c], part[3 * (id + c) + k]);
+  }
+};
+
+// (I + scaled coupling) x = r by conjugate gradients from x = 0 for the NC columns of a group; the
+// thread holds the rows of its site i (r = 0 past the last site).  Each column is scaled by a
+// power of two to unit size first (its squares stay in range) and stops when its residual has
+// fallen by tol.  Returns false (uniformly) when a direction of non-positive curvature shows up
+// (matrix not positive definite), on a non-finite value or after CG_MAXIT steps.
+template <int S, int NC>
+__device__ bool cg_solve(const CgSmem& sm, const CgGroup<S>& grp, int n1, int site, int c0, float tol,
+                         float (&r)[NC][3], float (&x)[NC][3]) {
+  const bool act = site < n1;
+  const int i = act ? site : n1 - 1;
+  const float4 own = sm.site[i].a;
+  float p[NC][3], rr[NC], thr[NC], unit[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) unit[c] = fmaxf(fabsf(r[c][0]), fmaxf(fabsf(r[c][1]), fabsf(r[c][2])));
+  grp.template max<NC>(unit, sm, 0);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    // 2^-e with the largest entry in [2^e, 2^(e+1)), from its biased exponent (0 for a zero column)
+    const int eb = min(max((__float_as_int(unit[c]) >> 23) & 0xff, 1), 253);
+    unit[c] = __int_as_float(eb << 23);
+    const float down = __int_as_float((254 - eb) << 23);
+    rr[c] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      p[c][a] = r[c][a] = r[c][a] * down;
+      x[c][a] = 0.f;
+      rr[c] += r[c][a] * r[c][a];
+    }
+  }
+  grp.template sum<NC>(rr, sm, 1);
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    thr[c] = tol * tol * rr[c];
+    ok = ok && rr[c] < 3e38f;   // also false for NaN
+  }
+  for (int it = 0; ok; ++it) {
+    bool more = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) more = more || rr[c] > thr[c];
+    if (!more) break;
+    if (it == CG_MAXIT) return false;
+    // every thread of the group is past the product of the step before (its sums synchronise)
+    if (S == 1) __syncwarp();
+    if (act) {
+      if (NC == 3) {
+        sm.site[i].a.w = p[2 % NC][2];
+        sm.site[i].b = make_float4(p[0][0], p[0][1], p[0][2], p[1 % NC][0]);
+        sm.site[i].c = make_float4(p[1 % NC][1], p[1 % NC][2], p[2 % NC][0], p[2 % NC][1]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) *cg_slot(sm.site[i], c0, a) = p[0][a];
+      }
+    }
+    grp.sync();
+    float q[NC][3];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) q[c][0] = q[c][1] = q[c][2] = 0.f;
+    // q += (3 x 3 coupling of the pair) p_j
+    auto partner = [&](int j, const float2 f) {
+      CgSite& t = sm.site[j];
+      const float4 ta = t.a;
+      float pj[NC][3];
+      if (NC == 3) {
+        const float4 tb = t.b, tc = t.c;
+        pj[0][0] = tb.x; pj[0][1] = tb.y; pj[0][2] = tb.z;
+        pj[1 % NC][0] = tb.w; pj[1 % NC][1] = tc.x; pj[1 % NC][2] = tc.y;
+        pj[2 % NC][0] = tc.z; pj[2 % NC][1] = tc.w; pj[2 % NC][2] = ta.w;
+      } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) pj[0][a] = *cg_slot(t, c0, a);
+      }
+      const float dx = ta.x - own.x, dy = ta.y - own.y, dz = ta.z - own.z;
+      const float ux = f.y * dx, uy = f.y * dy, uz = f.y * dz;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const float u = fmaf(dz, pj[c][2], fmaf(dy, pj[c][1], dx * pj[c][0]));
+        q[c][0] = fmaf(ux, u, fmaf(f.x, pj[c][0], q[c][0]));
+        q[c][1] = fmaf(uy, u, fmaf(f.x, pj[c][1], q[c][1]));
+        q[c][2] = fmaf(uz, u, fmaf(f.x, pj[c][2], q[c][2]));
+      }
+    };
+    // the row of site i in the triangle is contiguous up to j = i, then the column steps by j + 1;
+    // only the 32 partners around the warp's own sites need the choice
+    const int row = i * (i + 1) / 2, lo = S == 1 ? 0 : min(32 * grp.warp, n1), hi = S == 1 ? n1 : min(lo + 32, n1);
+    int j = 0;
+    if (S > 1)
+#pragma unroll 4
+      for (; j < lo; ++j) partner(j, sm.F[row + j]);
+    int col = j * (j + 1) / 2 + i;
+#pragma unroll 4
+    for (; j < hi; ++j) {
+      partner(j, sm.F[j <= i ? row + j : col]);
+      col += j + 1;
+    }
+    if (S > 1)
+#pragma unroll 4
+      for (; j < n1; ++j) {
+        partner(j, sm.F[col]);
+        col += j + 1;
+      }
+    float pq[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) q[c][a] = act ? q[c][a] : 0.f;
+      pq[c] = p[c][0] * q[c][0] + p[c][1] * q[c][1] + p[c][2] * q[c][2];
+    }
+    grp.template sum<NC>(pq, sm, 2);
+    float rn[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const bool go = rr[c] > thr[c];
+      if (go && !(pq[c] > 0.f)) ok = false;
+      const float al = go ? rr[c] / pq[c] : 0.f;
+      rn[c] = 0.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        x[c][a] += al * p[c][a];
+        r[c][a] -= al * q[c][a];
+        rn[c] += r[c][a] * r[c][a];
+      }
+    }
+    if (!ok) return false;
+    grp.template sum<NC>(rn, sm, 3);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const bool go = rr[c] > thr[c];
+      const float be = go ? rn[c] / rr[c] : 0.f;
+      if (go) rr[c] = rn[c];
+      ok = ok && rr[c] < 3e38f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) p[c][a] = r[c][a] + be * p[c][a];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) x[c][a] *= unit[c];
+  return ok;
+}
+
+// R <- R - B y for the FP32 vector y = p of the site records (the group's columns), in float-float arithmetic on the
+// FP32 pipe: F A0 y_j + F B0 r (r . y_j) over the adjacency row of every coupled site, error-free
+// products and compensated sums (ff.cuh), 1/alpha_bar on the diagonal.  Called with the FP32
+// solution it leaves the residual with an error ~2^-46 |B||x|, called with a correction it
+// carries the residual on.  Two lanes per (site, column), each half of the row; the halves are
+// combined in a fixed order.
+template <int S, int NC>
+__device__ void cg_residual_update(const Work& w, const DevParams& p, int c, int q, int n1, int c0, int nk1, int gt,
+                                   const CgSmem& sm, double* R) {
+  const long long offp = w.off_p[c], offa = w.off_a[c], rbase = w.off_k1[c] + c, sbase = (long long)c * w.site_cap;
+  const float4* rad = w.pr_rad4 + offp * p.nqs + (long long)q * nk1;
+  const int items = 2 * NC * n1;   // item e: half e % 2 of (site, column)
+  for (int base = 0; base < items; base += 32 * S) {
+    const int e = base + gt;
+    const bool on = e < items;
+    const int half = e & 1, cc = c0 + (NC == 1 ? 0 : (e >> 1) % NC), i = on ? (e >> 1) / NC : 0;
+    float h0 = 0.f, h1 = 0.f, h2 = 0.f, l0 = 0.f, l1 = 0.f, l2 = 0.f;
+    if (on) {
+      if (half == 0) {
+        const float2 ab = w.iabff[(long long)w.site_atom[sbase + i] * p.nqs + q];
+        const ff ia = ff_make(ab.x, ab.y);
+        const ff a = ff_scale(ia, *cg_slot(sm.site[i], cc, 0)), b = ff_scale(ia, *cg_slot(sm.site[i], cc, 1)),
+                 d = ff_scale(ia, *cg_slot(sm.site[i], cc, 2));
+        h0 = a.hi; l0 = a.lo; h1 = b.hi; l1 = b.lo; h2 = d.hi; l2 = d.lo;
+      }
+      const int b0 = w.arow[rbase + i], e0 = w.arow[rbase + i + 1];
+      const int mid = b0 + (e0 - b0 + 1) / 2;
+      const int tb = half == 0 ? b0 : mid, te = half == 0 ? mid : e0;
+      // the loads of an entry depend on its index pair: the indices run two entries ahead and the
+      // data one entry ahead of the arithmetic
+      const int2* ap = reinterpret_cast<const int2*>(w.adj) + offa;
+      const float4* gp = reinterpret_cast<const float4*>(w.pr_gff) + 3 * offp;
+      int2 ad = make_int2(0, 0), an = ad;
+      float4 n0, n1v, nf;
+      if (tb < te) {
+        an = __ldg(ap + tb);
+        n0 = __ldg(gp + 3 * an.y); n1v = __ldg(gp + 3 * an.y + 1); nf = rad[an.y];
+        ad = __ldg(ap + min(tb + 1, te - 1));
+      }
+      for (int t = tb; t < te; ++t) {
+        const float4 g0 = n0, g1 = n1v, f = nf;     // rx, ry | rz, F (hi, lo each) | F A0, F B0
+        CgSite& sj = sm.site[an.x];
+        const float3 d = make_float3(*cg_slot(sj, cc, 0), *cg_slot(sj, cc, 1), *cg_slot(sj, cc, 2));
+        an = ad;
+        n0 = __ldg(gp + 3 * an.y); n1v = __ldg(gp + 3 * an.y + 1); nf = rad[an.y];
+        ad = __ldg(ap + min(t + 2, te - 1));
+        // s = r . y
+        const float p0 = __fmul_rn(g0.x, d.x), p1 = __fmul_rn(g0.z, d.y), p2 = __fmul_rn(g1.x, d.z);
+        float s0 = __fmaf_rn(g0.y, d.x, __fmaf_rn(g0.x, d.x, -p0));
+        const float s1 = __fmaf_rn(g0.w, d.y, __fmaf_rn(g0.z, d.y, -p1));
+        const float s2 = __fmaf_rn(g1.y, d.z, __fmaf_rn(g1.x, d.z, -p2));
+        const ff a = ff_two_sum(p0, p1), b = ff_two_sum(a.hi, p2);
+        s0 = __fadd_rn(__fadd_rn(s0, s1), __fadd_rn(s2, __fadd_rn(a.lo, b.lo)));
+        const ff s = ff_quick_two_sum(b.hi, s0);
+        // u = F B0 s
+        const float uh = __fmul_rn(f.z, s.hi);
+        const float ul = __fmaf_rn(f.w, s.hi, __fmaf_rn(f.z, s.lo, __fmaf_rn(f.z, s.hi, -uh)));
+        auto add = [&](float& h, float& l, float dk, float rh, float rl) {
+          const float v = __fmul_rn(f.x, dk);
+          const float ve = __fmaf_rn(f.y, dk, __fmaf_rn(f.x, dk, -v));
+          const float z = __fmul_rn(uh, rh);
+          const float ze = __fmaf_rn(ul, rh, __fmaf_rn(uh, rl, __fmaf_rn(uh, rh, -z)));
+          const ff m = ff_two_sum(h, v), n = ff_two_sum(m.hi, z);
+          h = n.hi;
+          l = __fadd_rn(l, __fadd_rn(__fadd_rn(m.lo, n.lo), __fadd_rn(ve, ze)));
+        };
+        add(h0, l0, d.x, g0.x, g0.y);
+        add(h1, l1, d.y, g0.z, g0.w);
+        add(h2, l2, d.z, g1.x, g1.y);
+      }
+    }
+    const ff o0 = ff_make(__shfl_xor_sync(0xffffffffu, h0, 1), __shfl_xor_sync(0xffffffffu, l0, 1));
+    const ff o1 = ff_make(__shfl_xor_sync(0xffffffffu, h1, 1), __shfl_xor_sync(0xffffffffu, l1, 1));
+    const ff o2 = ff_make(__shfl_xor_sync(0xffffffffu, h2, 1), __shfl_xor_sync(0xffffffffu, l2, 1));
+    if (on && half == 0) {
+      double* Ri = R + 9 * i + cc;
+      Ri[0] -= ff_to_double(ff_add(ff_quick_two_sum(h0, l0), ff_quick_two_sum(o0.hi, o0.lo)));
+      Ri[3] -= ff_to_double(ff_add(ff_quick_two_sum(h1, l1), ff_quick_two_sum(o1.hi, o1.lo)));
+      Ri[6] -= ff_to_double(ff_add(ff_quick_two_sum(h2, l2), ff_quick_two_sum(o2.hi, o2.lo)));
+    }
   }
 }
 
-// ---------------------------------------------------------------------------------------
-// forward: one block per (central atom, frequency)
-// ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 3) k_scs_factor(Work w, DevParams p, const int* order, int c0, int max_n1,
-                                                  int max_n12) {
-  extern __shared__ unsigned char smem_raw[];
-  const int c = order ? order[c0 + blockIdx.x / p.nqs] : c0 + blockIdx.x / p.nqs;
-  const int q = blockIdx.x % p.nqs;
-  if (c >= w.n_atoms) return;
-  const Counts cn = w.counts[c];
-  const int n1 = cn.n1, n12 = cn.n12, N1 = 3 * n1;
-  Scs2Smem sm = scs2_carve(smem_raw, max_n1, max_n12, false);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  const long long sbase = (long long)c * w.site_cap;
-  const long long offp = w.off_p[c], offa = w.off_a[c], rbase = w.off_k1[c] + c;
-  const int np = w.prow[rbase + n1];
-  __shared__ int bad, fail;
-  if (tid == 0) { bad = 0; fail = 0; }
-  scs2_load_abar(w, p, c, q, n1, n12, sm);
-  const long long nA = (long long)N1 * (N1 + 1) / 2;
-  for (long long e = tid; e < nA; e += blockDim.x) sm.A[e] = 0.f;
-  __syncthreads();
-  // damped radial terms F A0, F B0 of every pair at this frequency in float-float (F times the
-  // atom-pair table entry, on the FP32 pipe), stored for the residuals and the adjoint, and the
-  // K1 blocks of B in FP32 (the factor needs FP32 values only)
-  for (int t = tid; t < np; t += blockDim.x) {
-    const long long pq = offp + t;
-    const int i = w.pr_ij[2 * pq], j = w.pr_ij[2 * pq + 1];
-    const int gi = w.pr_g[pq];
-    const float2* gf = w.pr_gff + 6 * pq;
-    ff fa, fb;
-    if (gi >= 0) {
-      const float2* ra = w.rad_ff + 4 * ((long long)gi * p.nqs + q);
-      const ff F = ff_make(gf[3].x, gf[3].y);
-      fa = ff_mul(F, ff_make(ra[0].x, ra[0].y));
-      fb = ff_mul(F, ff_make(ra[1].x, ra[1].y));
-    } else {   // no table entry (a distance that ties r_SCS to rounding): evaluate in FP64
-      double da, db;
-      pair_rad64(w, p, c, q, pq, da, db);
-      fa = ff_from_double(da);
-      fb = ff_from_double(db);
-    }
-    float2* rf = w.pr_rad_ff + 2 * (pq * p.nqs + q);
-    rf[0] = make_float2(fa.hi, fa.lo);
-    rf[1] = make_float2(fb.hi, fb.lo);
-    if (j < n1) {
-      const float rr[3] = {gf[0].x, gf[1].x, gf[2].x};
-#pragma unroll
-      for (int al = 0; al < 3; ++al) {
-        float* row = sm.A + packed_idx(3 * i + al, 3 * j);
-#pragma unroll
-        for (int be = 0; be < 3; ++be) row[be] = fb.hi * rr[al] * rr[be] + (al == be ? fa.hi : 0.f);
+// Compensated accumulation of the product a b (float-float operands) into (h, l).
+__device__ __forceinline__ void ff_mac(float& h, float& l, ff a, ff b) {
+  const float v = __fmul_rn(a.hi, b.hi);
+  const float e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -v)));
+  const ff m = ff_two_sum(h, v);
+  h = m.hi;
+  l = __fadd_rn(l, __fadd_rn(m.lo, e));
+}
+
+// Damped radial terms F A0, F B0 of pair t (of centre c) at SCS frequency q in float-float: F times
+// the atom-pair table entry, on the FP32 pipe.
+__device__ __noinline__ void pair_rad_slow(const Work& w, const DevParams& p, int c, int q, long long pq, ff& fa,
+                                           ff& fb) {
+  double da, db;   // no table entry (a distance that ties r_SCS to rounding): evaluate in FP64
+  pair_rad64(w, p, c, q, pq, da, db);
+  fa = ff_from_double(da);
+  fb = ff_from_double(db);
+}
+// the table row of entry gi at frequency q: A0, B0 (row 0 where there is no entry)
+__device__ __forceinline__ float4 rad_row(const Work& w, const DevParams& p, int gi, int q) {
+  return __ldg(reinterpret_cast<const float4*>(w.rad_ff + 4 * ((long long)max(gi, 0) * p.nqs + q)));
+}
+__device__ __forceinline__ void pair_rad_ff(const Work& w, const DevParams& p, int c, int q, long long pq, int gi,
+                                            float4 ra, ff F, ff& fa, ff& fb) {
+  if (gi >= 0) {
+    fa = ff_mul(F, ff_make(ra.x, ra.y));
+    fb = ff_mul(F, ff_make(ra.z, ra.w));
+  } else {
+    pair_rad_slow(w, p, c, q, pq, fa, fb);
+  }
+}
+
+// Right-hand side d_i = 1 - sum_{j in K2} T_SR,ij alpha_bar_j (Eq. local_pol) into R: float-float
+// sums (fixed order) of the six distinct entries of the symmetric block, four lanes per site.
+__device__ void cg_build_rhs(const Work& w, const DevParams& p, int c, int q, int n1, double* R) {
+  const long long offp = w.off_p[c], rbase = w.off_k1[c] + c;
+  for (int base = 0; base < 4 * n1; base += blockDim.x) {
+    const int e = base + threadIdx.x, i = e >> 2;
+    const bool on = i < n1;
+    float h[7] = {}, l[7] = {};   // xx, yy, zz, xy, xz, yz of F B0 alpha_bar r r^T, then F A0 alpha_bar
+    if (on) {
+      const int tb = w.prow_k2[rbase + i] + (e & 3), en = w.prow_k2[rbase + i + 1];
+      // as in the residual: indices two pairs ahead, data one pair ahead
+      const float4* gp = reinterpret_cast<const float4*>(w.pr_gff) + 3 * offp;
+      int2 gn = make_int2(-1, 0), ga = gn;
+      float4 n0, n1v, nr;
+      float2 na;
+      if (tb < en) {
+        gn = __ldg(w.pr_ga + offp + tb);
+        n0 = __ldg(gp + 3 * tb); n1v = __ldg(gp + 3 * tb + 1);
+        nr = rad_row(w, p, gn.x, q);
+        na = __ldg(w.abff + (long long)gn.y * p.nqs + q);
+        ga = __ldg(w.pr_ga + offp + min(tb + 4, en - 1));
+      }
+      for (int t = tb; t < en; t += 4) {
+        const float4 g0 = n0, g1 = n1v, ra = nr;
+        const float2 ab = na;
+        const int gi = gn.x, tn = min(t + 4, en - 1);
+        gn = ga;
+        n0 = __ldg(gp + 3 * tn); n1v = __ldg(gp + 3 * tn + 1);
+        nr = rad_row(w, p, gn.x, q);
+        na = __ldg(w.abff + (long long)gn.y * p.nqs + q);
+        ga = __ldg(w.pr_ga + offp + min(t + 8, en - 1));
+        ff fa, fb;
+        pair_rad_ff(w, p, c, q, offp + t, gi, ra, ff_make(g1.z, g1.w), fa, fb);
+        const ff aj = ff_make(ab.x, ab.y);
+        const ff rx = ff_make(g0.x, g0.y), ry = ff_make(g0.z, g0.w), rz = ff_make(g1.x, g1.y);
+        const ff wb = ff_mul(aj, fb);
+        const ff ux = ff_mul(wb, rx), uy = ff_mul(wb, ry), uz = ff_mul(wb, rz);
+        ff_mac(h[0], l[0], ux, rx);
+        ff_mac(h[1], l[1], uy, ry);
+        ff_mac(h[2], l[2], uz, rz);
+        ff_mac(h[3], l[3], ux, ry);
+        ff_mac(h[4], l[4], ux, rz);
+        ff_mac(h[5], l[5], uy, rz);
+        ff_mac(h[6], l[6], aj, fa);
       }
     }
-  }
-  for (int i = tid; i < n1; i += blockDim.x)
+    ff s[7];
 #pragma unroll
-    for (int al = 0; al < 3; ++al) sm.A[packed_idx(3 * i + al, 3 * i + al)] = (float)sm.iab[i];
+    for (int u = 0; u < 7; ++u) {
+      s[u] = ff_quick_two_sum(h[u], l[u]);
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1)
+        s[u] = ff_add(s[u], ff_make(__shfl_xor_sync(0xffffffffu, s[u].hi, o), __shfl_xor_sync(0xffffffffu, s[u].lo, o)));
+    }
+    if (on && (e & 3) == 0) {
+      double v[6];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) v[u] = 1.0 - ff_to_double(ff_add(s[u], s[6]));
+#pragma unroll
+      for (int u = 3; u < 6; ++u) v[u] = -ff_to_double(s[u]);
+      double* Ri = R + 9 * i;
+      Ri[0] = v[0]; Ri[1] = Ri[3] = v[3]; Ri[2] = Ri[6] = v[4];
+      Ri[4] = v[1]; Ri[5] = Ri[7] = v[5]; Ri[8] = v[2];
+    }
+  }
+}
+
+// Systems on the LU list: forward ones and, should the adjoint solve of a system stall, that one.
+__device__ __forceinline__ void scs_list_for_lu(const Work& w, int id) {
+  w.fb_flag[id] = 1;
+  const int e = atomicAdd(w.fb, 1);
+  w.fb[1 + e] = id;
+}
+
+// One (centre, frequency) system per block of 32 S (3 / NC) threads.  ADJ = false: X = B^-1 d to FP64
+// accuracy (2^-52), alpha_K and alpha_I.  ADJ = true: lambda = B^-1 dL/dX, to 2^-30 of its largest
+// value or better (it feeds the forces only).  The refinement measures its own contraction.
+constexpr int cg_min_blocks(int S, int NC) { return NC == 1 ? (S == 1 ? 7 : (S == 2 ? 4 : 2)) : (S == 1 ? 20 : (S == 2 ? 12 : 5)); }
+template <int S, int NC, bool ADJ>
+__global__ void __launch_bounds__(32 * S * (3 / NC), cg_min_blocks(S, NC))
+    k_scs_solve(Work w, DevParams p, const int* order, int b0, int ld) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int c = order ? order[b0 + blockIdx.x / p.nqs] : b0 + blockIdx.x / p.nqs;
+  const int q = blockIdx.x % p.nqs;
+  if (c >= w.n_atoms) return;
+  const int id = c * p.nqs + q;
+  if (ADJ && w.fb_flag[id]) return;   // solved by the LU fallback (k_scs_lu_adjoint)
+  const int n1 = w.counts[c].n1;
+  const CgSmem sm = cg_carve(smem_raw, ld);
+  const int tid = threadIdx.x, gt = tid % (32 * S);   // thread within its group
+  const CgGroup<S> grp{tid / (32 * S), gt >> 5};
+  const int c0 = grp.id;
+  const long long sbase = (long long)c * w.site_cap, offk1 = w.off_k1[c];
+  const long long offp = w.off_p[c], rbase = offk1 + c;
+  const int nk1 = w.prow[rbase + n1];
+  float4* rad = w.pr_rad4 + offp * p.nqs + (long long)q * nk1;
+  // the system's slot of the solution array holds its FP64 residual until the solution is known
+  double* R = (ADJ ? w.lsol : w.xsol) + offk1 * p.nqs * 9 + (long long)q * n1 * 9;
+  for (int s = tid; s < n1; s += blockDim.x) {
+    const double* x = w.site_x + 3 * (sbase + s);
+    const float ab = w.abff[(long long)w.site_atom[sbase + s] * p.nqs + q].x;
+    const float fx = (float)x[0], fy = (float)x[1], fz = (float)x[2];
+    sm.site[s].a = make_float4(fx, fy, fz, 0.f);
+    sm.s[s] = sqrtf(ab);
+  }
+  for (int e = tid; e < n1 * (n1 + 1) / 2; e += blockDim.x) sm.F[e] = make_float2(0.f, 0.f);
+  __syncthreads();
+  for (int s = tid; s < n1; s += blockDim.x) sm.F[s * (s + 1) / 2 + s] = make_float2(1.f, 0.f);
+#pragma unroll 2
+  for (int t = tid; t < nk1; t += blockDim.x) {
+    const int2 ij = __ldg(reinterpret_cast<const int2*>(w.pr_ij) + offp + t);
+    float4 f;
+    if (ADJ) {
+      f = __ldg(rad + t);
+    } else {
+      const int gi = __ldg(w.pr_ga + offp + t).x;
+      const float4 g1 = __ldg(reinterpret_cast<const float4*>(w.pr_gff + 6 * (offp + t)) + 1);
+      ff fa, fb;
+      pair_rad_ff(w, p, c, q, offp + t, gi, rad_row(w, p, gi, q), ff_make(g1.z, g1.w), fa, fb);
+      f = make_float4(fa.hi, fa.lo, fb.hi, fb.lo);
+      rad[t] = f;
+    }
+    const float s = sm.s[ij.x] * sm.s[ij.y];
+    sm.F[ij.x * (ij.x + 1) / 2 + ij.y] = make_float2(f.x * s, f.z * s);
+  }
+  double scale = 1.0;
+  if (!ADJ) {
+    cg_build_rhs(w, p, c, q, n1, R);
+  } else {
+    // dL/dX_i = delta/3 times dL/dalpha_K,i, plus dL/dalpha_I,c on the centre's block, scaled by
+    // a power of two to unit size (the weights of a caller may be of any magnitude)
+    double gv = 0.0;
+    int top = 0;
+    for (int i = tid & 31; i < n1; i += 32) {   // every warp finds the largest exponent of all sites
+      double v = w.alphaK_bar[(offk1 + i) * p.nqs + q];
+      if (i == 0) v += w.alphaI_bar[id];
+      v *= 1.0 / 3.0;
+      if (i == gt) gv = v;
+      top = max(top, (int)((__double_as_longlong(v) >> 52) & 0x7ff));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (top == 0x7ff) {   // not finite: no solution (uniform over the block)
+      if (tid == 0) atomicOr(w.status, LMBD_FLAG_NOT_CONVERGED);
+      return;
+    }
+    top = min(max(top, 1), 2045);
+    const double up = __longlong_as_double((long long)(2046 - top) << 52);
+    scale = __longlong_as_double((long long)top << 52);
+    if (gt < n1)
+#pragma unroll
+      for (int k = 0; k < NC; ++k)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) R[9 * gt + 3 * a + c0 + k] = a == c0 + k ? gv * up : 0.0;
+  }
   __threadfence_block();
   __syncthreads();
-  scs2_build_rhs(w, p, n1, offp, rbase, q, sm.abf, sm.rhs);
-  __syncthreads();
-  chol32_packed(sm.A, N1, &bad, sm.sinv, sm.binv);
-  // a non-positive pivot (B_K not positive definite: Sec. III.A, polarisation catastrophe) or
-  // a refinement that does not converge sends the system to the LU fallback (k_scs_lu_forward)
-  if (!bad) scs2_refine(w, p, n1, offp, offa, rbase, q, sm, &fail, 2.220446049250313e-16);
-  __syncthreads();
-  if (bad || fail) {
-    if (tid == 0) {
-      w.fb_flag[(long long)c * p.nqs + q] = 1;
-      const int e = atomicAdd(w.fb, 1);
-      w.fb[1 + e] = c * p.nqs + q;
+
+  const float rel = ADJ ? 9.313225746154785e-10f : 2.220446049250313e-16f;
+  const float inner = ADJ ? 1e-6f : 2e-6f;
+  const bool act = gt < n1;
+  const float si = act ? sm.s[gt] : 0.f;
+  double* const Ri = R + 9 * (act ? gt : 0);
+  double xd[NC][3];
+#pragma unroll
+  for (int k = 0; k < NC; ++k)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) xd[k][a] = 0.0;
+  float lim = 0.f, prev = 0.f, tol = inner;
+  bool ok = true;
+  for (int it = 0;; ++it) {
+    float r[NC][3], x[NC][3], dm[1] = {0.f};
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) r[k][a] = si * (float)Ri[3 * a + c0 + k];
+    ok = cg_solve<S, NC>(sm, grp, n1, gt, c0, tol, r, x);
+    if (!ok) break;
+    grp.sync();
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        x[k][a] *= si;
+        xd[k][a] += (double)x[k][a];
+        dm[0] = fmaxf(dm[0], fabsf(x[k][a]));
+        if (act) *cg_slot(sm.site[gt], c0 + k, a) = x[k][a];
+      }
+    grp.template max<1>(dm, sm, 2);
+    const float dmax = dm[0];
+    // contraction estimate rho = |delta_k| / |delta_{k-1}| (delta_0 = the FP32 solution): the error
+    // left after correction k is about rho |delta_k|, or tol |delta_k| where its solve was looser
+    const float rho = it > 0 ? dmax / prev : 0.f;
+    if (it == 0) {
+      lim = rel * dmax;
+      if (dmax == 0.f) break;
+    } else {
+      if (dmax <= lim) break;
+      if (ADJ && 10.f * rho * dmax <= lim && it == 1) break;
+      if (it >= 2 && rho < 0.5f && fmaxf(rho, tol) * dmax <= lim) break;
+      if (it == CG_OUTER) { ok = false; break; }
+      // the next correction (about rho dmax) only needs the digits down to the limit
+      if (!ADJ) tol = fminf(fmaxf(0.25f * lim / (rho * dmax), inner), 1e-2f);
     }
+    prev = dmax;
+    grp.sync();
+    cg_residual_update<S, NC>(w, p, c, q, n1, c0, nk1, gt, sm, R);
+    grp.sync();
+  }
+  // a direction of non-positive curvature (B_K not positive definite: Sec. III.A, polarisation
+  // catastrophe) or a refinement that does not converge sends the system to the LU fallback
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) scs_list_for_lu(w, id);
     return;
   }
-  if (tid == 0) w.fb_flag[(long long)c * p.nqs + q] = 0;
-  // outputs: X, alpha_K, alpha_I and the FP32 factor for the adjoint
-  scs2_store_solution(w, p, c, q, n1, sm.x);
-  float* Lg = w.lfac + w.off_b[c] + (long long)q * nA;
-  for (long long e = tid; e < nA; e += blockDim.x) Lg[e] = sm.A[e];
-  // the inverses of the diagonal blocks as well, so that the adjoint need not form them again
-  float* Bg = w.binvg + ((long long)c * p.nqs + q) * w.binv_slot;
-  for (int e = tid; e < (N1 + CB - 1) / CB * CBP; e += blockDim.x) Bg[e] = sm.binv[e];
-}
-
-// Adjoint right-hand side dL/dX of one (centre, frequency) into sm.rhs (dL/dX_i = delta/3 times
-// dL/dalpha_K,i, plus dL/dalpha_I,c on the centre's block), and the forward solution X into sm.xs.
-__device__ __forceinline__ void scs2_load_adjoint_rhs(const Work& w, const DevParams& p, int c, int q, int n1, Scs2Smem& sm) {
-  const int N1 = 3 * n1;
-  const long long offk1 = w.off_k1[c];
-  const double* X = w.xsol + offk1 * p.nqs * 9 + (long long)q * N1 * 3;
-  for (int e = threadIdx.x; e < N1 * 3; e += blockDim.x) {
-    sm.xs[e] = X[e];
-    int row = e / 3, col = e % 3, i = row / 3, al = row % 3;
-    double gval = 0.0;
-    if (al == col) {
-      gval = w.alphaK_bar[(offk1 + i) * p.nqs + q];
-      if (i == 0) gval += w.alphaI_bar[(long long)c * p.nqs + q];
-      gval *= (1.0 / 3.0);
+  if (!ADJ && tid == 0) w.fb_flag[id] = 0;
+  if (act)
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) Ri[3 * a + c0 + k] = ADJ ? xd[k][a] * scale : xd[k][a];
+  if (!ADJ) {   // alpha_K,i = Tr(X_i) / 3, alpha_I,c = alpha_K,0
+    __threadfence_block();
+    __syncthreads();
+    for (int i = tid; i < n1; i += blockDim.x) {
+      const double a = (R[9 * i] + R[9 * i + 4] + R[9 * i + 8]) / 3.0;
+      w.alphaK[(offk1 + i) * p.nqs + q] = a;
+      if (i == 0) w.alphaI[id] = a;
     }
-    sm.rhs[e] = gval;
   }
 }
 
-// Adjoint contraction of one (centre, frequency) given lambda = B^-1 dL/dX in sm.x and the
-// forward solution X in sm.xs (both N1 x 3, FP64): per pair <M, dT_SR/dr> with
-// M = -(lambda_i X_j^T + lambda_j X_i^T) (K1 pairs) or M = -alpha_bar_j lambda_i (K2 pairs),
-// symmetrised; g = dL/dr_j = -dL/dr_i per pair, staged in global scratch (L2-resident), then
-// summed per site in a fixed order.  The contraction runs in float-float arithmetic (ff.cuh,
-// ~2^-46 relative) on the FP32 pipe: lambda and X are converted once per site, geometry and
-// radial terms come converted from the tables.  sm.rhs and sm.xs are overwritten.
-__device__ __forceinline__ void scs2_adjoint_contract(const Work& w, const DevParams& p, int c, int q, int n1, int n12, Scs2Smem& sm) {
-  const int N1 = 3 * n1, tid = threadIdx.x;
+// ---------------------------------------------------------------------------------------
+// adjoint contraction: one block per central atom, all frequencies
+// ---------------------------------------------------------------------------------------
+// Per pair <M, dT_SR/dr> with M = -(lambda_i X_j^T + lambda_j X_i^T) (K1 pairs) or
+// M = -alpha_bar_j lambda_i (K2 pairs), symmetrised, T_SR = F (A0 + B0 r r^T):
+//   dL/dr_j = r [F dB0 r.M.r + F dA0 Tr M + dF (B0 r.M.r + A0 Tr M)] / |r| + 2 F B0 M r.
+// Geometry, F and dF do not depend on the frequency, so a thread runs its pair over all
+// frequencies, summing W = sum B0 M, W' = sum dB0 M (six entries each) and the scalars
+// sum A0 Tr M, sum dA0 Tr M, and applies geometry once; lambda and X of every frequency are staged
+// in shared memory as float-float (97 KB at |K1| = 52 and 13 frequencies, two blocks per SM).
+// Float-float throughout (compensated sums, ~2^-46): 4.1 ms per 4096-atom step, bound by its FP32
+// instructions; one block per (centre, frequency) with the gradients of each frequency staged in
+// global memory took about half of a 22.8 ms adjoint.
+// More frequencies than fit in shared memory are taken in chunks, the sums kept in `gstage`; small
+// structures split the frequencies of a centre over several blocks (the gradient is linear in the
+// sums, so each block finishes its own part).
+#define CON_W 14   // 6 + 6 + 2 float-float sums per pair
+
+__device__ __forceinline__ ff ff_ld(const float2* p) {
+  const float2 v = *p;
+  return ff_make(v.x, v.y);
+}
+
+struct ConSum {
+  float h[CON_W], l[CON_W];
+  __device__ __forceinline__ void add(const ff (&M)[6], ff A0, ff B0, ff dA0, ff dB0) {
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+      ff_mac(h[u], l[u], B0, M[u]);
+      ff_mac(h[6 + u], l[6 + u], dB0, M[u]);
+    }
+    const ff tr = ff_add(ff_add(M[0], M[1]), M[2]);
+    ff_mac(h[12], l[12], A0, tr);
+    ff_mac(h[13], l[13], dA0, tr);
+  }
+  __device__ __forceinline__ ff get(int u) const { return ff_quick_two_sum(h[u], l[u]); }
+};
+
+// A0, B0, dA0, dB0 of pair pq at frequency q (float-float)
+__device__ __noinline__ void pair_terms_slow(const Work& w, const DevParams& p, int c, int q, long long pq, ff& A0,
+                                             ff& B0, ff& dA0, ff& dB0) {
+  const long long sbase = (long long)c * w.site_cap;
+  const double* g = w.pr_geo + 8 * pq;
+  const double si = w.sig[(long long)w.site_atom[sbase + w.pr_ij[2 * pq]] * p.nqs + q];
+  const double sj = w.sig[(long long)w.site_atom[sbase + w.pr_ij[2 * pq + 1]] * p.nqs + q];
+  double a, b, da, db;
+  tsr_radial_fast(g[3], g[6], si * si + sj * sj, a, b, da, db);
+  A0 = ff_from_double(a); B0 = ff_from_double(b); dA0 = ff_from_double(da); dB0 = ff_from_double(db);
+}
+__device__ __forceinline__ void pair_terms(const Work& w, const DevParams& p, int c, int q, long long pq, int gi, float4 u,
+                                           float4 v, ff& A0, ff& B0, ff& dA0, ff& dB0) {
+  if (gi >= 0) {
+    A0 = ff_make(u.x, u.y); B0 = ff_make(u.z, u.w); dA0 = ff_make(v.x, v.y); dB0 = ff_make(v.z, v.w);
+  } else {
+    pair_terms_slow(w, p, c, q, pq, A0, B0, dA0, dB0);
+  }
+}
+
+// dL/dr_j of the pair from its frequency sums (W carries no minus sign and, for the off-diagonal
+// entries, both orders: the symmetrised M is half of them)
+__device__ __forceinline__ void con_finish(const Work& w, long long pq, const ConSum& S, ff (&g)[3]) {
+  const float4* gf = reinterpret_cast<const float4*>(w.pr_gff + 6 * pq);
+  const float4 g0 = gf[0], g1 = gf[1], g2 = gf[2];
+  const ff rr[3] = {ff_make(g0.x, g0.y), ff_make(g0.z, g0.w), ff_make(g1.x, g1.y)};
+  const ff F = ff_make(g1.z, g1.w), dF = ff_make(g2.x, g2.y), ir = ff_make(g2.z, g2.w);
+  ff V[3], rW[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const ff a = S.get(6 * k), b = S.get(6 * k + 1), d = S.get(6 * k + 2);
+    const ff xy = ff_scale(S.get(6 * k + 3), 0.5f), xz = ff_scale(S.get(6 * k + 4), 0.5f), yz = ff_scale(S.get(6 * k + 5), 0.5f);
+    const ff v0 = ff_fma(xz, rr[2], ff_fma(xy, rr[1], ff_mul(a, rr[0])));
+    const ff v1 = ff_fma(yz, rr[2], ff_fma(b, rr[1], ff_mul(xy, rr[0])));
+    const ff v2 = ff_fma(d, rr[2], ff_fma(yz, rr[1], ff_mul(xz, rr[0])));
+    rW[k] = ff_fma(rr[2], v2, ff_fma(rr[1], v1, ff_mul(rr[0], v0)));
+    if (k == 0) { V[0] = v0; V[1] = v1; V[2] = v2; }
+  }
+  const ff phi = ff_add(rW[0], S.get(12)), inner = ff_add(rW[1], S.get(13));
+  const ff radial = ff_mul(ff_fma(F, inner, ff_mul(dF, phi)), ir);
+  const ff tang = ff_scale(F, 2.0f);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) g[d] = ff_neg(ff_fma(tang, V[d], ff_mul(radial, rr[d])));
+}
+
+__global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, int c0, int nsplit, int smem, int scratch) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int c = c0 + blockIdx.x / nsplit, split = blockIdx.x % nsplit;
+  if (c >= w.n_atoms) return;
+  // this block's frequencies
+  const int per = (p.nqs + nsplit - 1) / nsplit, qb = split * per, qe = min(p.nqs, qb + per);
+  if (qb >= qe) return;
+  const int n1 = w.counts[c].n1, n12 = w.counts[c].n12, tid = threadIdx.x;
   const long long sbase = (long long)c * w.site_cap;
   const long long offp = w.off_p[c], offa = w.off_a[c], rbase = w.off_k1[c] + c;
-  const int np = w.prow[rbase + n1];
-  ff* lf = reinterpret_cast<ff*>(sm.rhs);   // lambda, 9 n1 (rhs is no longer needed)
-  ff* xf = reinterpret_cast<ff*>(sm.xs);    // X, 9 n1 (in place: one element per thread)
-  for (int e = tid; e < N1 * 3; e += blockDim.x) {
-    const double xv = sm.xs[e];
-    lf[e] = ff_from_double(sm.x[e]);
-    xf[e] = ff_from_double(xv);
-  }
-  __syncthreads();
-  // pair gradients as float-float (the per-site sums below stay on the FP32 pipe)
-  float2* gst = reinterpret_cast<float2*>(w.gstage) + (offp * p.nqs + (long long)q * np) * 3;
-  for (int t = tid; t < np; t += blockDim.x) {
-    const long long pq = offp + t;
-    const int i = w.pr_ij[2 * pq], j = w.pr_ij[2 * pq + 1];
-    const int gi = w.pr_g[pq];
-    const ff* li = lf + 9 * i;
-    ff M[6];
-    if (j < n1) {
-      const ff* lj = lf + 9 * j;
-      const ff* xi = xf + 9 * i;
-      const ff* xj = xf + 9 * j;
-      ff Mf[3][3];
+  const int nk1 = w.prow[rbase + n1], np = w.prow_k2[rbase + n1];
+  const double* Xg = w.xsol + w.off_k1[c] * p.nqs * 9;
+  const double* Lg = w.lsol + w.off_k1[c] * p.nqs * 9;
+  const int qc = max(1, min(per, smem / (144 * n1)));   // frequencies staged at once
+  float2* Ls = reinterpret_cast<float2*>(smem_raw);   // [qc][9 n1] lambda
+  float2* Xs = Ls + qc * 9 * n1;                      // [qc][9 n1] X
+  // gradient of each pair, then (frequencies in chunks) its CON_W sums of the chunks so far
+  float2* gst = w.gstage + (scratch / nsplit) * (offp * nsplit + (long long)split * np);
+  float2* sums = gst + 3LL * np;
+  for (int q0 = qb; q0 < qe; q0 += qc) {
+    const int nqc = min(qc, qe - q0);
+    const bool first = q0 == qb, last = q0 + nqc == qe;
+    __syncthreads();
+    for (int e = tid; e < nqc * 9 * n1; e += blockDim.x) {
+      const ff l = ff_from_double(Lg[(long long)q0 * 9 * n1 + e]), x = ff_from_double(Xg[(long long)q0 * 9 * n1 + e]);
+      Ls[e] = make_float2(l.hi, l.lo);
+      Xs[e] = make_float2(x.hi, x.lo);
+    }
+    __syncthreads();
+    // K1 pairs (whole warps), then K2 pairs
+    for (int kind = 0; kind < 2; ++kind) {
+      const int tb = kind == 0 ? 0 : nk1, te = kind == 0 ? nk1 : np;
+      for (int t = tb + tid; t < te; t += blockDim.x) {
+        const long long pq = offp + t;
+        const int2 ij = reinterpret_cast<const int2*>(w.pr_ij)[pq];
+        const int2 ga = w.pr_ga[pq];
+        const int gi = ga.x;
+        // table rows of this pair, one frequency ahead of the arithmetic
+        const float4* ra = reinterpret_cast<const float4*>(w.rad_ff + 4 * ((long long)max(gi, 0) * p.nqs + q0));
+        float4 nu = ra[0], nv = ra[1];
+        ConSum S;
 #pragma unroll
-      for (int al = 0; al < 3; ++al)
-#pragma unroll
-        for (int be = 0; be < 3; ++be) {
-          ff s = ff_mul(li[3 * al], xj[3 * be]);
-          s = ff_fma(lj[3 * al], xi[3 * be], s);
-#pragma unroll
-          for (int ga = 1; ga < 3; ++ga) {
-            s = ff_fma(li[3 * al + ga], xj[3 * be + ga], s);
-            s = ff_fma(lj[3 * al + ga], xi[3 * be + ga], s);
+        for (int u = 0; u < CON_W; ++u) {
+          S.h[u] = S.l[u] = 0.f;
+          if (!first) {
+            const float2 v = sums[(long long)CON_W * t + u];
+            S.h[u] = v.x;
+            S.l[u] = v.y;
           }
-          Mf[al][be] = ff_neg(s);
         }
-      M[0] = Mf[0][0]; M[1] = Mf[1][1]; M[2] = Mf[2][2];
-      M[3] = ff_scale(ff_add(Mf[0][1], Mf[1][0]), 0.5f);
-      M[4] = ff_scale(ff_add(Mf[0][2], Mf[2][0]), 0.5f);
-      M[5] = ff_scale(ff_add(Mf[1][2], Mf[2][1]), 0.5f);
-    } else {
-      const ff aj = ff_neg(sm.abf[j]);
-      M[0] = ff_mul(aj, li[0]); M[1] = ff_mul(aj, li[4]); M[2] = ff_mul(aj, li[8]);
-      M[3] = ff_scale(ff_mul(aj, ff_add(li[1], li[3])), 0.5f);
-      M[4] = ff_scale(ff_mul(aj, ff_add(li[2], li[6])), 0.5f);
-      M[5] = ff_scale(ff_mul(aj, ff_add(li[5], li[7])), 0.5f);
-    }
-    const float2* gf = w.pr_gff + 6 * pq;
-    const ff rr[3] = {ff_make(gf[0].x, gf[0].y), ff_make(gf[1].x, gf[1].y), ff_make(gf[2].x, gf[2].y)};
-    const ff F = ff_make(gf[3].x, gf[3].y), dF = ff_make(gf[4].x, gf[4].y), ir = ff_make(gf[5].x, gf[5].y);
-    ff A0, B0, dA0, dB0;
-    if (gi >= 0) {
-      const float2* ra = w.rad_ff + 4 * ((long long)gi * p.nqs + q);
-      A0 = ff_make(ra[0].x, ra[0].y); B0 = ff_make(ra[1].x, ra[1].y);
-      dA0 = ff_make(ra[2].x, ra[2].y); dB0 = ff_make(ra[3].x, ra[3].y);
-    } else {
-      const double* g = w.pr_geo + 8 * pq;
-      const double si = w.sig[(long long)w.site_atom[sbase + i] * p.nqs + q];
-      const double sj = w.sig[(long long)w.site_atom[sbase + j] * p.nqs + q];
-      double a0d, b0d, da0d, db0d;
-      tsr_radial_fast(g[3], g[6], si * si + sj * sj, a0d, b0d, da0d, db0d);
-      A0 = ff_from_double(a0d); B0 = ff_from_double(b0d); dA0 = ff_from_double(da0d); dB0 = ff_from_double(db0d);
-    }
-    const ff Mr[3] = {ff_fma(M[4], rr[2], ff_fma(M[3], rr[1], ff_mul(M[0], rr[0]))),
-                      ff_fma(M[5], rr[2], ff_fma(M[1], rr[1], ff_mul(M[3], rr[0]))),
-                      ff_fma(M[2], rr[2], ff_fma(M[5], rr[1], ff_mul(M[4], rr[0])))};
-    const ff trM = ff_add(ff_add(M[0], M[1]), M[2]);
-    const ff rMr = ff_fma(rr[2], Mr[2], ff_fma(rr[1], Mr[1], ff_mul(rr[0], Mr[0])));
-    const ff phi = ff_fma(B0, rMr, ff_mul(A0, trM));
-    const ff inner = ff_fma(dB0, rMr, ff_mul(dA0, trM));
-    const ff radial = ff_mul(ff_fma(F, inner, ff_mul(dF, phi)), ir);
-    const ff tang = ff_scale(ff_mul(F, B0), 2.0f);
+        if (kind == 0) {
+          for (int q = 0; q < nqc; ++q) {
+            const float4 u4 = nu, v4 = nv;
+            const int qn = min(q + 1, nqc - 1);
+            nu = ra[2 * qn];
+            nv = ra[2 * qn + 1];
+            const float2* li = Ls + (q * n1 + ij.x) * 9;
+            const float2* lj = Ls + (q * n1 + ij.y) * 9;
+            const float2* xi = Xs + (q * n1 + ij.x) * 9;
+            const float2* xj = Xs + (q * n1 + ij.y) * 9;
+            float h[6] = {}, l[6] = {};
+            // row a of lambda times row b of X, summed over the three right-hand sides
+            constexpr int idx[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const ff g = ff_fma(tang, Mr[d], ff_mul(radial, rr[d]));
-      gst[3 * t + d] = make_float2(g.hi, g.lo);
+            for (int k = 0; k < 3; ++k) {
+              ff xa[3], xb[3];
+#pragma unroll
+              for (int b = 0; b < 3; ++b) { xa[b] = ff_ld(xi + 3 * b + k); xb[b] = ff_ld(xj + 3 * b + k); }
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                const ff va = ff_ld(li + 3 * a + k), vb = ff_ld(lj + 3 * a + k);
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                  ff_mac(h[idx[a][b]], l[idx[a][b]], va, xb[b]);
+                  ff_mac(h[idx[a][b]], l[idx[a][b]], vb, xa[b]);
+                }
+              }
+            }
+            ff M[6];
+#pragma unroll
+            for (int u = 0; u < 6; ++u) M[u] = ff_quick_two_sum(h[u], l[u]);
+            ff A0, B0, dA0, dB0;
+            pair_terms(w, p, c, q0 + q, pq, gi, u4, v4, A0, B0, dA0, dB0);
+            S.add(M, A0, B0, dA0, dB0);
+          }
+        } else {
+          const float2* abj = w.abff + (long long)ga.y * p.nqs + q0;
+          float2 na = abj[0];
+          for (int q = 0; q < nqc; ++q) {
+            const float4 u4 = nu, v4 = nv;
+            const ff a = ff_make(na.x, na.y);
+            const int qn = min(q + 1, nqc - 1);
+            nu = ra[2 * qn];
+            nv = ra[2 * qn + 1];
+            na = abj[qn];
+            const float2* li = Ls + (q * n1 + ij.x) * 9;
+            const ff M[6] = {ff_ld(li), ff_ld(li + 4), ff_ld(li + 8), ff_add(ff_ld(li + 1), ff_ld(li + 3)),
+                             ff_add(ff_ld(li + 2), ff_ld(li + 6)), ff_add(ff_ld(li + 5), ff_ld(li + 7))};
+            ff A0, B0, dA0, dB0;
+            pair_terms(w, p, c, q0 + q, pq, gi, u4, v4, A0, B0, dA0, dB0);
+            S.add(M, ff_mul(a, A0), ff_mul(a, B0), ff_mul(a, dA0), ff_mul(a, dB0));
+          }
+        }
+        if (!last) {
+#pragma unroll
+          for (int u = 0; u < CON_W; ++u) sums[(long long)CON_W * t + u] = make_float2(S.h[u], S.l[u]);
+        } else {
+          ff g[3];
+          con_finish(w, pq, S, g);
+#pragma unroll
+          for (int d = 0; d < 3; ++d) gst[3LL * t + d] = make_float2(g[d].hi, g[d].lo);
+        }
+      }
     }
   }
+  __threadfence_block();
   __syncthreads();
-  // per site (fixed order): owner of its row's pairs (-g), partner of K1 pairs owned by later
-  // rows (+g, from the adjacency row) and of K2 pairs (+g, from the reverse list)
-  double* sgq = w.sgq + (sbase * p.nqs + q) * 3;
-  auto gld = [&](long long k) { const float2 v = gst[k]; return ff_make(v.x, v.y); };
+  // per site (fixed order): owner of its row's pairs (-g), partner of K1 pairs owned by later rows
+  // (+g, from the adjacency row) and of K2 pairs (+g, from the reverse list)
   for (int s = tid; s < n12; s += blockDim.x) {
-    ff gx = ff_make(0.f, 0.f), gy = gx, gz = gx;
-    if (s < n1) {
-      for (int t = w.prow[rbase + s]; t < w.prow[rbase + s + 1]; ++t) {
-        gx = ff_sub(gx, gld(3 * t)); gy = ff_sub(gy, gld(3 * t + 1)); gz = ff_sub(gz, gld(3 * t + 2));
+    const int a = w.site_atom[sbase + s];
+    if (p.paper && a != c) continue;     // the paper's forces: only atom c's own gradient
+    ff gs[3] = {ff_make(0.f, 0.f), ff_make(0.f, 0.f), ff_make(0.f, 0.f)};
+    auto acc = [&](int t, bool plus) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const ff v = ff_ld(gst + 3LL * t + d);
+        gs[d] = plus ? ff_add(gs[d], v) : ff_sub(gs[d], v);
       }
-      for (int t = w.arow[rbase + s]; t < w.arow[rbase + s + 1]; ++t) {
-        const int j = w.adj[2 * (offa + t)], pp = w.adj[2 * (offa + t) + 1];
-        if (j > s) { gx = ff_add(gx, gld(3 * pp)); gy = ff_add(gy, gld(3 * pp + 1)); gz = ff_add(gz, gld(3 * pp + 2)); }
+    };
+    if (s < n1) {
+      const int e1 = w.prow[rbase + s + 1], e2 = w.prow_k2[rbase + s + 1], e3 = w.arow[rbase + s + 1];
+#pragma unroll 4
+      for (int t = w.prow[rbase + s]; t < e1; ++t) acc(t, false);
+#pragma unroll 4
+      for (int t = w.prow_k2[rbase + s]; t < e2; ++t) acc(t, false);
+      const int2* ad = reinterpret_cast<const int2*>(w.adj) + offa;
+#pragma unroll 4
+      for (int t = w.arow[rbase + s]; t < e3; ++t) {
+        const int2 v = __ldg(ad + t);
+        if (v.x > s) acc(v.y, true);
       }
     } else {
-      for (int t = w.k2ptr[sbase + s]; t < w.k2ptr[sbase + s + 1]; ++t) {
-        const int pp = w.k2rev[offp + t];
-        gx = ff_add(gx, gld(3 * pp)); gy = ff_add(gy, gld(3 * pp + 1)); gz = ff_add(gz, gld(3 * pp + 2));
-      }
+      const int e = w.k2ptr[sbase + s + 1];
+#pragma unroll 4
+      for (int t = w.k2ptr[sbase + s]; t < e; ++t) acc(__ldg(w.k2rev + offp + t), true);
     }
-    sgq[(long long)s * p.nqs * 3] = ff_to_double(gx);
-    sgq[(long long)s * p.nqs * 3 + 1] = ff_to_double(gy);
-    sgq[(long long)s * p.nqs * 3 + 2] = ff_to_double(gz);
+    const double gx = ff_to_double(gs[0]), gy = ff_to_double(gs[1]), gz = ff_to_double(gs[2]);
+    if (gx != 0.0 || gy != 0.0 || gz != 0.0) atomic_add3(w.gacc + 3 * a, gx, gy, gz);
   }
-}
-
-// ---------------------------------------------------------------------------------------
-// adjoint: one block per (central atom, frequency)
-// ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 3) k_scs_adjoint2(Work w, DevParams p, const int* order, int c0, int max_n1,
-                                                  int max_n12) {
-  extern __shared__ unsigned char smem_raw[];
-  const int c = order ? order[c0 + blockIdx.x / p.nqs] : c0 + blockIdx.x / p.nqs;
-  const int q = blockIdx.x % p.nqs;
-  if (c >= w.n_atoms) return;
-  if (w.fb_flag[(long long)c * p.nqs + q]) return;   // solved by the LU fallback (k_scs_lu_adjoint)
-  const Counts cn = w.counts[c];
-  const int n1 = cn.n1, n12 = cn.n12, N1 = 3 * n1;
-  Scs2Smem sm = scs2_carve(smem_raw, max_n1, max_n12, true);
-  const int tid = threadIdx.x;
-  const long long offp = w.off_p[c], offa = w.off_a[c], rbase = w.off_k1[c] + c;
-  __shared__ int fail;
-  if (tid == 0) fail = 0;
-  scs2_load_abar(w, p, c, q, n1, n12, sm);
-  const long long nA = (long long)N1 * (N1 + 1) / 2;
-  const float* Lg = w.lfac + w.off_b[c] + (long long)q * nA;
-  for (long long e = tid; e < nA; e += blockDim.x) sm.A[e] = Lg[e];
-  // the inverses of the diagonal blocks, as the factor kernel formed them (the solves need no more)
-  const float* Bg = w.binvg + ((long long)c * p.nqs + q) * w.binv_slot;
-  for (int e = tid; e < (N1 + CB - 1) / CB * CBP; e += blockDim.x) sm.binv[e] = Bg[e];
-  __syncthreads();
-  scs2_load_adjoint_rhs(w, p, c, q, n1, sm);
-  __syncthreads();
-  scs2_refine(w, p, n1, offp, offa, rbase, q, sm, &fail, 9.313225746154785e-10);   // lambda, 2^-30
-  __syncthreads();
-  scs2_adjoint_contract(w, p, c, q, n1, n12, sm);
-  if (tid == 0 && fail) atomicOr(w.status, LMBD_FLAG_NOT_CONVERGED);
 }
 
 // ---------------------------------------------------------------------------------------
 // LU fallback for screening matrices that are not positive definite (Sec. III.A: the
-// polarisation catastrophe makes B_K indefinite) or on which the FP32-factor refinement does
-// not converge.  Such systems are rare; each is solved in FP64 by Gaussian elimination with
+// polarisation catastrophe makes B_K indefinite) or on which the refinement does not converge.
+// Such systems are rare; each is solved in FP64 by Gaussian elimination with
 // partial pivoting (row interchanges), the same factorisation a library dense solve uses, on
 // the dense B_K assembled from the pair list into a per-block slot of global memory.  A pivot
 // that is exactly zero (B_K singular) sets LMBD_FLAG_NOT_SPD.
 // ---------------------------------------------------------------------------------------
+struct LuSmem {
+  double* x;      // 9 n1: right-hand side, then solution
+  double* red;    // 64
+  int* piv;       // 3 n1
+  int* redi;      // 64
+};
+__host__ __device__ inline size_t lu_smem_bytes(int max_n1) {
+  return (size_t)max_n1 * (9 * sizeof(double) + 3 * sizeof(int)) + 64 * (sizeof(double) + sizeof(int));
+}
+__device__ inline LuSmem lu_carve(unsigned char* base, int max_n1) {
+  LuSmem s;
+  s.x = reinterpret_cast<double*>(base);
+  s.red = s.x + 9 * max_n1;
+  s.piv = reinterpret_cast<int*>(s.red + 64);
+  s.redi = s.piv + 3 * max_n1;
+  return s;
+}
+
 // dense B_K (N1 x N1 row-major, FP64) of one (centre, frequency): diag(1/alpha_bar) plus the
 // T_SR blocks of the K1 pairs (symmetric 3 x 3 blocks, F A0 delta + F B0 r r^T)
-__device__ void scs2_dense_b(const Work& w, const DevParams& p, int c, int q, int n1, const Scs2Smem& sm, double* A) {
+__device__ void scs2_dense_b(const Work& w, const DevParams& p, int c, int q, int n1, double* A) {
   const int N1 = 3 * n1;
-  const long long offp = w.off_p[c], rbase = w.off_k1[c] + c;
-  const int np = w.prow[rbase + n1];
+  const long long offp = w.off_p[c], rbase = w.off_k1[c] + c, sbase = (long long)c * w.site_cap;
+  const int nk1 = w.prow[rbase + n1];
   for (long long e = threadIdx.x; e < (long long)N1 * N1; e += blockDim.x) A[e] = 0.0;
   __syncthreads();
-  for (int i = threadIdx.x; i < n1; i += blockDim.x)
-    for (int al = 0; al < 3; ++al) A[(long long)(3 * i + al) * N1 + 3 * i + al] = sm.iab[i];
-  for (int t = threadIdx.x; t < np; t += blockDim.x) {
+  for (int i = threadIdx.x; i < n1; i += blockDim.x) {
+    const double ia = 1.0 / w.abar[(long long)w.site_atom[sbase + i] * p.nqs + q];
+    for (int al = 0; al < 3; ++al) A[(long long)(3 * i + al) * N1 + 3 * i + al] = ia;
+  }
+  for (int t = threadIdx.x; t < nk1; t += blockDim.x) {
     const long long pq = offp + t;
     const int i = w.pr_ij[2 * pq], j = w.pr_ij[2 * pq + 1];
-    if (j >= n1) continue;
     const double* g = w.pr_geo + 8 * pq;
     double fa, fb;
     pair_rad64(w, p, c, q, pq, fa, fb);
@@ -1216,82 +1382,68 @@ __device__ void lu_solve3_dense(const double* A, int n, const int* piv, double* 
 
 // Forward LU fallback: persistent over the listed (centre, frequency) systems, one dense slot
 // of lu_slot doubles per block.
-__global__ void __launch_bounds__(256) k_scs_lu_forward(Work w, DevParams p, int max_n1, int max_n12, int tally) {
-  extern __shared__ unsigned char smem_raw[];
-  Scs2Smem sm = scs2_carve(smem_raw, max_n1, max_n12, true);
-  int* piv = reinterpret_cast<int*>(sm.A);
-  int* redi = reinterpret_cast<int*>(sm.y);
+__global__ void __launch_bounds__(256) k_scs_lu_forward(Work w, DevParams p, int max_n1, int tally) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const LuSmem sm = lu_carve(smem_raw, max_n1);
   double* A = w.lu + (long long)blockIdx.x * w.lu_slot;
   const int count = w.fb[0];
   if (tally && blockIdx.x == 0 && threadIdx.x == 0 && count > 0) atomicAdd(w.status + 2, count);
   for (int e = blockIdx.x; e < count; e += gridDim.x) {
     const int id = w.fb[1 + e], c = id / p.nqs, q = id % p.nqs;
-    const int n1 = w.counts[c].n1, n12 = w.counts[c].n12, N1 = 3 * n1;
-    const long long offp = w.off_p[c], rbase = w.off_k1[c] + c;
-    scs2_load_abar(w, p, c, q, n1, n12, sm);
-    __syncthreads();
+    const int n1 = w.counts[c].n1, N1 = 3 * n1;
+    const long long offk1 = w.off_k1[c];
     scs2_build_rhs64(w, p, c, n1, q, sm.x);
-    scs2_dense_b(w, p, c, q, n1, sm, A);
-    if (!lu_factor_dense(A, N1, piv, sm.red, redi)) {
+    scs2_dense_b(w, p, c, q, n1, A);
+    if (!lu_factor_dense(A, N1, sm.piv, sm.red, sm.redi)) {
       if (threadIdx.x == 0) atomicOr(w.status, LMBD_FLAG_NOT_SPD);
       __syncthreads();
       continue;
     }
-    lu_solve3_dense(A, N1, piv, sm.x);
-    scs2_store_solution(w, p, c, q, n1, sm.x);
+    lu_solve3_dense(A, N1, sm.piv, sm.x);
+    double* X = w.xsol + offk1 * p.nqs * 9 + (long long)q * N1 * 3;
+    for (int u = threadIdx.x; u < N1 * 3; u += blockDim.x) X[u] = sm.x[u];
+    for (int i = threadIdx.x; i < n1; i += blockDim.x) {
+      const double a = (sm.x[9 * i] + sm.x[9 * i + 4] + sm.x[9 * i + 8]) / 3.0;
+      w.alphaK[(offk1 + i) * p.nqs + q] = a;
+      if (i == 0) w.alphaI[id] = a;
+    }
     __syncthreads();
   }
 }
 
 // Adjoint LU fallback for the listed systems of centres [c0, c1): B_K is factored again (it is
-// symmetric, so lambda = B_K^-T dL/dX = B_K^-1 dL/dX), then the same pair contraction as the
-// Cholesky path.
-__global__ void __launch_bounds__(256) k_scs_lu_adjoint(Work w, DevParams p, int c0, int c1, int max_n1,
-                                                         int max_n12) {
-  extern __shared__ unsigned char smem_raw[];
-  Scs2Smem sm = scs2_carve(smem_raw, max_n1, max_n12, true);
-  int* piv = reinterpret_cast<int*>(sm.A);
-  int* redi = reinterpret_cast<int*>(sm.y);
+// symmetric, so lambda = B_K^-T dL/dX = B_K^-1 dL/dX).
+__global__ void __launch_bounds__(256) k_scs_lu_adjoint(Work w, DevParams p, int c0, int c1, int max_n1) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const LuSmem sm = lu_carve(smem_raw, max_n1);
   double* A = w.lu + (long long)blockIdx.x * w.lu_slot;
   const int count = w.fb[0];
   for (int e = blockIdx.x; e < count; e += gridDim.x) {
     const int id = w.fb[1 + e], c = id / p.nqs, q = id % p.nqs;
     if (c < c0 || c >= c1) continue;
-    const int n1 = w.counts[c].n1, n12 = w.counts[c].n12, N1 = 3 * n1;
-    scs2_load_abar(w, p, c, q, n1, n12, sm);
-    __syncthreads();
-    scs2_dense_b(w, p, c, q, n1, sm, A);
-    if (!lu_factor_dense(A, N1, piv, sm.red, redi)) {
+    const int n1 = w.counts[c].n1, N1 = 3 * n1;
+    const long long offk1 = w.off_k1[c];
+    scs2_dense_b(w, p, c, q, n1, A);
+    if (!lu_factor_dense(A, N1, sm.piv, sm.red, sm.redi)) {
       if (threadIdx.x == 0) atomicOr(w.status, LMBD_FLAG_NOT_SPD);
       __syncthreads();
       continue;
     }
-    scs2_load_adjoint_rhs(w, p, c, q, n1, sm);
-    for (int u = threadIdx.x; u < 3 * N1; u += blockDim.x) sm.x[u] = sm.rhs[u];
-    __syncthreads();
-    lu_solve3_dense(A, N1, piv, sm.x);
-    scs2_adjoint_contract(w, p, c, q, n1, n12, sm);
-    __syncthreads();
-  }
-}
-
-// Sum of the per-frequency site gradients of the SCS adjoint, scattered to atoms.
-__global__ void __launch_bounds__(256) k_scs_site_reduce(Work w, DevParams p, int c0) {
-  const int c = c0 + blockIdx.x;
-  if (c >= w.n_atoms) return;
-  const int n12 = w.counts[c].n12;
-  const long long sbase = (long long)c * w.site_cap;
-  for (int s = threadIdx.x; s < n12; s += blockDim.x) {
-    const double* g = w.sgq + (sbase + s) * p.nqs * 3;
-    double gx = 0.0, gy = 0.0, gz = 0.0;
-    for (int q = 0; q < p.nqs; ++q) {
-      gx += g[3 * q];
-      gy += g[3 * q + 1];
-      gz += g[3 * q + 2];
+    for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x) {
+      const int i = u / 9, a = (u % 9) / 3, k = u % 3;
+      double g = 0.0;
+      if (a == k) {
+        g = w.alphaK_bar[(offk1 + i) * p.nqs + q];
+        if (i == 0) g += w.alphaI_bar[id];
+        g *= 1.0 / 3.0;
+      }
+      sm.x[u] = g;
     }
-    const int a = w.site_atom[sbase + s];
-    if (p.paper && a != c) continue;     // the paper's forces: only atom c's own gradient
-    if (gx != 0.0 || gy != 0.0 || gz != 0.0) atomic_add3(w.gacc + 3 * a, gx, gy, gz);
+    __syncthreads();
+    lu_solve3_dense(A, N1, sm.piv, sm.x);
+    double* lam = w.lsol + offk1 * p.nqs * 9 + (long long)q * N1 * 3;
+    for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x) lam[u] = sm.x[u];
+    __syncthreads();
   }
 }
 
@@ -1308,7 +1460,7 @@ void launch_scs_count(const Work& w, const DevParams& p, int max_n12, cudaStream
 void launch_scs_fill(const Work& w, const DevParams& p, int c0, int c1, int max_n12, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
   size_t sm = sizeof(double) * 3 * (size_t)max_n12 +
-              sizeof(int) * ((size_t)max_n1 * max_n1 + 6 * (size_t)max_n1 + 2 + (size_t)max_n12 + 8 * (size_t)max_n1) +
+              sizeof(int) * ((size_t)max_n1 * max_n1 + 7 * (size_t)max_n1 + 3 + (size_t)max_n12 + 8 * (size_t)max_n1) +
               sizeof(float) * 3 * (size_t)max_n12;
   raise_smem_limit((const void*)k_scs_fill, sm);
   k_scs_fill<<<c1 - c0, 256, sm, s>>>(w, p, c0, max_n12, max_n1);
@@ -1319,44 +1471,82 @@ void launch_pair_radial(const Work& w, const DevParams& p, cudaStream_t s) {
   k_pair_radial<<<w.n_atoms, 128, 0, s>>>(w, p);
 }
 
-size_t scs2_forward_smem(int max_n1, int max_n12) { return scs2_smem_bytes(max_n1, max_n12, false); }
-size_t scs2_adjoint_smem(int max_n1, int max_n12) { return scs2_smem_bytes(max_n1, max_n12, true); }
-
-// Centres order[c0..c1) (or c0..c1 when order is NULL), shared memory sized for the largest
-// K1 and K1 u K2 among them.
-void launch_scs_factor(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, int max_n12,
-                       cudaStream_t s) {
-  if (c1 <= c0) return;
-  size_t sm = scs2_smem_bytes(max_n1, max_n12, false);
-  raise_smem_limit((const void*)k_scs_factor, sm);
-  k_scs_factor<<<(c1 - c0) * p.nqs, 256, sm, s>>>(w, p, order, c0, max_n1, max_n12);
+// Sites one screening system may hold: |K1| <= 96 (three warps), and with it the combined size of
+// its lists, a limit of the entry points in terms of |K1| and |K1 u K2|.
+bool scs_capacity(int max_n1, int max_n12) {
+  const size_t N1 = 3 * (size_t)max_n1;
+  const size_t fl = (N1 * (N1 + 1) / 2 + 7 * N1 + (N1 + 15) / 16 * 136 + 1) & ~size_t(1);
+  return max_n1 <= 96 && fl * sizeof(float) + (9 * N1 + (size_t)max_n12 + max_n1 + 64) * sizeof(double) <= 227 * 1024;
 }
 
-void launch_scs_adjoint2(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1,
-                         int max_n12, cudaStream_t s) {
+template <int S, int NC, bool ADJ>
+static void run_solve(const Work& w, const DevParams& p, const int* order, int c0, int c1, int ld, cudaStream_t s) {
+  const size_t sm = cg_smem_bytes(ld);
+  raise_smem_limit((const void*)k_scs_solve<S, NC, ADJ>, sm);
+  k_scs_solve<S, NC, ADJ><<<(c1 - c0) * p.nqs, 32 * S * (3 / NC), sm, s>>>(w, p, order, c0, ld);
+}
+
+// Centres order[c0..c1) (or c0..c1 when order is NULL), shared memory sized for the largest K1 among
+// them.  A structure whose systems are all resident at once is bound by the time of one solve:
+// there a group of warps per right-hand side shortens it (64-atom box, forward solves 0.72 ->
+// 0.52 ms; 24-atom cluster 82 -> 47 us); larger ones are bound by the issue slots and take the three
+// right-hand sides together (4096 atoms: 14.0 against 18.5 ms).  The choice depends on the
+// structure, not on the wave, so that energies are the same bits in every partition.
+template <bool ADJ>
+static void run_solve_any(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
-  size_t sm = scs2_smem_bytes(max_n1, max_n12, true);
-  raise_smem_limit((const void*)k_scs_adjoint2, sm);
-  k_scs_adjoint2<<<(c1 - c0) * p.nqs, 256, sm, s>>>(w, p, order, c0, max_n1, max_n12);
+  const bool split = (long long)w.n_atoms * p.nqs <= 152 * 12;
+  if (split) {
+    if (max_n1 <= 32) run_solve<1, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
+    else if (max_n1 <= 64) run_solve<2, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
+    else run_solve<3, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
+  } else {
+    if (max_n1 <= 32) run_solve<1, 3, ADJ>(w, p, order, c0, c1, max_n1, s);
+    else if (max_n1 <= 64) run_solve<2, 3, ADJ>(w, p, order, c0, c1, max_n1, s);
+    else run_solve<3, 3, ADJ>(w, p, order, c0, c1, max_n1, s);
+  }
+}
+void launch_scs_solve(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s) {
+  run_solve_any<false>(w, p, order, c0, c1, max_n1, s);
+}
+void launch_scs_adjoint(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s) {
+  run_solve_any<true>(w, p, order, c0, c1, max_n1, s);
+}
+
+// Blocks per centre of the contraction: structures of fewer centres than fill the chip twice split
+// the frequencies (64-atom box, SCS adjoint phase 0.76 -> 0.57 ms, of which the solves 0.2).
+int scs_contract_split(int n_atoms, int nqs) {
+  const int want = (2 * 152 + n_atoms - 1) / (n_atoms > 0 ? n_atoms : 1);
+  const int per = (nqs + want - 1) / want;
+  return (nqs + per - 1) / per;
+}
+// Shared memory of its blocks: lambda and X of all a block's frequencies, or two blocks per SM; a centre
+// whose |K1| does not fit takes its frequencies in chunks.
+static size_t scs_contract_smem(int n_atoms, int max_n1, int nqs) {
+  const int split = scs_contract_split(n_atoms, nqs), per = (nqs + split - 1) / split;
+  return std::min((size_t)144 * max_n1 * per, (size_t)112 * 1024);
+}
+// float2 of gradient scratch per pair: 3, and 14 sums when the frequencies go in chunks, per block
+int scs_contract_scratch(int n_atoms, int max_n1, int nqs) {
+  const int split = scs_contract_split(n_atoms, nqs), per = (nqs + split - 1) / split;
+  return split * (scs_contract_smem(n_atoms, max_n1, nqs) < (size_t)144 * max_n1 * per ? 3 + CON_W : 3);
+}
+
+void launch_scs_contract(const Work& w, const DevParams& p, int c0, int c1, int max_n1, cudaStream_t s) {
+  if (c1 <= c0) return;
+  const int split = scs_contract_split(w.n_atoms, p.nqs);
+  const size_t sm = scs_contract_smem(w.n_atoms, max_n1, p.nqs);
+  raise_smem_limit((const void*)k_scs_contract, sm);
+  k_scs_contract<<<(c1 - c0) * split, 256, sm, s>>>(w, p, c0, split, (int)sm,
+                                                    scs_contract_scratch(w.n_atoms, max_n1, p.nqs));
 }
 
 // LU fallback launches: a fixed grid of lu_blocks persistent blocks (one dense slot each);
 // with an empty list every block exits at once.
-void launch_scs_lu_forward(const Work& w, const DevParams& p, int lu_blocks, int max_n1, int max_n12, int tally,
-                           cudaStream_t s) {
-  size_t sm = scs2_smem_bytes(max_n1, max_n12, true);
-  raise_smem_limit((const void*)k_scs_lu_forward, sm);
-  k_scs_lu_forward<<<lu_blocks, 256, sm, s>>>(w, p, max_n1, max_n12, tally);
+void launch_scs_lu_forward(const Work& w, const DevParams& p, int lu_blocks, int max_n1, int tally, cudaStream_t s) {
+  k_scs_lu_forward<<<lu_blocks, 256, lu_smem_bytes(max_n1), s>>>(w, p, max_n1, tally);
 }
 
-void launch_scs_lu_adjoint(const Work& w, const DevParams& p, int lu_blocks, int c0, int c1, int max_n1,
-                           int max_n12, cudaStream_t s) {
-  size_t sm = scs2_smem_bytes(max_n1, max_n12, true);
-  raise_smem_limit((const void*)k_scs_lu_adjoint, sm);
-  k_scs_lu_adjoint<<<lu_blocks, 256, sm, s>>>(w, p, c0, c1, max_n1, max_n12);
-}
-
-void launch_scs_site_reduce(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s) {
-  if (c1 <= c0) return;
-  k_scs_site_reduce<<<c1 - c0, 256, 0, s>>>(w, p, c0);
+void launch_scs_lu_adjoint(const Work& w, const DevParams& p, int lu_blocks, int c0, int c1, int max_n1, cudaStream_t s) {
+  k_scs_lu_adjoint<<<lu_blocks, 256, lu_smem_bytes(max_n1), s>>>(w, p, c0, c1, max_n1);
 }

@@ -107,7 +107,7 @@ struct Ctx {
   DevBuf table_d, pos_d, species_d, nu_d, weights_d, out_e_d, out_f_d;
   DevBuf abar, sig, rvdw, a0, r0, wpos, cell_of, cell_count, cell_start, cell_atoms, grid;
   DevBuf site_atom, site_x, site_img, wrap, counts, offs, totals, status, pcount;
-  DevBuf alphaK, alphaI, energies, trbuf, wexp, alphaK_bar, alphaI_bar, gacc, rad_ab, rad_ff;
+  DevBuf alphaK, alphaI, energies, trbuf, wexp, alphaK_bar, alphaI_bar, gacc, rad_ab, rad_ff, abff;
   DevBuf order1_d, order3_d, fitw, cfit, lam, gl64, fb, fb_flag, lu, sp_cnt, sp_np;
   DevBuf arena;
   std::vector<Counts> counts_h;
@@ -120,7 +120,7 @@ struct Ctx {
     DevBuf* l[] = {&table_d, &pos_d, &species_d, &nu_d, &weights_d, &out_e_d, &out_f_d, &abar, &sig, &rvdw,
                    &a0, &r0, &wpos, &cell_of, &cell_count, &cell_start, &cell_atoms, &grid, &site_atom,
                    &site_x, &counts, &offs, &totals, &status, &pcount, &alphaK, &alphaI, &energies, &trbuf,
-                   &wexp, &alphaK_bar, &alphaI_bar, &gacc, &order1_d, &order3_d, &rad_ab, &rad_ff, &fitw, &cfit, &lam, &gl64,
+                   &wexp, &alphaK_bar, &alphaI_bar, &gacc, &order1_d, &order3_d, &rad_ab, &rad_ff, &abff, &fitw, &cfit, &lam, &gl64,
                    &fb, &fb_flag, &lu, &theta_f, &theta_out, &site_img, &wrap, &ref_pos, &ref_spec, &kept_pos, &kept_spec,
                    &sp_cnt, &sp_np};
     static_assert(sizeof(l) / sizeof(l[0]) <= kMaxWhole, "whole-structure buffer list exceeds its array");
@@ -276,7 +276,7 @@ struct Layout {
   int nqs;   // frequencies of the SCS solves (stage-1 arrays)
   int tk;    // tcgen05 path: row pitch of the T and W digit planes (0: per-centre Kpad)
   bool sparse;   // block-sparse T_LR: coupled pairs and float-float chain/pair operands
-  int binv_slot; // floats of the diagonal-block inverses of one SCS system (largest |K1|)
+  int gs_ld;     // float2 per pair of the SCS adjoint's gradient scratch
 
   // stage 1 (SCS): pair lists, FP32 factors and solutions of centres [c0, c1)
   size_t stage1(const Offs& o, int c0, int c1, char* base, Work* w) const {
@@ -285,12 +285,10 @@ struct Layout {
     const long long a0 = o.at(O_A, c0), na = o.span(O_A, c0, c1);
     const long long k0 = o.at(O_K1, c0), nk = o.span(O_K1, c0, c1);
     const long long n = c1 - c0;
-    float* lfac = cv.take<float>(o.span(O_B, c0, c1), o.at(O_B, c0));
-    float* binvg = cv.take<float>((long long)binv_slot * nqs * n, (long long)binv_slot * nqs * c0);
     int* pr_ij = cv.take<int>(2 * (np + 1), 2 * p0);
     double* pr_geo = cv.take<double>(8 * (np + 1), 8 * p0);
-    float2* pr_rad_ff = cv.take<float2>(2LL * nqs * (np + 1), 2LL * nqs * p0);
-    int* pr_g = cv.take<int>(np + 1, p0);
+    float4* pr_rad4 = cv.take<float4>(nqs * (np + 1), nqs * p0);
+    int2* pr_ga = cv.take<int2>(np + 1, p0);
     float2* pr_gff = cv.take<float2>(6 * (np + 1), 6 * p0);
     int* k2rev = cv.take<int>(np + 1, p0);
     int* prow = cv.take<int>(nk + n, k0 + c0);
@@ -300,13 +298,10 @@ struct Layout {
     int* k2ptr = cv.take<int>(n * site_cap + 1, (long long)c0 * site_cap);
     double* xsol = cv.take<double>(9LL * nqs * nk, 9LL * nqs * k0);
     if (w) {
-      w->lfac = lfac;
-      w->binvg = binvg;
-      w->binv_slot = binv_slot;
       w->pr_ij = pr_ij;
       w->pr_geo = pr_geo;
-      w->pr_rad_ff = pr_rad_ff;
-      w->pr_g = pr_g;
+      w->pr_rad4 = pr_rad4;
+      w->pr_ga = pr_ga;
       w->pr_gff = pr_gff;
       w->k2rev = k2rev;
       w->prow = prow;
@@ -319,15 +314,16 @@ struct Layout {
     return align256(cv.used);
   }
 
-  // scratch of the SCS adjoint: pair and site gradients of centres [c0, c1)
+  // scratch of the SCS adjoint: its solutions and the pair gradients of centres [c0, c1)
   size_t scs_adjoint(const Offs& o, int c0, int c1, char* base, Work* w) const {
     Carver cv{base, 0};
     const long long p0 = o.at(O_P, c0), np = o.span(O_P, c0, c1);
-    double* gstage = cv.take<double>(3LL * nqs * (np + 1), 3LL * nqs * p0);
-    double* sgq = cv.take<double>(3LL * nqs * (c1 - c0) * site_cap, 3LL * nqs * c0 * site_cap);
+    const long long k0 = o.at(O_K1, c0), nk = o.span(O_K1, c0, c1);
+    float2* gstage = cv.take<float2>((long long)gs_ld * (np + 1), (long long)gs_ld * p0);
+    double* lsol = cv.take<double>(9LL * nqs * nk, 9LL * nqs * k0);
     if (w) {
       w->gstage = gstage;
-      w->sgq = sgq;
+      w->lsol = lsol;
     }
     return align256(cv.used);
   }
@@ -835,7 +831,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   // (the block-sparse T_LR path keeps no dense 3 ns x 3 ns matrix: spheres up to the site capacity)
   if (max_n1 > 96 || max_ns > (c->sparse ? 4096 : 1024) || max_n12 > 4096) return LMBD_ECAPACITY;
   const int max_pairs = (int)c->totals_h[11];
-  if (scs2_adjoint_smem(max_n1, max_n12) > 227 * 1024) return LMBD_ECAPACITY;
+  if (!scs_capacity(max_n1, max_n12)) return LMBD_ECAPACITY;
   // dense FP64 slots of the LU fallback, one per persistent block
   const int lu_blocks = 32;
   w.lu_slot = 9LL * max_n1 * max_n1;
@@ -867,6 +863,9 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   w.alphaK = (double*)c->alphaK.p;
   w.rad_ab = (double*)c->rad_ab.p;
   w.rad_ff = (float2*)c->rad_ff.p;
+  TRY(ensure(c->abff, sizeof(float2) * 2 * (size_t)N * nq));
+  w.abff = (float2*)c->abff.p;
+  w.iabff = w.abff + (size_t)N * nq;
   w.nvec = nvec;
   w.ncol = ncol;
   if (sliced_chain) {
@@ -911,7 +910,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   // ---- waves under the memory budget --------------------------------------------------------
   const Layout L{nq, ncv, nvec, ncol, (ncol + 15) / 16 * 16, ST, DIG_P, c->site_cap, forces, sliced_chain,
                  sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 15) / 16 * 16 : 0, sparse,
-                 (3 * max_n1 + 15) / 16 * 136};
+                 scs_contract_scratch(N, max_n1, dp.nqs)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };
   auto s1x = [&](int a, int b) { return forces ? L.scs_adjoint(o, a, b, nullptr, nullptr) : (size_t)0; };
   auto s2 = [&](int a, int b) { return L.stage2(o, a, b, nullptr, nullptr, nullptr); };
@@ -1006,7 +1005,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
     ++phase_launch[LMBD_PHASE_SCS];
     if (per_atom) {
       for (int cc = c0; cc < c1; ++cc)
-        launch_scs_factor(w, dp, nullptr, cc, cc + 1, c->counts_h[cc].n1, c->counts_h[cc].n12, s);
+        launch_scs_solve(w, dp, nullptr, cc, cc + 1, c->counts_h[cc].n1, s);
       phase_launch[LMBD_PHASE_SCS] += c1 - c0;
     } else {
       if (kmark_fwd) cudaEventRecord(c->kev[0], s);
@@ -1014,14 +1013,14 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
       Fork fk(c, s, (int)bk[wv].size());
       for (size_t i = 0; i < bk[wv].size(); ++i) {
         const Bucket& b = bk[wv][i];
-        launch_scs_factor(w, dp, order, b.b0, b.b1, b.n1, b.n12, fk.stream((int)i));
+        launch_scs_solve(w, dp, order, b.b0, b.b1, b.n1, fk.stream((int)i));
       }
       fk.join();
       nvtxRangePop();
       if (kmark_fwd) cudaEventRecord(c->kev[1], s);
       phase_launch[LMBD_PHASE_SCS] += (int)bk[wv].size();
     }
-    launch_scs_lu_forward(w, dp, lu_blocks, max_n1, max_n12, tally_lu ? 1 : 0, s);
+    launch_scs_lu_forward(w, dp, lu_blocks, max_n1, tally_lu ? 1 : 0, s);
     ++phase_launch[LMBD_PHASE_SCS];
     CK(cudaGetLastError());
     return LMBD_OK;
@@ -1185,9 +1184,9 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
       L.scs_adjoint(o, c0, c1, arena + x_at, &w);
       if (per_atom) {
         for (int cc = c0; cc < c1; ++cc)
-          launch_scs_adjoint2(w, dp, nullptr, cc, cc + 1, c->counts_h[cc].n1, c->counts_h[cc].n12, s);
-        launch_scs_lu_adjoint(w, dp, lu_blocks, c0, c1, max_n1, max_n12, s);
-        for (int cc = c0; cc < c1; ++cc) launch_scs_site_reduce(w, dp, cc, cc + 1, s);
+          launch_scs_adjoint(w, dp, nullptr, cc, cc + 1, c->counts_h[cc].n1, s);
+        launch_scs_lu_adjoint(w, dp, lu_blocks, c0, c1, max_n1, s);
+        for (int cc = c0; cc < c1; ++cc) launch_scs_contract(w, dp, cc, cc + 1, max_n1, s);
         phase_launch[LMBD_PHASE_ADJ_SCS] += 2 * (c1 - c0) + 1;
       } else {
         if (prof) cudaEventRecord(c->kev[2], s);
@@ -1195,13 +1194,13 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
         Fork fk(c, s, (int)bucketsC[wv].size());
         for (size_t i = 0; i < bucketsC[wv].size(); ++i) {
           const Bucket& b = bucketsC[wv][i];
-          launch_scs_adjoint2(w, dp, orderC, b.b0, b.b1, b.n1, b.n12, fk.stream((int)i));
+          launch_scs_adjoint(w, dp, orderC, b.b0, b.b1, b.n1, fk.stream((int)i));
         }
         fk.join();
         nvtxRangePop();
         if (prof) cudaEventRecord(c->kev[3], s);
-        launch_scs_lu_adjoint(w, dp, lu_blocks, c0, c1, max_n1, max_n12, s);
-        launch_scs_site_reduce(w, dp, c0, c1, s);
+        launch_scs_lu_adjoint(w, dp, lu_blocks, c0, c1, max_n1, s);
+        launch_scs_contract(w, dp, c0, c1, max_n1, s);
         phase_launch[LMBD_PHASE_ADJ_SCS] += (int)bucketsC[wv].size() + 2;
       }
       CK(cudaGetLastError());

@@ -120,30 +120,28 @@ struct Work {
   int* pcount;                 // N x 2: pairs, adjacency entries
   int* pr_ij;                  // pairs x 2: owner row i (K1), partner j (K1 with j < i, or K2)
   double* pr_geo;              // pairs x 8: r = x_j - x_i (3), |r|, F, dF/dr, 1/|r|, unused
-  float2* pr_rad_ff;           // pairs x nq x 2: F A0, F B0 as float-float (residual updates)
-  int* pr_g;                   // pairs: index of the pair in the atom-pair radial table, -1 = none
+  float4* pr_rad4;             // per centre (off_p nq) [nq][K1 pairs]: F A0, F B0 as float-float (hi, lo)
+  int2* pr_ga;                 // pairs: index of the pair in the atom-pair radial table (-1 = none), atom of j
   // radial terms of T_SR per atom pair and frequency, independent of the central atom: entry
   // off_k1[a] + s is atom a with site s (1 <= s < n1) of its own K1 list
   double* rad_ab;              // sum n1 x nq x 2: A0, B0
   float2* rad_ff;              // sum n1 x nq x 4: A0, B0, dA0/dr, dB0/dr as float-float (hi, lo)
   float2* pr_gff;              // pairs x 6: r (3), F, dF/dr, 1/|r| as float-float (SCS adjoint)
-  int* prow;                   // (sum n1 + N): first pair of each row, per centre n1 + 1 entries
-  int* prow_k2;                // (sum n1 + N): first K2 pair of each row
+  int* prow;                   // (sum n1 + N): first K1 pair of each row, per centre n1 + 1 entries
+  int* prow_k2;                // (sum n1 + N): first K2 pair of each row (after all K1 pairs)
   int* arow;                   // (sum n1 + N): first adjacency entry of each row
   int* adj;                    // entries x 2: K1 partner j, pair index
   int* k2ptr;                  // N x site_cap: first reverse-list entry of each K2 site
   int* k2rev;                  // per centre (off_p): pair indices grouped by K2 partner
-  double* sgq;                 // N x site_cap x nq x 3: SCS-adjoint site gradients per frequency
-  double* gstage;              // sum pairs x nq x 3: SCS-adjoint pair gradients (scratch; 8-byte
-                               // entries, written and read as float-float pairs)
-  float* lfac;                 // packed FP32 Cholesky factors, off_b
-  float* binvg;                // inverses of their 16 x 16 diagonal blocks, binv_slot floats per
-                               // (centre, SCS frequency), indexed by the global centre
-  int binv_slot;
-  // LU fallback of the SCS solves (systems whose FP32 Cholesky pivot is not positive or whose
-  // refinement does not converge): fb[0] = count, fb[1 + e] = c * nqs + q; fb_flag[c * nqs + q]
-  // = 1 for such a system (its FP32 factor is not used); lu: per-block dense slots of lu_slot
-  // doubles ((3 max n1)^2)
+  float2* gstage;              // SCS-adjoint pair gradients, 3 float-float per pair and block of a centre
+                               // (with frequencies in chunks: 14 sums)
+  double* lsol;                // adjoint solutions lambda = B^-1 dL/dX, off_k1 * nq * 9
+  float2* abff;                // N x nqs: alpha_bar as float-float
+  float2* iabff;               // N x nqs: 1 / alpha_bar as float-float
+  // LU fallback of the SCS solves (systems in which the conjugate gradients meet a direction of
+  // non-positive curvature or whose refinement does not converge): fb[0] = count, fb[1 + e] =
+  // c * nqs + q; fb_flag[c * nqs + q] = 1 for such a system; lu: per-block dense slots of
+  // lu_slot doubles ((3 max n1)^2)
   int* fb;
   int* fb_flag;
   double* lu;
@@ -393,17 +391,15 @@ void launch_offsets(const Work& w, const DevParams& p, cudaStream_t s);
 void launch_scs_count(const Work& w, const DevParams& p, int max_n12, cudaStream_t s);
 void launch_scs_fill(const Work& w, const DevParams& p, int c0, int c1, int max_n12, int max_n1, cudaStream_t s);
 void launch_pair_radial(const Work& w, const DevParams& p, cudaStream_t s);
-void launch_scs_factor(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, int max_n12,
-                       cudaStream_t s);
-void launch_scs_adjoint2(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1,
-                         int max_n12, cudaStream_t s);
-void launch_scs_site_reduce(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s);
-void launch_scs_lu_forward(const Work& w, const DevParams& p, int lu_blocks, int max_n1, int max_n12, int tally,
-                           cudaStream_t s);
+void launch_scs_solve(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s);
+void launch_scs_adjoint(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1,
+                        cudaStream_t s);
+void launch_scs_lu_forward(const Work& w, const DevParams& p, int lu_blocks, int max_n1, int tally, cudaStream_t s);
 void launch_scs_lu_adjoint(const Work& w, const DevParams& p, int lu_blocks, int c0, int c1, int max_n1,
-                           int max_n12, cudaStream_t s);
-size_t scs2_forward_smem(int max_n1, int max_n12);
-size_t scs2_adjoint_smem(int max_n1, int max_n12);
+                           cudaStream_t s);
+void launch_scs_contract(const Work& w, const DevParams& p, int c0, int c1, int max_n1, cudaStream_t s);
+int scs_contract_scratch(int n_atoms, int max_n1, int nqs);   // float2 of gradient scratch per pair
+bool scs_capacity(int max_n1, int max_n12);
 void launch_mbd_prepare_sized(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
 void launch_mbd_chain_sized(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, cudaStream_t s);
 void launch_mbd_energy(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s);
