@@ -67,3 +67,12 @@ __device__ __forceinline__ ff ff_scale(ff a, float s) {   // a * s for an exact 
   e = __fmaf_rn(a.lo, s, e);
   return ff_quick_two_sum(p, e);
 }
+
+// Compensated accumulation of the product a b (float-float operands) into (h, l).
+__device__ __forceinline__ void ff_mac(float& h, float& l, ff a, ff b) {
+  const float v = __fmul_rn(a.hi, b.hi);
+  const float e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -v)));
+  const ff m = ff_two_sum(h, v);
+  h = m.hi;
+  l = __fadd_rn(l, __fadd_rn(m.lo, e));
+}

@@ -22,9 +22,77 @@
 #include "ozaki.cuh"
 #include "pair_epilogue.cuh"
 
+// padded rows and columns of a centre's digit planes
+__device__ __forceinline__ int oz_mpad(int n) { return (n + 63) / 64 * 64; }
+__device__ __forceinline__ int oz_kpad(int n) { return (n + 15) / 16 * 16; }
+
 // ---------------------------------------------------------------------------------------
 // prepare: blended polarisabilities, SCS radii, T_LR and the first Krylov block
 // ---------------------------------------------------------------------------------------
+// The FP64 pipe bounds this kernel, so only what needs it runs there: each warp screens 32 pairs in
+// FP32 (pairs within a relative 1e-4 of the cutoff take the FP64 test, so the decision is the FP64
+// one), queues the coupled ones (47 % at the benchmark cutoffs), and evaluates 32 queued pairs with
+// all lanes: distance, exponential and the two divisions in FP64, the products of the record in
+// float-float on the FP32 pipe.  1024-atom step: 2.51 ms with every pair in FP64
+// and T_LR stored, 1.11 ms now (FP64 pipe 62 % busy over a launch of 1.7 waves).
+// DENSE: the FP64 blocks of T_LR and / or the FP64 coefficients are wanted as well (Lanczos-based
+// modes, the paper's forces, FP64 and warp-level products).
+
+// The record of a coupled pair at displacement rr: see Work::trec; with f = 1 / (1 + e^(-d (x - 1))),
+// x = r / S~, C = f_LR f:  k1 = 6 C' / r^6 - 30 C / r^7,  k2 = 6 C / r^5 - 2 C' / r^4,  k3 = 12 C / r^5,
+// k4 = 6 beta f_LR f_S / r^5,  k5 = -2 beta f_LR f_S / r^3 (C' = dC/dr, f_S = df/dS~).  top[a]: a
+// bound of the largest entry of row a of the block, as FP32 bits.
+struct PairRec {
+  float4 v[4];
+  int top[3];
+};
+__device__ __forceinline__ float4 two_ff(ff a, ff b) { return make_float4(a.hi, a.lo, b.hi, b.lo); }
+__device__ __forceinline__ PairRec tlr_pair_record(const DevParams& p, ff d_ff, ff beta_ff, ff ib_ff, const double (&rr)[3],
+                                                   double rc, double rts, double rtt, bool full) {
+  const double r2 = rr[0] * rr[0] + rr[1] * rr[1] + rr[2] * rr[2];
+  const double ird = rsqrt(r2), r = r2 * ird;
+  const double xd = r / (p.beta * (rts + rtt));
+  const double e = exp(-p.d * (xd - 1.0));
+  const double fd = 1.0 / (1.0 + e);
+  const ff x = ff_from_double(rr[0]), y = ff_from_double(rr[1]), z = ff_from_double(rr[2]);
+  const ff ir = ff_from_double(ird), ir2 = ff_mul(ir, ir), ir4 = ff_mul(ir2, ir2), ir5 = ff_mul(ir4, ir);
+  const ff f = ff_from_double(fd);
+  // f_LR = 1 - 3 t^2 + 2 t^3, f_LR' = (-6 t + 6 t^2) / r_b, t = (r - rc + r_b) / r_b in the buffer
+  const double tb = r - (rc - p.r_buf);
+  const bool buffer = tb >= 0.0;
+  ff flr = ff_make(1.f, 0.f), dflr = ff_make(0.f, 0.f);
+  if (buffer) {
+    const ff t = ff_mul(ff_from_double(tb), ib_ff), t2 = ff_mul(t, t);
+    flr = ff_add(ff_make(1.f, 0.f), ff_sub(ff_scale(ff_mul(t2, t), 2.f), ff_scale(t2, 3.f)));
+    dflr = ff_mul(ff_scale(ff_sub(t2, t), 6.f), ib_ff);
+    if (!(r < rc)) flr = dflr = ff_make(0.f, 0.f);
+  }
+  const ff C = buffer ? ff_mul(flr, f) : f;
+  const ff u = ff_mul(C, ir5);
+  PairRec o;
+  o.v[0] = two_ff(x, y);
+  o.v[1] = two_ff(z, ff_scale(u, 12.f));
+  if (full) {
+    const ff sx = ff_from_double(xd);
+    const ff dfr = ff_mul(ff_mul(ff_from_double(fd * (1.0 - fd)), d_ff), ff_mul(sx, ir));   // df/dr
+    const ff dlr = buffer ? ff_mul(flr, dfr) : dfr;
+    const ff dC = buffer ? ff_add(ff_mul(dflr, f), dlr) : dfr;
+    const ff v = ff_mul(ff_mul(ff_mul(ff_neg(dlr), sx), ff_mul(ir2, ir)), beta_ff);   // beta f_LR f_S / r^3
+    o.v[2] = two_ff(ff_sub(ff_scale(ff_mul(dC, ff_mul(ir4, ir2)), 6.f), ff_scale(ff_mul(u, ir2), 30.f)),
+                    ff_sub(ff_scale(u, 6.f), ff_scale(ff_mul(dC, ir4), 2.f)));
+    o.v[3] = two_ff(ff_scale(ff_mul(v, ir2), 6.f), ff_scale(v, -2.f));
+  }
+  // FP32 bound of the rows' entries: 3 u r_a r_b - u r^2 delta_ab, raised by 2^-20
+  const float a3 = 3.00001f * fabsf(u.hi), b = fabsf(u.hi) * (float)r2;
+  const float ax = fabsf(x.hi), ay = fabsf(y.hi), az = fabsf(z.hi);
+  const float xy = a3 * ax * ay, xz = a3 * ax * az, yz = a3 * ay * az, up = 1e-5f * b;
+  o.top[0] = __float_as_int(fmaxf(fabsf(a3 * ax * ax - b) + up, fmaxf(xy, xz)));
+  o.top[1] = __float_as_int(fmaxf(fabsf(a3 * ay * ay - b) + up, fmaxf(xy, yz)));
+  o.top[2] = __float_as_int(fmaxf(fabsf(a3 * az * az - b) + up, fmaxf(xz, yz)));
+  return o;
+}
+
+template <bool DENSE>
 __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0, int max_ns) {
   extern __shared__ double smem_d[];
   const int c = c0 + blockIdx.x;
@@ -33,54 +101,148 @@ __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0
   const int ns = cn.ns, n1 = cn.n1, N = 3 * ns;
   double* xs = smem_d;                 // 3 x max_ns
   double* rt = xs + 3 * max_ns;        // max_ns
-  const int tid = threadIdx.x;
+  double* col = rt + max_ns;           // 9 x max_ns: column block of the central site
+  float* xf = reinterpret_cast<float*>(col + 9 * max_ns);   // 3 x max_ns, FP32 copies of xs
+  int* ex = reinterpret_cast<int*>(xf + 3 * max_ns);        // 3 x max_ns: largest entry of each row of T_LR
+  int* queue = ex + 3 * max_ns;                             // 64 per warp
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
   const long long sbase = (long long)c * w.site_cap;
   const long long offs = w.off_s[c], offk1 = w.off_k1[c];
   for (int s = tid; s < ns; s += blockDim.x) {
     int a = w.site_atom[sbase + s];
     double x0 = w.site_x[3 * (sbase + s)], x1 = w.site_x[3 * (sbase + s) + 1], x2 = w.site_x[3 * (sbase + s) + 2];
     xs[s] = x0; xs[max_ns + s] = x1; xs[2 * max_ns + s] = x2;
+    xf[s] = (float)x0; xf[max_ns + s] = (float)x1; xf[2 * max_ns + s] = (float)x2;
     rt[s] = mbd_blend_site(w, p, s, a, n1, offs, offk1, x0, x1, x2);
   }
+  for (int e = tid; e < 9 * ns; e += blockDim.x) col[e] = 0.0;
+  for (int e = tid; e < N; e += blockDim.x) ex[e] = 0;
+  double* T = DENSE && w.tlr ? w.tlr + w.off_t[c] : nullptr;
+  if (T)   // diagonal blocks are zero
+    for (int e = tid; e < ns * 9; e += blockDim.x) {
+      int s = e / 9, t = e % 9;
+      T[(long long)(3 * s + t / 3) * N + 3 * s + t % 3] = 0.0;
+    }
   __syncthreads();
-  double* T = w.tlr + w.off_t[c];
-  // diagonal blocks are zero
-  for (int e = tid; e < ns * 9; e += blockDim.x) {
-    int s = e / 9, t = e % 9;
-    T[(long long)(3 * s + t / 3) * N + 3 * s + t % 3] = 0.0;
+  float4* rec = w.trec ? pair_record(w, c, 1, 0) : nullptr;
+  double* pco = DENSE && w.pcoef ? w.pcoef + w.off_t[c] : nullptr;
+  const ff d_ff = ff_from_double(p.d), beta_ff = ff_from_double(p.beta), ib_ff = ff_from_double(1.0 / p.r_buf);
+  const bool full = w.trec_full != 0;
+  auto pair = [&](int i, int j) {   // a coupled pair, i > j
+    const double rr[3] = {xs[j] - xs[i], xs[max_ns + j] - xs[max_ns + i], xs[2 * max_ns + j] - xs[2 * max_ns + i]};
+    const double rc = (j == 0) ? p.r_mbd1 : p.r_mbd2;
+    const int e = i * (i - 1) / 2 + j;
+    if (!DENSE || rec) {
+      const PairRec o = tlr_pair_record(p, d_ff, beta_ff, ib_ff, rr, rc, rt[i], rt[j], full);
+      rec[4LL * e] = o.v[0];
+      rec[4LL * e + 1] = o.v[1];
+      if (full) {
+        rec[4LL * e + 2] = o.v[2];
+        rec[4LL * e + 3] = o.v[3];
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        atomicMax(ex + 3 * i + a, o.top[a]);
+        atomicMax(ex + 3 * j + a, o.top[a]);
+      }
+    }
+    if (DENSE) {
+      double blk[3][3], kc[5];
+      tlr_pair_block(p, rr, rc, rt[i], rt[j], blk, pco ? kc : nullptr);
+      if (pco) {
+        double* pc = pco + 8LL * e;
+        pc[0] = rr[0]; pc[1] = rr[1]; pc[2] = rr[2];
+        pc[3] = kc[0]; pc[4] = kc[1]; pc[5] = kc[2]; pc[6] = kc[3]; pc[7] = kc[4];
+      }
+      if (T)
+#pragma unroll
+        for (int al = 0; al < 3; ++al)
+#pragma unroll
+          for (int be = 0; be < 3; ++be) {
+            T[(long long)(3 * i + al) * N + 3 * j + be] = blk[al][be];
+            T[(long long)(3 * j + al) * N + 3 * i + be] = blk[al][be];
+          }
+    }
+  };
+  auto empty = [&](int i, int j, int e) {   // an uncoupled pair
+    if (!DENSE || rec) {
+      rec[4LL * e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      rec[4LL * e + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (pco)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) pco[8LL * e + u] = 0.0;
+    if (T)
+#pragma unroll
+      for (int al = 0; al < 3; ++al)
+#pragma unroll
+        for (int be = 0; be < 3; ++be) {
+          T[(long long)(3 * i + al) * N + 3 * j + be] = 0.0;
+          T[(long long)(3 * j + al) * N + 3 * i + be] = 0.0;
+        }
+  };
+  // the column block of the central site in FP64: v_1 is formed from it below
+  for (int i = 1 + tid; i < ns; i += blockDim.x) {
+    const double rr[3] = {xs[0] - xs[i], xs[max_ns] - xs[max_ns + i], xs[2 * max_ns] - xs[2 * max_ns + i]};
+    double blk[3][3];
+    tlr_pair_block(p, rr, p.r_mbd1, rt[i], rt[0], blk, nullptr);
+#pragma unroll
+    for (int u = 0; u < 9; ++u) col[9 * i + u] = blk[u / 3][u % 3];
   }
   const int npair = ns * (ns - 1) / 2;
-  for (int e = tid; e < npair; e += blockDim.x) {
-    int i = (int)((sqrtf(8.0f * e + 1.0f) + 1.0f) * 0.5f);
-    while (i * (i - 1) / 2 > e) --i;
-    while ((i + 1) * i / 2 <= e) ++i;
-    int j = e - i * (i - 1) / 2;     // i > j
-    double rr[3] = {xs[j] - xs[i], xs[max_ns + j] - xs[max_ns + i], xs[2 * max_ns + j] - xs[2 * max_ns + i]};
-    double blk[3][3], kc[5];
-    tlr_pair_block(p, rr, (j == 0) ? p.r_mbd1 : p.r_mbd2, rt[i], rt[j], blk, w.pcoef ? kc : nullptr);
-    if (w.pcoef) {
-      double* pc = w.pcoef + w.off_t[c] + 8LL * (i * (i - 1) / 2 + j);
-      pc[0] = rr[0]; pc[1] = rr[1]; pc[2] = rr[2];
-      pc[3] = kc[0]; pc[4] = kc[1]; pc[5] = kc[2]; pc[6] = kc[3]; pc[7] = kc[4];
-    }
-#pragma unroll
-    for (int al = 0; al < 3; ++al)
-#pragma unroll
-      for (int be = 0; be < 3; ++be) {
-        T[(long long)(3 * i + al) * N + 3 * j + be] = blk[al][be];
-        T[(long long)(3 * j + al) * N + 3 * i + be] = blk[al][be];
+  int* qw = queue + 64 * warp;
+  int queued = 0;
+  for (int e0 = 32 * warp; e0 < npair; e0 += 32 * nw) {
+    const int e = e0 + lane;
+    bool in = false;
+    int i = 0, j = 0;
+    if (e < npair) {
+      i = (int)((sqrtf(8.0f * e + 1.0f) + 1.0f) * 0.5f);
+      while (i * (i - 1) / 2 > e) --i;
+      while ((i + 1) * i / 2 <= e) ++i;
+      j = e - i * (i - 1) / 2;     // i > j
+      const double rc = j == 0 ? p.r_mbd1 : p.r_mbd2, rc2 = rc * rc;
+      const float dx = xf[j] - xf[i], dy = xf[max_ns + j] - xf[max_ns + i], dz = xf[2 * max_ns + j] - xf[2 * max_ns + i];
+      const float r2 = dx * dx + dy * dy + dz * dz, c2 = (float)rc2;
+      if (r2 < c2 * (1.f - 1e-4f)) {
+        in = true;
+      } else if (!(r2 > c2 * (1.f + 1e-4f))) {
+        const double ex = xs[j] - xs[i], ey = xs[max_ns + j] - xs[max_ns + i], ez = xs[2 * max_ns + j] - xs[2 * max_ns + i];
+        in = ex * ex + ey * ey + ez * ez < rc2;
       }
+      if (!in) empty(i, j, e);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (in) qw[queued + __popc(m & ((1u << lane) - 1u))] = i << 16 | j;
+    queued += __popc(m);
+    __syncwarp();
+    if (queued >= 32) {
+      const int v = qw[lane];
+      pair(v >> 16, v & 0xffff);
+      queued -= 32;
+      const int rest = lane < queued ? qw[32 + lane] : 0;
+      __syncwarp();
+      if (lane < queued) qw[lane] = rest;
+      __syncwarp();
+    }
   }
-  __threadfence_block();
+  if (lane < queued) {
+    const int v = qw[lane];
+    pair(v >> 16, v & 0xffff);
+  }
   __syncthreads();
+  // row exponents of the digit planes: |T_row| < 2^e
+  if (rec && w.texp)
+    for (int e = tid; e < oz_mpad(N); e += blockDim.x)
+      w.texp[w.off_tr[c] + e] = e < N ? (ex[e] >> 23) - 126 : 0;
   // v_1 = G e_k: column block of the central site, scaled by D_s D_0 (per frequency)
   const int ncv = 3 * p.n_freq;
   double* V1 = w.vkr + (offs * 3) * ncv;
   for (int e = tid; e < N * ncv; e += blockDim.x) {
-    int row = e / ncv, col = e % ncv;
-    int s = row / 3, q = col / 3 + 1, be = col % 3;
+    int row = e / ncv, cc = e % ncv;
+    int s = row / 3, q = cc / 3 + 1, be = cc % 3;
     double d = w.dsq[(offs + s) * p.nq + q] * w.dsq[offs * p.nq + q];
-    V1[(long long)row * ncv + col] = d * T[(long long)row * N + be];
+    V1[(long long)row * ncv + cc] = d * col[3 * row + be];
   }
 }
 
@@ -965,9 +1127,14 @@ __global__ void __launch_bounds__(256) k_mbd_energy(Work w, DevParams p, int c0)
 
 void launch_mbd_prepare_sized(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return;
-  size_t sm = sizeof(double) * 4 * (size_t)max_ns;
-  raise_smem_limit((const void*)k_mbd_prepare, sm);
-  k_mbd_prepare<<<c1 - c0, 256, sm, s>>>(w, p, c0, max_ns);
+  const size_t sm = (sizeof(double) * 13 + sizeof(float) * 6) * (size_t)max_ns + sizeof(int) * 64 * 8;
+  if (w.tlr || w.pcoef) {
+    raise_smem_limit((const void*)k_mbd_prepare<true>, sm);
+    k_mbd_prepare<true><<<c1 - c0, 256, sm, s>>>(w, p, c0, max_ns);
+  } else {
+    raise_smem_limit((const void*)k_mbd_prepare<false>, sm);
+    k_mbd_prepare<false><<<c1 - c0, 256, sm, s>>>(w, p, c0, max_ns);
+  }
 }
 
 void launch_mbd_chain_sized(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, cudaStream_t s) {
@@ -1486,60 +1653,121 @@ void launch_forces_out(const Work& w, double* forces, cudaStream_t s) {
 // Kpad = 16 ceil(N/16); W^T digit planes [48][Kpad]; P and Q digit planes [3 ns16][Kp] with
 // ns16 = 16 ceil(ns/16) and Kp = 16 ceil(ncol/16).
 // =======================================================================================
-__device__ __forceinline__ int oz_mpad(int n) { return (n + 63) / 64 * 64; }
-__device__ __forceinline__ int oz_kpad(int n) { return (n + 15) / 16 * 16; }
 
-// T_LR digit planes and row exponents (one block per central atom, one warp per row).  Rows of
-// at most 32 SLT_REG entries are read once into registers; longer rows are read twice.
-#define SLT_REG 18
-template <int st>
-__global__ void __launch_bounds__(256) k_slice_t(Work w, int c0) {
+// T_LR digit planes from the pair records (the row exponents come with them): one block per central
+// atom, a warp per (site, 64 partners), a lane per two neighbouring partners: three rows by six
+// columns of every plane.  T_st = a r r^T - (a r^2 / 3) I with a = k3 / 4 is formed in float-float on
+// the FP32 pipe (~2^-45 against the 2^-42 of the digits), so T_LR itself is never stored: the FP64
+// matrix cost 12.3 GB of traffic per 4096-atom step on its way here.  The digits of a row pass
+// through shared memory into 16-byte stores; written straight from the lanes (4 bytes every 12) the
+// partial sectors took 1.22 ms per 1024 atoms, 0.99 ms now (65 % of the issue slots).
+struct TBlock {
+  ff v[6];   // xx, yy, zz, xy, xz, yz
+};
+__device__ __forceinline__ ff ff_prod(ff a, ff b) {   // a b, not renormalised
+  const float v = __fmul_rn(a.hi, b.hi);
+  return ff_make(v, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -v))));
+}
+__device__ __forceinline__ TBlock t_block(const float4* rec, int s, int t) {
+  const int i = max(s, t), j = min(s, t);
+  const float4* r = rec + 4u * (unsigned)(i * (i - 1) / 2 + j);
+  const float4 u = __ldg(r), v = __ldg(r + 1);
+  const ff x = ff_make(u.x, u.y), y = ff_make(u.z, u.w), z = ff_make(v.x, v.y);
+  const ff a = ff_make(0.25f * v.z, 0.25f * v.w);
+  const ff ax = ff_prod(a, x), ay = ff_prod(a, y), az = ff_prod(a, z);
+  const ff xx = ff_prod(ax, x), yy = ff_prod(ay, y), zz = ff_prod(az, z);
+  const ff s1 = ff_two_sum(xx.hi, yy.hi), s2 = ff_two_sum(s1.hi, zz.hi);
+  const ff sum = ff_make(s2.hi, (s1.lo + s2.lo) + (xx.lo + yy.lo + zz.lo));
+  const ff b = ff_prod(sum, ff_make(-0.33333334f, 9.934108e-9f));   // -a r^2 / 3
+  TBlock o;
+  auto diag = [&](ff q) {
+    const ff m = ff_two_sum(q.hi, b.hi);
+    return ff_quick_two_sum(m.hi, m.lo + (q.lo + b.lo));
+  };
+  o.v[0] = diag(xx); o.v[1] = diag(yy); o.v[2] = diag(zz);
+  const ff xy = ff_prod(ax, y), xz = ff_prod(ax, z), yz = ff_prod(ay, z);
+  o.v[3] = ff_quick_two_sum(xy.hi, xy.lo); o.v[4] = ff_quick_two_sum(xz.hi, xz.lo); o.v[5] = ff_quick_two_sum(yz.hi, yz.lo);
+  return o;
+}
+// index of entry (a, b) of the symmetric block
+__host__ __device__ constexpr int t_idx(int a, int b) { return a == b ? a : (a + b == 1 ? 3 : (a + b == 2 ? 4 : 5)); }
+
+// Six signed 7-bit digits of v relative to 2^e (s1 s2 = 2^(42 - e)), rounded to nearest (the first may
+// be 128), as bf16 bits in the upper half of each word: |v| 2^(42-e) as two 21-bit integers, read
+// off the mantissas of FP32 sums with 1.5 2^23.
+__device__ __forceinline__ void t_digits(ff v, float s1, float s2, unsigned (&d)[6]) {
+  const float big = 12582912.f;
+  const unsigned sg = __float_as_uint(v.hi) & 0x80000000u;
+  const float h = fabsf(v.hi) * s1 * s2, l = __uint_as_float(__float_as_uint(v.lo) ^ sg) * s1 * s2;
+  const float tm = __fmaf_rn(h, 0x1p-21f, big);
+  const float r = __fadd_rn(__fmaf_rn(__fsub_rn(tm, big), -0x1p21f, h), l);
+  const int b = __float_as_int(__fadd_rn(r, big)) - 0x4B400000;   // in (-2^21, 2^21)
+  const unsigned a = (__float_as_uint(tm) & 0x3fffffu) + (unsigned)(b >> 21), lo = (unsigned)b & 0x1fffffu;
+  const float one = __uint_as_float(0x3f800000u | sg), off = -8388608.f * one;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const unsigned x = (k < 3 ? a : lo) >> (7 * (2 - k % 3));
+    const unsigned q = k % 3 == 0 ? x : x & 127u;
+    d[k] = __float_as_uint(__fmaf_rn(__uint_as_float(0x4B000000u | q), one, off));
+  }
+}
+
+#define SLT_W 96   // words of a row that a warp forms at once (64 partners)
+__global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
+  extern __shared__ float2 sl_scale[];   // 2^(42 - e) of every row in two factors (it can pass the FP32 range)
+  __shared__ __align__(16) unsigned stage[8][6 * SLT_W];
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
-  const int N = 3 * w.counts[c].ns, Mpad = oz_mpad(N), Kpad = oz_kpad(N);
-  const double* T = w.tlr + w.off_t[c];
+  constexpr int st = 6;
+  const int ns = w.counts[c].ns, N = 3 * ns, Mpad = oz_mpad(N), Kpad = oz_kpad(N);
+  const float4* rec = pair_record(w, c, 1, 0);
   // row pitch: the centre's Kpad, or the common pitch tk of the tcgen05 path (zeros past N)
   const int ld = w.tk > 0 ? w.tk : Kpad;
-  unsigned short* base = w.tk > 0 ? w.tdig + w.off_tr[c] * st * w.tk : w.tdig + w.off_tq[c] * st;
-  const long long plane = (long long)Mpad * ld;
+  unsigned* base = reinterpret_cast<unsigned*>(w.tk > 0 ? w.tdig + w.off_tr[c] * st * w.tk : w.tdig + w.off_tq[c] * st);
+  const int lw = ld / 2;                            // words per row, a multiple of 8
+  const long long plane = (long long)Mpad * lw;
+  const int* texp = w.texp + w.off_tr[c];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (N <= 32 * SLT_REG) {
-    // one read of T: the row stays in registers between its exponent and its digits
-    for (int row = warp; row < Mpad; row += nw) {
-      double v[SLT_REG];
-      int mx = 0;
-#pragma unroll
-      for (int k = 0; k < SLT_REG; ++k) {
-        const int j = lane + 32 * k;
-        v[k] = (row < N && j < N) ? T[(long long)row * N + j] : 0.0;
-        mx = max(mx, oz_biased_exp(v[k]));
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const int e = oz_scale_exp(mx);
-      if (lane == 0) w.texp[w.off_tr[c] + row] = e;
-#pragma unroll
-      for (int k = 0; k < SLT_REG; ++k) {
-        const int j = lane + 32 * k;
-        if (j < ld) oz_store_digits<st>(base + (long long)row * ld + j, plane, v[k], e);
-      }
-      for (int j = lane + 32 * SLT_REG; j < ld; j += 32) oz_store_digits<st>(base + (long long)row * ld + j, plane, 0.0, e);
-    }
-    return;
+  for (int r = threadIdx.x; r < N; r += blockDim.x) {
+    const int up = 42 - texp[r], u1 = min(up, 100);
+    sl_scale[r] = make_float2(__int_as_float((u1 + 127) << 23), __int_as_float((up - u1 + 127) << 23));
   }
-  for (int row = warp; row < Mpad; row += nw) {
-    int mx = 0;
-    if (row < N)
-      for (int j = lane; j < N; j += 32) mx = max(mx, oz_biased_exp(T[(long long)row * N + j]));
+  __syncthreads();
+  const int nch = (lw + SLT_W - 1) / SLT_W;
+  unsigned* buf = stage[warp];
+  for (int e = warp; e < ns * nch; e += nw) {
+    const int s = e / nch, ch = e - s * nch;
+    TBlock o[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    const int e = oz_scale_exp(mx);
-    if (lane == 0) w.texp[w.off_tr[c] + row] = e;
-    for (int j = lane; j < ld; j += 32) {
-      const double v = (row < N && j < N) ? T[(long long)row * N + j] : 0.0;
-      oz_store_digits<st>(base + (long long)row * ld + j, plane, v, e);
+    for (int h = 0; h < 2; ++h) {
+      const int t = 64 * ch + 2 * lane + h;
+#pragma unroll
+      for (int u = 0; u < 6; ++u) o[h].v[u] = ff_make(0.f, 0.f);
+      if (t < ns && t != s) o[h] = t_block(rec, s, t);
+    }
+    const int quads = min(SLT_W, lw - SLT_W * ch) / 4;   // 16-byte pieces of the chunk
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float2 sc = sl_scale[3 * s + a];
+      unsigned d[6][6];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) t_digits(o[q / 3].v[t_idx(a, q % 3)], sc.x, sc.y, d[q]);
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < st; ++k)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) buf[k * SLT_W + 3 * lane + q] = __byte_perm(d[2 * q][k], d[2 * q + 1][k], 0x7632);
+      __syncwarp();
+      uint4* row = reinterpret_cast<uint4*>(base + (long long)(3 * s + a) * lw + SLT_W * ch);
+      for (int i = lane; i < 6 * (SLT_W / 4); i += 32) {
+        const int k = i / (SLT_W / 4), u = i % (SLT_W / 4);
+        if (u < quads) row[k * (plane / 4) + u] = reinterpret_cast<const uint4*>(buf)[i];
+      }
     }
   }
+  // rows past N
+  for (int k = 0; k < st; ++k)
+    for (int j = threadIdx.x; j < (Mpad - N) * lw; j += blockDim.x) base[k * plane + (long long)N * lw + j] = 0u;
 }
 
 // W = D v_m digit planes (stored by column) and column exponents (one block per atom).
@@ -1629,14 +1857,6 @@ __global__ void __launch_bounds__(256) k_slice_pq(Work w, int c0) {
 }
 
 // Slicing launches for the digit counts in use (4 to 7; the products use 5 and 6).
-static void run_slice_t(const Work& w, int c0, int n, int st, cudaStream_t s) {
-  switch (st) {
-    case 4: k_slice_t<4><<<n, 256, 0, s>>>(w, c0); break;
-    case 5: k_slice_t<5><<<n, 256, 0, s>>>(w, c0); break;
-    case 6: k_slice_t<6><<<n, 256, 0, s>>>(w, c0); break;
-    default: k_slice_t<7><<<n, 256, 0, s>>>(w, c0); break;
-  }
-}
 static void run_slice_w(const Work& w, const DevParams& p, int m, int c0, int n, int sw, cudaStream_t s) {
   switch (sw) {
     case 4: k_slice_w<4><<<n, 256, 0, s>>>(w, p, m, c0); break;
@@ -1655,9 +1875,11 @@ static void run_slice_pq(const Work& w, int c0, int n, int sp, cudaStream_t s) {
   }
 }
 
-void launch_slice_t(const Work& w, int c0, int c1, int st, cudaStream_t s) {
+void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return;
-  run_slice_t(w, c0, c1 - c0, st, s);
+  const size_t sm = sizeof(float2) * 3 * (size_t)max_ns;
+  raise_smem_limit((const void*)k_slice_t, sm);
+  k_slice_t<<<c1 - c0, 256, sm, s>>>(w, c0);
 }
 
 void launch_slice_pq(const Work& w, int c0, int c1, int digits, cudaStream_t s) {

@@ -738,15 +738,6 @@ __device__ void cg_residual_update(const Work& w, const DevParams& p, int c, int
   }
 }
 
-// Compensated accumulation of the product a b (float-float operands) into (h, l).
-__device__ __forceinline__ void ff_mac(float& h, float& l, ff a, ff b) {
-  const float v = __fmul_rn(a.hi, b.hi);
-  const float e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -v)));
-  const ff m = ff_two_sum(h, v);
-  h = m.hi;
-  l = __fadd_rn(l, __fadd_rn(m.lo, e));
-}
-
 // Damped radial terms F A0, F B0 of pair t (of centre c) at SCS frequency q in float-float: F times
 // the atom-pair table entry, on the FP32 pipe.
 __device__ __noinline__ void pair_rad_slow(const Work& w, const DevParams& p, int c, int q, long long pq, ff& fa,
@@ -844,6 +835,23 @@ __device__ __forceinline__ void scs_list_for_lu(const Work& w, int id) {
   w.fb[1 + e] = id;
 }
 
+// dL/dX_i = delta/3 times this: dL/dalpha_K,i, plus dL/dalpha_I,c on the centre's block.
+__device__ __forceinline__ double adjoint_seed(const Work& w, const DevParams& p, int c, int q, int i) {
+  double v = w.alphaK_bar[(w.off_k1[c] + i) * p.nqs + q];
+  if (i == 0) v += w.alphaI_bar[(long long)c * p.nqs + q];
+  return v * (1.0 / 3.0);
+}
+// Biased exponent of the largest seed of a system (every warp by itself), 0x7ff if one is not finite:
+// the adjoint systems are solved, and their solutions kept, at unit size (lambda = 2^lexp lsol),
+// since a caller's weights may be of any magnitude.
+__device__ __forceinline__ int adjoint_exponent(const Work& w, const DevParams& p, int c, int q, int n1) {
+  int top = 1;
+  for (int i = threadIdx.x & 31; i < n1; i += 32)
+    top = max(top, (int)((__double_as_longlong(adjoint_seed(w, p, c, q, i)) >> 52) & 0x7ff));
+  top = __reduce_max_sync(0xffffffffu, top);
+  return top == 0x7ff ? top : min(top, 2045);
+}
+
 // One (centre, frequency) system per block of 32 S (3 / NC) threads.  ADJ = false: X = B^-1 d to FP64
 // accuracy (2^-52), alpha_K and alpha_I.  ADJ = true: lambda = B^-1 dL/dX, to 2^-30 of its largest
 // value or better (it feeds the forces only).  The refinement measures its own contraction.
@@ -895,29 +903,17 @@ __global__ void __launch_bounds__(32 * S * (3 / NC), cg_min_blocks(S, NC))
     const float s = sm.s[ij.x] * sm.s[ij.y];
     sm.F[ij.x * (ij.x + 1) / 2 + ij.y] = make_float2(f.x * s, f.z * s);
   }
-  double scale = 1.0;
   if (!ADJ) {
     cg_build_rhs(w, p, c, q, n1, R);
   } else {
-    // dL/dX_i = delta/3 times dL/dalpha_K,i, plus dL/dalpha_I,c on the centre's block, scaled by
-    // a power of two to unit size (the weights of a caller may be of any magnitude)
-    double gv = 0.0;
-    int top = 0;
-    for (int i = tid & 31; i < n1; i += 32) {   // every warp finds the largest exponent of all sites
-      double v = w.alphaK_bar[(offk1 + i) * p.nqs + q];
-      if (i == 0) v += w.alphaI_bar[id];
-      v *= 1.0 / 3.0;
-      if (i == gt) gv = v;
-      top = max(top, (int)((__double_as_longlong(v) >> 52) & 0x7ff));
-    }
-    top = __reduce_max_sync(0xffffffffu, top);
+    const int top = adjoint_exponent(w, p, c, q, n1);
     if (top == 0x7ff) {   // not finite: no solution (uniform over the block)
       if (tid == 0) atomicOr(w.status, LMBD_FLAG_NOT_CONVERGED);
       return;
     }
-    top = min(max(top, 1), 2045);
+    if (tid == 0) w.lexp[id] = top - 1023;
     const double up = __longlong_as_double((long long)(2046 - top) << 52);
-    scale = __longlong_as_double((long long)top << 52);
+    const double gv = gt < n1 ? adjoint_seed(w, p, c, q, gt) : 0.0;
     if (gt < n1)
 #pragma unroll
       for (int k = 0; k < NC; ++k)
@@ -989,7 +985,7 @@ __global__ void __launch_bounds__(32 * S * (3 / NC), cg_min_blocks(S, NC))
 #pragma unroll
     for (int k = 0; k < NC; ++k)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) Ri[3 * a + c0 + k] = ADJ ? xd[k][a] * scale : xd[k][a];
+      for (int a = 0; a < 3; ++a) Ri[3 * a + c0 + k] = xd[k][a];
   if (!ADJ) {   // alpha_K,i = Tr(X_i) / 3, alpha_I,c = alpha_K,0
     __threadfence_block();
     __syncthreads();
@@ -1097,6 +1093,8 @@ __global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, in
   const int nk1 = w.prow[rbase + n1], np = w.prow_k2[rbase + n1];
   const double* Xg = w.xsol + w.off_k1[c] * p.nqs * 9;
   const double* Lg = w.lsol + w.off_k1[c] * p.nqs * 9;
+  int lexp = -2000;   // the block works at the largest scale of its frequencies
+  for (int q = qb; q < qe; ++q) lexp = max(lexp, w.lexp[(long long)c * p.nqs + q]);
   const int qc = max(1, min(per, smem / (144 * n1)));   // frequencies staged at once
   float2* Ls = reinterpret_cast<float2*>(smem_raw);   // [qc][9 n1] lambda
   float2* Xs = Ls + qc * 9 * n1;                      // [qc][9 n1] X
@@ -1108,8 +1106,10 @@ __global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, in
     const bool first = q0 == qb, last = q0 + nqc == qe;
     __syncthreads();
     for (int e = tid; e < nqc * 9 * n1; e += blockDim.x) {
+      const int down = w.lexp[(long long)c * p.nqs + q0 + e / (9 * n1)] - lexp;
+      const float f = down < -126 ? 0.f : __int_as_float((down + 127) << 23);
       const ff l = ff_from_double(Lg[(long long)q0 * 9 * n1 + e]), x = ff_from_double(Xg[(long long)q0 * 9 * n1 + e]);
-      Ls[e] = make_float2(l.hi, l.lo);
+      Ls[e] = make_float2(l.hi * f, l.lo * f);
       Xs[e] = make_float2(x.hi, x.lo);
     }
     __syncthreads();
@@ -1201,6 +1201,7 @@ __global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, in
   }
   __threadfence_block();
   __syncthreads();
+  const double scale = __longlong_as_double((long long)(min(max(lexp, -1022), 1023) + 1023) << 52);
   // per site (fixed order): owner of its row's pairs (-g), partner of K1 pairs owned by later rows
   // (+g, from the adjacency row) and of K2 pairs (+g, from the reverse list)
   for (int s = tid; s < n12; s += blockDim.x) {
@@ -1231,7 +1232,7 @@ __global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, in
 #pragma unroll 4
       for (int t = w.k2ptr[sbase + s]; t < e; ++t) acc(__ldg(w.k2rev + offp + t), true);
     }
-    const double gx = ff_to_double(gs[0]), gy = ff_to_double(gs[1]), gz = ff_to_double(gs[2]);
+    const double gx = ff_to_double(gs[0]) * scale, gy = ff_to_double(gs[1]) * scale, gz = ff_to_double(gs[2]) * scale;
     if (gx != 0.0 || gy != 0.0 || gz != 0.0) atomic_add3(w.gacc + 3 * a, gx, gy, gz);
   }
 }
@@ -1422,26 +1423,20 @@ __global__ void __launch_bounds__(256) k_scs_lu_adjoint(Work w, DevParams p, int
     const int id = w.fb[1 + e], c = id / p.nqs, q = id % p.nqs;
     if (c < c0 || c >= c1) continue;
     const int n1 = w.counts[c].n1, N1 = 3 * n1;
-    const long long offk1 = w.off_k1[c];
     scs2_dense_b(w, p, c, q, n1, A);
     if (!lu_factor_dense(A, N1, sm.piv, sm.red, sm.redi)) {
       if (threadIdx.x == 0) atomicOr(w.status, LMBD_FLAG_NOT_SPD);
       __syncthreads();
       continue;
     }
-    for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x) {
-      const int i = u / 9, a = (u % 9) / 3, k = u % 3;
-      double g = 0.0;
-      if (a == k) {
-        g = w.alphaK_bar[(offk1 + i) * p.nqs + q];
-        if (i == 0) g += w.alphaI_bar[id];
-        g *= 1.0 / 3.0;
-      }
-      sm.x[u] = g;
-    }
+    const int top = min(adjoint_exponent(w, p, c, q, n1), 2045);   // not finite: stays so
+    const double up = __longlong_as_double((long long)(2046 - top) << 52);
+    if (threadIdx.x == 0) w.lexp[id] = top - 1023;
+    for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x)
+      sm.x[u] = (u % 9) / 3 == u % 3 ? adjoint_seed(w, p, c, q, u / 9) * up : 0.0;
     __syncthreads();
     lu_solve3_dense(A, N1, sm.piv, sm.x);
-    double* lam = w.lsol + offk1 * p.nqs * 9 + (long long)q * N1 * 3;
+    double* lam = w.lsol + w.off_k1[c] * p.nqs * 9 + (long long)q * N1 * 3;
     for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x) lam[u] = sm.x[u];
     __syncthreads();
   }

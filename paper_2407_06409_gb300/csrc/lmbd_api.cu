@@ -276,6 +276,8 @@ struct Layout {
   int nqs;   // frequencies of the SCS solves (stage-1 arrays)
   int tk;    // tcgen05 path: row pitch of the T and W digit planes (0: per-centre Kpad)
   bool sparse;   // block-sparse T_LR: coupled pairs and float-float chain/pair operands
+  bool dense_t;  // FP64 T_LR kept (Lanczos-based modes, the paper's forces, FP64 products)
+  bool rec_pair; // the pair adjoint reads float-float records instead of FP64 coefficients
   int gs_ld;     // float2 per pair of the SCS adjoint's gradient scratch
 
   // stage 1 (SCS): pair lists, FP32 factors and solutions of centres [c0, c1)
@@ -336,12 +338,15 @@ struct Layout {
     const long long np0 = o.at(O_NP, c0), npn = o.span(O_NP, c0, c1);
     double* alphaT = cv.take<double>((long long)nq * ns, (long long)nq * s0);
     double* dsq = cv.take<double>((long long)nq * ns, (long long)nq * s0);
-    double* tlr = sparse ? nullptr : cv.take<double>(nt, t0);
+    double* tlr = dense_t ? cv.take<double>(nt, t0) : nullptr;
+    float4* trec = sliced_chain || rec_pair ? cv.take<float4>(2 * (nt / 9), 2 * (t0 / 9)) : nullptr;
     double* vkr = cv.take<double>((long long)nvec * ns * 3 * ncv, s0 * 3 * ncv);
     if (w) {
       w->alphaT = alphaT;
       w->dsq = dsq;
       w->tlr = tlr;
+      w->trec = trec;
+      w->trec_full = rec_pair;
       w->vkr = vkr;
       w->vstride = ns * 3 * ncv;
     }
@@ -391,7 +396,7 @@ struct Layout {
       float2* pff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       float2* qff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       double* x0buf = cv.take<double>(9 * ns, 9 * s0);
-      double* pcoef = sparse ? cv.take<double>(8 * npn, 8 * np0) : cv.take<double>(nt, t0);
+      double* pcoef = rec_pair ? nullptr : (sparse ? cv.take<double>(8 * npn, 8 * np0) : cv.take<double>(nt, t0));
       double* rbar = cv.take<double>(ns, s0);
       if (w) {
         w->gbar = gbar;
@@ -863,9 +868,10 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   w.alphaK = (double*)c->alphaK.p;
   w.rad_ab = (double*)c->rad_ab.p;
   w.rad_ff = (float2*)c->rad_ff.p;
-  TRY(ensure(c->abff, sizeof(float2) * 2 * (size_t)N * nq));
+  TRY(ensure(c->abff, (sizeof(float2) * 2 + sizeof(int)) * (size_t)N * nq));
   w.abff = (float2*)c->abff.p;
   w.iabff = w.abff + (size_t)N * nq;
+  w.lexp = reinterpret_cast<int*>(w.iabff + (size_t)N * nq);
   w.nvec = nvec;
   w.ncol = ncol;
   if (sliced_chain) {
@@ -910,6 +916,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   // ---- waves under the memory budget --------------------------------------------------------
   const Layout L{nq, ncv, nvec, ncol, (ncol + 15) / 16 * 16, ST, DIG_P, c->site_cap, forces, sliced_chain,
                  sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 15) / 16 * 16 : 0, sparse,
+                 !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), forces && sliced_pair && tc05 && !dp.paper,
                  scs_contract_scratch(N, max_n1, dp.nqs)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };
   auto s1x = [&](int a, int b) { return forces ? L.scs_adjoint(o, a, b, nullptr, nullptr) : (size_t)0; };
@@ -1063,7 +1070,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
           launch_sp_prepare(w, dp, cc, cc + 1, max_ns, s);
         else
           launch_mbd_prepare_sized(w, dp, cc, cc + 1, max_ns, s);
-        if (sliced_chain) launch_slice_t(w, cc, cc + 1, ST, s);
+        if (sliced_chain) launch_slice_t(w, cc, cc + 1, max_ns, s);
         if (dp.lanczos) {
           if (!launch_series_coefficients(w, dp, cc, cc + 1, max_ns, s)) return LMBD_ECAPACITY;
           phase_launch[LMBD_PHASE_PREPARE] += 2;
@@ -1092,7 +1099,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
         launch_sp_prepare(w, dp, c0, c1, max_ns, s);
       else
         launch_mbd_prepare_sized(w, dp, c0, c1, max_ns, s);
-      if (sliced_chain) launch_slice_t(w, c0, c1, ST, s);
+      if (sliced_chain) launch_slice_t(w, c0, c1, max_ns, s);
       if (dp.lanczos) {
         if (!launch_series_coefficients(w, dp, c0, c1, max_ns, s)) return LMBD_ECAPACITY;
         phase_launch[LMBD_PHASE_PREPARE] += 2;

@@ -135,7 +135,8 @@ struct Work {
   int* k2rev;                  // per centre (off_p): pair indices grouped by K2 partner
   float2* gstage;              // SCS-adjoint pair gradients, 3 float-float per pair and block of a centre
                                // (with frequencies in chunks: 14 sums)
-  double* lsol;                // adjoint solutions lambda = B^-1 dL/dX, off_k1 * nq * 9
+  double* lsol;                // adjoint solutions lambda = B^-1 dL/dX 2^-lexp, off_k1 * nq * 9
+  int* lexp;                   // N x nqs: their exponents
   float2* abff;                // N x nqs: alpha_bar as float-float
   float2* iabff;               // N x nqs: 1 / alpha_bar as float-float
   // LU fallback of the SCS solves (systems in which the conjugate gradients meet a direction of
@@ -174,7 +175,11 @@ struct Work {
   double* alphaI;              // N x nq
   // stage 2 (MBD)
   double* alphaT;              // blended alpha, off_s * nq
-  double* tlr;                 // T_LR, off_t
+  double* tlr;                 // T_LR, off_t (NULL when only its digit planes and records are needed)
+  // site-pair records in float-float, 4 float4 per pair (s > t) from 2 off_t / 9: (rx, ry),
+  // (rz, k3), then with forces (k1, k2), (k4, k5); k3 = 12 f_LR f / r^5 = 0 for uncoupled pairs
+  float4* trec;
+  int trec_full;               // the second half is written (the tcgen05 pair kernel reads it)
   double* dsq;                 // sqrt(alpha~), off_s * nq
   double* vkr;                 // Krylov vectors: nvec blocks of (off_s total * 3) x (3 n_freq)
   int nvec;
@@ -371,6 +376,11 @@ __device__ __forceinline__ void tlr_pair_block(const DevParams& p, const double 
   }
 }
 
+// the record of site pair (s, t), s > t, of centre c
+__device__ __forceinline__ float4* pair_record(const Work& w, int c, int s, int t) {
+  return w.trec + 2 * (w.off_t[c] / 9) + 4LL * (s * (s - 1) / 2 + t);
+}
+
 // atomicAdd for doubles is native on sm_60+.
 __device__ __forceinline__ void atomic_add3(double* p, double a, double b, double c) {
   atomicAdd(p, a);
@@ -431,7 +441,7 @@ void launch_sp_prepare(const Work& w, const DevParams& p, int c0, int c1, int ma
 void launch_sp_chain(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, cudaStream_t s);
 void launch_sp_adj_pair(const Work& w, const DevParams& p, int c0, int c1, int max_pairs, cudaStream_t s);
 void launch_forces_out(const Work& w, double* forces, cudaStream_t s);
-void launch_slice_t(const Work& w, int c0, int c1, int st, cudaStream_t s);
+void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s);   // T_LR digit planes, 6 digits
 void launch_chain_oz2(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, int digits, int st,
                       cudaStream_t s);
 // W = D v_m digit planes for chain step m (one block per central atom)

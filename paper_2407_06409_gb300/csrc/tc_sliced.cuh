@@ -38,15 +38,16 @@
 #define TCS_TMEM_COLS 512            // tensor-memory allocation per CTA
 #define TCS_WAIT_CYCLES (1LL << 32)  // about two seconds at 2 GHz
 
-template <int S, int NB>
+// NBUF slots and COLS tensor-memory columns: 3 and 512 for one CTA per SM, 2 and 256 for two.
+template <int S, int NB, int NBUF = TCS_NBUF, int COLS = TCS_TMEM_COLS>
 struct TcsShape {
   static constexpr int kAPlane = TCS_M * TCS_KS * 2;
   static constexpr int kBPlane = NB * TCS_KS * 2;
   static constexpr int kSlot = S * (kAPlane + kBPlane);
-  static constexpr int kBytes = TCS_NBUF * kSlot + 1024;  // + slack to align the ring to 1024 B
+  static constexpr int kBytes = NBUF * kSlot + 1024;  // + slack to align the ring to 1024 B
   static constexpr int kGroupCols = NB;                    // TMEM columns per digit order
   static constexpr int kPlanesPerMma = 256 / NB;           // B planes per MMA (N <= 256)
-  static_assert(S * kGroupCols <= TCS_TMEM_COLS, "accumulators exceed the tensor-memory allocation");
+  static_assert(NBUF <= TCS_NBUF && S * kGroupCols <= COLS, "accumulators exceed the tensor-memory allocation");
   static_assert(NB % 16 == 0 && NB >= 16 && NB <= 256, "N of an M = 128 tcgen05.mma");
   static_assert(kBPlane % 512 == 0, "swizzled tiles start on 512-byte boundaries");
 };
@@ -72,15 +73,16 @@ struct TcsBarriers {
 };
 
 // Block-wide set-up: tensor memory (warp 0) and the mbarriers.  Returns the TMEM base.
+template <int NBUF = TCS_NBUF, int COLS = TCS_TMEM_COLS>
 __device__ __forceinline__ uint32_t tcs_setup(TcsBarriers& bar) {
   const int warp = threadIdx.x >> 5;
   if (warp == 0) {
-    tc_alloc(&bar.tmem, TCS_TMEM_COLS);
+    tc_alloc(&bar.tmem, COLS);
     tc_relinquish();
   }
   if (threadIdx.x == 32) {
 #pragma unroll
-    for (int b = 0; b < TCS_NBUF; ++b) {
+    for (int b = 0; b < NBUF; ++b) {
       tc_mbar_init(&bar.full[b], 1);
       tc_mbar_init(&bar.empty[b], 1);
     }
@@ -102,20 +104,21 @@ struct TcsProgress {
 // Block-wide tear-down.  After an abort, thread 0 waits (bounded) for the copies it issued, the
 // MMAs it committed and their commits' arrivals, so nothing lands in shared or tensor memory
 // after the block is gone; then tensor memory is freed.
+template <int NBUF = TCS_NBUF, int COLS = TCS_TMEM_COLS>
 __device__ __forceinline__ void tcs_teardown(TcsBarriers& bar, bool abort, const TcsProgress& pr, int* status) {
   if (abort && threadIdx.x == 0) {
     atomicOr(status, LMBD_FLAG_TIMEOUT);
     for (int s = pr.committed + 1; s <= pr.issued; ++s)
-      tc_mbar_wait(&bar.full[s % TCS_NBUF], (s / TCS_NBUF) & 1, TCS_WAIT_CYCLES);
+      tc_mbar_wait(&bar.full[s % NBUF], (s / NBUF) & 1, TCS_WAIT_CYCLES);
     if (pr.committed >= 0)
-      tc_mbar_wait(&bar.empty[pr.committed % TCS_NBUF], (pr.committed / TCS_NBUF) & 1, TCS_WAIT_CYCLES);
+      tc_mbar_wait(&bar.empty[pr.committed % NBUF], (pr.committed / NBUF) & 1, TCS_WAIT_CYCLES);
     if (pr.acc >= 0) tc_mbar_wait(&bar.acc, pr.acc & 1, TCS_WAIT_CYCLES);
   }
   tc_fence_before();
   __syncthreads();
   if ((threadIdx.x >> 5) == 0) {
     tc_fence_after();
-    tc_dealloc(bar.tmem, TCS_TMEM_COLS);
+    tc_dealloc(bar.tmem, COLS);
   }
 }
 
@@ -128,16 +131,16 @@ __device__ __forceinline__ uint32_t tcs_lane_addr(uint32_t tmem, int col) {
 // consume() runs block-wide at the end of every K chunk with the accumulators complete in TMEM.
 // Every wait is bounded by `budget` cycles; returns false if one ran out.  `pr` (thread 0) keeps
 // what is in flight, for the tear-down.
-template <int S, int NB, class Consume>
+template <int S, int NB, int NBUF = TCS_NBUF, int COLS = TCS_TMEM_COLS, class Consume>
 __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B, int K, uint32_t sbase,
                                              TcsBarriers& bar, long long budget, TcsProgress& pr, Consume&& consume) {
-  using Sh = TcsShape<S, NB>;
+  using Sh = TcsShape<S, NB, NBUF, COLS>;
   const int tid = threadIdx.x;
   const int nst = (K + TCS_KS - 1) / TCS_KS;
   constexpr int kPerChunk = OZ_KCHUNK / TCS_KS;
   const uint32_t tmem = bar.tmem;
   auto load = [&](int s) {
-    const int slot = s % TCS_NBUF;
+    const int slot = s % NBUF;
     const uint32_t sA = sbase + slot * Sh::kSlot;
     const uint32_t sB = sA + S * Sh::kAPlane;
     tc_mbar_expect_tx(&bar.full[slot], (uint32_t)Sh::kSlot);
@@ -148,15 +151,15 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
     pr.issued = s;
   };
   if (tid == 0)
-    for (int s = 0; s < TCS_NBUF && s < nst; ++s) load(s);
+    for (int s = 0; s < NBUF && s < nst; ++s) load(s);
   const int nchunk = (nst + kPerChunk - 1) / kPerChunk;
   for (int ch = 0; ch < nchunk; ++ch) {
     const int s0 = ch * kPerChunk, s1 = min(nst, s0 + kPerChunk);
     bool to = false;
     if (tid == 0) {
       for (int s = s0; s < s1; ++s) {
-        const int slot = s % TCS_NBUF;
-        if (!tc_mbar_wait(&bar.full[slot], (s / TCS_NBUF) & 1, budget)) {
+        const int slot = s % NBUF;
+        if (!tc_mbar_wait(&bar.full[slot], (s / NBUF) & 1, budget)) {
           to = true;
           break;
         }
@@ -179,10 +182,10 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
           }
         tc_commit(&bar.empty[slot]);
         pr.committed = s;
-        // refill the slot of stage s - 1 with stage s - 1 + TCS_NBUF once its MMAs are done
-        const int r = s - 1 + TCS_NBUF;
+        // refill the slot of stage s - 1 with stage s - 1 + NBUF once its MMAs are done
+        const int r = s - 1 + NBUF;
         if (s >= 1 && r < nst) {
-          if (!tc_mbar_wait(&bar.empty[(s - 1) % TCS_NBUF], ((s - 1) / TCS_NBUF) & 1, budget)) {
+          if (!tc_mbar_wait(&bar.empty[(s - 1) % NBUF], ((s - 1) / NBUF) & 1, budget)) {
             to = true;
             break;
           }
