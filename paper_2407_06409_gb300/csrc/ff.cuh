@@ -24,6 +24,18 @@ __device__ __forceinline__ ff ff_from_double(double x) {
   return ff_make(hi, lo);
 }
 
+// The same up to truncation (47 bits kept) by integer and FP32 instructions, for kernels whose FP64
+// pipe is the bound: hi = the top 24 bits, lo = the next 23.  Finite values in the FP32 range;
+// smaller ones give zero.
+__device__ __forceinline__ ff ff_split(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), sg = h & 0x80000000u;
+  const int e = (int)((h >> 20) & 0x7ffu) - (1023 - 127);   // biased FP32 exponent
+  const unsigned hb = ((unsigned)max(e, 0) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);
+  const float low = __fsub_rn(__uint_as_float(0x4B000000u | ((l >> 6) & 0x7fffffu)), 8388608.f);
+  const float unit = __uint_as_float(sg | ((unsigned)max(e - 46, 0) << 23));   // 2^-46 of the leading bit
+  return e > 0 ? ff_make(__uint_as_float(sg | hb), __fmul_rn(low, unit)) : ff_make(0.f, 0.f);
+}
+
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 
 __device__ __forceinline__ ff ff_quick_two_sum(float a, float b) {   // |a| >= |b|

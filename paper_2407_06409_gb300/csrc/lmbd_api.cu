@@ -278,6 +278,7 @@ struct Layout {
   bool sparse;   // block-sparse T_LR: coupled pairs and float-float chain/pair operands
   bool dense_t;  // FP64 T_LR kept (Lanczos-based modes, the paper's forces, FP64 products)
   bool rec_pair; // the pair adjoint reads float-float records instead of FP64 coefficients
+  bool pq_fp64;  // FP64 P and Q kept (FP64 products, more than 32 integrand frequencies)
   int gs_ld;     // float2 per pair of the SCS adjoint's gradient scratch
 
   // stage 1 (SCS): pair lists, FP32 factors and solutions of centres [c0, c1)
@@ -391,8 +392,8 @@ struct Layout {
       const long long nc = ncol > 0 ? ncol : 1;
       double* gbar = cv.take<double>((long long)nq * ns, (long long)nq * s0);
       // P and Q: FP64 for the dense products, float-float for the sparse pair products
-      double* pmat = sparse ? nullptr : cv.take<double>(3 * ns * nc, 3 * s0 * nc);
-      double* qmat = sparse ? nullptr : cv.take<double>(3 * ns * nc, 3 * s0 * nc);
+      double* pmat = pq_fp64 ? cv.take<double>(3 * ns * nc, 3 * s0 * nc) : nullptr;
+      double* qmat = pq_fp64 ? cv.take<double>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       float2* pff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       float2* qff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       double* x0buf = cv.take<double>(9 * ns, 9 * s0);
@@ -917,6 +918,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   const Layout L{nq, ncv, nvec, ncol, (ncol + 15) / 16 * 16, ST, DIG_P, c->site_cap, forces, sliced_chain,
                  sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 15) / 16 * 16 : 0, sparse,
                  !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), forces && sliced_pair && tc05 && !dp.paper,
+                 !sparse && (!sliced_pair || dp.paper || nf > 32),
                  scs_contract_scratch(N, max_n1, dp.nqs)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };
   auto s1x = [&](int a, int b) { return forces ? L.scs_adjoint(o, a, b, nullptr, nullptr) : (size_t)0; };

@@ -192,7 +192,7 @@ struct Work {
   double* cfit;                // N x n_freq x LMBD_MAX_ORDER_P1: fitted c_n per centre and frequency
   double* lam;                 // N x n_freq x 2: Lanczos estimate of G's spectral interval
   const double* gl64;          // 64 Gauss-Legendre nodes on [-1, 1], then their weights
-  double* pmat;                // off_s*3 x ncol
+  double* pmat;                // off_s*3 x ncol (NULL: the series adjoint writes the digit planes of P and Q)
   double* qmat;                // off_s*3 x ncol
   int ncol;                    // 3 n_freq (n_max - 2)
   double* x0buf;               // off_s x 9, central-column term of the pair matrix
