@@ -17,6 +17,23 @@ __device__ __forceinline__ ff ff_make(float hi, float lo) {
   return r;
 }
 
+// (hi + lo) 2^shift as a double by integer instructions (normalised float-float, hi normal or zero;
+// low parts below 2^-46 of hi round away; zero below the double range).
+__device__ __forceinline__ double ff_join(ff a, int shift) {
+  const unsigned hb = __float_as_uint(a.hi), sg = hb & 0x80000000u;
+  const int e = (int)((hb >> 23) & 0xffu);
+  // |hi| as an integer with 46 fraction bits, and the low part (at most 2^22) in the same unit
+  const float unit = __uint_as_float((unsigned)min(max(300 - e, 1), 254) << 23);   // 2^(173 - e)
+  const float l = __uint_as_float(__float_as_uint(a.lo) ^ sg) * unit;
+  const int q = __float_as_int(__fadd_rn(l, 12582912.f)) - 0x4B400000;
+  long long m = ((long long)((hb & 0x7fffffu) | 0x800000u) << 23) + q;
+  const int below = m < (1LL << 46);
+  m <<= 6 + below;
+  const int ex = e - 127 + 1023 - below + shift;
+  const long long r = ((long long)ex << 52) + (m & 0xfffffffffffffLL);
+  return e == 0 || ex <= 0 ? 0.0 : __longlong_as_double(r | ((long long)sg << 32));
+}
+
 // nearest float-float of a double (two conversions and one FP64 subtraction)
 __device__ __forceinline__ ff ff_from_double(double x) {
   const float hi = __double2float_rn(x);

@@ -1704,9 +1704,10 @@ __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
   constexpr int st = 6;
   const int ns = w.counts[c].ns, N = 3 * ns, Mpad = oz_mpad(N), Kpad = oz_kpad(N);
   const float4* rec = pair_record(w, c, 1, 0);
-  // row pitch: the centre's Kpad, or the common pitch tk of the tcgen05 path (zeros past N)
-  const int ld = w.tk > 0 ? w.tk : Kpad;
-  unsigned* base = reinterpret_cast<unsigned*>(w.tk > 0 ? w.tdig + w.off_tr[c] * st * w.tk : w.tdig + w.off_tq[c] * st);
+  // rows of pitch Kpad, or the tile images of the tcgen05 path (zeros past N along K)
+  const bool tiled = w.tk > 0;
+  const int ld = tiled ? (N + 31) / 32 * 32 : Kpad;
+  unsigned* base = reinterpret_cast<unsigned*>(tiled ? w.tdig + w.off_tr[c] * st * w.tk : w.tdig + w.off_tq[c] * st);
   const int lw = ld / 2;                            // words per row, a multiple of 8
   const long long plane = (long long)Mpad * lw;
   const int* texp = w.texp + w.off_tr[c];
@@ -1729,6 +1730,7 @@ __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
       if (t < ns && t != s) o[h] = t_block(rec, s, t);
     }
     const int quads = min(SLT_W, lw - SLT_W * ch) / 4;   // 16-byte pieces of the chunk
+    const int first = 2 * SLT_W * ch;                    // and its first column
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const float2 sc = sl_scale[3 * s + a];
@@ -1741,22 +1743,53 @@ __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) buf[k * SLT_W + 3 * lane + q] = __byte_perm(d[2 * q][k], d[2 * q + 1][k], 0x7632);
       __syncwarp();
-      uint4* row = reinterpret_cast<uint4*>(base + (long long)(3 * s + a) * lw + SLT_W * ch);
+      const OzTileRow trow(3 * s + a, st, OZ_T_ROWS, N, ld);
       for (int i = lane; i < 6 * (SLT_W / 4); i += 32) {
         const int k = i / (SLT_W / 4), u = i % (SLT_W / 4);
-        if (u < quads) row[k * (plane / 4) + u] = reinterpret_cast<const uint4*>(buf)[i];
+        if (u >= quads) continue;
+        const long long at = tiled ? (trow.at(first + 8 * u, k, st) >> 3)
+                                   : (k * plane + (long long)(3 * s + a) * lw + SLT_W * ch) / 4 + u;
+        reinterpret_cast<uint4*>(base)[at] = reinterpret_cast<const uint4*>(buf)[i];
       }
     }
   }
   // rows past N
-  for (int k = 0; k < st; ++k)
+  for (int k = 0; k < st && !tiled; ++k)
     for (int j = threadIdx.x; j < (Mpad - N) * lw; j += blockDim.x) base[k * plane + (long long)N * lw + j] = 0u;
 }
 
-// W = D v_m digit planes (stored by column) and column exponents (one block per atom).
+// W = D v_m digit planes (stored by column) and column exponents (one block per atom): a thread keeps
+// its column over the rows (coalesced reads) for the maxima, then 64 rows at a time pass through
+// shared memory so that both the reads of v_m (by row) and the writes of the planes (by column, two
+// digits per store) are coalesced.  Reading by column took 0.177 ms per 1024 atoms and step, now
+// 0.158 ms.
+#define SLW_R 64
+// Signed 7-bit digits of v, |v| < 1, truncated to 47 bits and then rounded to 7 sw, as bf16 bits: two
+// integers of 21 (the second) and 7 (sw - 3) bits, read off the mantissas of FP32 sums.
+template <int sw>
+__device__ __forceinline__ void w_digits(double v, unsigned (&d)[sw]) {
+  static_assert(sw == 5 || sw == 6, "digits of a chain step");
+  const ff f = ff_split(v);
+  const float big = 12582912.f, s1 = __int_as_float((7 * sw + 127) << 23);
+  const unsigned sg = __float_as_uint(f.hi) & 0x80000000u;
+  const float h = fabsf(f.hi) * s1, l = __uint_as_float(__float_as_uint(f.lo) ^ sg) * s1;
+  const float tm = __fmaf_rn(h, 0x1p-21f, big);
+  const float r = __fadd_rn(__fmaf_rn(__fsub_rn(tm, big), -0x1p21f, h), l);
+  const int b = __float_as_int(__fadd_rn(r, big)) - 0x4B400000;   // in (-2^21, 2^21)
+  const unsigned a = (__float_as_uint(tm) & 0x3fffffu) + (unsigned)(b >> 21), lo = (unsigned)b & 0x1fffffu;
+  const float one = __uint_as_float(0x3f800000u | sg), off = -8388608.f * one;
+#pragma unroll
+  for (int k = 0; k < sw; ++k) {
+    const unsigned x = k < sw - 3 ? a >> (7 * (sw - 4 - k)) : lo >> (7 * (sw - 1 - k));
+    const unsigned q = k == 0 || k == sw - 3 ? x : x & 127u;
+    d[k] = __float_as_uint(__fmaf_rn(__uint_as_float(0x4B000000u | q), one, off)) >> 16;
+  }
+}
+
 template <int sw>
 __global__ void __launch_bounds__(256) k_slice_w(Work w, DevParams p, int m, int c0) {
   __shared__ int cmax[48];
+  __shared__ double tile[48][SLW_R + 1];
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
   const int N = 3 * w.counts[c].ns, Kpad = oz_kpad(N);
@@ -1764,24 +1797,46 @@ __global__ void __launch_bounds__(256) k_slice_w(Work w, DevParams p, int m, int
   const int ncv = 3 * p.n_freq;
   const double* Vin = w.vkr + (long long)(m - 1) * w.vstride + (offs * 3) * ncv;
   const double* dsq = w.dsq + offs * p.nq;
-  const int ld = w.tk > 0 ? w.tk : Kpad;
-  unsigned short* base = w.tk > 0 ? w.wdig + (long long)c * 48 * sw * w.tk : w.wdig + w.off_kp[c] * 48 * sw;
-  const long long plane = 48LL * ld;
-  const int tid = threadIdx.x;
+  const bool tiled = w.tk > 0;   // tile images of the tcgen05 path, or columns of pitch Kpad
+  const int ld = tiled ? (N + 31) / 32 * 32 : Kpad;
+  unsigned short* base = tiled ? w.wdig + (long long)c * 48 * sw * w.tk : w.wdig + w.off_kp[c] * 48 * sw;
+  const int tid = threadIdx.x, groups = blockDim.x / ncv, col = tid % ncv, r0 = tid / ncv;
   if (tid < 48) cmax[tid] = 0;
+  for (int e = tid; e < (48 - ncv) * SLW_R; e += blockDim.x) tile[ncv + e / SLW_R][e % SLW_R] = 0.0;
   __syncthreads();
-  for (int e = tid; e < N * ncv; e += blockDim.x) {
-    const int j = e / ncv, col = e % ncv;
-    const double v = dsq[(j / 3) * p.nq + col / 3 + 1] * Vin[(long long)j * ncv + col];
-    atomicMax(&cmax[col], oz_biased_exp(v));
+  if (r0 < groups) {
+    int mx = 0;
+#pragma unroll 4
+    for (int j = r0; j < N; j += groups)
+      mx = max(mx, oz_biased_exp(dsq[(j / 3) * p.nq + col / 3 + 1] * Vin[(long long)j * ncv + col]));
+    atomicMax(&cmax[col], mx);
   }
   __syncthreads();
   if (tid < 48) w.wexp[(long long)c * 48 + tid] = oz_scale_exp(cmax[tid]);
-  for (int e = tid; e < 48 * ld; e += blockDim.x) {
-    const int col = e / ld, j = e % ld;
-    double v = 0.0;
-    if (col < ncv && j < N) v = dsq[(j / 3) * p.nq + col / 3 + 1] * Vin[(long long)j * ncv + col];
-    oz_store_digits<sw>(base + (long long)col * ld + j, plane, v, oz_scale_exp(cmax[col]));
+  const int down = oz_scale_exp(cmax[col]);
+  for (int j0 = 0; j0 < ld; j0 += SLW_R) {
+    __syncthreads();
+    if (r0 < groups)
+#pragma unroll 4
+      for (int r = r0; r < SLW_R; r += groups) {
+        const int j = j0 + r;
+        // times 2^-e of the column by its exponent field: |value| < 1
+        const long long v = j < N ? __double_as_longlong(dsq[(j / 3) * p.nq + col / 3 + 1] * Vin[(long long)j * ncv + col]) : 0;
+        const int ex = (int)((v >> 52) & 0x7ff) - down;
+        tile[col][r] = ex > 0 ? __longlong_as_double(v - ((long long)down << 52)) : 0.0;
+      }
+    __syncthreads();
+    for (int e = tid; e < 48 * (SLW_R / 2); e += blockDim.x) {
+      const int cl = e / (SLW_R / 2), r = 2 * (e % (SLW_R / 2));
+      if (j0 + r >= ld) continue;
+      unsigned d[2][sw];
+      w_digits<sw>(tile[cl][r], d[0]);
+      w_digits<sw>(tile[cl][r + 1], d[1]);
+      unsigned short* o = base + (tiled ? oz_tile_offset(cl, j0 + r, 0, sw, OZ_W_ROWS, 48, ld) : (long long)cl * ld + j0 + r);
+      const int step = tiled ? 48 * 32 : 48 * ld;
+#pragma unroll
+      for (int k = 0; k < sw; ++k) *reinterpret_cast<unsigned*>(o + k * step) = d[0][k] | d[1][k] << 16;
+    }
   }
 }
 
@@ -1792,7 +1847,8 @@ __global__ void __launch_bounds__(256) k_slice_w(Work w, DevParams p, int m, int
 // every Krylov value is read once and P and Q never exist in FP64.  All arithmetic is float-float on the
 // FP32 pipe (2^-46, against the 2^-35 of the digits); the frequency weights are scaled to unit size
 // (callers' weights may be of any magnitude), the exponent goes to Q's rows and the sums.  FP64 P and Q
-// and their separate slicing took 5.2 + 1.75 ms per 4096-atom step; now 4.4 ms.
+// and their separate slicing took 5.2 + 1.75 ms per 4096-atom step; now 4.9 ms with the tile images that
+// save the pair product 0.4 ms.
 // Five signed 7-bit digits of v relative to 2^e (s1 = 2^(35 - e)), rounded to nearest, as bf16 bits.
 __device__ __forceinline__ void pq_digits(ff v, float s1, unsigned (&d)[5]) {
   const float big = 12582912.f;
@@ -1811,14 +1867,15 @@ __device__ __forceinline__ void pq_digits(ff v, float s1, unsigned (&d)[5]) {
   }
 }
 
-template <int NM>
+template <int NM, bool TILED>
 __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p, int c0, int seg) {
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
   constexpr int NV = 3 * (NM - 2);   // columns of P and Q per frequency
   constexpr int SP = 5;
   const int ns = w.counts[c].ns, N = 3 * ns, R = 3 * ((ns + 15) / 16 * 16);
-  const int nf = p.n_freq, ncv = 3 * nf, Kp = oz_kpad(w.ncol);
+  // TILED: tile images of the tcgen05 path, else rows of pitch Kp
+  const int nf = p.n_freq, ncv = 3 * nf, Kp = TILED ? (w.ncol + 31) / 32 * 32 : oz_kpad(w.ncol);
   const long long offs = w.off_s[c];
   const double wk = w.weights ? w.weights[c] : 1.0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1871,11 +1928,14 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
       for (int n = 2; n <= NM; ++n) {
         float h = 0.f, l = 0.f;
 #pragma unroll
-        for (int be = 0; be < 3; ++be) {
+        for (int be = 0; be < 3; ++be)
 #pragma unroll
-          for (int j = 1; 2 * j < n; ++j) ff_mac(h, l, ff_scale(u[j][be], 2.f), u[n - j][be]);
+          for (int j = 1; 2 * j < n; ++j) ff_mac(h, l, u[j][be], u[n - j][be]);
+        h *= 2.f;   // the pairs j, n - j and n - j, j
+        l *= 2.f;
+#pragma unroll
+        for (int be = 0; be < 3; ++be)
           if (n % 2 == 0) ff_mac(h, l, u[n / 2][be], u[n / 2][be]);
-        }
         ff_mac(gh, gl, ff_quick_two_sum(h, l), cf[n]);
       }
       // X0 of this row: sum over the frequencies of D_q0 sum_n c_n u_(n-1)
@@ -1910,28 +1970,32 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
           w.pexp[w.off_sp[c] * 3 + row] = fp;
           w.qexp[w.off_sp[c] * 3 + row] = fq + lift;
         }
-        unsigned short* dst[2] = {w.pdig + dbase + (long long)row * Kp + qq * NV, w.qdig + dbase + (long long)row * Kp + qq * NV};
         // digits of G neighbouring columns at a time, one store per plane
         constexpr int G = NV % 4 == 0 ? 4 : (NV % 2 == 0 ? 2 : 1);
 #pragma unroll
-        for (int side = 0; side < 2; ++side)
+        for (int side = 0; side < 2; ++side) {
+          unsigned short* dst = (side == 0 ? w.pdig : w.qdig) + dbase;   // a centre's planes fit 32-bit offsets
+          const OzTileRow at(row, SP, side == 0 ? OZ_P_ROWS : OZ_W_ROWS, N, Kp);
+          const unsigned row_at = TILED ? (unsigned)at.base : (unsigned)(row * Kp), step = TILED ? (unsigned)at.step : (unsigned)plane;
 #pragma unroll
           for (int v0 = 0; v0 < NV; v0 += G) {
+            const int cl = qq * NV + v0;
+            unsigned o = row_at + (TILED ? (unsigned)((cl >> 5) * SP * at.step + ((((cl >> 3) & 3) ^ at.sw) << 3) + (cl & 7)) : (unsigned)cl);
             unsigned d[G][SP];
 #pragma unroll
             for (int g = 0; g < G; ++g)
               pq_digits(side == 0 ? u[(v0 + g) / 3 + 1][(v0 + g) % 3] : qv[v0 + g], side == 0 ? sp : sq, d[g]);
 #pragma unroll
-            for (int k = 0; k < SP; ++k) {
-              unsigned short* o = dst[side] + k * plane + v0;
+            for (int k = 0; k < SP; ++k, o += step) {
               if (G == 4)
-                *reinterpret_cast<uint2*>(o) = make_uint2(d[0][k] | d[1 % G][k] << 16, d[2 % G][k] | d[3 % G][k] << 16);
+                *reinterpret_cast<uint2*>(dst + o) = make_uint2(d[0][k] | d[1 % G][k] << 16, d[2 % G][k] | d[3 % G][k] << 16);
               else if (G == 2)
-                *reinterpret_cast<unsigned*>(o) = d[0][k] | d[1 % G][k] << 16;
+                *reinterpret_cast<unsigned*>(dst + o) = d[0][k] | d[1 % G][k] << 16;
               else
-                *o = (unsigned short)d[0][k];
+                dst[o] = (unsigned short)d[0][k];
             }
           }
+        }
       }
     }
     if (on) {
@@ -1944,85 +2008,66 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
       w.gbar[(offs + s) * p.nq + qq + 1] = g * ia;
     }
   }
-  // columns past n_col (the K padding of the product)
-  const int pad = Kp - w.ncol;
-  for (int e = threadIdx.x; e < 2 * SP * N * pad; e += blockDim.x) {
-    const int col = w.ncol + e % pad, t = e / pad, row = t % N, k = (t / N) % SP, side = t / N / SP;
-    (side ? w.qdig : w.pdig)[dbase + k * plane + (long long)row * Kp + col] = 0;
+  // columns past n_col (the product runs to the next multiple of 16), 8 at a time where they are aligned
+  const int kend = oz_kpad(w.ncol);
+  for (int e = threadIdx.x; e < 2 * SP * N && w.ncol < kend; e += blockDim.x) {
+    const int row = e % N, k = (e / N) % SP, side = e / N / SP;
+    unsigned short* dst = (side ? w.qdig : w.pdig) + dbase;
+    const OzTileRow at(row, SP, side == 0 ? OZ_P_ROWS : OZ_W_ROWS, N, Kp);
+    for (int col = w.ncol; col < kend;) {
+      unsigned short* o = dst + (TILED ? at.at(col, k, SP) : k * plane + (long long)row * Kp + col);
+      if (col % 8 == 0) {
+        *reinterpret_cast<uint4*>(o) = make_uint4(0u, 0u, 0u, 0u);
+        col += 8;
+      } else {
+        *o = 0;
+        ++col;
+      }
+    }
   }
 }
 
-// P and Q digit planes and row exponents (blockIdx.y = 0: P, 1: Q); rows of at most 32 SLP_REG
-// columns are read once into registers.
-#define SLP_REG 6
+// P and Q digit planes and row exponents from FP64 P, Q (more than 32 integrand frequencies;
+// blockIdx.y = 0: P, 1: Q), one warp per row.
 template <int sp>
 __global__ void __launch_bounds__(256) k_slice_pq(Work w, int c0) {
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
+  const bool tiled = w.trec_full != 0;   // tile images of the tcgen05 path, or rows of pitch Kp
   const int ns = w.counts[c].ns, R = 3 * ((ns + 15) / 16 * 16), rows = 3 * ns;
-  const int ncol = w.ncol, Kp = oz_kpad(ncol);
+  const int ncol = w.ncol, Kp = tiled ? (ncol + 31) / 32 * 32 : oz_kpad(ncol);
   const long long offs = w.off_s[c];
   const double* src = (blockIdx.y == 0 ? w.pmat : w.qmat) + offs * 3 * (long long)ncol;
   unsigned short* base = (blockIdx.y == 0 ? w.pdig : w.qdig) + w.off_sp[c] * 3 * (long long)Kp * sp;
   int* ex = (blockIdx.y == 0 ? w.pexp : w.qexp) + w.off_sp[c] * 3;
   const long long plane = (long long)R * Kp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (ncol <= 32 * SLP_REG) {
-    // one read of P or Q: the row stays in registers between its exponent and its digits
-    for (int row = warp; row < R; row += nw) {
-      double v[SLP_REG];
-      int mx = 0;
-#pragma unroll
-      for (int k = 0; k < SLP_REG; ++k) {
-        const int j = lane + 32 * k;
-        v[k] = (row < rows && j < ncol) ? src[(long long)row * ncol + j] : 0.0;
-        mx = max(mx, oz_biased_exp(v[k]));
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const int e = oz_scale_exp(mx);
-      if (lane == 0) ex[row] = e;
-#pragma unroll
-      for (int k = 0; k < SLP_REG; ++k) {
-        const int j = lane + 32 * k;
-        if (j < Kp) oz_store_digits<sp>(base + (long long)row * Kp + j, plane, v[k], e);
-      }
-      for (int j = lane + 32 * SLP_REG; j < Kp; j += 32) oz_store_digits<sp>(base + (long long)row * Kp + j, plane, 0.0, e);
-    }
-    return;
-  }
-  for (int row = warp; row < R; row += nw) {
+  for (int row = warp; row < rows; row += nw) {
     int mx = 0;
-    if (row < rows)
-      for (int j = lane; j < ncol; j += 32) mx = max(mx, oz_biased_exp(src[(long long)row * ncol + j]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int j = lane; j < ncol; j += 32) mx = max(mx, oz_biased_exp(src[(long long)row * ncol + j]));
+    mx = __reduce_max_sync(0xffffffffu, mx);
     const int e = oz_scale_exp(mx);
     if (lane == 0) ex[row] = e;
     for (int j = lane; j < Kp; j += 32) {
-      const double v = (row < rows && j < ncol) ? src[(long long)row * ncol + j] : 0.0;
-      oz_store_digits<sp>(base + (long long)row * Kp + j, plane, v, e);
+      unsigned d[sp];
+      oz_digits<sp>(j < ncol ? src[(long long)row * ncol + j] : 0.0, e, d);
+#pragma unroll
+      for (int k = 0; k < sp; ++k)
+        base[tiled ? oz_tile_offset(row, j, k, sp, blockIdx.y == 0 ? OZ_P_ROWS : OZ_W_ROWS, rows, Kp)
+                   : k * plane + (long long)row * Kp + j] = (unsigned short)d[k];
     }
   }
 }
 
-// Slicing launches for the digit counts in use (4 to 7; the products use 5 and 6).
+// Slicing launches for the digit counts in use (5 and 6).
 static void run_slice_w(const Work& w, const DevParams& p, int m, int c0, int n, int sw, cudaStream_t s) {
-  switch (sw) {
-    case 4: k_slice_w<4><<<n, 256, 0, s>>>(w, p, m, c0); break;
-    case 5: k_slice_w<5><<<n, 256, 0, s>>>(w, p, m, c0); break;
-    case 6: k_slice_w<6><<<n, 256, 0, s>>>(w, p, m, c0); break;
-    default: k_slice_w<7><<<n, 256, 0, s>>>(w, p, m, c0); break;
-  }
+  if (sw == 5) k_slice_w<5><<<n, 256, 0, s>>>(w, p, m, c0);
+  else k_slice_w<6><<<n, 256, 0, s>>>(w, p, m, c0);
 }
 static void run_slice_pq(const Work& w, int c0, int n, int sp, cudaStream_t s) {
   const dim3 g2(n, 2);
-  switch (sp) {
-    case 4: k_slice_pq<4><<<g2, 256, 0, s>>>(w, c0); break;
-    case 5: k_slice_pq<5><<<g2, 256, 0, s>>>(w, c0); break;
-    case 6: k_slice_pq<6><<<g2, 256, 0, s>>>(w, c0); break;
-    default: k_slice_pq<7><<<g2, 256, 0, s>>>(w, c0); break;
-  }
+  if (sp == 5) k_slice_pq<5><<<g2, 256, 0, s>>>(w, c0);
+  else k_slice_pq<6><<<g2, 256, 0, s>>>(w, c0);
 }
 
 void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
@@ -2277,8 +2322,10 @@ void launch_mbd_adj_series(const Work& w, const DevParams& p, int c0, int c1, cu
       k_mbd_adj_site<N, true><<<c1 - c0, 256, 0, s>>>(w, p, c0);                       \
     else if (w.pmat || N == 2) /* order 2 has no P, Q */                               \
       k_mbd_adj_site<N, false><<<c1 - c0, 256, 0, s>>>(w, p, c0);                      \
+    else if (w.trec_full)                                                              \
+      k_adj_site_digits<(N > 2 ? N : 3), true><<<c1 - c0, 256, 0, s>>>(w, p, c0, seg); \
     else                                                                               \
-      k_adj_site_digits<(N > 2 ? N : 3)><<<c1 - c0, 256, 0, s>>>(w, p, c0, seg);       \
+      k_adj_site_digits<(N > 2 ? N : 3), false><<<c1 - c0, 256, 0, s>>>(w, p, c0, seg);\
     break;
     ADJ_SITE_CASE(2) ADJ_SITE_CASE(3) ADJ_SITE_CASE(4) ADJ_SITE_CASE(5) ADJ_SITE_CASE(6)
     ADJ_SITE_CASE(7) ADJ_SITE_CASE(8) ADJ_SITE_CASE(9) ADJ_SITE_CASE(10)

@@ -11,7 +11,7 @@
 //
 // Everything between the accumulators and the atomics is float-float on the FP32 pipe (2^-46,
 // against the 2^-35 of the digits), and only coupled pairs are evaluated: with an FP64 tile and
-// epilogue over all pairs two thirds of a tile's time was FP64 issue (1024-atom step: 3.55 ms, now 1.33 ms).
+// epilogue over all pairs two thirds of a tile's time was FP64 issue (1024-atom step: 3.55 ms, now 1.22 ms).
 // Two CTAs share an SM (256 tensor-memory columns and a two-slot ring each), so that one tile's
 // copies and MMAs run under the other's epilogue; the 42 x 32 tile of one CTA per SM re-read less of
 // P but left the SM at 24 % of its issue slots (1.77 against 1.33 ms).
@@ -71,13 +71,11 @@ __device__ __forceinline__ void ptc_epilogue(const float4* rec, const ff (&acc)[
   out[3] = dot2(k4, rMr, k5, tr);
 }
 
-__device__ __forceinline__ int ptc_kpad(int n) { return (n + 15) / 16 * 16; }
-inline long long ptc_kpad_host(int n) { return (n + 15) / 16 * 16; }
+__device__ __forceinline__ int ptc_k(int n) { return (n + 31) / 32 * 32; }
 
 template <int S>
 __global__ void __launch_bounds__(256, 2)
-    k_pair_tc(Work w, DevParams p, int c0, int nb_max, int tiles_per_c, const __grid_constant__ CUtensorMap tmP,
-              const __grid_constant__ CUtensorMap tmQ) {
+    k_pair_tc(Work w, DevParams p, int c0, int nb_max, int tiles_per_c) {
   using Sh = TcsShape<S, PTC_NB, PTC_BUF, PTC_COLS>;
   extern __shared__ unsigned char tc_dyn[];
   __shared__ TcsBarriers bar;
@@ -90,11 +88,11 @@ __global__ void __launch_bounds__(256, 2)
   const int s0 = PTC_SA * (tile / nb_max), t0 = PTC_SB * (tile % nb_max);
   // tiles without a site pair s > t inside the sphere have nothing to do
   if (s0 >= ns || t0 >= ns || min(s0 + PTC_SA, ns) - 1 <= t0) return;
-  const int R = 3 * ((ns + 15) / 16 * 16), Kp = ptc_kpad(w.ncol);
-  // P and Q digit planes of this centre: rows off_sp[c] 3 S + k R + r of the wave's maps (pitch Kp)
-  const int prow = (int)(w.off_sp[c] * 3 * S - w.prow0);
-  const TcsTile A{&tmP, prow + 3 * s0, R};
-  const TcsTile B{&tmQ, prow + 3 * t0, R};
+  const int K = ptc_k(w.ncol);
+  // P and Q tile images of this centre
+  const long long dig = w.off_sp[c] * 3LL * K * S;
+  const TcsImage A{w.pdig + dig + 3LL * s0 * K * S, min(3 * PTC_SA, 3 * (ns - s0)), S};
+  const TcsImage B{w.qdig + dig + 3LL * t0 * K * S, min(PTC_NB, 3 * (ns - t0)), S};
   const uint32_t sraw = tc_smem_u32(tc_dyn);
   const uint32_t sbase = (sraw + 1023u) & ~1023u;
   if (threadIdx.x == 64) {
@@ -147,7 +145,13 @@ __global__ void __launch_bounds__(256, 2)
   float Yh[24], Yl[24];
   bool first = true;
   TcsProgress pr;
-  const bool ok = tcs_mainloop<S, PTC_NB, PTC_BUF, PTC_COLS>(A, B, Kp, sbase, bar, p.tc_wait, pr, [&]() {
+  const bool ok = tcs_mainloop_with<S, PTC_NB, PTC_BUF, PTC_COLS>(
+      [&](int s, uint32_t sA, uint32_t sB, uint64_t* mbar) {
+        tc_mbar_expect_tx(mbar, tcs_image_bytes<S>(A) + tcs_image_bytes<S>(B));
+        tcs_image_copy<S>(A, s, sA, Sh::kAPlane, mbar);
+        tcs_image_copy<S>(B, s, sB, Sh::kBPlane, mbar);
+      },
+      (w.ncol + 15) / 16 * 16, sbase, bar, p.tc_wait, pr, [&]() {
 #pragma unroll
     for (int j8 = 0; j8 < 3; ++j8) {
       float h[8], l[8];
@@ -251,6 +255,7 @@ __global__ void __launch_bounds__(256, 2)
   }
 }
 
+static_assert(3 * PTC_SA == OZ_P_ROWS && PTC_NB == OZ_W_ROWS, "tiles of the digit images");
 static_assert(TcsShape<5, PTC_NB, PTC_BUF, PTC_COLS>::kBytes <= 113 * 1024, "two staging rings exceed the shared memory of an SM");
 static_assert(3 * PTC_SA * PTC_LD * 8 % 16 == 0, "pair results start on a 16-byte boundary");
 static_assert((3 * PTC_SA * PTC_LD + 4 * PTC_SA * PTC_GL) * 8 <= TcsShape<5, PTC_NB, PTC_BUF, PTC_COLS>::kBytes - 1024,
@@ -258,19 +263,15 @@ static_assert((3 * PTC_SA * PTC_LD + 4 * PTC_SA * PTC_GL) * 8 <= TcsShape<5, PTC
 
 }  // namespace
 
-// Digit planes of P and Q (k_slice_pq), then the tcgen05 pair kernel; digits must be 5.
+// The tcgen05 pair kernel on the digit images of P and Q (written by the series adjoint, or here from
+// FP64 P, Q); digits must be 5.
 bool launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits, cudaStream_t s) {
   if (c1 <= c0) return true;
   if (digits != 5) return false;
   launch_slice_pq(w, c0, c1, digits, s);
   const int na = (max_ns + PTC_SA - 1) / PTC_SA, nb = (max_ns + PTC_SB - 1) / PTC_SB;
-  const long long Kp = ptc_kpad_host(w.ncol);
-  CUtensorMap tmP, tmQ;
-  if (!tc_encode_map(&tmP, w.pdig + w.prow0 * Kp, Kp, Kp, w.prows, TCS_M) ||
-      !tc_encode_map(&tmQ, w.qdig + w.prow0 * Kp, Kp, Kp, w.prows, PTC_NB))
-    return false;
   using Sh = TcsShape<5, PTC_NB, PTC_BUF, PTC_COLS>;
   raise_smem_limit((const void*)k_pair_tc<5>, Sh::kBytes);
-  k_pair_tc<5><<<(c1 - c0) * na * nb, 256, Sh::kBytes, s>>>(w, p, c0, nb, na * nb, tmP, tmQ);
+  k_pair_tc<5><<<(c1 - c0) * na * nb, 256, Sh::kBytes, s>>>(w, p, c0, nb, na * nb);
   return true;
 }

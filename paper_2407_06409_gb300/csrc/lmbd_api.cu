@@ -274,7 +274,7 @@ struct Layout {
   int nq, ncv, nvec, ncol, kp_pair, st, dig_p, site_cap;
   bool forces, sliced_chain, sliced_pair;
   int nqs;   // frequencies of the SCS solves (stage-1 arrays)
-  int tk;    // tcgen05 path: row pitch of the T and W digit planes (0: per-centre Kpad)
+  int tk;    // tcgen05 path: longest K of the T and W tile images (0: rows of pitch Kpad)
   bool sparse;   // block-sparse T_LR: coupled pairs and float-float chain/pair operands
   bool dense_t;  // FP64 T_LR kept (Lanczos-based modes, the paper's forces, FP64 products)
   bool rec_pair; // the pair adjoint reads float-float records instead of FP64 coefficients
@@ -289,9 +289,9 @@ struct Layout {
     const long long k0 = o.at(O_K1, c0), nk = o.span(O_K1, c0, c1);
     const long long n = c1 - c0;
     int* pr_ij = cv.take<int>(2 * (np + 1), 2 * p0);
-    double* pr_geo = cv.take<double>(8 * (np + 1), 8 * p0);
     float4* pr_rad4 = cv.take<float4>(nqs * (np + 1), nqs * p0);
     int2* pr_ga = cv.take<int2>(np + 1, p0);
+    double* pr_geo = cv.take<double>(8 * (np + 1), 8 * p0);
     float2* pr_gff = cv.take<float2>(6 * (np + 1), 6 * p0);
     int* k2rev = cv.take<int>(np + 1, p0);
     int* prow = cv.take<int>(nk + n, k0 + c0);
@@ -302,9 +302,9 @@ struct Layout {
     double* xsol = cv.take<double>(9LL * nqs * nk, 9LL * nqs * k0);
     if (w) {
       w->pr_ij = pr_ij;
-      w->pr_geo = pr_geo;
       w->pr_rad4 = pr_rad4;
       w->pr_ga = pr_ga;
+      w->pr_geo = pr_geo;
       w->pr_gff = pr_gff;
       w->k2rev = k2rev;
       w->prow = prow;
@@ -368,8 +368,8 @@ struct Layout {
       }
     }
     if (sliced_chain) {
-      // T planes: per centre st planes of Mpad rows, row pitch Kpad (warp-level path) or the
-      // common pitch tk (tcgen05 path: one tensor map covers the wave)
+      // T planes: per centre st planes of Mpad rows of pitch Kpad (warp-level path), or its tile
+      // images (tcgen05 path: at most Mpad rows of tk, the largest K rounded to 32)
       unsigned short* tdig =
           tk > 0 ? cv.take<unsigned short>((long long)st * o.span(O_TR, c0, c1) * tk, (long long)st * o.at(O_TR, c0) * tk)
                  : cv.take<unsigned short>((long long)st * o.span(O_TQ, c0, c1), (long long)st * o.at(O_TQ, c0));
@@ -382,10 +382,6 @@ struct Layout {
         w->texp = texp;
         *wdig_raw = wdig;
         w->tk = tk;
-        w->trow0 = (long long)st * o.at(O_TR, c0);
-        w->trows = (long long)st * o.span(O_TR, c0, c1);
-        w->wc0 = c0;
-        w->wcn = c1 - c0;
       }
     }
     if (forces) {
@@ -421,8 +417,6 @@ struct Layout {
           w->qdig = qdig;
           w->pexp = pexp;
           w->qexp = qexp;
-          w->prow0 = 3LL * dig_p * sp0;
-          w->prows = 3LL * dig_p * nsp;
         }
       }
     }
@@ -915,9 +909,11 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   }
 
   // ---- waves under the memory budget --------------------------------------------------------
-  const Layout L{nq, ncv, nvec, ncol, (ncol + 15) / 16 * 16, ST, DIG_P, c->site_cap, forces, sliced_chain,
-                 sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 15) / 16 * 16 : 0, sparse,
-                 !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), forces && sliced_pair && tc05 && !dp.paper,
+  const bool rec_pair = forces && sliced_pair && tc05 && !dp.paper;   // tcgen05 pair adjoint
+  const int kp_pair = rec_pair ? (ncol + 31) / 32 * 32 : (ncol + 15) / 16 * 16;   // K of the P, Q planes
+  const Layout L{nq, ncv, nvec, ncol, kp_pair, ST, DIG_P, c->site_cap, forces, sliced_chain,
+                 sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 31) / 32 * 32 : 0, sparse,
+                 !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), rec_pair,
                  !sparse && (!sliced_pair || dp.paper || nf > 32),
                  scs_contract_scratch(N, max_n1, dp.nqs)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };

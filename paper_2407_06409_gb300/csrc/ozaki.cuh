@@ -24,6 +24,36 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+// Digit planes of the tcgen05 kernels lie in memory as the images of their shared-memory tiles: for a
+// tile of `tile` rows (the last one of a matrix has fewer, nrows) and every slice of 32 along K the
+// planes one after another, each nrows x 64 bytes with the 16-byte chunk q of row r at chunk
+// q ^ ((r >> 1) & 3) (64-byte swizzle).  A stage of a full tile is then one contiguous bulk copy; boxes
+// of 64-byte rows through tensor maps moved 64 bytes in about four cycles.
+// Offset in elements of (row, column) of plane k of a `rows` x K matrix (K a multiple of 32).
+__host__ __device__ __forceinline__ long long oz_tile_offset(int row, int col, int k, int planes, int tile, int rows, int K) {
+  const int t = row / tile, r = row - t * tile;
+  const int nrows = rows - t * tile < tile ? rows - t * tile : tile;
+  const int q = ((col >> 3) & 3) ^ ((r >> 1) & 3);
+  return (long long)t * tile * K * planes + ((long long)(col >> 5) * planes + k) * nrows * 32 + r * 32 + q * 8 + (col & 7);
+}
+// The same with the part of the row done once.
+struct OzTileRow {
+  long long base;
+  int step, sw;   // elements per plane of a K slice; chunk swizzle of the row
+  __device__ __forceinline__ OzTileRow(int row, int planes, int tile, int rows, int K) {
+    const int t = row / tile, r = row - t * tile;
+    step = min(tile, rows - t * tile) * 32;
+    base = (long long)t * tile * K * planes + r * 32;
+    sw = (r >> 1) & 3;
+  }
+  __device__ __forceinline__ long long at(int col, int k, int planes) const {
+    return base + ((col >> 5) * planes + k) * step + ((((col >> 3) & 3) ^ sw) << 3) + (col & 7);
+  }
+};
+#define OZ_T_ROWS 128   // T_LR: rows of a tile
+#define OZ_W_ROWS 48    // W and Q
+#define OZ_P_ROWS 126   // P: 42 sites
+
 // Exponent e with |v| < 2^e for the largest |v| (biased exponent of v, 0 for zero).
 __device__ __forceinline__ int oz_biased_exp(double v) {
   return (int)((__double_as_longlong(v) >> 52) & 0x7ff);
@@ -58,6 +88,26 @@ __device__ __forceinline__ void oz_store_digits(unsigned short* dst, long long p
   const int sg = bits < 0 ? -1 : 1;
 #pragma unroll
   for (int k = 0; k < S; ++k) dst[k * plane] = oz_bf16_bits(sg * (int)((U >> (7 * (S - 1 - k))) & 127ULL));
+}
+
+// The same digits as bf16 bits in d[0..S-1].
+template <int S>
+__device__ __forceinline__ void oz_digits(double v, int e, unsigned (&d)[S]) {
+  const long long bits = __double_as_longlong(v);
+  const int ex = (int)((bits >> 52) & 0x7ff);
+  unsigned long long U = 0;
+  if (ex != 0) {
+    const unsigned long long mant = (unsigned long long)(bits & 0xFFFFFFFFFFFFFLL) | (1ULL << 52);
+    const int sh = (ex - 1075) + 7 * S - e;
+    if (sh >= 0) U = mant << sh;
+    else if (sh > -64) U = mant >> (-sh);
+  }
+  const unsigned sg = (unsigned)(bits >> 48) & 0x8000u;
+#pragma unroll
+  for (int k = 0; k < S; ++k) {   // an integer below 2^7 read off the mantissa of an FP32 sum
+    const unsigned q = (unsigned)(U >> (7 * (S - 1 - k))) & 127u;
+    d[k] = (__float_as_uint(__uint_as_float(0x4B000000u | q) - 8388608.f) >> 16) | sg;
+  }
 }
 
 // 2^E as a double (E clamped to the normal range; tiny scales flush to zero).

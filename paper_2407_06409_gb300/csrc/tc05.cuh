@@ -78,6 +78,23 @@ __device__ __forceinline__ bool tc_mbar_wait(uint64_t* mbar, uint32_t parity, lo
   return true;
 }
 
+// The same for one of several cooperating roles: gives up as well when another role has set *stop, and
+// sets it when the budget runs out.
+__device__ __forceinline__ bool tc_mbar_wait_or_stop(uint64_t* mbar, uint32_t parity, long long budget, volatile int* stop) {
+  const long long t0 = clock64();
+  while (!tc_mbar_test_wait(mbar, parity)) {
+    if (*stop) return false;
+    if (clock64() - t0 > budget) {
+      *stop = 1;
+      return false;
+    }
+  }
+  return true;
+}
+__device__ __forceinline__ void tc_mbar_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem_u32(mbar)) : "memory");
+}
+
 // TMEM allocation (one whole warp); the column base is written to shared memory.
 __device__ __forceinline__ void tc_alloc(uint32_t* holder, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem_u32(holder)),
@@ -121,4 +138,12 @@ __device__ __forceinline__ void tc_tma_load_2d(uint32_t sdst, const CUtensorMap*
           sdst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(tc_smem_u32(mbar))
       : "memory");
+}
+
+// Bulk copy of `bytes` (a multiple of 16) from 16-byte aligned global memory into shared memory;
+// completion is counted in bytes on the mbarrier.
+__device__ __forceinline__ void tc_bulk_load(uint32_t sdst, const void* gsrc, uint32_t bytes, uint64_t* mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sdst),
+               "l"(gsrc), "r"(bytes), "r"(tc_smem_u32(mbar))
+               : "memory");
 }

@@ -127,13 +127,14 @@ __device__ __forceinline__ uint32_t tcs_lane_addr(uint32_t tmem, int col) {
   return tmem + ((uint32_t)(32 * ((threadIdx.x >> 5) & 3)) << 16) + (uint32_t)col;
 }
 
-// The main loop (all 256 threads; thread 0 issues copies and MMAs and waits for them).
+// The main loop (all 256 threads; thread 0 issues copies and MMAs and waits for them).  copy(s, sA, sB,
+// mbar) sets the bytes the slot's barrier waits for and issues the copies of stage s.
 // consume() runs block-wide at the end of every K chunk with the accumulators complete in TMEM.
 // Every wait is bounded by `budget` cycles; returns false if one ran out.  `pr` (thread 0) keeps
 // what is in flight, for the tear-down.
-template <int S, int NB, int NBUF = TCS_NBUF, int COLS = TCS_TMEM_COLS, class Consume>
-__device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B, int K, uint32_t sbase,
-                                             TcsBarriers& bar, long long budget, TcsProgress& pr, Consume&& consume) {
+template <int S, int NB, int NBUF, int COLS, class Copy, class Consume>
+__device__ __forceinline__ bool tcs_mainloop_with(Copy&& copy, int K, uint32_t sbase, TcsBarriers& bar,
+                                                  long long budget, TcsProgress& pr, Consume&& consume) {
   using Sh = TcsShape<S, NB, NBUF, COLS>;
   const int tid = threadIdx.x;
   const int nst = (K + TCS_KS - 1) / TCS_KS;
@@ -143,11 +144,7 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
     const int slot = s % NBUF;
     const uint32_t sA = sbase + slot * Sh::kSlot;
     const uint32_t sB = sA + S * Sh::kAPlane;
-    tc_mbar_expect_tx(&bar.full[slot], (uint32_t)Sh::kSlot);
-#pragma unroll
-    for (int k = 0; k < S; ++k) tc_tma_load_2d(sA + k * Sh::kAPlane, A.map, s * TCS_KS, A.y0 + k * A.plane_rows, &bar.full[slot]);
-#pragma unroll
-    for (int k = 0; k < S; ++k) tc_tma_load_2d(sB + k * Sh::kBPlane, B.map, s * TCS_KS, B.y0 + k * B.plane_rows, &bar.full[slot]);
+    copy(s, sA, sB, &bar.full[slot]);
     pr.issued = s;
   };
   if (tid == 0)
@@ -167,7 +164,8 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
         const uint32_t sA = sbase + slot * Sh::kSlot;
         const uint32_t sB = sA + S * Sh::kAPlane;
 #pragma unroll
-        for (int kk = 0; kk < TCS_KS / 16; ++kk)
+        for (int kk = 0; kk < TCS_KS / 16; ++kk) {
+          if (s * TCS_KS + kk * 16 >= K) break;   // the second half of the last slice may be past K
 #pragma unroll
           for (int k = 0; k < S; ++k) {
             const uint64_t ad = tc_desc_k_sw64(sA + k * Sh::kAPlane + kk * 32);
@@ -180,6 +178,7 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
                           (s == s0 && kk == 0 && k == 0) ? 0u : 1u);
             }
           }
+        }
         tc_commit(&bar.empty[slot]);
         pr.committed = s;
         // refill the slot of stage s - 1 with stage s - 1 + NBUF once its MMAs are done
@@ -207,4 +206,41 @@ __device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B,
     __syncthreads();
   }
   return true;
+}
+
+// The main loop on operand tiles addressed through tensor maps.
+template <int S, int NB, class Consume>
+__device__ __forceinline__ bool tcs_mainloop(const TcsTile& A, const TcsTile& B, int K, uint32_t sbase,
+                                             TcsBarriers& bar, long long budget, TcsProgress& pr, Consume&& consume) {
+  using Sh = TcsShape<S, NB>;
+  return tcs_mainloop_with<S, NB, TCS_NBUF, TCS_TMEM_COLS>(
+      [&](int s, uint32_t sA, uint32_t sB, uint64_t* mbar) {
+        tc_mbar_expect_tx(mbar, (uint32_t)Sh::kSlot);
+#pragma unroll
+        for (int k = 0; k < S; ++k) tc_tma_load_2d(sA + k * Sh::kAPlane, A.map, s * TCS_KS, A.y0 + k * A.plane_rows, mbar);
+#pragma unroll
+        for (int k = 0; k < S; ++k) tc_tma_load_2d(sB + k * Sh::kBPlane, B.map, s * TCS_KS, B.y0 + k * B.plane_rows, mbar);
+      },
+      K, sbase, bar, budget, pr, consume);
+}
+
+// One operand tile as an image in memory (oz_tile_offset): `rows` rows of `planes` planes; copies the
+// first S planes of K slice s to sdst (plane stride `stride` bytes).  The stage has
+// tcs_image_bytes bytes.
+struct TcsImage {
+  const unsigned short* at;   // of the tile
+  int rows, planes;
+};
+template <int S>
+__device__ __forceinline__ uint32_t tcs_image_bytes(const TcsImage& t) { return (uint32_t)(S * t.rows * TCS_KS * 2); }
+template <int S>
+__device__ __forceinline__ void tcs_image_copy(const TcsImage& t, int s, uint32_t sdst, int stride, uint64_t* mbar) {
+  const unsigned short* src = t.at + (long long)s * t.planes * t.rows * TCS_KS;
+  const uint32_t plane = (uint32_t)(t.rows * TCS_KS * 2);
+  if ((int)plane == stride) {   // a full tile: one piece
+    tc_bulk_load(sdst, src, S * plane, mbar);
+  } else {
+#pragma unroll
+    for (int k = 0; k < S; ++k) tc_bulk_load(sdst + k * stride, src + (long long)k * t.rows * TCS_KS, plane, mbar);
+  }
 }
