@@ -41,10 +41,11 @@ __device__ __forceinline__ ff ff_from_double(double x) {
   return ff_make(hi, lo);
 }
 
-// The same up to truncation (47 bits kept) by integer and FP32 instructions, for kernels whose FP64
-// pipe is the bound: hi = the top 24 bits, lo = the next 23.  Finite values in the FP32 range;
-// smaller ones give zero.
-__device__ __forceinline__ ff ff_split(double x) {
+// The same to 47 bits (nearest) by integer and FP32 instructions, for kernels whose FP64 pipe is the
+// bound: hi = the top 24 bits, lo = the next 23.  Finite values in the FP32 range; smaller ones give
+// zero.
+__device__ __forceinline__ ff ff_split(double v) {
+  const double x = __longlong_as_double(__double_as_longlong(v) + 32);   // half of the last bit kept
   const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), sg = h & 0x80000000u;
   const int e = (int)((h >> 20) & 0x7ffu) - (1023 - 127);   // biased FP32 exponent
   const unsigned hb = ((unsigned)max(e, 0) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);

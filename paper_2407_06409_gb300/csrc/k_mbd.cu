@@ -34,7 +34,8 @@ __device__ __forceinline__ int oz_kpad(int n) { return (n + 15) / 16 * 16; }
 // one), queues the coupled ones (47 % at the benchmark cutoffs), and evaluates 32 queued pairs with
 // all lanes: distance, exponential and the two divisions in FP64, the products of the record in
 // float-float on the FP32 pipe.  1024-atom step: 2.51 ms with every pair in FP64
-// and T_LR stored, 1.11 ms now (FP64 pipe 62 % busy over a launch of 1.7 waves).
+// and T_LR stored, 1.11 ms with the records and FP64 conversions to float-float (FP64 pipe 62 % busy),
+// 0.78 ms with integer ones (ff_split).
 // DENSE: the FP64 blocks of T_LR and / or the FP64 coefficients are wanted as well (Lanczos-based
 // modes, the paper's forces, FP64 and warp-level products).
 
@@ -54,15 +55,15 @@ __device__ __forceinline__ PairRec tlr_pair_record(const DevParams& p, ff d_ff, 
   const double xd = r / (p.beta * (rts + rtt));
   const double e = exp(-p.d * (xd - 1.0));
   const double fd = 1.0 / (1.0 + e);
-  const ff x = ff_from_double(rr[0]), y = ff_from_double(rr[1]), z = ff_from_double(rr[2]);
-  const ff ir = ff_from_double(ird), ir2 = ff_mul(ir, ir), ir4 = ff_mul(ir2, ir2), ir5 = ff_mul(ir4, ir);
-  const ff f = ff_from_double(fd);
+  const ff x = ff_split(rr[0]), y = ff_split(rr[1]), z = ff_split(rr[2]);
+  const ff ir = ff_split(ird), ir2 = ff_mul(ir, ir), ir4 = ff_mul(ir2, ir2), ir5 = ff_mul(ir4, ir);
+  const ff f = ff_split(fd);
   // f_LR = 1 - 3 t^2 + 2 t^3, f_LR' = (-6 t + 6 t^2) / r_b, t = (r - rc + r_b) / r_b in the buffer
   const double tb = r - (rc - p.r_buf);
   const bool buffer = tb >= 0.0;
   ff flr = ff_make(1.f, 0.f), dflr = ff_make(0.f, 0.f);
   if (buffer) {
-    const ff t = ff_mul(ff_from_double(tb), ib_ff), t2 = ff_mul(t, t);
+    const ff t = ff_mul(ff_split(tb), ib_ff), t2 = ff_mul(t, t);
     flr = ff_add(ff_make(1.f, 0.f), ff_sub(ff_scale(ff_mul(t2, t), 2.f), ff_scale(t2, 3.f)));
     dflr = ff_mul(ff_scale(ff_sub(t2, t), 6.f), ib_ff);
     if (!(r < rc)) flr = dflr = ff_make(0.f, 0.f);
@@ -73,8 +74,8 @@ __device__ __forceinline__ PairRec tlr_pair_record(const DevParams& p, ff d_ff, 
   o.v[0] = two_ff(x, y);
   o.v[1] = two_ff(z, ff_scale(u, 12.f));
   if (full) {
-    const ff sx = ff_from_double(xd);
-    const ff dfr = ff_mul(ff_mul(ff_from_double(fd * (1.0 - fd)), d_ff), ff_mul(sx, ir));   // df/dr
+    const ff sx = ff_split(xd);
+    const ff dfr = ff_mul(ff_mul(ff_split(fd * (1.0 - fd)), d_ff), ff_mul(sx, ir));   // df/dr
     const ff dlr = buffer ? ff_mul(flr, dfr) : dfr;
     const ff dC = buffer ? ff_add(ff_mul(dflr, f), dlr) : dfr;
     const ff v = ff_mul(ff_mul(ff_mul(ff_neg(dlr), sx), ff_mul(ir2, ir)), beta_ff);   // beta f_LR f_S / r^3

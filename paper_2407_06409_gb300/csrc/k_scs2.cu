@@ -106,8 +106,7 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
   int* adjcnt = k2start + max_n1 + 1;              // max_n1
   int* adjstart = adjcnt + max_n1;                 // max_n1 + 1
   int* k2cnt = adjstart + max_n1 + 1;              // max_n12
-  int* klist = k2cnt + max_n12;                    // per warp max_n1: atoms of one K1 list
-  float* xf = (float*)(klist + 8 * max_n1);        // 3 x max_n12, FP32 copies of xs
+  float* xf = (float*)(k2cnt + max_n12);           // 3 x max_n12, FP32 copies of xs
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
   const Counts cn = w.counts[c];
@@ -149,16 +148,8 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     k2start[n1] = run;
   }
   __syncthreads();
-  // phase 2a: pairs in order (row, partner) and their entry in the atom-pair radial table
-  int* lst = klist + warp * max_n1;
+  // phase 2a: pairs in order (row, partner)
   for (int i = warp; i < n1; i += nw) {
-    // atoms of the K1 list of site i's atom, for the radial-table lookup below
-    const int ai = w.site_atom[sbase + i];
-    const int na = w.counts[ai].n1;
-    const long long ab = (long long)ai * w.site_cap;
-    __syncwarp();
-    for (int t = lane; t < na; t += 32) lst[t] = w.site_atom[ab + t];
-    __syncwarp();
     for (int pass = 0; pass < 2; ++pass) {
       int jb = pass == 0 ? 0 : n1, je = pass == 0 ? i : n12;
       int pos = pass == 0 ? k1start[i] : k2start[i];
@@ -171,23 +162,6 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
           long long q = offp + slot;
           w.pr_ij[2 * q] = i;
           w.pr_ij[2 * q + 1] = j;
-          // the same atom pair in the radial table: the site of atom aj at displacement
-          // r = x_j - x_i in atom ai's own K1 list (periodic images of one atom are far apart,
-          // so an FP32 match is unambiguous; none only if r ties r_SCS to rounding)
-          const int aj = w.site_atom[sbase + j];
-          const float rxf = xf[j] - xf[i], ryf = xf[max_n12 + j] - xf[max_n12 + i],
-                      rzf = xf[2 * max_n12 + j] - xf[2 * max_n12 + i];
-          int gi = -1;
-          for (int t = 1; t < na; ++t) {
-            if (lst[t] != aj) continue;
-            const double* xt = w.site_x + 3 * (ab + t);
-            const float dx = (float)xt[0] - rxf, dy = (float)xt[1] - ryf, dz = (float)xt[2] - rzf;
-            if (dx * dx + dy * dy + dz * dz < 1e-4f) {
-              gi = (int)(w.off_k1[ai] + t);
-              break;
-            }
-          }
-          w.pr_ga[q] = make_int2(gi, aj);
           if (pass == 0) pid[i * max_n1 + j] = slot;
         }
         pos += __popc(m);
@@ -203,34 +177,77 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     w.prow_k2[rbase + n1] = k2start[n1];
   }
   __syncthreads();
-  // phase 2b: FP64 geometry and damping of every pair, one thread per pair
+  // phase 2b, one thread per pair: its entry in the atom-pair radial table, geometry and damping.
+  // Searching the table here, with every lane a pair, instead of by the few coupled lanes of phase 2a
+  // took three quarters of this kernel's instructions away; distance, exponential and divisions
+  // run in FP64, the products of the damping in float-float (1024 atoms: 1.14 -> 0.77 ms).
+  const ff d_ff = ff_from_double(p.d), ibuf_ff = ff_from_double(1.0 / p.r_buf), iin_ff = ff_from_double(1.0 / p.r_inner);
   for (int t = tid; t < k2start[n1]; t += blockDim.x) {
     const long long q = offp + t;
-    const int i = w.pr_ij[2 * q], j = w.pr_ij[2 * q + 1];
+    const int2 ij = reinterpret_cast<const int2*>(w.pr_ij)[q];
+    const int i = ij.x, j = ij.y;
+    const int ai = w.site_atom[sbase + i], aj = w.site_atom[sbase + j];
     double rx, ry, rz, r2;
     scs_pair_in(xs, max_n12, i, j, rc2, rx, ry, rz, r2);
+    // the same atom pair in the radial table: the site of atom aj at displacement r = x_j - x_i in
+    // atom ai's own K1 list (periodic images of one atom are far apart, so an FP32 match is
+    // unambiguous; none only if r ties r_SCS to rounding)
+    int gi = -1;
+    {
+      const long long ab = (long long)ai * w.site_cap;   // site lists start on 16-byte boundaries
+      const int na = w.counts[ai].n1;
+      const int4* list = reinterpret_cast<const int4*>(w.site_atom + ab);
+      const float fx = (float)rx, fy = (float)ry, fz = (float)rz;
+      auto match = [&](int u) {
+        const double* xt = w.site_x + 3 * (ab + u);
+        const float dx = (float)xt[0] - fx, dy = (float)xt[1] - fy, dz = (float)xt[2] - fz;
+        if (dx * dx + dy * dy + dz * dz < 1e-4f) gi = (int)(w.off_k1[ai] + u);
+      };
+#pragma unroll 2
+      for (int u = 0; u < na && gi < 0; u += 4) {
+        const int4 a = __ldg(list + u / 4);
+        if (a.x == aj && u > 0) match(u);
+        if (a.y == aj && u + 1 < na && gi < 0) match(u + 1);
+        if (a.z == aj && u + 2 < na && gi < 0) match(u + 2);
+        if (a.w == aj && u + 3 < na && gi < 0) match(u + 3);
+      }
+    }
+    w.pr_ga[q] = make_int2(gi, aj);
     // 1/r from one reciprocal square root; the Fermi damping (Eq. damping-function) through
     // x = r / S_vdW, its r-derivative f (1 - f) d / S_vdW as f (1 - f) d x / r
-    const double ir = rsqrt(r2);
-    const double r = r2 * ir;
-    const int ai = w.site_atom[sbase + i], aj = w.site_atom[sbase + j];
-    double fsr, dfsr, fin = 1.0, dfin = 0.0;
-    cutoff_buf(r, p.r_scs, p.r_buf, fsr, dfsr);
-    if (j >= n1) finner(r, p.r_inner, fin, dfin);
+    const double ird = rsqrt(r2);
+    const double r = r2 * ird;
     const double x = r / (p.beta * (w.rvdw[ai] + w.rvdw[aj]));
     const double f = 1.0 / (1.0 + exp(-p.d * (x - 1.0)));
-    const double dfr = f * (1.0 - f) * p.d * x * ir;
-    const double F = fin * fsr * (1.0 - f);
-    const double dF = dfin * fsr * (1.0 - f) + fin * dfsr * (1.0 - f) - fin * fsr * dfr;
-    double* g = w.pr_geo + 8 * q;
-    g[0] = rx; g[1] = ry; g[2] = rz; g[3] = r; g[4] = F; g[5] = dF; g[6] = ir; g[7] = 0.0;
-    float2* gf = w.pr_gff + 6 * q;
-#pragma unroll
-    for (int u = 0; u < 7; ++u) {
-      if (u == 3) continue;
-      const ff v = ff_from_double(g[u]);
-      gf[u < 3 ? u : u - 1] = make_float2(v.hi, v.lo);
+    const ff ir = ff_split(ird), omf = ff_split(1.0 - f);
+    const ff dfr = ff_mul(ff_mul(ff_split(f * (1.0 - f)), d_ff), ff_mul(ff_split(x), ir));
+    // F = f_inner f_SR (1 - f); c = f_inner f_SR and its derivative where either differs from 1
+    ff F = omf, dF = ff_neg(dfr);
+    const double tb = r - (p.r_scs - p.r_buf);
+    const bool buffer = tb >= 0.0, inner = j >= n1 && r < p.r_inner;
+    if (buffer || inner) {
+      ff cs = ff_make(1.f, 0.f), dc = ff_make(0.f, 0.f);
+      if (buffer) {
+        const ff u = ff_mul(ff_split(tb), ibuf_ff), u2 = ff_mul(u, u);
+        cs = ff_add(cs, ff_sub(ff_scale(ff_mul(u2, u), 2.f), ff_scale(u2, 3.f)));
+        dc = ff_mul(ff_scale(ff_sub(u2, u), 6.f), ibuf_ff);
+        if (!(r < p.r_scs)) cs = dc = ff_make(0.f, 0.f);
+      }
+      if (inner) {
+        const ff u = ff_mul(ff_split(r), iin_ff), u2 = ff_mul(u, u);
+        const ff fi = ff_sub(ff_scale(u2, 3.f), ff_scale(ff_mul(u2, u), 2.f));
+        const ff di = ff_mul(ff_scale(ff_sub(u, u2), 6.f), iin_ff);
+        dc = ff_add(ff_mul(di, cs), ff_mul(fi, dc));
+        cs = ff_mul(fi, cs);
+      }
+      F = ff_mul(cs, omf);
+      dF = ff_sub(ff_mul(dc, omf), ff_mul(cs, dfr));
     }
+    float4* gf = reinterpret_cast<float4*>(w.pr_gff + 6 * q);
+    const ff gx = ff_split(rx), gy = ff_split(ry), gz = ff_split(rz);
+    gf[0] = make_float4(gx.hi, gx.lo, gy.hi, gy.lo);
+    gf[1] = make_float4(gz.hi, gz.lo, F.hi, F.lo);
+    gf[2] = make_float4(dF.hi, dF.lo, ir.hi, ir.lo);
   }
   __syncthreads();
   // phase 3: adjacency rows (K1 partners of every coupled site, both directions)
@@ -267,34 +284,41 @@ __global__ void __launch_bounds__(256) k_scs_fill(Work w, DevParams p, int c0, i
     if (lane == 0) w.arow[rbase + i] = adjstart[i];
   }
   if (tid == 0) w.arow[rbase + n1] = adjstart[n1];
-  // phase 4: for every K2 site the pairs in which it is the partner (rows ascending)
-  if (tid < 32) {
-    for (int j = n1 + lane; j < n12; j += 32) k2cnt[j] = 0;
-    __syncwarp();
-    for (int i = 0; i < n1; ++i) {
-      const int b = k2start[i], e = k2start[i + 1];
-      for (int t = b + lane; t < e; t += 32) ++k2cnt[w.pr_ij[2 * (offp + t) + 1]];
-      __syncwarp();
-    }
-    if (lane == 0) {
-      int run = 0;
-      for (int j = n1; j < n12; ++j) {
-        int cj = k2cnt[j];
-        w.k2ptr[sbase + j] = run;
-        k2cnt[j] = run;
-        run += cj;
+  // phase 4: for every K2 site the pairs in which it is the partner, ascending (rows ascending): a
+  // counting sort by the whole block, whose lists (a few entries each) are then put in order.  One warp
+  // going through the rows took as long as the rest of the kernel.
+  const int kb = k2start[0], ke = k2start[n1];
+  for (int j = n1 + tid; j < n12; j += blockDim.x) k2cnt[j] = 0;
+  __syncthreads();
+  for (int t = kb + tid; t < ke; t += blockDim.x) atomicAdd(&k2cnt[w.pr_ij[2 * (offp + t) + 1]], 1);
+  __syncthreads();
+  if (warp == 0) {
+    int run = 0;
+    for (int j0 = n1; j0 < n12; j0 += 32) {
+      const int j = j0 + lane, v = j < n12 ? k2cnt[j] : 0;
+      int x = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
       }
-      w.k2ptr[sbase + n12] = run;
+      if (j < n12) w.k2ptr[sbase + j] = k2cnt[j] = run + x - v;
+      run += __shfl_sync(0xffffffffu, x, 31);
     }
-    __syncwarp();
-    for (int i = 0; i < n1; ++i) {
-      const int b = k2start[i], e = k2start[i + 1];
-      for (int t = b + lane; t < e; t += 32) {
-        const int j = w.pr_ij[2 * (offp + t) + 1];
-        w.k2rev[offp + k2cnt[j]] = t;
-        ++k2cnt[j];
-      }
-      __syncwarp();
+    if (lane == 0) w.k2ptr[sbase + n12] = run;
+  }
+  __syncthreads();
+  for (int t = kb + tid; t < ke; t += blockDim.x) w.k2rev[offp + atomicAdd(&k2cnt[w.pr_ij[2 * (offp + t) + 1]], 1)] = t;
+  __threadfence_block();
+  __syncthreads();
+  for (int j = n1 + tid; j < n12; j += blockDim.x) {   // k2cnt[j] is the end of list j now
+    int* list = w.k2rev + offp;
+    const int first = w.k2ptr[sbase + j], end = k2cnt[j];
+    for (int u = first + 1; u < end; ++u) {
+      const int v = list[u];
+      int k = u;
+      for (; k > first && list[k - 1] > v; --k) list[k] = list[k - 1];
+      list[k] = v;
     }
   }
 }
@@ -351,17 +375,37 @@ __global__ void __launch_bounds__(128) k_pair_radial(Work w, DevParams p) {
     const double v[4] = {A0, B0, dA0, dB0};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const ff t = ff_from_double(v[u]);
+      const ff t = ff_split(v[u]);
       w.rad_ff[4 * o + u] = make_float2(t.hi, t.lo);
     }
   }
 }
 
-// FP64 damped radial terms F A0, F B0 of pair pq at SCS frequency q (LU fallback): from the
-// atom-pair table, or evaluated when the pair has no table entry
-__device__ __forceinline__ void pair_rad64(const Work& w, const DevParams& p, int c, int q, long long pq, double& fa,
-                                           double& fb) {
-  const double* g = w.pr_geo + 8 * pq;
+// FP64 geometry and damping of pair pq of centre c (LU fallback, and pairs without a table entry).
+struct PairGeo64 {
+  double x[3], r, ir, F;
+};
+__device__ PairGeo64 pair_geo64(const Work& w, const DevParams& p, int c, long long pq) {
+  const long long sbase = (long long)c * w.site_cap;
+  const int i = w.pr_ij[2 * pq], j = w.pr_ij[2 * pq + 1];
+  const double *xi = w.site_x + 3 * (sbase + i), *xj = w.site_x + 3 * (sbase + j);
+  PairGeo64 g;
+  for (int d = 0; d < 3; ++d) g.x[d] = xj[d] - xi[d];
+  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(g.x[0], g.x[0]), __dmul_rn(g.x[1], g.x[1])), __dmul_rn(g.x[2], g.x[2]));
+  g.ir = rsqrt(r2);
+  g.r = r2 * g.ir;
+  double fsr, dfsr, fin = 1.0, dfin = 0.0;
+  cutoff_buf(g.r, p.r_scs, p.r_buf, fsr, dfsr);
+  if (j >= w.counts[c].n1) finner(g.r, p.r_inner, fin, dfin);
+  const double x = g.r / (p.beta * (w.rvdw[w.site_atom[sbase + i]] + w.rvdw[w.site_atom[sbase + j]]));
+  g.F = fin * fsr * (1.0 - 1.0 / (1.0 + exp(-p.d * (x - 1.0))));
+  return g;
+}
+
+// FP64 damped radial terms F A0, F B0 of the pair at SCS frequency q: from the atom-pair table, or
+// evaluated when the pair has no table entry
+__device__ __forceinline__ void pair_rad64(const Work& w, const DevParams& p, int c, int q, long long pq,
+                                           const PairGeo64& g, double& fa, double& fb) {
   const int gi = w.pr_ga[pq].x;
   double A0, B0;
   if (gi >= 0) {
@@ -374,10 +418,10 @@ __device__ __forceinline__ void pair_rad64(const Work& w, const DevParams& p, in
     const double si = w.sig[(long long)w.site_atom[sbase + i] * p.nqs + q];
     const double sj = w.sig[(long long)w.site_atom[sbase + j] * p.nqs + q];
     double dA0, dB0;
-    tsr_radial_fast(g[3], g[6], si * si + sj * sj, A0, B0, dA0, dB0);
+    tsr_radial_fast(g.r, g.ir, si * si + sj * sj, A0, B0, dA0, dB0);
   }
-  fa = g[4] * A0;
-  fb = g[4] * B0;
+  fa = g.F * A0;
+  fb = g.F * B0;
 }
 
 // the right-hand side of Eq. local_pol in FP64 (LU fallback), alpha_bar from global memory
@@ -390,15 +434,15 @@ __device__ void scs2_build_rhs64(const Work& w, const DevParams& p, int c, int n
     for (int t = b; t < en; ++t) {
       const long long pq = offp + t;
       const int j = w.pr_ij[2 * pq + 1];
-      const double* g = w.pr_geo + 8 * pq;
+      const PairGeo64 g = pair_geo64(w, p, c, pq);
       double fa, fb;
-      pair_rad64(w, p, c, q, pq, fa, fb);
+      pair_rad64(w, p, c, q, pq, g, fa, fb);
       const double abj = w.abar[(long long)w.site_atom[sbase + j] * p.nqs + q];
       ad += abj * fa;
-      const double wb = abj * fb * g[cc];
-      a0 += wb * g[0];
-      a1 += wb * g[1];
-      a2 += wb * g[2];
+      const double wb = abj * fb * g.x[cc];
+      a0 += wb * g.x[0];
+      a1 += wb * g.x[1];
+      a2 += wb * g.x[2];
     }
     double* y = rhs + 9 * i;
     y[cc] = (cc == 0 ? 1.0 : 0.0) - a0 - (cc == 0 ? ad : 0.0);
@@ -743,7 +787,7 @@ __device__ void cg_residual_update(const Work& w, const DevParams& p, int c, int
 __device__ __noinline__ void pair_rad_slow(const Work& w, const DevParams& p, int c, int q, long long pq, ff& fa,
                                            ff& fb) {
   double da, db;   // no table entry (a distance that ties r_SCS to rounding): evaluate in FP64
-  pair_rad64(w, p, c, q, pq, da, db);
+  pair_rad64(w, p, c, q, pq, pair_geo64(w, p, c, pq), da, db);
   fa = ff_from_double(da);
   fb = ff_from_double(db);
 }
@@ -1039,11 +1083,11 @@ struct ConSum {
 __device__ __noinline__ void pair_terms_slow(const Work& w, const DevParams& p, int c, int q, long long pq, ff& A0,
                                              ff& B0, ff& dA0, ff& dB0) {
   const long long sbase = (long long)c * w.site_cap;
-  const double* g = w.pr_geo + 8 * pq;
+  const PairGeo64 g = pair_geo64(w, p, c, pq);
   const double si = w.sig[(long long)w.site_atom[sbase + w.pr_ij[2 * pq]] * p.nqs + q];
   const double sj = w.sig[(long long)w.site_atom[sbase + w.pr_ij[2 * pq + 1]] * p.nqs + q];
   double a, b, da, db;
-  tsr_radial_fast(g[3], g[6], si * si + sj * sj, a, b, da, db);
+  tsr_radial_fast(g.r, g.ir, si * si + sj * sj, a, b, da, db);
   A0 = ff_from_double(a); B0 = ff_from_double(b); dA0 = ff_from_double(da); dB0 = ff_from_double(db);
 }
 __device__ __forceinline__ void pair_terms(const Work& w, const DevParams& p, int c, int q, long long pq, int gi, float4 u,
@@ -1108,7 +1152,7 @@ __global__ void __launch_bounds__(256, 2) k_scs_contract(Work w, DevParams p, in
     for (int e = tid; e < nqc * 9 * n1; e += blockDim.x) {
       const int down = w.lexp[(long long)c * p.nqs + q0 + e / (9 * n1)] - lexp;
       const float f = down < -126 ? 0.f : __int_as_float((down + 127) << 23);
-      const ff l = ff_from_double(Lg[(long long)q0 * 9 * n1 + e]), x = ff_from_double(Xg[(long long)q0 * 9 * n1 + e]);
+      const ff l = ff_split(Lg[(long long)q0 * 9 * n1 + e]), x = ff_split(Xg[(long long)q0 * 9 * n1 + e]);
       Ls[e] = make_float2(l.hi * f, l.lo * f);
       Xs[e] = make_float2(x.hi, x.lo);
     }
@@ -1278,12 +1322,12 @@ __device__ void scs2_dense_b(const Work& w, const DevParams& p, int c, int q, in
   for (int t = threadIdx.x; t < nk1; t += blockDim.x) {
     const long long pq = offp + t;
     const int i = w.pr_ij[2 * pq], j = w.pr_ij[2 * pq + 1];
-    const double* g = w.pr_geo + 8 * pq;
+    const PairGeo64 g = pair_geo64(w, p, c, pq);
     double fa, fb;
-    pair_rad64(w, p, c, q, pq, fa, fb);
+    pair_rad64(w, p, c, q, pq, g, fa, fb);
     for (int al = 0; al < 3; ++al)
       for (int be = 0; be < 3; ++be) {
-        const double v = fb * g[al] * g[be] + (al == be ? fa : 0.0);
+        const double v = fb * g.x[al] * g.x[be] + (al == be ? fa : 0.0);
         A[(long long)(3 * i + al) * N1 + 3 * j + be] = v;
         A[(long long)(3 * j + be) * N1 + 3 * i + al] = v;
       }
@@ -1455,7 +1499,7 @@ void launch_scs_count(const Work& w, const DevParams& p, int max_n12, cudaStream
 void launch_scs_fill(const Work& w, const DevParams& p, int c0, int c1, int max_n12, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
   size_t sm = sizeof(double) * 3 * (size_t)max_n12 +
-              sizeof(int) * ((size_t)max_n1 * max_n1 + 7 * (size_t)max_n1 + 3 + (size_t)max_n12 + 8 * (size_t)max_n1) +
+              sizeof(int) * ((size_t)max_n1 * max_n1 + 7 * (size_t)max_n1 + 3 + (size_t)max_n12) +
               sizeof(float) * 3 * (size_t)max_n12;
   raise_smem_limit((const void*)k_scs_fill, sm);
   k_scs_fill<<<c1 - c0, 256, sm, s>>>(w, p, c0, max_n12, max_n1);

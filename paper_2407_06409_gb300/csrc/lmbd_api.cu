@@ -291,7 +291,6 @@ struct Layout {
     int* pr_ij = cv.take<int>(2 * (np + 1), 2 * p0);
     float4* pr_rad4 = cv.take<float4>(nqs * (np + 1), nqs * p0);
     int2* pr_ga = cv.take<int2>(np + 1, p0);
-    double* pr_geo = cv.take<double>(8 * (np + 1), 8 * p0);
     float2* pr_gff = cv.take<float2>(6 * (np + 1), 6 * p0);
     int* k2rev = cv.take<int>(np + 1, p0);
     int* prow = cv.take<int>(nk + n, k0 + c0);
@@ -304,7 +303,6 @@ struct Layout {
       w->pr_ij = pr_ij;
       w->pr_rad4 = pr_rad4;
       w->pr_ga = pr_ga;
-      w->pr_geo = pr_geo;
       w->pr_gff = pr_gff;
       w->k2rev = k2rev;
       w->prow = prow;

@@ -119,14 +119,13 @@ struct Work {
   // SCS pair lists (one list per central atom; rows = coupled sites of K1)
   int* pcount;                 // N x 2: pairs, adjacency entries
   int* pr_ij;                  // pairs x 2: owner row i (K1), partner j (K1 with j < i, or K2)
-  double* pr_geo;              // pairs x 8: r = x_j - x_i (3), |r|, F, dF/dr, 1/|r|, unused
   float4* pr_rad4;             // per centre (off_p nq) [nq][K1 pairs]: F A0, F B0 as float-float (hi, lo)
   int2* pr_ga;                 // pairs: index of the pair in the atom-pair radial table (-1 = none), atom of j
   // radial terms of T_SR per atom pair and frequency, independent of the central atom: entry
   // off_k1[a] + s is atom a with site s (1 <= s < n1) of its own K1 list
   double* rad_ab;              // sum n1 x nq x 2: A0, B0
   float2* rad_ff;              // sum n1 x nq x 4: A0, B0, dA0/dr, dB0/dr as float-float (hi, lo)
-  float2* pr_gff;              // pairs x 6: r (3), F, dF/dr, 1/|r| as float-float (SCS adjoint)
+  float2* pr_gff;              // pairs x 6: r = x_j - x_i (3), F, dF/dr, 1/|r| as float-float
   int* prow;                   // (sum n1 + N): first K1 pair of each row, per centre n1 + 1 entries
   int* prow_k2;                // (sum n1 + N): first K2 pair of each row (after all K1 pairs)
   int* arow;                   // (sum n1 + N): first adjacency entry of each row
