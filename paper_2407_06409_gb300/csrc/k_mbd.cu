@@ -320,9 +320,11 @@ __device__ __forceinline__ double series_c(const Work& w, const DevParams& p, in
 // G = D T_LR D from m Lanczos steps (three-term recurrence, no reorthogonalisation, start
 // vector from SplitMix64), then c_n, n = 1..n_max, of the L2 fit of ln(1 - lambda) on it.
 // ---------------------------------------------------------------------------------------
-#define LZ_THREADS 256
+#define LZ_THREADS 256    // log mode
 #define LZ_RPT 4          // rows per thread: 3 ns <= 1024
-#define LZ_QC 12          // frequencies per pass
+#define LZ_QC 12          // vectors per pass
+#define LF_THREADS 512    // fit coefficients: two rows per thread
+#define LF_CHUNK 8        // products summed up between two additions to the running float-float sum
 
 // SplitMix64 output for counter i (state 0 advanced i + 1 times), mapped to [-1, 1).
 __device__ __forceinline__ double splitmix_unit(unsigned long long i) {
@@ -437,16 +439,194 @@ __device__ bool tridiag_ql_first_row(double* a, double* b, double* z, int m) {
   return true;
 }
 
-// Lanczos recurrences on G(omega) = D T_LR D for every frequency of this pass (frequencies
-// q0 ..), nd start vectors per frequency (vector v <-> frequency q0 + v / nd, direction v % nd):
-//  * nd = 1 (polynomial-fit coefficients, Sec. III.A): SplitMix64 start vector, the extreme
-//    Ritz values go to w.lam;
-//  * nd = 3 (log mode): start vectors e_alpha, the centre's three rows; the Gauss rule of the
-//    tridiagonal matrix J (Ritz values theta_i, squared first components z_i^2) gives
-//    e_alpha^T ln(1 - G) e_alpha ~ sum_i z_i^2 ln(1 - theta_i) (exact once the Krylov space is
-//    exhausted, b = 0), and the three directions sum to the k-block trace of ln(1 - G)
-//    (Eq. series-expansion, the n_max -> infinity limit), stored per frequency in trbuf row 0.
-__global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int c0, int q0, int qc, int L3, int nd) {
+// Sums the QC (at most 16) per-thread partials v[q] over the block into tot[q] (shared).  Each exchange
+// halves the number of values a lane holds: 16 additions a warp instead of five for every value.
+template <int QC>
+__device__ __forceinline__ void lf_block_sum(const double* v, double* red, double* tot) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double t[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) t[q] = q < QC ? v[q] : 0.0;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int half = 8 >> b;
+    const bool up = (lane >> b) & 1;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const double send = up ? t[j] : t[j + half];
+      t[j] = (up ? t[j + half] : t[j]) + __shfl_xor_sync(0xffffffffu, send, 1 << b);
+    }
+  }
+  t[0] += __shfl_xor_sync(0xffffffffu, t[0], 16);
+  const int q = (lane & 1) * 8 + (lane >> 1 & 1) * 4 + (lane >> 2 & 1) * 2 + (lane >> 3 & 1);
+  if (lane < 16 && q < QC) red[q * (LF_THREADS / 32) + warp] = t[0];
+  __syncthreads();
+  if (threadIdx.x < QC) {
+    double u = 0.0;
+    for (int k = 0; k < LF_THREADS / 32; ++k) u += red[threadIdx.x * (LF_THREADS / 32) + k];
+    tot[threadIdx.x] = u;
+  }
+  __syncthreads();
+}
+
+// Extreme Ritz values of G(omega) = D T_LR D for the qc <= QC frequencies q0 .. of this pass, from
+// p.lanczos steps with the SplitMix64 start vector, into w.lam (polynomial-fit coefficients, Sec. III.A).
+// The products with T_LR are all of the work, QC N^2 multiply-adds a step: in FP64 they kept that pipe
+// busy for 13 of this kernel's 26 ms (300 atoms, 12 frequencies, 12 steps), and every thread adding up
+// the block sums took most of the rest.  Here a product is float-float (a lane per row, QC columns at a
+// time, so an element of T_LR is read and split once for all of them), LF_CHUNK products are summed with
+// their rounding errors and then added to the running sum, which keeps its error at that of an
+// FP64 sum of this length.  The recurrence itself stays in FP64: v and the vector that becomes the
+// next one lie in shared memory, column-major and touched only by the thread of their row.
+// 300 atoms (spheres of 143 sites), 12 frequencies, 12 steps: 25.8 -> 6.1 ms.
+template <int QC>
+__global__ void __launch_bounds__(LF_THREADS) k_lanczos_fit(Work w, DevParams p, int c0, int q0, int qc, int L3) {
+  extern __shared__ double lfs[];
+  const int c = c0 + blockIdx.x;
+  if (c >= w.n_atoms) return;
+  const int ns = w.counts[c].ns, N = 3 * ns;
+  double* V = lfs;                                  // QC x L3
+  double* U = V + (size_t)L3 * QC;                  // QC x L3: previous vector, then the next one
+  float2* X = reinterpret_cast<float2*>(U + (size_t)L3 * QC);   // (L3 + LF_CHUNK) x QC: D v as float-float
+  double* al = reinterpret_cast<double*>(X + (size_t)(L3 + LF_CHUNK) * QC);   // QC x LMBD_MAX_LANCZOS
+  double* be = al + QC * LMBD_MAX_LANCZOS;
+  double* red = be + QC * LMBD_MAX_LANCZOS;         // QC x (threads / 32)
+  __shared__ int mq[QC];                            // steps taken per frequency, negative when finished
+  __shared__ double tot[QC], binv[QC], bprev[QC];
+  const int tid = threadIdx.x;
+  const double* T = w.tlr + w.off_t[c];
+  const double* dq = w.dsq + w.off_s[c] * p.nq + q0 + 1;
+  const int m = min(p.lanczos, N);
+  double part[QC];
+  // start vector u / |u| for every frequency
+  for (int q = 0; q < QC; ++q) part[q] = 0.0;
+  for (int i = tid; i < N; i += LF_THREADS) {
+    const double u = splitmix_unit((unsigned long long)i);
+    part[0] += u * u;
+  }
+  lf_block_sum<QC>(part, red, tot);
+  {
+    const double inv = 1.0 / sqrt(tot[0]);
+    for (int i = tid; i < N; i += LF_THREADS) {
+      const double u = splitmix_unit((unsigned long long)i) * inv;
+#pragma unroll
+      for (int q = 0; q < QC; ++q) {
+        V[q * L3 + i] = u;
+        U[q * L3 + i] = 0.0;
+      }
+    }
+  }
+  for (int e = tid; e < LF_CHUNK * QC; e += LF_THREADS) X[N * QC + e] = make_float2(0.f, 0.f);
+  if (tid < QC) {
+    mq[tid] = tid < qc ? 0 : -1;
+    bprev[tid] = 0.0;
+  }
+  for (int j = 0; j < m; ++j) {
+    for (int i = tid; i < N; i += LF_THREADS)
+#pragma unroll
+      for (int q = 0; q < QC; ++q) {
+        const ff x = ff_split(q < qc ? dq[(long long)(i / 3) * p.nq + q] * V[q * L3 + i] : 0.0);
+        X[i * QC + q] = make_float2(x.hi, x.lo);
+      }
+    __syncthreads();
+    // u <- D T x - beta v_prev: T is symmetric, so lane i reads column i of row k (coalesced)
+    for (int i0 = tid & ~31; i0 < N; i0 += LF_THREADS) {
+      const int i = i0 + (tid & 31);
+      const double* Tc = T + min(i, N - 1);
+      ff y[QC];
+#pragma unroll
+      for (int q = 0; q < QC; ++q) y[q] = ff_make(0.f, 0.f);
+      double tn[LF_CHUNK];
+#pragma unroll
+      for (int u = 0; u < LF_CHUNK; ++u) tn[u] = u < N ? Tc[(long long)u * N] : 0.0;
+#pragma unroll 1
+      for (int k = 0; k < N; k += LF_CHUNK) {
+        double t[LF_CHUNK];
+#pragma unroll
+        for (int u = 0; u < LF_CHUNK; ++u) {
+          t[u] = tn[u];
+          tn[u] = k + LF_CHUNK + u < N ? Tc[(long long)(k + LF_CHUNK + u) * N] : 0.0;
+        }
+        float h[QC], l[QC];
+#pragma unroll
+        for (int q = 0; q < QC; ++q) h[q] = l[q] = 0.f;
+#pragma unroll
+        for (int u = 0; u < LF_CHUNK; ++u) {
+          const ff a = ff_split(t[u]);
+          const float4* xk = reinterpret_cast<const float4*>(X + (k + u) * QC);
+#pragma unroll
+          for (int q = 0; q < QC; q += 2) {
+            const float4 x = xk[q / 2];
+            ff_mac(h[q], l[q], a, ff_make(x.x, x.y));
+            ff_mac(h[q + 1], l[q + 1], a, ff_make(x.z, x.w));
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < QC; ++q) y[q] = ff_add(y[q], ff_quick_two_sum(h[q], l[q]));
+      }
+      if (i < N)
+#pragma unroll
+        for (int q = 0; q < QC; ++q) {
+          const double d = q < qc ? dq[(long long)(i / 3) * p.nq + q] : 0.0;
+          U[q * L3 + i] = d * ff_to_double(y[q]) - bprev[q] * U[q * L3 + i];
+        }
+    }
+    // alpha = <v, u>
+    for (int q = 0; q < QC; ++q) part[q] = 0.0;
+    for (int i = tid; i < N; i += LF_THREADS)
+#pragma unroll
+      for (int q = 0; q < QC; ++q) part[q] += V[q * L3 + i] * U[q * L3 + i];
+    lf_block_sum<QC>(part, red, tot);
+    if (tid < QC && mq[tid] == j) al[tid * LMBD_MAX_LANCZOS + j] = tot[tid];
+    // u <- u - alpha v, beta = |u|
+    for (int q = 0; q < QC; ++q) part[q] = 0.0;
+    for (int i = tid; i < N; i += LF_THREADS)
+#pragma unroll
+      for (int q = 0; q < QC; ++q) {
+        const double u = U[q * L3 + i] - tot[q] * V[q * L3 + i];
+        U[q * L3 + i] = u;
+        part[q] += u * u;
+      }
+    lf_block_sum<QC>(part, red, tot);
+    if (tid < QC) {
+      const double beta = sqrt(tot[tid]);
+      bool on = mq[tid] == j;                // still running
+      if (on) {
+        mq[tid] = j + 1;
+        on = j < m - 1 && beta != 0.0;
+        if (on) be[tid * LMBD_MAX_LANCZOS + j] = beta;
+        else mq[tid] = -(j + 1);             // finished with j + 1 steps
+      }
+      bprev[tid] = beta;
+      binv[tid] = on ? 1.0 / beta : 0.0;     // a finished column goes on with zeros
+    }
+    __syncthreads();
+    bool running = false;
+    for (int q = 0; q < QC; ++q) running |= mq[q] > 0;
+    if (!running) break;
+    for (int i = tid; i < N; i += LF_THREADS)
+#pragma unroll
+      for (int q = 0; q < QC; ++q) U[q * L3 + i] *= binv[q];
+    double* t = V;
+    V = U;
+    U = t;
+  }
+  // extremes of the tridiagonal matrices
+  if (tid < 2 * qc) {
+    const int q = tid >> 1, mm = abs(mq[q]);
+    w.lam[((long long)c * p.n_freq + q0) * 2 + tid] =
+        lz_eig(al + q * LMBD_MAX_LANCZOS, be + q * LMBD_MAX_LANCZOS, mm, tid & 1 ? mm - 1 : 0);
+  }
+}
+
+// Log mode: Lanczos recurrences on G(omega) = D T_LR D for every frequency of this pass (frequencies
+// q0 ..) with the three start vectors e_alpha of the centre's rows (vector v <-> frequency q0 + v / 3,
+// direction v % 3).  The Gauss rule of the tridiagonal matrix J (Ritz values theta_i, squared first
+// components z_i^2) gives e_alpha^T ln(1 - G) e_alpha ~ sum_i z_i^2 ln(1 - theta_i) (exact once the
+// Krylov space is exhausted, b = 0), and the three directions sum to the k-block trace of ln(1 - G)
+// (Eq. series-expansion, the n_max -> infinity limit), stored per frequency in trbuf row 0.  The
+// products stay in FP64: whether the space is exhausted is decided at FP64 rounding.
+__global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int c0, int q0, int qc, int L3) {
   extern __shared__ double lzs[];
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
@@ -462,30 +642,13 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int
   const int tid = threadIdx.x;
   const double* T = w.tlr + w.off_t[c];
   const long long offs = w.off_s[c];
-  const bool logm = nd == 3;
-  const int m = min(logm ? p.logmode : p.lanczos, N);
-  // start vectors: u / |u| for every frequency, or e_alpha
+  const int m = min(p.logmode, N);
   double part[LZ_QC];
-  double tot[LZ_QC];
-  for (int q = 0; q < LZ_QC; ++q) part[q] = 0.0;
-  double inv = 1.0;
-  if (!logm) {
-    for (int r = 0; r < LZ_RPT; ++r) {
-      const int i = tid + r * LZ_THREADS;
-      if (i < N) {
-        const double u = splitmix_unit((unsigned long long)i);
-        part[0] += u * u;
-      }
-    }
-    lz_block_sum(part, 1, red, tot);
-    inv = 1.0 / sqrt(tot[0]);
-  }
   for (int r = 0; r < LZ_RPT; ++r) {
     const int i = tid + r * LZ_THREADS;
     if (i < N) {
-      const double u = logm ? 0.0 : splitmix_unit((unsigned long long)i) * inv;
       for (int q = 0; q < qc; ++q) {
-        V[i * qc + q] = logm ? (i == q % 3 ? 1.0 : 0.0) : u;
+        V[i * qc + q] = i == q % 3 ? 1.0 : 0.0;   // e_alpha
         Vp[i * qc + q] = 0.0;
       }
     }
@@ -499,7 +662,7 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int
     // X = D V
     for (int e = tid; e < N * qc; e += LZ_THREADS) {
       const int i = e / qc, q = e % qc;
-      X[e] = w.dsq[(offs + i / 3) * p.nq + q0 + q / nd + 1] * V[e];
+      X[e] = w.dsq[(offs + i / 3) * p.nq + q0 + q / 3 + 1] * V[e];
     }
     __syncthreads();
     // Y = D (T X): T symmetric, so thread i reads column i of row k (coalesced)
@@ -531,7 +694,7 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int
 #pragma unroll
         for (int q = 0; q < LZ_QC; ++q)
           if (q < qc) {
-            y[r][q] *= w.dsq[(offs + i / 3) * p.nq + q0 + q / nd + 1];
+            y[r][q] *= w.dsq[(offs + i / 3) * p.nq + q0 + q / 3 + 1];
             part[q] += V[i * qc + q] * y[r][q];
           }
       }
@@ -559,13 +722,12 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int
     if (tid < qc && mq[tid] == j) {           // frequency still running: record step j
       al[tid * LMBD_MAX_LANCZOS + j] = alpha[tid];
       mq[tid] = j + 1;
-      // log mode: a beta below 1e-13 of the largest recurrence coefficient so far means the
+      // a beta below 1e-13 of the largest recurrence coefficient so far means the
       // Krylov space is exhausted to rounding (the Gauss rule is then exact)
       double scale = 0.0;
-      if (logm)
-        for (int u = 0; u <= j; ++u)
-          scale = fmax(scale, fabs(al[tid * LMBD_MAX_LANCZOS + u]) + (u < j ? be[tid * LMBD_MAX_LANCZOS + u] : 0.0));
-      if (j < m - 1 && beta[tid] != 0.0 && !(logm && beta[tid] <= 1e-13 * scale)) {
+      for (int u = 0; u <= j; ++u)
+        scale = fmax(scale, fabs(al[tid * LMBD_MAX_LANCZOS + u]) + (u < j ? be[tid * LMBD_MAX_LANCZOS + u] : 0.0));
+      if (j < m - 1 && beta[tid] != 0.0 && !(beta[tid] <= 1e-13 * scale)) {
         be[tid * LMBD_MAX_LANCZOS + j] = beta[tid];
       } else {
         mq[tid] = -(j + 1);                   // finished with j + 1 steps
@@ -590,18 +752,6 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(Work w, DevParams p, int
     bool running = false;
     for (int q = 0; q < qc; ++q) running |= mq[q] > 0;
     if (!running) break;
-  }
-  if (!logm) {
-    // extremes of the tridiagonal matrices
-    if (tid < qc) {
-      const int mm = mq[tid] < 0 ? -mq[tid] : mq[tid];
-      const double* a = al + tid * LMBD_MAX_LANCZOS;
-      const double* b = be + tid * LMBD_MAX_LANCZOS;
-      double* out = w.lam + ((long long)c * p.n_freq + q0 + tid) * 2;
-      out[0] = lz_eig(a, b, mm, 0);
-      out[1] = lz_eig(a, b, mm, mm - 1);
-    }
-    return;
   }
   // log mode: Gauss rule of every tridiagonal, then the sum over the three directions
   double* lq = red;                               // qc partial traces (red is free now)
@@ -693,26 +843,51 @@ __global__ void __launch_bounds__(128) k_series_fit(Work w, DevParams p, int c0,
   }
 }
 
-// Lanczos passes over the frequencies: nd vectors per frequency, three L3 x (vectors) arrays in
-// shared memory next to the recurrence coefficients; frequencies of one pass share T_LR reads.
-static bool launch_lanczos(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int nd, cudaStream_t s) {
+// Lanczos passes over the frequencies, which share the reads of T_LR within a pass: as many as the
+// vectors in shared memory leave room for, in a kernel for 4, 8 or 12 columns.
+template <int QC>
+static size_t lanczos_fit_smem(int L3) {
+  return sizeof(double) * QC * (3 * (size_t)L3 + LF_CHUNK + 2 * LMBD_MAX_LANCZOS + LF_THREADS / 32);
+}
+
+template <int QC>
+static void run_lanczos_fit(const Work& w, const DevParams& p, int c0, int c1, int q0, int n, int L3, cudaStream_t s) {
+  const size_t sm = lanczos_fit_smem<QC>(L3);
+  raise_smem_limit((const void*)k_lanczos_fit<QC>, sm);
+  k_lanczos_fit<QC><<<c1 - c0, LF_THREADS, sm, s>>>(w, p, c0, q0, n, L3);
+}
+
+static bool launch_lanczos_fit(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
   const int L3 = 3 * max_ns;
   if (L3 > LZ_THREADS * LZ_RPT) return false;
-  const size_t per_v = sizeof(double) * (3 * (size_t)L3 + 2 * LMBD_MAX_LANCZOS + LZ_THREADS / 32);
-  int qf = (int)((200 * 1024) / (per_v * nd));       // frequencies per pass
-  qf = std::max(1, std::min(std::min(qf, LZ_QC / nd), p.n_freq));
+  const size_t room = 216 * 1024;
+  const int qf = lanczos_fit_smem<12>(L3) <= room ? 12 : lanczos_fit_smem<8>(L3) <= room ? 8 : 4;
   for (int q0 = 0; q0 < p.n_freq; q0 += qf) {
     const int n = std::min(qf, p.n_freq - q0);
-    const size_t sm = per_v * n * nd;
-    raise_smem_limit((const void*)k_lanczos, sm);
-    k_lanczos<<<c1 - c0, LZ_THREADS, sm, s>>>(w, p, c0, q0, n * nd, L3, nd);
+    if (n > 8) run_lanczos_fit<12>(w, p, c0, c1, q0, n, L3, s);
+    else if (n > 4) run_lanczos_fit<8>(w, p, c0, c1, q0, n, L3, s);
+    else run_lanczos_fit<4>(w, p, c0, c1, q0, n, L3, s);
+  }
+  return true;
+}
+
+static bool launch_lanczos(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
+  const int L3 = 3 * max_ns;
+  if (L3 > LZ_THREADS * LZ_RPT) return false;
+  const size_t per_f = 3 * sizeof(double) * (3 * (size_t)L3 + 2 * LMBD_MAX_LANCZOS + LZ_THREADS / 32);
+  int qf = (int)((200 * 1024) / per_f);              // frequencies per pass
+  qf = std::max(1, std::min(std::min(qf, LZ_QC / 3), p.n_freq));
+  for (int q0 = 0; q0 < p.n_freq; q0 += qf) {
+    const int n = std::min(qf, p.n_freq - q0);
+    raise_smem_limit((const void*)k_lanczos, per_f * n);
+    k_lanczos<<<c1 - c0, LZ_THREADS, per_f * n, s>>>(w, p, c0, q0, n * 3, L3);
   }
   return true;
 }
 
 bool launch_series_coefficients(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return true;
-  if (!launch_lanczos(w, p, c0, c1, max_ns, 1, s)) return false;
+  if (!launch_lanczos_fit(w, p, c0, c1, max_ns, s)) return false;
   const long long items = (long long)(c1 - c0) * p.n_freq;
   k_series_fit<<<(unsigned)((items + 127) / 128), 128, 0, s>>>(w, p, c0, c1);
   return true;
@@ -720,7 +895,7 @@ bool launch_series_coefficients(const Work& w, const DevParams& p, int c0, int c
 
 bool launch_log_mode(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return true;
-  return launch_lanczos(w, p, c0, c1, max_ns, 3, s);
+  return launch_lanczos(w, p, c0, c1, max_ns, s);
 }
 
 // ---------------------------------------------------------------------------------------
