@@ -27,15 +27,15 @@ if ROOT not in sys.path:
 METRIC = "atoms/s for lMBD energy+forces on 1 GB300 (batched vs per-atom launch); serve p50/p99"
 FP64_PEAK_TFLOPS = 1.25          # nominal GB300 FP64 (DFMA and DMMA), profiling recipe table
 FP32_PEAK_TFLOPS = 80.5          # 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz (unit counts and clock)
-# DRAM bytes (read + write) of the SCS factor kernel (k_scs_factor alone) per atom: ncu on the
-# 512-atom box, profiles/ncu_scs_factor_box512.md; scaled to a launch by atoms / launches
-SCS_FACTOR_DRAM_BYTES_PER_ATOM = 1.189e6
+# DRAM bytes (read + write) of the forward SCS solves (k_scs_solve) per atom: ncu on the
+# 512-atom box, profiles/ncu_all_kernels_box512.md; scaled to a launch by atoms / launches
+SCS_SOLVE_DRAM_BYTES_PER_ATOM = 0.314e6
 PRECISION = ("chain products: 6-digit (energy blocks) / 5-digit (adjoint-only blocks) bf16 Ozaki slices "
-             "of the FP64 operands, exact integer recombination, FP64 scaling; adjoint pair product: "
-             "5-digit slices; SCS: FP32 Cholesky and solves with FP64 iterative refinement to FP64 "
-             "accuracy; everything else FP64")
-PRECISION_FP64 = ("chain and adjoint pair products in FP64; SCS: FP32 Cholesky and solves with FP64 "
-                  "iterative refinement to FP64 accuracy; everything else FP64")
+             "of the operands, exact recombination; adjoint pair product: 5-digit slices, float-float "
+             "operands and epilogue; SCS: FP32 conjugate gradients with iterative refinement to FP64 "
+             "accuracy (float-float residuals); everything else FP64")
+PRECISION_FP64 = ("chain and adjoint pair products in FP64; SCS: FP32 conjugate gradients with "
+                  "iterative refinement to FP64 accuracy (float-float residuals); everything else FP64")
 WORKLOAD = ("periodic random box, 4096 atoms, 0.1 atoms/A^3, 4 species; r_SCS 5 A, MBD sphere 7 A "
             "(r_MBD,1 = r_MBD,2 = 7 A), 12 omega, n_max 6; energies + forces within 1e-10 rel. / "
             "1e-8 eV/A of the FP64 oracle (see precision)")
@@ -343,16 +343,16 @@ def run_ours(args, world, rank, local):
     fp64 = ("scs", "chain", "adj_pair", "adj_scs")
     dom = max(fp64, key=lambda ph: phase_ms.get(ph, 0.0))
     avg_ms = phase_ms[dom] / max(1, phase_launch[dom])
-    kernel_names = {"scs": "k_scs_factor", "chain": "k_chain_tc" if args.mma == "tc05" else "k_chain_oz2",
+    kernel_names = {"scs": "k_scs_solve", "chain": "k_chain_tc" if args.mma == "tc05" else "k_chain_oz2",
                     "adj_pair": "k_pair_tc" if args.mma == "tc05" else "k_mbd_adj_pair_oz2",
-                    "adj_scs": "k_scs_adjoint2"}
+                    "adj_scs": "k_scs_solve"}
     st_last = model.stats()
     if dom == "scs":
-        # The SCS factor kernel.  Method work (the dense linear algebra of the local screening
+        # The forward SCS solves.  Method work (the dense linear algebra of the local screening
         # solves): per centre and SCS frequency a Cholesky factorisation, (3 n1)^3 / 3 flops, and
         # 12 (3 n1)^2 for the triangular solves with 3 right-hand sides (the count of the work
-        # estimate of the scope table, independent of how many refinement corrections the
-        # kernel makes).  The factor runs on the FP32 SIMT pipe, so the peak is that pipe's
+        # estimate of the scope table; the kernel solves the same systems by conjugate gradients on
+        # their sparse pair lists).  It runs on the FP32 SIMT pipe, so the peak is that pipe's
         # nominal rate from unit counts and the maximum clock.  Time: the kernel's own bucket
         # launches, fork to join (CUDA events around them in the library).
         nq = 2 if args.omega_ref > 0 else (args.fit_nodes + 2 if args.fit_nodes > 0 else 13)
@@ -363,27 +363,24 @@ def run_ours(args, world, rank, local):
         t_fac = kernel_ms["scs_factor"] / args.steps * 1e-3 if kernel_ms["scs_factor"] > 0 else avg_ms * 1e-3
         work = w_method / n_fac
         achieved = work / (t_fac / n_fac) / 1e12
-        # the composite bound of the kernel's full instruction mix, as a second figure: FP32 work
-        # (factor, three solves of 3 right-hand sides) plus the float-float right-hand side and
-        # residuals (the FP64-equivalent flop count of those sums, each float-float multiply-add
-        # about 20 FP32 operations, i.e. 10 per FP64 flop), all on the FP32 pipe
-        w32 = nq * float(np.sum(N1 ** 3 / 3.0 + 18.0 * N1 ** 2))
+        # a second figure: the part of the kernel's instruction mix that the pair counts fix, the
+        # float-float right-hand side and residuals (the FP64-equivalent flop count of those sums, each
+        # float-float multiply-add about 20 FP32 operations, i.e. 10 per FP64 flop)
         pairs, adj = float(st_last["scs_pairs"]), float(st_last["scs_adjacency"])
         wff = nq * (60.0 * adj + 36.0 * (pairs - adj / 2.0) + 2.0 * pairs)
-        t_star = (w32 + 10.0 * wff) / (FP32_PEAK_TFLOPS * 1e12)
+        t_star = 10.0 * wff / (FP32_PEAK_TFLOPS * 1e12)
         roofline = {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP32_PEAK_TFLOPS,
-                    "traffic": SCS_FACTOR_DRAM_BYTES_PER_ATOM * args.atoms / n_fac,
+                    "traffic": SCS_SOLVE_DRAM_BYTES_PER_ATOM * args.atoms / n_fac,
                     "kernel": kernel_names[dom], "launches_per_step": n_fac, "ms_per_step": t_fac * 1e3,
                     "work_per_step": w_method,
-                    "peak_note": "method flops sum_k nq [(3 n1)^3/3 + 12 (3 n1)^2] over the kernel's own time, "
-                                 "against the FP32 SIMT pipe it runs on: 152 SMs x 128 lanes x 2 flops x "
+                    "peak_note": "flops of a dense solve, sum_k nq [(3 n1)^3/3 + 12 (3 n1)^2], over the time of "
+                                 "the kernel, which solves by conjugate gradients on the sparse pair lists, against the FP32 SIMT pipe it runs on: 152 SMs x 128 lanes x 2 flops x "
                                  "2.07 GHz = 80.5 TFLOP/s nominal (unit counts and maximum clock)",
-                    "composite": {"peak_note": "the kernel's whole instruction mix on the FP32 pipe (80.5 "
-                                               "TFLOP/s): factor, solves and refinement corrections, plus the "
-                                               "float-float right-hand side and residuals at 10 FP32 operations "
-                                               "per FP64-equivalent flop",
-                                  "work_fp32": w32, "work_float_float_fp64_equiv": wff, "t_star_ms": t_star * 1e3,
+                    "composite": {"peak_note": "the float-float right-hand side and residuals alone, at 10 "
+                                               "FP32 operations per FP64-equivalent flop, on the FP32 pipe "
+                                               "(80.5 TFLOP/s)",
+                                  "work_float_float_fp64_equiv": wff, "t_star_ms": t_star * 1e3,
                                   "frac": t_star / t_fac}}
     elif dom in ("chain", "adj_pair"):
         # sliced products on the bf16 tensor cores: the bf16 work is the FP64 product's flops times

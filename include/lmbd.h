@@ -85,7 +85,7 @@ typedef struct {
 
 /* Phases of one call, in launch order (index into the lmbd_stats arrays). */
 #define LMBD_PHASE_NEIGHBORS   0  /* free-atom terms, cell list, site lists, offsets          */
-#define LMBD_PHASE_SCS         1  /* T_SR assembly + Cholesky + solves, all atoms/frequencies */
+#define LMBD_PHASE_SCS         1  /* T_SR radial terms, pair lists, solves, all frequencies     */
 #define LMBD_PHASE_PREPARE     2  /* blend, SCS radii, T_LR, first Krylov block               */
 #define LMBD_PHASE_CHAIN       3  /* Krylov products v_{m+1} = D T D v_m                       */
 #define LMBD_PHASE_ENERGY      4  /* k-block traces and quadrature                            */
@@ -116,10 +116,10 @@ typedef struct {
   long long scs_pairs;     /* SCS site pairs over all central atoms (r < r_SCS, K1 x (K1 u K2)) */
   long long scs_adjacency; /* directed K1-K1 pair entries (two per K1-K1 pair)                 */
   double ms_kernel[2];     /* with profiling, one wave: device time of the bucket launches of
-                              [0] the SCS factor kernel, [1] the SCS adjoint kernel (all side
+                              [0] the forward SCS solves, [1] the adjoint SCS solves (all side
                               streams, fork to join; without the pair-list kernels)            */
   long long scs_lu_systems; /* (centre, frequency) screening systems solved by the LU fallback:
-                              the FP32 Cholesky met a non-positive pivot (B_K indefinite) or
+                              the FP32 solver met a non-positive curvature (B_K indefinite) or
                               its FP64 refinement did not converge                              */
   int sites_refreshed;     /* 1 if the call refreshed resident site lists (lmbd_set_verlet_skin)
                               instead of building them                                         */

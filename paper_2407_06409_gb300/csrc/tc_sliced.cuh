@@ -2,8 +2,9 @@
 // the Krylov-chain kernel (k_chain_tc.cu) and the adjoint pair-matrix kernel (k_pair_tc.cu).
 //
 // One CTA of 256 threads owns a 128 x NB output tile.  A (128 rows) and B (NB rows) are S digit
-// planes of signed 7-bit integers stored as bf16 (ozaki.cuh), K-major, addressed through 2-D
-// tensor maps (inner dimension K, one row per matrix row, 64-byte swizzle).  The loop
+// planes of signed 7-bit integers stored as bf16 (ozaki.cuh), K-major, brought
+// in by the caller's copy function: tile images (tcs_image_copy), or boxes of 2-D tensor maps (inner
+// dimension K, one row per matrix row, 64-byte swizzle) in tcs_mainloop.  The loop
 //   * stages K slices of 32 of every plane of A and B into a three-deep ring of 64-byte-swizzled
 //     shared-memory tiles with bulk tensor copies (TMA, cp.async.bulk.tensor) issued by one
 //     thread; each slot has a "full" mbarrier counting the bytes in flight (K past the tensor's
