@@ -475,8 +475,8 @@ __device__ __forceinline__ void lf_block_sum(const double* v, double* red, doubl
 // busy for 13 of this kernel's 26 ms (300 atoms, 12 frequencies, 12 steps), and every thread adding up
 // the block sums took most of the rest.  Here a product is float-float (a lane per row, QC columns at a
 // time, so an element of T_LR is read and split once for all of them), LF_CHUNK products are summed with
-// their rounding errors and then added to the running sum, which keeps its error at that of an
-// FP64 sum of this length.  The recurrence itself stays in FP64: v and the vector that becomes the
+// their rounding errors and then added to the running sum, so the low words stay small (energies of the
+// fitted series, error against 64 bits: 3.7e-13 with FP64 products, 3.3e-13 now).  The recurrence itself stays in FP64: v and the vector that becomes the
 // next one lie in shared memory, column-major and touched only by the thread of their row.
 // 300 atoms (spheres of 143 sites), 12 frequencies, 12 steps: 25.8 -> 6.1 ms.
 template <int QC>
