@@ -18,7 +18,8 @@ __device__ __forceinline__ ff ff_make(float hi, float lo) {
 }
 
 // (hi + lo) 2^shift as a double by integer instructions (normalised float-float, hi normal or zero;
-// low parts below 2^-46 of hi round away; zero below the double range).
+// low parts below 2^-46 of hi round away; zero below the double range, infinite above it, NaN when hi
+// is not finite).
 __device__ __forceinline__ double ff_join(ff a, int shift) {
   const unsigned hb = __float_as_uint(a.hi), sg = hb & 0x80000000u;
   const int e = (int)((hb >> 23) & 0xffu);
@@ -30,7 +31,8 @@ __device__ __forceinline__ double ff_join(ff a, int shift) {
   const int below = m < (1LL << 46);
   m <<= 6 + below;
   const int ex = e - 127 + 1023 - below + shift;
-  const long long r = ((long long)ex << 52) + (m & 0xfffffffffffffLL);
+  long long r = ((long long)ex << 52) + (m & 0xfffffffffffffLL);
+  if (e == 255 || ex >= 2047) r = e == 255 ? 0x7ff8000000000000LL : 0x7ff0000000000000LL;
   return e == 0 || ex <= 0 ? 0.0 : __longlong_as_double(r | ((long long)sg << 32));
 }
 
@@ -42,12 +44,14 @@ __device__ __forceinline__ ff ff_from_double(double x) {
 }
 
 // The same to 47 bits (nearest) by integer and FP32 instructions, for kernels whose FP64 pipe is the
-// bound: hi = the top 24 bits, lo = the next 23.  Finite values in the FP32 range; smaller ones give
-// zero.
+// bound: hi = the top 24 bits, lo = the next 23.  Values below 2^-126 give zero, the low part of those
+// below 2^-80 is zero; from 2^128 on, and for infinities and NaN, hi is not finite.
 __device__ __forceinline__ ff ff_split(double v) {
-  const double x = __longlong_as_double(__double_as_longlong(v) + 32);   // half of the last bit kept
-  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), sg = h & 0x80000000u;
-  const int e = (int)((h >> 20) & 0x7ffu) - (1023 - 127);   // biased FP32 exponent
+  const unsigned hv = (unsigned)__double2hiint(v), sg = hv & 0x80000000u;
+  // half of the last bit kept is added to |v|, in words: as one 64-bit mask it becomes an FP64 abs, whose
+  // result for a NaN has no fixed sign.  NaN of any payload stays at or above the exponent 0x7ff.
+  const unsigned l = (unsigned)__double2loint(v) + 32u, h = (hv & 0x7fffffffu) + (l < 32u ? 1u : 0u);
+  const int e = min((int)(h >> 20) - (1023 - 127), 255);   // biased FP32 exponent
   const unsigned hb = ((unsigned)max(e, 0) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);
   const float low = __fsub_rn(__uint_as_float(0x4B000000u | ((l >> 6) & 0x7fffffu)), 8388608.f);
   const float unit = __uint_as_float(sg | ((unsigned)max(e - 46, 0) << 23));   // 2^-46 of the leading bit
