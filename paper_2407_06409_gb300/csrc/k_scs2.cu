@@ -896,6 +896,13 @@ __device__ __forceinline__ int adjoint_exponent(const Work& w, const DevParams& 
   return top == 0x7ff ? top : min(top, 2045);
 }
 
+// A seed that is not finite (a caller's weight, a negative polarisability) makes the whole solution NaN: the
+// gradient it belongs to says so, and the other centres' stay as they are.
+__device__ __forceinline__ void adjoint_not_finite(const Work& w, int id, int n1, double* lam) {
+  for (int e = threadIdx.x; e < 9 * n1; e += blockDim.x) lam[e] = __longlong_as_double(0x7ff8000000000000LL);
+  if (threadIdx.x == 0) w.lexp[id] = 0;
+}
+
 // One (centre, frequency) system per block of 32 S (3 / NC) threads.  ADJ = false: X = B^-1 d to FP64
 // accuracy (2^-52), alpha_K and alpha_I.  ADJ = true: lambda = B^-1 dL/dX, to 2^-30 of its largest
 // value or better (it feeds the forces only).  The refinement measures its own contraction.
@@ -951,8 +958,8 @@ __global__ void __launch_bounds__(32 * S * (3 / NC), cg_min_blocks(S, NC))
     cg_build_rhs(w, p, c, q, n1, R);
   } else {
     const int top = adjoint_exponent(w, p, c, q, n1);
-    if (top == 0x7ff) {   // not finite: no solution (uniform over the block)
-      if (tid == 0) atomicOr(w.status, LMBD_FLAG_NOT_CONVERGED);
+    if (top == 0x7ff) {   // uniform over the block
+      adjoint_not_finite(w, id, n1, R);
       return;
     }
     if (tid == 0) w.lexp[id] = top - 1023;
@@ -1467,20 +1474,24 @@ __global__ void __launch_bounds__(256) k_scs_lu_adjoint(Work w, DevParams p, int
     const int id = w.fb[1 + e], c = id / p.nqs, q = id % p.nqs;
     if (c < c0 || c >= c1) continue;
     const int n1 = w.counts[c].n1, N1 = 3 * n1;
+    double* lam = w.lsol + w.off_k1[c] * p.nqs * 9 + (long long)q * N1 * 3;
+    const int top = adjoint_exponent(w, p, c, q, n1);
+    if (top == 0x7ff) {   // uniform over the block
+      adjoint_not_finite(w, id, n1, lam);
+      continue;
+    }
     scs2_dense_b(w, p, c, q, n1, A);
     if (!lu_factor_dense(A, N1, sm.piv, sm.red, sm.redi)) {
       if (threadIdx.x == 0) atomicOr(w.status, LMBD_FLAG_NOT_SPD);
       __syncthreads();
       continue;
     }
-    const int top = min(adjoint_exponent(w, p, c, q, n1), 2045);   // not finite: stays so
     const double up = __longlong_as_double((long long)(2046 - top) << 52);
     if (threadIdx.x == 0) w.lexp[id] = top - 1023;
     for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x)
       sm.x[u] = (u % 9) / 3 == u % 3 ? adjoint_seed(w, p, c, q, u / 9) * up : 0.0;
     __syncthreads();
     lu_solve3_dense(A, N1, sm.piv, sm.x);
-    double* lam = w.lsol + w.off_k1[c] * p.nqs * 9 + (long long)q * N1 * 3;
     for (int u = threadIdx.x; u < 9 * n1; u += blockDim.x) lam[u] = sm.x[u];
     __syncthreads();
   }
