@@ -45,13 +45,14 @@ __device__ __forceinline__ ff ff_from_double(double x) {
 
 // The same to 47 bits (nearest) by integer and FP32 instructions, for kernels whose FP64 pipe is the
 // bound: hi = the top 24 bits, lo = the next 23.  Values below 2^-126 give zero, the low part of those
-// below 2^-80 is zero; from 2^128 on, and for infinities and NaN, hi is not finite.
-__device__ __forceinline__ ff ff_split(double v) {
+// below 2^-80 is zero; from 2^128 on, and for infinities and NaN, hi is not finite.  With `shift` the same
+// of v 2^shift (|shift| < 800).
+__device__ __forceinline__ ff ff_split(double v, int shift = 0) {
   const unsigned hv = (unsigned)__double2hiint(v), sg = hv & 0x80000000u;
   // half of the last bit kept is added to |v|, in words: as one 64-bit mask it becomes an FP64 abs, whose
   // result for a NaN has no fixed sign.  NaN of any payload stays at or above the exponent 0x7ff.
   const unsigned l = (unsigned)__double2loint(v) + 32u, h = (hv & 0x7fffffffu) + (l < 32u ? 1u : 0u);
-  const int e = min((int)(h >> 20) - (1023 - 127), 255);   // biased FP32 exponent
+  const int e = min((int)(h >> 20) - (1023 - 127) + shift, 255);   // biased FP32 exponent
   const unsigned hb = ((unsigned)max(e, 0) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);
   const float low = __fsub_rn(__uint_as_float(0x4B000000u | ((l >> 6) & 0x7fffffu)), 8388608.f);
   const float unit = __uint_as_float(sg | ((unsigned)max(e - 46, 0) << 23));   // 2^-46 of the leading bit

@@ -309,6 +309,18 @@ __global__ void __launch_bounds__(256) k_mbd_chain(Work w, DevParams p, int m, i
   }
 }
 
+// Exponent h of G's scale at frequency column qq, |lambda| < 2^h, for the sliced products of the fitted
+// coefficients (0 otherwise).  The fit works in lambda / rho, so c_n = s_n / rho^n with s_n of one size, while
+// v_n falls like rho^n: at the highest frequencies c_10 reaches 2^100 and more.  With G 2^-h in place of G,
+//   v^_n = 2^(-n h) v_n,  c^_n = 2^(n h) c_n,  sum c_(j+k+1) v_j v_k = 2^-h sum c^_(j+k+1) v^_j v^_k,
+// all exact, both have one size and the digits of P and Q go to what counts in P Q^T.  Where the interval is a
+// point the coefficients are -1/n and need no scale.
+__device__ __forceinline__ int series_scale(const Work& w, const DevParams& p, int c, int qq) {
+  if (!p.lanczos) return 0;
+  const double lo = w.lam[((long long)c * p.n_freq + qq) * 2], hi = w.lam[((long long)c * p.n_freq + qq) * 2 + 1];
+  return hi - lo > 1e-12 ? min(max(oz_biased_exp(fmax(fabs(lo), fabs(hi))) - 1022, -85), 85) : 0;
+}
+
 // Series coefficient c_n of centre c at frequency column qq: -1/n (Eq. E_k), or the fitted one.
 __device__ __forceinline__ double series_c(const Work& w, const DevParams& p, int c, int qq, int n) {
   return p.lanczos ? w.cfit[((long long)c * p.n_freq + qq) * LMBD_MAX_ORDER_P1 + n] : p.cn[n];
@@ -2021,8 +2033,9 @@ __global__ void __launch_bounds__(256) k_slice_w(Work w, DevParams p, int m, int
 // frequency): a site takes a segment of the power of two of lanes that covers the frequencies, so
 // the row maxima over the frequencies, dL/dalpha~ and X0 need only shuffles inside the segment,
 // every Krylov value is read once and P and Q never exist in FP64.  All arithmetic is float-float on the
-// FP32 pipe (2^-46, against the 2^-35 of the digits); the frequency weights are scaled to unit size
-// (callers' weights may be of any magnitude), the exponent goes to Q's rows and the sums.  FP64 P and Q
+// FP32 pipe (2^-46, against the 2^-35 of the digits); the weights c_n of each frequency are scaled to unit
+// size (callers' weights may be of any magnitude, and fitted coefficients differ by 2^150 between
+// frequencies; see series_scale), the exponent goes to Q's rows and the sums.  FP64 P and Q
 // and their separate slicing took 5.2 + 1.75 ms per 4096-atom step; now 4.9 ms with the tile images that
 // save the pair product 0.4 ms.
 // Five signed 7-bit digits of v relative to 2^e (s1 = 2^(35 - e)), rounded to nearest, as bf16 bits.
@@ -2057,24 +2070,25 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int per = 32 / seg, qq = lane % seg;
   const bool freq = qq < nf;
-  // series weights of this lane's frequency at unit size: ct 2^lift
+  // series weights of this lane's frequency at unit size: c^_n = cf 2^lift; P Q^T and X0 of the lane are
+  // 2^(lift - h) times what it sums, 2^up times that after 2^rel (up: the largest over the frequencies)
   double ct[NM + 1];
-  int lift = 0;
+  int lift = -4000;
   ct[0] = ct[1] = 0.0;
+  const int h = freq ? series_scale(w, p, c, qq) : 0;
   {
     const double cwq = freq ? (p.fit ? w.fitw[(long long)c * LMBD_FITW + qq] : p.cweight[qq + 1]) : 0.0;
 #pragma unroll
     for (int n = 2; n <= NM; ++n) {
       ct[n] = freq ? wk * cwq * series_c(w, p, c, qq, n) : 0.0;
-      lift = max(lift, oz_biased_exp(ct[n]));
+      if (ct[n] != 0.0) lift = max(lift, max(oz_biased_exp(ct[n]), 1) - 1023 + n * h);
     }
   }
-  lift = min(max((int)__reduce_max_sync(0xffffffffu, lift), 1), 2045) - 1023;
   ff cf[NM + 1];
 #pragma unroll
-  for (int n = 2; n <= NM; ++n) cf[n] = ff_from_double(ct[n] * oz_pow2(-lift));
-  const double up = oz_pow2(lift);
-  const ff d0 = freq ? ff_from_double(w.dsq[offs * p.nq + qq + 1]) : ff_make(0.f, 0.f);
+  for (int n = 2; n <= NM; ++n) cf[n] = ff_from_double(oz_ldexp(ct[n], n * h - lift));
+  const int up = __reduce_max_sync(0xffffffffu, freq ? lift - h : -8000), rel = freq ? lift - h - up : 0;
+  const ff d0 = freq ? ff_scale(ff_from_double(w.dsq[offs * p.nq + qq + 1]), oz_down(rel)) : ff_make(0.f, 0.f);
   auto segmax = [&](int v) {
     for (int o = seg >> 1; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
@@ -2099,7 +2113,8 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
       for (int m = 1; m < NM; ++m)
 #pragma unroll
         for (int be = 0; be < 3; ++be)
-          u[m][be] = on ? ff_mul(ds, ff_split(V[(long long)(m - 1) * w.vstride + (long long)al * ncv + be])) : ff_make(0.f, 0.f);
+          u[m][be] = on ? ff_mul(ds, ff_split(V[(long long)(m - 1) * w.vstride + (long long)al * ncv + be], -m * h))
+                        : ff_make(0.f, 0.f);
 #pragma unroll
       for (int n = 2; n <= NM; ++n) {
         float h = 0.f, l = 0.f;
@@ -2121,7 +2136,7 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
 #pragma unroll
         for (int n = 2; n <= NM; ++n) ff_mac(h, l, cf[n], u[n - 1][be]);
         const ff x = segsum(ff_mul(ff_quick_two_sum(h, l), d0));
-        if (on && qq == 0) w.x0buf[(offs + s) * 9 + al * 3 + be] = ff_to_double(x) * up;
+        if (on && qq == 0) w.x0buf[(offs + s) * 9 + al * 3 + be] = oz_ldexp(ff_to_double(x), up);
       }
       int mp = 0, mq = 0;
 #pragma unroll
@@ -2136,15 +2151,15 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
           mq = max(mq, (__float_as_int(q.hi) >> 23) & 0xff);
           mp = max(mp, (__float_as_int(u[j][be].hi) >> 23) & 0xff);
         }
-      const int ep = segmax(mp) - 126, eq = segmax(mq) - 126;   // |row| < 2^e
+      const int ep = segmax(mp) - 126, eq = segmax(mq + rel) - 126;   // |row| < 2^e, Q's without 2^up
       // rows far below the FP32 range keep the digits that fit (2^(35 - e) must stay a float)
       const int fp = max(ep, -90), fq = max(eq, -90);
-      const float sp = __int_as_float((35 - fp + 127) << 23), sq = __int_as_float((35 - fq + 127) << 23);
+      const float sp = __int_as_float((35 - fp + 127) << 23), sq = oz_down(35 - fq + rel);
       const int row = 3 * s + al;
       if (on) {
         if (qq == 0) {
           w.pexp[w.off_sp[c] * 3 + row] = fp;
-          w.qexp[w.off_sp[c] * 3 + row] = fq + lift;
+          w.qexp[w.off_sp[c] * 3 + row] = fq + up;
         }
         // digits of G neighbouring columns at a time, one store per plane
         constexpr int G = NV % 4 == 0 ? 4 : (NV % 2 == 0 ? 2 : 1);
@@ -2177,7 +2192,7 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
     if (on) {
       // dL/dalpha~ = (sum_n c_n (<u, u>_n / alpha~ + [s = 0] tr_n)) / alpha~
       const double ia = 1.0 / w.alphaT[(offs + s) * p.nq + qq + 1];
-      double g = ff_to_double(ff_quick_two_sum(gh, gl)) * up * ia;
+      double g = oz_ldexp(ff_to_double(ff_quick_two_sum(gh, gl)), lift) * ia;
       if (s == 0)
 #pragma unroll
         for (int n = 2; n <= NM; ++n) g += ct[n] * w.trbuf[((long long)c * LMBD_MAX_ORDER_P1) * 64 + n * 64 + qq];
@@ -2206,7 +2221,7 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
 // P and Q digit planes and row exponents from FP64 P, Q (more than 32 integrand frequencies;
 // blockIdx.y = 0: P, 1: Q), one warp per row.
 template <int sp>
-__global__ void __launch_bounds__(256) k_slice_pq(Work w, int c0) {
+__global__ void __launch_bounds__(256) k_slice_pq(Work w, DevParams p, int c0) {
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
   const bool tiled = w.trec_full != 0;   // tile images of the tcgen05 path, or rows of pitch Kp
@@ -2218,15 +2233,22 @@ __global__ void __launch_bounds__(256) k_slice_pq(Work w, int c0) {
   int* ex = (blockIdx.y == 0 ? w.pexp : w.qexp) + w.off_sp[c] * 3;
   const long long plane = (long long)R * Kp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  // P_j 2^(-j h) and Q_j 2^(j h) of a frequency: one size for all columns of P (series_scale)
+  auto value = [&](int row, int j) {
+    const double v = src[(long long)row * ncol + j];
+    if (!p.lanczos) return v;
+    const int per = ncol / p.n_freq, e = (j % per / 3 + 1) * series_scale(w, p, c, j / per);
+    return oz_ldexp(v, blockIdx.y == 0 ? -e : e);
+  };
   for (int row = warp; row < rows; row += nw) {
     int mx = 0;
-    for (int j = lane; j < ncol; j += 32) mx = max(mx, oz_biased_exp(src[(long long)row * ncol + j]));
+    for (int j = lane; j < ncol; j += 32) mx = max(mx, oz_biased_exp(value(row, j)));
     mx = __reduce_max_sync(0xffffffffu, mx);
     const int e = oz_scale_exp(mx);
     if (lane == 0) ex[row] = e;
     for (int j = lane; j < Kp; j += 32) {
       unsigned d[sp];
-      oz_digits<sp>(j < ncol ? src[(long long)row * ncol + j] : 0.0, e, d);
+      oz_digits<sp>(j < ncol ? value(row, j) : 0.0, e, d);
 #pragma unroll
       for (int k = 0; k < sp; ++k)
         base[tiled ? oz_tile_offset(row, j, k, sp, blockIdx.y == 0 ? OZ_P_ROWS : OZ_W_ROWS, rows, Kp)
@@ -2240,10 +2262,10 @@ static void run_slice_w(const Work& w, const DevParams& p, int m, int c0, int n,
   if (sw == 5) k_slice_w<5><<<n, 256, 0, s>>>(w, p, m, c0);
   else k_slice_w<6><<<n, 256, 0, s>>>(w, p, m, c0);
 }
-static void run_slice_pq(const Work& w, int c0, int n, int sp, cudaStream_t s) {
+static void run_slice_pq(const Work& w, const DevParams& p, int c0, int n, int sp, cudaStream_t s) {
   const dim3 g2(n, 2);
-  if (sp == 5) k_slice_pq<5><<<g2, 256, 0, s>>>(w, c0);
-  else k_slice_pq<6><<<g2, 256, 0, s>>>(w, c0);
+  if (sp == 5) k_slice_pq<5><<<g2, 256, 0, s>>>(w, p, c0);
+  else k_slice_pq<6><<<g2, 256, 0, s>>>(w, p, c0);
 }
 
 void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
@@ -2253,9 +2275,9 @@ void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
   k_slice_t<<<c1 - c0, 256, sm, s>>>(w, c0);
 }
 
-void launch_slice_pq(const Work& w, int c0, int c1, int digits, cudaStream_t s) {
+void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, int digits, cudaStream_t s) {
   if (c1 <= c0 || !w.pmat) return;   // no FP64 P, Q: the series kernel wrote their digits
-  run_slice_pq(w, c0, c1 - c0, digits, s);
+  run_slice_pq(w, p, c0, c1 - c0, digits, s);
 }
 
 void launch_slice_w(const Work& w, const DevParams& p, int m, int c0, int c1, int digits, cudaStream_t s) {
@@ -2473,7 +2495,7 @@ __global__ void __launch_bounds__(288) k_mbd_adj_pair_oz2(Work w, DevParams p, i
 void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits,
                              cudaStream_t s) {
   if (c1 <= c0) return;
-  launch_slice_pq(w, c0, c1, digits, s);
+  launch_slice_pq(w, p, c0, c1, digits, s);
   const int nt = (max_ns + PT - 1) / PT;
   const int tiles = nt * (nt + 1) / 2;
   if (digits == 6) {

@@ -268,7 +268,7 @@ static_assert((3 * PTC_SA * PTC_LD + 4 * PTC_SA * PTC_GL) * 8 <= TcsShape<5, PTC
 bool launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits, cudaStream_t s) {
   if (c1 <= c0) return true;
   if (digits != 5) return false;
-  launch_slice_pq(w, c0, c1, digits, s);
+  launch_slice_pq(w, p, c0, c1, digits, s);
   const int na = (max_ns + PTC_SA - 1) / PTC_SA, nb = (max_ns + PTC_SB - 1) / PTC_SB;
   using Sh = TcsShape<5, PTC_NB, PTC_BUF, PTC_COLS>;
   raise_smem_limit((const void*)k_pair_tc<5>, Sh::kBytes);

@@ -446,7 +446,7 @@ bool launch_chain_tc(const Work& w, const DevParams& p, int m, int c0, int c1, i
                      cudaStream_t s);
 size_t chain_tc_smem(int digits);
 // P and Q digit planes (blockIdx.y = 0: P, 1: Q)
-void launch_slice_pq(const Work& w, int c0, int c1, int digits, cudaStream_t s);
+void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, int digits, cudaStream_t s);
 // adjoint pair matrix and its per-pair contraction on the tcgen05 tensor cores (digits 5 only;
 // returns false for another digit count)
 bool launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits, cudaStream_t s);

@@ -117,6 +117,14 @@ __device__ __forceinline__ double oz_pow2(int E) {
   return __longlong_as_double((long long)(E + 1023) << 52);
 }
 
+// v 2^E for any E (two exact factors).
+__device__ __forceinline__ double oz_ldexp(double v, int E) {
+  const int a = E >> 1;
+  return v * oz_pow2(a) * oz_pow2(E - a);
+}
+// 2^e as a float for e <= 127, zero below the normal range.
+__device__ __forceinline__ float oz_down(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
+
 // d += a b for one m16n8k16 bf16 tile (row-major A, column-major B, FP32 accumulate).
 __device__ __forceinline__ void oz_mma(float* d, const uint32_t* a, const uint32_t* b) {
   asm volatile(
