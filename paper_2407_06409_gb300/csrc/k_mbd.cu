@@ -2475,7 +2475,7 @@ __global__ void __launch_bounds__(288) k_mbd_adj_pair_oz2(Work w, DevParams p, i
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const int rr = wr * 16 + g + (v >> 1) * 8, cc = wc * 16 + n8 * 8 + 2 * tq + (v & 1);
-      Ms[rr * 49 + cc] = (double)Y[n8][v] * oz_pow2(pe[bi * 48 + rr] + qe[bj * 48 + cc] - 7 * (S + 1));
+      Ms[rr * 49 + cc] = oz_ldexp((double)Y[n8][v], pe[bi * 48 + rr] + qe[bj * 48 + cc] - 7 * (S + 1));
     }
   __syncthreads();
   if (tid < PT * PT) {

@@ -31,9 +31,6 @@
 
 namespace {
 
-// 2^e as a float for e <= 0 (zero below the normal range)
-__device__ __forceinline__ float ptc_down(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
-
 // Contribution of a coupled pair to dL/dr (out[0..2]: g = dL/dr_t = -dL/dr_s) and the SCS-radius
 // seed beta dL/dS~ (out[3]) from its block of the pair matrix and its record (lmbd_internal.cuh).
 __device__ __forceinline__ void ptc_epilogue(const float4* rec, const ff (&acc)[3][3], ff (&out)[4]) {
@@ -192,27 +189,25 @@ __global__ void __launch_bounds__(256, 2)
   const int erow = emax[0], ecol = emax[1];
   int scale = erow + ecol - 14;                    // the digits are 2^(er + ec - 14) sum acc_g 2^(-7 g)
   if (t0 == 0) scale = max(scale, emax[2]);
-  scale = min(max(scale, -900), 900);
   const int row = 32 * (warp & 3) + lane;
   if (row < 3 * PTC_SA) {
     const bool rv = 3 * s0 + row < 3 * ns;
-    const float fr = rv ? ptc_down(min(pe[row] - erow, 0)) * ptc_down(min(erow + ecol - 14 - scale, 0)) : 0.f;
+    const float fr = rv ? oz_down(min(pe[row] - erow, 0)) * oz_down(min(erow + ecol - 14 - scale, 0)) : 0.f;
 #pragma unroll
     for (int j = 0; j < 24; ++j) {
       const int col = cb + j;
-      const float f = rv && 3 * t0 + col < 3 * ns ? fr * ptc_down(min(qe[col] - ecol, 0)) : 0.f;
+      const float f = rv && 3 * t0 + col < 3 * ns ? fr * oz_down(min(qe[col] - ecol, 0)) : 0.f;
       Ms[row * PTC_LD + col] = make_float2(Yh[j] * f, Yl[j] * f);
     }
   }
   for (int e = tid; e < 2 * PTC_SA * PTC_GL; e += blockDim.x) gp[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   if (t0 == 0) {   // central column: the further term X0
-    const double down = oz_pow2(-scale);
     for (int e = tid; e < 9 * PTC_SA; e += blockDim.x) {
       const int sl = e / 9, u = e % 9;
       if (s0 + sl >= ns) continue;
       float2& m = Ms[(3 * sl + u / 3) * PTC_LD + u % 3];
-      const ff v = ff_add(ff_make(m.x, m.y), ff_from_double(w.x0buf[(offs + s0 + sl) * 9 + u] * down));
+      const ff v = ff_add(ff_make(m.x, m.y), ff_from_double(oz_ldexp(w.x0buf[(offs + s0 + sl) * 9 + u], -scale)));
       m = make_float2(v.hi, v.lo);
     }
     __syncthreads();
@@ -248,7 +243,7 @@ __global__ void __launch_bounds__(256, 2)
       const float2 v = g2[4 * (first + o * step) + d];
       s2[o & 1] = ff_add(s2[o & 1], ff_make(v.x, v.y));
     }
-    const double sum = ff_to_double(ff_add(s2[0], s2[1])) * oz_pow2(scale);
+    const double sum = oz_ldexp(ff_to_double(ff_add(s2[0], s2[1])), scale);
     if (sum == 0.0) continue;
     if (d == 3) atomicAdd(&w.rbar[offs + ss], sum);
     else atomicAdd(w.gacc + 3 * w.site_atom[(long long)c * w.site_cap + ss] + d, rs ? -sum : sum);

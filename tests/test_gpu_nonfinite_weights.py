@@ -1,10 +1,11 @@
-"""Weights (upstream gradients) that are not finite, and polarisabilities that turn negative: the call
+"""Weights (upstream gradients) at the ends of the FP64 range or not finite, and polarisabilities that turn negative: the call
 returns, the forces that depend on them are NaN, and all others are those of the same call without them.
 
 Two clusters 200 Angstrom apart share no site list, so the weights of one never reach the other.  Once
 with few screening systems (a group of warps per right-hand side) and once with many (63 frequencies:
 three right-hand sides together); on the LU fallback (a polarisation catastrophe); and with the digit
-planes of the warp-level path."""
+planes of the warp-level path.  Finite weights scaled by a power of two scale the forces, to 1e-12
+eV/Angstrom of the unscaled ones (rounding is relative; the smallest scale leaves 2^-60 of a force)."""
 import numpy as np
 import pytest
 import torch
@@ -98,3 +99,16 @@ def test_negative_polarisabilities(lm):
                                torch.tensor(s.hirshfeld, device="cuda"))
     assert (model.central_polarizabilities(64).numpy() < 0).any()
     assert torch.isnan(e).all() and torch.isnan(f).all()
+
+
+@pytest.mark.parametrize("path", ["tc05", "warp"])
+@pytest.mark.parametrize("power", [-1000, -950, 920, 990])
+def test_weights_at_the_ends_of_the_range(lm, power, path):
+    table, args, _ = _two_clusters()
+    model = lm.LMBD(table, lm.default_params(r_scs=5.0, r_mbd1=5.0, r_mbd2=5.0, r_sphere=5.0), 12, 6)
+    if path == "warp":
+        model.set_mma_path(lm.MMA_WARP)
+    w = torch.linspace(0.5, 1.5, 48, device="cuda", dtype=torch.float64)
+    f0 = model.energy_forces(*args, weights=w)[1]
+    f = model.energy_forces(*args, weights=w * 2.0 ** power)[1]
+    assert (f * 2.0 ** -power - f0).abs().max().item() < 1e-12
