@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0
     }
   __syncthreads();
   float4* rec = w.trec ? pair_record(w, c, 1, 0) : nullptr;
-  double* pco = DENSE && w.pcoef ? w.pcoef + w.off_t[c] : nullptr;
+  double* pco = DENSE && w.pcoef ? pair_coefs(w, w.off_t[c]) : nullptr;
   const ff d_ff = ff_from_double(p.d), beta_ff = ff_from_double(p.beta), ib_ff = ff_from_double(1.0 / p.r_buf);
   const bool full = w.trec_full != 0;
   auto pair = [&](int i, int j) {   // a coupled pair, i > j
@@ -141,11 +141,12 @@ __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0
         rec[4LL * e + 2] = o.v[2];
         rec[4LL * e + 3] = o.v[3];
       }
+      if (!DENSE || !w.t64)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        atomicMax(ex + 3 * i + a, o.top[a]);
-        atomicMax(ex + 3 * j + a, o.top[a]);
-      }
+        for (int a = 0; a < 3; ++a) {
+          atomicMax(ex + 3 * i + a, o.top[a]);
+          atomicMax(ex + 3 * j + a, o.top[a]);
+        }
     }
     if (DENSE) {
       double blk[3][3], kc[5];
@@ -155,6 +156,13 @@ __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0
         pc[0] = rr[0]; pc[1] = rr[1]; pc[2] = rr[2];
         pc[3] = kc[0]; pc[4] = kc[1]; pc[5] = kc[2]; pc[6] = kc[3]; pc[7] = kc[4];
       }
+      if (w.t64)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int top = __float_as_int(__double2float_ru(fmax(fmax(fabs(blk[a][0]), fabs(blk[a][1])), fabs(blk[a][2]))));
+          atomicMax(ex + 3 * i + a, top);
+          atomicMax(ex + 3 * j + a, top);
+        }
       if (T)
 #pragma unroll
         for (int al = 0; al < 3; ++al)
@@ -233,7 +241,7 @@ __global__ void __launch_bounds__(256) k_mbd_prepare(Work w, DevParams p, int c0
   }
   __syncthreads();
   // row exponents of the digit planes: |T_row| < 2^e
-  if (rec && w.texp)
+  if (w.texp)
     for (int e = tid; e < oz_mpad(N); e += blockDim.x)
       w.texp[w.off_tr[c] + e] = e < N ? (ex[e] >> 23) - 126 : 0;
   // v_1 = G e_k: column block of the central site, scaled by D_s D_0 (per frequency)
@@ -1764,7 +1772,7 @@ __global__ void __launch_bounds__(256) k_f3_pair(Work w, DevParams p, int c0, in
   if (s < ns && t < ns && s > t) {
     double gamma = 0.0;
     for (int qq = 0; qq < nf; ++qq) gamma += cq[qq] * alt[0][ty][qq] * alt[1][tx][qq];
-    const double* pc = w.pcoef + w.off_t[c] + 8LL * (s * (s - 1) / 2 + t);
+    const double* pc = pair_coefs(w, w.off_t[c]) + 8LL * (s * (s - 1) / 2 + t);
     const double rr[3] = {pc[0], pc[1], pc[2]};
     const double r2 = rr[0] * rr[0] + rr[1] * rr[1] + rr[2] * rr[2];
     const double cg = gamma * pc[5] / 12.0;      // pc[5] = 12 f_LR f / r^5
@@ -1825,7 +1833,8 @@ void launch_forces_out(const Work& w, double* forces, cudaStream_t s) {
 // ns16 = 16 ceil(ns/16) and Kp = 16 ceil(ncol/16).
 // =======================================================================================
 
-// T_LR digit planes from the pair records (the row exponents come with them): one block per central
+// T_LR digit planes from the pair records, or from the FP64 T_LR that fitted coefficients need anyway
+// (FP64T; the row exponents come from the prepare kernel in both cases): one block per central
 // atom, a warp per (site, 64 partners), a lane per two neighbouring partners: three rows by six
 // columns of every plane.  T_st = a r r^T - (a r^2 / 3) I with a = k3 / 4 is formed in float-float on
 // the FP32 pipe (~2^-45 against the 2^-42 of the digits), so T_LR itself is never stored: the FP64
@@ -1860,6 +1869,13 @@ __device__ __forceinline__ TBlock t_block(const float4* rec, int s, int t) {
   o.v[3] = ff_quick_two_sum(xy.hi, xy.lo); o.v[4] = ff_quick_two_sum(xz.hi, xz.lo); o.v[5] = ff_quick_two_sum(yz.hi, yz.lo);
   return o;
 }
+__device__ __forceinline__ TBlock t_block(const double* T, int N, int s, int t) {
+  const double* r = T + (long long)(3 * s) * N + 3 * t;
+  TBlock o;
+  o.v[0] = ff_split(r[0]); o.v[1] = ff_split(r[N + 1]); o.v[2] = ff_split(r[2 * N + 2]);
+  o.v[3] = ff_split(r[1]); o.v[4] = ff_split(r[2]); o.v[5] = ff_split(r[N + 2]);
+  return o;
+}
 // index of entry (a, b) of the symmetric block
 __host__ __device__ constexpr int t_idx(int a, int b) { return a == b ? a : (a + b == 1 ? 3 : (a + b == 2 ? 4 : 5)); }
 
@@ -1884,6 +1900,7 @@ __device__ __forceinline__ void t_digits(ff v, float s1, float s2, unsigned (&d)
 }
 
 #define SLT_W 96   // words of a row that a warp forms at once (64 partners)
+template <bool FP64T>
 __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
   extern __shared__ float2 sl_scale[];   // 2^(42 - e) of every row in two factors (it can pass the FP32 range)
   __shared__ __align__(16) unsigned stage[8][6 * SLT_W];
@@ -1891,7 +1908,8 @@ __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
   if (c >= w.n_atoms) return;
   constexpr int st = 6;
   const int ns = w.counts[c].ns, N = 3 * ns, Mpad = oz_mpad(N), Kpad = oz_kpad(N);
-  const float4* rec = pair_record(w, c, 1, 0);
+  const float4* rec = FP64T ? nullptr : pair_record(w, c, 1, 0);
+  const double* T = FP64T ? w.tlr + w.off_t[c] : nullptr;
   // rows of pitch Kpad, or the tile images of the tcgen05 path (zeros past N along K)
   const bool tiled = w.tk > 0;
   const int ld = tiled ? (N + 31) / 32 * 32 : Kpad;
@@ -1915,7 +1933,7 @@ __global__ void __launch_bounds__(256, 3) k_slice_t(Work w, int c0) {
       const int t = 64 * ch + 2 * lane + h;
 #pragma unroll
       for (int u = 0; u < 6; ++u) o[h].v[u] = ff_make(0.f, 0.f);
-      if (t < ns && t != s) o[h] = t_block(rec, s, t);
+      if (t < ns && t != s) o[h] = FP64T ? t_block(T, N, s, t) : t_block(rec, s, t);
     }
     const int quads = min(SLT_W, lw - SLT_W * ch) / 4;   // 16-byte pieces of the chunk
     const int first = 2 * SLT_W * ch;                    // and its first column
@@ -2271,8 +2289,13 @@ static void run_slice_pq(const Work& w, const DevParams& p, int c0, int n, int s
 void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return;
   const size_t sm = sizeof(float2) * 3 * (size_t)max_ns;
-  raise_smem_limit((const void*)k_slice_t, sm);
-  k_slice_t<<<c1 - c0, 256, sm, s>>>(w, c0);
+  if (!w.t64) {
+    raise_smem_limit((const void*)k_slice_t<false>, sm);
+    k_slice_t<false><<<c1 - c0, 256, sm, s>>>(w, c0);
+  } else {
+    raise_smem_limit((const void*)k_slice_t<true>, sm);
+    k_slice_t<true><<<c1 - c0, 256, sm, s>>>(w, c0);
+  }
 }
 
 void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, int digits, cudaStream_t s) {

@@ -277,6 +277,7 @@ struct Layout {
   int tk;    // tcgen05 path: longest K of the T and W tile images (0: rows of pitch Kpad)
   bool sparse;   // block-sparse T_LR: coupled pairs and float-float chain/pair operands
   bool dense_t;  // FP64 T_LR kept (Lanczos-based modes, the paper's forces, FP64 products)
+  bool t64;      // T_LR's digit planes are cut from the FP64 matrix
   bool rec_pair; // the pair adjoint reads float-float records instead of FP64 coefficients
   bool pq_fp64;  // FP64 P and Q kept (FP64 products, more than 32 integrand frequencies)
   int gs_ld;     // float2 per pair of the SCS adjoint's gradient scratch
@@ -338,7 +339,8 @@ struct Layout {
     double* alphaT = cv.take<double>((long long)nq * ns, (long long)nq * s0);
     double* dsq = cv.take<double>((long long)nq * ns, (long long)nq * s0);
     double* tlr = dense_t ? cv.take<double>(nt, t0) : nullptr;
-    float4* trec = sliced_chain || rec_pair ? cv.take<float4>(2 * (nt / 9), 2 * (t0 / 9)) : nullptr;
+    // records: for the tcgen05 pair kernel, and for the digit planes unless these come from the FP64 T_LR
+    float4* trec = rec_pair || (sliced_chain && !t64) ? cv.take<float4>(2 * (nt / 9), 2 * (t0 / 9)) : nullptr;
     double* vkr = cv.take<double>((long long)nvec * ns * 3 * ncv, s0 * 3 * ncv);
     if (w) {
       w->alphaT = alphaT;
@@ -346,6 +348,7 @@ struct Layout {
       w->tlr = tlr;
       w->trec = trec;
       w->trec_full = rec_pair;
+      w->t64 = t64;
       w->vkr = vkr;
       w->vstride = ns * 3 * ncv;
     }
@@ -391,7 +394,7 @@ struct Layout {
       float2* pff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       float2* qff = sparse ? cv.take<float2>(3 * ns * nc, 3 * s0 * nc) : nullptr;
       double* x0buf = cv.take<double>(9 * ns, 9 * s0);
-      double* pcoef = rec_pair ? nullptr : (sparse ? cv.take<double>(8 * npn, 8 * np0) : cv.take<double>(nt, t0));
+      double* pcoef = rec_pair ? nullptr : (sparse ? cv.take<double>(8 * npn, 8 * np0) : cv.take<double>(4 * (nt / 9), 4 * (t0 / 9)));
       double* rbar = cv.take<double>(ns, s0);
       if (w) {
         w->gbar = gbar;
@@ -911,7 +914,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   const int kp_pair = rec_pair ? (ncol + 31) / 32 * 32 : (ncol + 15) / 16 * 16;   // K of the P, Q planes
   const Layout L{nq, ncv, nvec, ncol, kp_pair, ST, DIG_P, c->site_cap, forces, sliced_chain,
                  sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 31) / 32 * 32 : 0, sparse,
-                 !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), rec_pair,
+                 !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), sliced_chain && dp.lanczos, rec_pair,
                  !sparse && (!sliced_pair || dp.paper || nf > 32),
                  scs_contract_scratch(N, max_n1, dp.nqs)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };

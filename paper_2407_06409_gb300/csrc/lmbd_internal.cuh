@@ -173,6 +173,7 @@ struct Work {
   // site-pair records in float-float, 4 float4 per pair (s > t) from 2 off_t / 9: (rx, ry),
   // (rz, k3), then with forces (k1, k2), (k4, k5); k3 = 12 f_LR f / r^5 = 0 for uncoupled pairs
   float4* trec;
+  int t64;                     // the digit planes of T_LR are cut from tlr, not from the records
   int trec_full;               // the second half is written (the tcgen05 pair kernel reads it)
   double* dsq;                 // sqrt(alpha~), off_s * nq
   double* vkr;                 // Krylov vectors: nvec blocks of (off_s total * 3) x (3 n_freq)
@@ -190,7 +191,7 @@ struct Work {
   double* qmat;                // off_s*3 x ncol
   int ncol;                    // 3 n_freq (n_max - 2)
   double* x0buf;               // off_s x 9, central-column term of the pair matrix
-  double* pcoef;               // off_t: per site pair (s > t) r (3) and 5 derivative coefficients
+  double* pcoef;               // per site pair (s > t) r (3) and 5 derivative coefficients (pair_coefs)
   double* rbar;                // dL/d R~ per sphere site, off_s
   // block-sparse T_LR (Sec. III.A: only the central row and column reach r_MBD,1, every other
   // pair couples within r_MBD,2): per centre the coupled site pairs (s, t), s > t, in row order,
@@ -369,6 +370,10 @@ __device__ __forceinline__ void tlr_pair_block(const DevParams& p, const double 
     kc[4] = -2.0 * p.beta * CS * ir3;
   }
 }
+
+// FP64 pair coefficients of the dense layout, 8 per pair (s > t): 4 n_s^2 doubles for a centre at offset
+// offt = off_t[c] (9 n_s^2 a centre)
+__device__ __forceinline__ double* pair_coefs(const Work& w, long long offt) { return w.pcoef + 4 * (offt / 9); }
 
 // the record of site pair (s, t), s > t, of centre c
 __device__ __forceinline__ float4* pair_record(const Work& w, int c, int s, int t) {

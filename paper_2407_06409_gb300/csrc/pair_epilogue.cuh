@@ -41,5 +41,5 @@ __device__ __forceinline__ void pair_epilogue(const Work& w, long long offs, lon
     out[0] = out[1] = out[2] = out[3] = 0.0;
     return;
   }
-  pair_epilogue_at(w, offs, w.pcoef + offt + 8LL * (s * (s - 1) / 2 + t), s, t, acc, out);
+  pair_epilogue_at(w, offs, pair_coefs(w, offt) + 8LL * (s * (s - 1) / 2 + t), s, t, acc, out);
 }
