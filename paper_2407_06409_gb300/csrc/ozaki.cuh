@@ -117,8 +117,9 @@ __device__ __forceinline__ double oz_pow2(int E) {
   return __longlong_as_double((long long)(E + 1023) << 52);
 }
 
-// v 2^E for any E (two exact factors).
+// v 2^E for any E (two exact factors where one does not reach).
 __device__ __forceinline__ double oz_ldexp(double v, int E) {
+  if (E >= -1022 && E <= 1023) return v * oz_pow2(E);
   const int a = E >> 1;
   return v * oz_pow2(a) * oz_pow2(E - a);
 }
