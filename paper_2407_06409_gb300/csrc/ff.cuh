@@ -23,9 +23,10 @@ __device__ __forceinline__ ff ff_make(float hi, float lo) {
 __device__ __forceinline__ double ff_join(ff a, int shift) {
   const unsigned hb = __float_as_uint(a.hi), sg = hb & 0x80000000u;
   const int e = (int)((hb >> 23) & 0xffu);
-  // |hi| as an integer with 46 fraction bits, and the low part (at most 2^22) in the same unit
-  const float unit = __uint_as_float((unsigned)min(max(300 - e, 1), 254) << 23);   // 2^(173 - e)
-  const float l = __uint_as_float(__float_as_uint(a.lo) ^ sg) * unit;
+  // |hi| as an integer with 46 fraction bits, and the low part (at most 2^22) in the same unit, 2^(e - 173)
+  const int up = e < 64 ? 64 : 0;
+  const float unit = __uint_as_float((unsigned)max(300 - e - up, 1) << 23);
+  const float l = __uint_as_float(__float_as_uint(a.lo) ^ sg) * unit * (up ? 0x1p64f : 1.f);
   const int q = __float_as_int(__fadd_rn(l, 12582912.f)) - 0x4B400000;
   long long m = ((long long)((hb & 0x7fffffu) | 0x800000u) << 23) + q;
   const int below = m < (1LL << 46);
@@ -44,19 +45,27 @@ __device__ __forceinline__ ff ff_from_double(double x) {
 }
 
 // The same to 47 bits (nearest) by integer and FP32 instructions, for kernels whose FP64 pipe is the
-// bound: hi = the top 24 bits, lo = the next 23.  Values below 2^-126 give zero, the low part of those
-// below 2^-80 is zero; from 2^128 on, and for infinities and NaN, hi is not finite.  With `shift` the same
-// of v 2^shift (|shift| < 800).
-__device__ __forceinline__ ff ff_split(double v, int shift = 0) {
-  const unsigned hv = (unsigned)__double2hiint(v), sg = hv & 0x80000000u;
+// bound: hi = the top 24 bits, lo = the next 23 (rounded to FP32's smallest numbers below 2^-80 of the
+// value).  Values below 2^-126 give zero; from 2^128 on, and for infinities and NaN, hi is not finite.
+__device__ __forceinline__ ff ff_split(double v) {
+  const unsigned hv = (unsigned)__double2hiint(v), top = hv & 0x7fffffffu;
   // half of the last bit kept is added to |v|, in words: as one 64-bit mask it becomes an FP64 abs, whose
-  // result for a NaN has no fixed sign.  NaN of any payload stays at or above the exponent 0x7ff.
-  const unsigned l = (unsigned)__double2loint(v) + 32u, h = (hv & 0x7fffffffu) + (l < 32u ? 1u : 0u);
-  const int e = min((int)(h >> 20) - (1023 - 127) + shift, 255);   // biased FP32 exponent
-  const unsigned hb = ((unsigned)max(e, 0) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);
+  // result for a NaN has no fixed sign
+  const unsigned l = (unsigned)__double2loint(v) + 32u, h = top + (l < 32u ? 1u : 0u);
+  // exponent and 23 bits of the fraction, moved to FP32's place and bias: two upper exponent bits drop out, and
+  // 1023 - 127 = 896 is -128 modulo 2^9
+  unsigned hb = __funnelshift_l(l, h, 3) + (128u << 23);
+  hb = top < (897u << 20) ? 0u : (top >= (1151u << 20) ? 0x7fc00000u : hb);
+  hb |= hv & 0x80000000u;
   const float low = __fsub_rn(__uint_as_float(0x4B000000u | ((l >> 6) & 0x7fffffu)), 8388608.f);
-  const float unit = __uint_as_float(sg | ((unsigned)max(e - 46, 0) << 23));   // 2^-46 of the leading bit
-  return e > 0 ? ff_make(__uint_as_float(sg | hb), __fmul_rn(low, unit)) : ff_make(0.f, 0.f);
+  return ff_make(__uint_as_float(hb), __fmul_rn(__fmul_rn(low, 0x1p-46f), __uint_as_float(hb & 0xff800000u)));
+}
+
+// The same of v 2^shift, |shift| < 1000 (zero where that leaves the normal range of FP64 below).
+__device__ __forceinline__ ff ff_split_scaled(double v, int shift) {
+  const int hv = __double2hiint(v), e = (hv >> 20) & 0x7ff;
+  if (e == 0 || e + shift <= 0) return ff_make(0.f, 0.f);
+  return ff_split(e + shift >= 0x7ff ? v : __hiloint2double(hv + (shift << 20), __double2loint(v)));
 }
 
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }

@@ -2074,7 +2074,7 @@ __device__ __forceinline__ void pq_digits(ff v, float s1, unsigned (&d)[5]) {
   }
 }
 
-template <int NM, bool TILED>
+template <int NM, bool TILED, bool FIT>
 __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p, int c0, int seg) {
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
@@ -2093,7 +2093,7 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
   double ct[NM + 1];
   int lift = -4000;
   ct[0] = ct[1] = 0.0;
-  const int h = freq ? series_scale(w, p, c, qq) : 0;
+  const int h = FIT && freq ? series_scale(w, p, c, qq) : 0;
   {
     const double cwq = freq ? (p.fit ? w.fitw[(long long)c * LMBD_FITW + qq] : p.cweight[qq + 1]) : 0.0;
 #pragma unroll
@@ -2130,9 +2130,10 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
 #pragma unroll
       for (int m = 1; m < NM; ++m)
 #pragma unroll
-        for (int be = 0; be < 3; ++be)
-          u[m][be] = on ? ff_mul(ds, ff_split(V[(long long)(m - 1) * w.vstride + (long long)al * ncv + be], -m * h))
-                        : ff_make(0.f, 0.f);
+        for (int be = 0; be < 3; ++be) {
+          const double v = on ? V[(long long)(m - 1) * w.vstride + (long long)al * ncv + be] : 0.0;
+          u[m][be] = ff_mul(ds, FIT ? ff_split_scaled(v, -m * h) : ff_split(v));
+        }
 #pragma unroll
       for (int n = 2; n <= NM; ++n) {
         float h = 0.f, l = 0.f;
@@ -2532,6 +2533,19 @@ void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, 
   }
 }
 
+// FIT: the scale of fitted coefficients; the default series is compiled without it.
+template <int NM>
+static void run_adj_site_digits(const Work& w, const DevParams& p, int c0, int c1, int seg, cudaStream_t s) {
+  const int n = c1 - c0;
+  if (w.trec_full) {
+    if (p.lanczos) k_adj_site_digits<NM, true, true><<<n, 256, 0, s>>>(w, p, c0, seg);
+    else k_adj_site_digits<NM, true, false><<<n, 256, 0, s>>>(w, p, c0, seg);
+  } else {
+    if (p.lanczos) k_adj_site_digits<NM, false, true><<<n, 256, 0, s>>>(w, p, c0, seg);
+    else k_adj_site_digits<NM, false, false><<<n, 256, 0, s>>>(w, p, c0, seg);
+  }
+}
+
 void launch_mbd_adj_series(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s) {
   if (c1 <= c0) return;
   int seg = 1;   // lanes per site of the digits variant: the power of two that covers the frequencies
@@ -2543,10 +2557,8 @@ void launch_mbd_adj_series(const Work& w, const DevParams& p, int c0, int c1, cu
       k_mbd_adj_site<N, true><<<c1 - c0, 256, 0, s>>>(w, p, c0);                       \
     else if (w.pmat || N == 2) /* order 2 has no P, Q */                               \
       k_mbd_adj_site<N, false><<<c1 - c0, 256, 0, s>>>(w, p, c0);                      \
-    else if (w.trec_full)                                                              \
-      k_adj_site_digits<(N > 2 ? N : 3), true><<<c1 - c0, 256, 0, s>>>(w, p, c0, seg); \
     else                                                                               \
-      k_adj_site_digits<(N > 2 ? N : 3), false><<<c1 - c0, 256, 0, s>>>(w, p, c0, seg);\
+      run_adj_site_digits<(N > 2 ? N : 3)>(w, p, c0, c1, seg, s);                      \
     break;
     ADJ_SITE_CASE(2) ADJ_SITE_CASE(3) ADJ_SITE_CASE(4) ADJ_SITE_CASE(5) ADJ_SITE_CASE(6)
     ADJ_SITE_CASE(7) ADJ_SITE_CASE(8) ADJ_SITE_CASE(9) ADJ_SITE_CASE(10)
