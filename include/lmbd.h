@@ -97,9 +97,9 @@ typedef struct {
 #define LMBD_NPHASE           10
 
 /* Per-call statistics of the last lmbd_energy_forces call.  flops count the dense
- * linear algebra of each phase from the actual site counts (Cholesky n^3/3, two
- * triangular solves 6 n^2 per frequency, 2 n^2 k per product of an n x n with an
- * n x k matrix); ms are device times from CUDA events on the call's stream and are
+ * linear algebra of each phase from the actual site counts (direct solves: n^3/3 and two
+ * triangular solves 6 n^2 per frequency, whatever solver runs; 2 n^2 k per product of an
+ * n x n with an n x k matrix); ms are device times from CUDA events on the call's stream and are
  * filled only when profiling is on (lmbd_set_profiling), in batched launch mode. */
 typedef struct {
   double flops[LMBD_NPHASE];
@@ -172,7 +172,7 @@ int lmbd_energy_forces_weighted(lmbd_ctx* ctx, int n_atoms, const double* positi
 /* Energies now, forces later (a reverse-mode autograd: forward, then backward with the upstream
  * gradient as weights).  lmbd_energy_keep computes the energies like lmbd_energy_forces without
  * forces, but lays the workspaces out for forces and keeps the forward state (site lists, SCS
- * factors and solutions, T_LR, Krylov blocks, pair coefficients) on the device.
+ * pair terms and solutions, T_LR, Krylov blocks, pair coefficients) on the device.
  * lmbd_forces_kept then gives forces = -d(sum_k w_k E_k)/dR for weights w (NULL = ones) by the
  * reverse sweep alone on that state (the adjoint of Sec. III.D's derivative pieces, exact), when
  * the state is there: the context's last call was lmbd_energy_keep for the same atom count, its
@@ -197,10 +197,13 @@ int lmbd_set_launch_mode(lmbd_ctx* ctx, int mode);
 
 /* Arithmetic of the two large matrix products (the Krylov chain T_LR W and the adjoint pair
  * matrix P Q^T).  LMBD_PREC_SLICED (default) evaluates them on the bf16 tensor cores from
- * exact 7-bit integer slices of the FP64 operands, recombined in FP64 (6 slices for the
- * products that feed the energies, 5 for those that feed only the forces; truncation error
- * ~S 2^-7S relative to sum |a||b|); LMBD_PREC_FP64 uses FP64 FMA kernels.  Everything
- * else is FP64 (the SCS factorisation is FP32 with FP64 iterative refinement).            */
+ * 7-bit integer slices of the operands, recombined in float-float (tcgen05) or 64-bit integers
+ * (mma.sync) (6 slices for the products that feed the energies, 5 for those that feed only the
+ * forces; error ~S 2^-7S relative to sum |a||b|); LMBD_PREC_FP64 uses FP64 FMA kernels.  In both
+ * settings the SCS pair terms, solves (FP32 with float-float refinement) and adjoint contraction,
+ * and the Lanczos products of the fitted coefficients, are float-float (2^-46); with the sliced
+ * products so are T_LR's pair records and digits and the adjoint's series and pair sums.  The
+ * rest is FP64.                                                                            */
 #define LMBD_PREC_FP64   0
 #define LMBD_PREC_SLICED 1
 int lmbd_set_precision(lmbd_ctx* ctx, int mode);

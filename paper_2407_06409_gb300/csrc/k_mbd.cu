@@ -881,7 +881,7 @@ static bool launch_lanczos_fit(const Work& w, const DevParams& p, int c0, int c1
   const int L3 = 3 * max_ns;
   if (L3 > LZ_THREADS * LZ_RPT) return false;
   const size_t room = 216 * 1024;
-  const int qf = lanczos_fit_smem<12>(L3) <= room ? 12 : lanczos_fit_smem<8>(L3) <= room ? 8 : 4;
+  const int qf = lanczos_fit_smem<12>(L3) <= room ? 12 : 8;   // 8 columns fit up to 1024 rows
   for (int q0 = 0; q0 < p.n_freq; q0 += qf) {
     const int n = std::min(qf, p.n_freq - q0);
     if (n > 8) run_lanczos_fit<12>(w, p, c0, c1, q0, n, L3, s);
@@ -2239,10 +2239,10 @@ __global__ void __launch_bounds__(256, 2) k_adj_site_digits(Work w, DevParams p,
 
 // P and Q digit planes and row exponents from FP64 P, Q (more than 32 integrand frequencies;
 // blockIdx.y = 0: P, 1: Q), one warp per row.
-template <int sp>
 __global__ void __launch_bounds__(256) k_slice_pq(Work w, DevParams p, int c0) {
   const int c = c0 + blockIdx.x;
   if (c >= w.n_atoms) return;
+  constexpr int sp = 5;
   const bool tiled = w.trec_full != 0;   // tile images of the tcgen05 path, or rows of pitch Kp
   const int ns = w.counts[c].ns, R = 3 * ((ns + 15) / 16 * 16), rows = 3 * ns;
   const int ncol = w.ncol, Kp = tiled ? (ncol + 31) / 32 * 32 : oz_kpad(ncol);
@@ -2281,11 +2281,6 @@ static void run_slice_w(const Work& w, const DevParams& p, int m, int c0, int n,
   if (sw == 5) k_slice_w<5><<<n, 256, 0, s>>>(w, p, m, c0);
   else k_slice_w<6><<<n, 256, 0, s>>>(w, p, m, c0);
 }
-static void run_slice_pq(const Work& w, const DevParams& p, int c0, int n, int sp, cudaStream_t s) {
-  const dim3 g2(n, 2);
-  if (sp == 5) k_slice_pq<5><<<g2, 256, 0, s>>>(w, p, c0);
-  else k_slice_pq<6><<<g2, 256, 0, s>>>(w, p, c0);
-}
 
 void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return;
@@ -2299,9 +2294,9 @@ void launch_slice_t(const Work& w, int c0, int c1, int max_ns, cudaStream_t s) {
   }
 }
 
-void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, int digits, cudaStream_t s) {
+void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s) {
   if (c1 <= c0 || !w.pmat) return;   // no FP64 P, Q: the series kernel wrote their digits
-  run_slice_pq(w, p, c0, c1 - c0, digits, s);
+  k_slice_pq<<<dim3(c1 - c0, 2), 256, 0, s>>>(w, p, c0);
 }
 
 void launch_slice_w(const Work& w, const DevParams& p, int m, int c0, int c1, int digits, cudaStream_t s) {
@@ -2419,8 +2414,8 @@ void launch_chain_oz2(const Work& w, const DevParams& p, int m, int c0, int c1, 
 // Pair matrix M' = P Q^T on one 16 x 16 site tile with staged digit tiles (cp.async, two
 // stages of 32 K) and integer recombination; 9 warps of 16 x 16 outputs, then the per-pair
 // epilogue of the FP64 kernel.
-template <int S>
 __global__ void __launch_bounds__(288) k_mbd_adj_pair_oz2(Work w, DevParams p, int c0, int tiles_per_c) {
+  constexpr int S = 5;
   extern __shared__ __align__(16) unsigned short oz_sm[];
   __shared__ double xs[2][PT][3];
   __shared__ double rts[2][PT];
@@ -2516,21 +2511,14 @@ __global__ void __launch_bounds__(288) k_mbd_adj_pair_oz2(Work w, DevParams p, i
   pair_tile_reduce(w, offs, sbase, ns, bi, bj, gp);
 }
 
-void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits,
-                             cudaStream_t s) {
+void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
   if (c1 <= c0) return;
-  launch_slice_pq(w, p, c0, c1, digits, s);
+  launch_slice_pq(w, p, c0, c1, s);
   const int nt = (max_ns + PT - 1) / PT;
   const int tiles = nt * (nt + 1) / 2;
-  if (digits == 6) {
-    const size_t sm = 2 * 2 * sizeof(unsigned short) * 6 * 48 * OZ_LD;
-    raise_smem_limit((const void*)k_mbd_adj_pair_oz2<6>, sm);
-    k_mbd_adj_pair_oz2<6><<<(c1 - c0) * tiles, 288, sm, s>>>(w, p, c0, tiles);
-  } else {
-    const size_t sm = 2 * 2 * sizeof(unsigned short) * 5 * 48 * OZ_LD;
-    raise_smem_limit((const void*)k_mbd_adj_pair_oz2<5>, sm);
-    k_mbd_adj_pair_oz2<5><<<(c1 - c0) * tiles, 288, sm, s>>>(w, p, c0, tiles);
-  }
+  const size_t sm = 2 * 2 * sizeof(unsigned short) * 5 * 48 * OZ_LD;
+  raise_smem_limit((const void*)k_mbd_adj_pair_oz2, sm);
+  k_mbd_adj_pair_oz2<<<(c1 - c0) * tiles, 288, sm, s>>>(w, p, c0, tiles);
 }
 
 // FIT: the scale of fitted coefficients; the default series is compiled without it.

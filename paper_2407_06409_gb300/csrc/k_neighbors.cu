@@ -430,30 +430,28 @@ void launch_neighbors(const Work& w, const DevParams& p, const Grid& g, cudaStre
 
 // ---------------------------------------------------------------------------------------
 // per-centre offsets into the variable-size workspaces (one block, 64-bit scans)
-// totals: [0] sum n1, [1] sum ns, [2] sum nq N1(N1+1)/2 (packed factors, N1 = 3 n1),
-//         [3] sum (3 ns)^2, [4] max n1, [5] max ns, [6] max n12, [7] sum nt,
+// totals: [0] sum n1, [1] sum ns, [2] sum of coupled T_LR pairs (block-sparse T_LR), [3] sum (3 ns)^2,
+//         [4] max n1, [5] max ns, [6] max n12, [7] sum nt,
 //         [8] sum of SCS pairs, [9] sum of SCS adjacency entries, [10] max pairs,
 //         [11] max coupled T_LR pairs (block-sparse T_LR, 0 otherwise),
 //         [12] sum Mpad Kpad, [13] sum Mpad, [14] sum Kpad, [15] sum ns16 (sliced products)
 // ---------------------------------------------------------------------------------------
 #define OFF_T 256
-__global__ void k_offsets(Work w, int nq) {
-  __shared__ long long part[11][OFF_T];
+__global__ void k_offsets(Work w) {
+  __shared__ long long part[10][OFF_T];
   __shared__ int mx[5][OFF_T];
   __shared__ long long tot_nt[OFF_T];
   int N = w.n_atoms;
   int per = (N + blockDim.x - 1) / blockDim.x;
   int b = threadIdx.x * per, e = min(N, b + per);
-  long long s[11] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  long long s[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   int m[5] = {0, 0, 0, 0, 0};
   long long snt = 0;
   for (int i = b; i < e; ++i) {
     Counts c = w.counts[i];
-    long long N1 = 3LL * c.n1;
     int np = w.pcount ? w.pcount[2 * i] : 0, na = w.pcount ? w.pcount[2 * i + 1] : 0;
     s[0] += c.n1;
     s[1] += c.ns;
-    s[2] += (long long)nq * N1 * (N1 + 1) / 2;
     s[3] += 9LL * c.ns * c.ns;
     s[4] += np;
     s[5] += na;
@@ -463,7 +461,7 @@ __global__ void k_offsets(Work w, int nq) {
     s[8] += Kp;
     s[9] += (c.ns + 15) / 16 * 16;
     const int spn = w.sp_np ? w.sp_np[i] : 0;
-    s[10] += spn;
+    s[2] += spn;
     m[4] = max(m[4], spn);
     m[0] = max(m[0], c.n1);
     m[1] = max(m[1], c.ns);
@@ -471,29 +469,27 @@ __global__ void k_offsets(Work w, int nq) {
     m[3] = max(m[3], np);
     snt += c.nt;
   }
-  for (int t = 0; t < 11; ++t) part[t][threadIdx.x] = s[t];
+  for (int t = 0; t < 10; ++t) part[t][threadIdx.x] = s[t];
   for (int t = 0; t < 5; ++t) mx[t][threadIdx.x] = m[t];
   tot_nt[threadIdx.x] = snt;
   __syncthreads();
   for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-    long long v[11];
-    for (int t = 0; t < 11; ++t) v[t] = threadIdx.x >= off ? part[t][threadIdx.x - off] : 0;
+    long long v[10];
+    for (int t = 0; t < 10; ++t) v[t] = threadIdx.x >= off ? part[t][threadIdx.x - off] : 0;
     __syncthreads();
-    for (int t = 0; t < 11; ++t) part[t][threadIdx.x] += v[t];
+    for (int t = 0; t < 10; ++t) part[t][threadIdx.x] += v[t];
     __syncthreads();
   }
-  long long run[11];
-  for (int t = 0; t < 11; ++t) run[t] = part[t][threadIdx.x] - s[t];
+  long long run[10];
+  for (int t = 0; t < 10; ++t) run[t] = part[t][threadIdx.x] - s[t];
   for (int i = b; i < e; ++i) {
     Counts c = w.counts[i];
-    long long N1 = 3LL * c.n1;
     w.off_k1[i] = run[0];
     w.off_s[i] = run[1];
-    w.off_b[i] = run[2];
     w.off_t[i] = run[3];
     if (w.off_p) w.off_p[i] = run[4];
     if (w.off_a) w.off_a[i] = run[5];
-    if (w.off_np) w.off_np[i] = run[10];
+    if (w.off_np) w.off_np[i] = run[2];
     if (w.off_tq) {
       w.off_tq[i] = run[6];
       w.off_tr[i] = run[7];
@@ -507,11 +503,10 @@ __global__ void k_offsets(Work w, int nq) {
     run[9] += (c.ns + 15) / 16 * 16;
     run[0] += c.n1;
     run[1] += c.ns;
-    run[2] += (long long)nq * N1 * (N1 + 1) / 2;
     run[3] += 9LL * c.ns * c.ns;
     run[4] += w.pcount ? w.pcount[2 * i] : 0;
     run[5] += w.pcount ? w.pcount[2 * i + 1] : 0;
-    run[10] += w.sp_np ? w.sp_np[i] : 0;
+    run[2] += w.sp_np ? w.sp_np[i] : 0;
   }
   for (int st = blockDim.x / 2; st > 0; st >>= 1) {
     if (threadIdx.x < st) {
@@ -523,11 +518,10 @@ __global__ void k_offsets(Work w, int nq) {
   if (threadIdx.x == blockDim.x - 1) {
     w.off_k1[N] = part[0][threadIdx.x];
     w.off_s[N] = part[1][threadIdx.x];
-    w.off_b[N] = part[2][threadIdx.x];
     w.off_t[N] = part[3][threadIdx.x];
     if (w.off_p) w.off_p[N] = part[4][threadIdx.x];
     if (w.off_a) w.off_a[N] = part[5][threadIdx.x];
-    if (w.off_np) w.off_np[N] = part[10][threadIdx.x];
+    if (w.off_np) w.off_np[N] = part[2][threadIdx.x];
     for (int t = 0; t < 4; ++t) w.totals[t] = part[t][threadIdx.x];
     w.totals[8] = part[4][threadIdx.x];
     w.totals[9] = part[5][threadIdx.x];
@@ -549,7 +543,7 @@ __global__ void k_offsets(Work w, int nq) {
   }
 }
 
-void launch_offsets(const Work& w, const DevParams& p, cudaStream_t s) {
+void launch_offsets(const Work& w, cudaStream_t s) {
   if (w.n_atoms == 0) return;
-  k_offsets<<<1, OFF_T, 0, s>>>(w, p.nqs);
+  k_offsets<<<1, OFF_T, 0, s>>>(w);
 }

@@ -259,14 +259,12 @@ static_assert((3 * PTC_SA * PTC_LD + 4 * PTC_SA * PTC_GL) * 8 <= TcsShape<5, PTC
 }  // namespace
 
 // The tcgen05 pair kernel on the digit images of P and Q (written by the series adjoint, or here from
-// FP64 P, Q); digits must be 5.
-bool launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits, cudaStream_t s) {
-  if (c1 <= c0) return true;
-  if (digits != 5) return false;
-  launch_slice_pq(w, p, c0, c1, digits, s);
+// FP64 P, Q).
+void launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s) {
+  if (c1 <= c0) return;
+  launch_slice_pq(w, p, c0, c1, s);
   const int na = (max_ns + PTC_SA - 1) / PTC_SA, nb = (max_ns + PTC_SB - 1) / PTC_SB;
   using Sh = TcsShape<5, PTC_NB, PTC_BUF, PTC_COLS>;
   raise_smem_limit((const void*)k_pair_tc<5>, Sh::kBytes);
   k_pair_tc<5><<<(c1 - c0) * na * nb, 256, Sh::kBytes, s>>>(w, p, c0, nb, na * nb);
-  return true;
 }

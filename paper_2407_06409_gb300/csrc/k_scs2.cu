@@ -476,8 +476,11 @@ __device__ void scs2_build_rhs64(const Work& w, const DevParams& p, int c, int n
 // systems per SM); this kernel takes 14.0 + 7.7 ms and k_scs_contract 4.1 ms.  It is bound by the
 // FP32 issue rate and the latency of the pair loads in the float-float residuals (60 % of the
 // issue slots).  A warp per system with packed FP32 pairs (fma.rn.f32x2) measured 17.4 + 10.5 ms:
-// the pairs cost as many moves as they save, with half the warps.  A system whose condition number
-// is above about 10^3 needs more steps than a factor would cost; beyond CG_MAXIT it goes to LU.
+// the pairs cost as many moves as they save, with half the warps.  The steps grow with the condition
+// number, where a factor's time does not: with alpha0 raised until the smallest eigenvalue of B nears zero
+// (jittered lattices and chains, 36 to 1000 atoms, all polarisabilities still positive) the forward
+// solves of 1000 atoms rise from 4.1 to 5.6 ms (the factors took 10.7) and those of 64 atoms from 0.63 to 0.97 (1.10),
+// so no such call is slower than with the factor.  Beyond CG_MAXIT a system goes to LU.
 #define CG_MAXIT 250          // steps of one inner solve; systems that need more go to LU
 #define CG_OUTER 12           // refinement steps
 
@@ -903,8 +906,9 @@ __device__ __forceinline__ void adjoint_not_finite(const Work& w, int id, int n1
   if (threadIdx.x == 0) w.lexp[id] = 0;
 }
 
-// One (centre, frequency) system per block of 32 S (3 / NC) threads.  ADJ = false: X = B^-1 d to FP64
-// accuracy (2^-52), alpha_K and alpha_I.  ADJ = true: lambda = B^-1 dL/dX, to 2^-30 of its largest
+// One (centre, frequency) system per block of 32 S (3 / NC) threads.  ADJ = false: X = B^-1 d, refined until
+// a correction falls to 2^-52 of it, alpha_K and alpha_I; the couplings and the residuals are float-float, so
+// its error is about cond(B) 2^-46.  ADJ = true: lambda = B^-1 dL/dX, to 2^-30 of its largest
 // value or better (it feeds the forces only).  The refinement measures its own contraction.
 constexpr int cg_min_blocks(int S, int NC) { return NC == 1 ? (S == 1 ? 7 : (S == 2 ? 4 : 2)) : (S == 1 ? 20 : (S == 2 ? 12 : 5)); }
 template <int S, int NC, bool ADJ>
@@ -1521,8 +1525,9 @@ void launch_pair_radial(const Work& w, const DevParams& p, cudaStream_t s) {
   k_pair_radial<<<w.n_atoms, 128, 0, s>>>(w, p);
 }
 
-// Sites one screening system may hold: |K1| <= 96 (three warps), and with it the combined size of
-// its lists, a limit of the entry points in terms of |K1| and |K1 u K2|.
+// Sites one screening system may hold: |K1| <= 96 (three warps) and, for the largest of them, |K1 u K2| (at most
+// 3264 at |K1| = 96).  The second limit is the shared memory of a packed dense factor with its lists; the
+// kernels here need less (k_scs_fill 204 KB at 4096 sites), but it stays part of what the entry points accept.
 bool scs_capacity(int max_n1, int max_n12) {
   const size_t N1 = 3 * (size_t)max_n1;
   const size_t fl = (N1 * (N1 + 1) / 2 + 7 * N1 + (N1 + 15) / 16 * 136 + 1) & ~size_t(1);
@@ -1545,7 +1550,7 @@ static void run_solve(const Work& w, const DevParams& p, const int* order, int c
 template <bool ADJ>
 static void run_solve_any(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
-  const bool split = (long long)w.n_atoms * p.nqs <= 152 * 12;
+  const bool split = (long long)w.n_atoms * p.nqs <= 12LL * device_sms();
   if (split) {
     if (max_n1 <= 32) run_solve<1, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
     else if (max_n1 <= 64) run_solve<2, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
@@ -1566,7 +1571,7 @@ void launch_scs_adjoint(const Work& w, const DevParams& p, const int* order, int
 // Blocks per centre of the contraction: structures of fewer centres than fill the chip twice split
 // the frequencies (64-atom box, SCS adjoint phase 0.76 -> 0.57 ms, of which the solves 0.2).
 int scs_contract_split(int n_atoms, int nqs) {
-  const int want = (2 * 152 + n_atoms - 1) / (n_atoms > 0 ? n_atoms : 1);
+  const int want = (2 * device_sms() + n_atoms - 1) / (n_atoms > 0 ? n_atoms : 1);
   const int per = (nqs + want - 1) / want;
   return (nqs + per - 1) / per;
 }

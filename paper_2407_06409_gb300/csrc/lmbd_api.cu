@@ -32,6 +32,13 @@ void raise_smem_limit(const void* func, size_t bytes) {
     cur = bytes;
 }
 
+int device_sms() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    cudaGetLastError();
+  return n > 0 ? n : 152;
+}
+
 namespace {
 
 constexpr int LMBD_ESTALE = -1;   // internal: the kept forward state does not match the inputs
@@ -91,7 +98,7 @@ struct Ctx {
   DevBuf theta_f, theta_out;       // force integrands at the samples (J x N x 3); fitted forces
   int last_nqs = 0;                // columns of the central polarisabilities of the last call
   cudaEvent_t ev[LMBD_NPHASE + 1] = {};
-  // around the bucket launches of the SCS factor (pass A) and SCS adjoint (pass C): their own
+  // around the bucket launches of the SCS solves (pass A) and of their adjoint (pass C): their own
   // wall time, fork to join, without the pair-list and radial-table kernels of the phase
   cudaEvent_t kev[4] = {};
   // side streams for independent bucket launches (same priority as the caller's stream)
@@ -245,7 +252,7 @@ int stage_input(DevBuf& buf, const void* src, size_t bytes, cudaStream_t s, cons
 // Central atoms are processed in contiguous waves [c0, c1) whose per-centre arrays fit the
 // memory budget.  The arrays of a wave live in one arena; every pointer is rebased by the
 // wave's first offset, so kernels index them with the whole-structure offsets unchanged.
-enum { O_K1, O_S, O_B, O_T, O_P, O_A, O_TQ, O_TR, O_KP, O_SP, O_NP, O_COUNT };
+enum { O_K1, O_S, O_T, O_P, O_A, O_TQ, O_TR, O_KP, O_SP, O_NP, O_COUNT };
 
 struct Offs {
   const long long* h;
@@ -282,7 +289,7 @@ struct Layout {
   bool pq_fp64;  // FP64 P and Q kept (FP64 products, more than 32 integrand frequencies)
   int gs_ld;     // float2 per pair of the SCS adjoint's gradient scratch
 
-  // stage 1 (SCS): pair lists, FP32 factors and solutions of centres [c0, c1)
+  // stage 1 (SCS): pair lists, radial terms and solutions of centres [c0, c1)
   size_t stage1(const Offs& o, int c0, int c1, char* base, Work* w) const {
     Carver cv{base, 0};
     const long long p0 = o.at(O_P, c0), np = o.span(O_P, c0, c1);
@@ -444,7 +451,7 @@ bool partition(int N, size_t cap, F size, std::vector<int>& cuts) {
 // Size buckets for the SCS kernels: within each wave, centres sorted by |K1|, one launch per
 // bucket of width 6 in |K1| with shared memory sized to the bucket.
 struct Bucket {
-  int b0, b1, n1, n12;
+  int b0, b1, n1;
 };
 void make_buckets(const std::vector<Counts>& cnt, const std::vector<int>& cuts, std::vector<int>& order,
                   std::vector<std::vector<Bucket>>& buckets, int width) {
@@ -458,13 +465,12 @@ void make_buckets(const std::vector<Counts>& cnt, const std::vector<int>& cuts, 
     int b0 = c0;
     while (b0 < c1) {
       const int lo = cnt[order[b0]].n1;
-      int b1 = b0, n1m = 0, n12m = 0;
+      int b1 = b0, n1m = 0;
       while (b1 < c1 && cnt[order[b1]].n1 < lo + width) {
         n1m = std::max(n1m, cnt[order[b1]].n1);
-        n12m = std::max(n12m, cnt[order[b1]].n12);
         ++b1;
       }
-      buckets[wv].push_back({b0, b1, n1m, n12m});
+      buckets[wv].push_back({b0, b1, n1m});
       b0 = b1;
     }
   }
@@ -698,7 +704,6 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   long long* const ob = (long long*)c->offs.p;
   w.off_k1 = ob + (size_t)O_K1 * (N + 1);
   w.off_s = ob + (size_t)O_S * (N + 1);
-  w.off_b = ob + (size_t)O_B * (N + 1);
   w.off_t = ob + (size_t)O_T * (N + 1);
   w.off_p = ob + (size_t)O_P * (N + 1);
   w.off_a = ob + (size_t)O_A * (N + 1);
@@ -799,7 +804,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
       ++launches;
     }
     launch_scs_count(w, dp, w.site_cap, s);
-    launch_offsets(w, dp, s);
+    launch_offsets(w, s);
     launches += 2;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(c->totals_h, w.totals, sizeof(long long) * 16, cudaMemcpyDeviceToHost, s));
@@ -999,8 +1004,8 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   const bool one_wave = nwA == 1 && nw2 == 1 && nwC == 1;
   const bool per_atom = c->launch_mode == LMBD_LAUNCH_PER_ATOM;
 
-  // stage-1 forward of one wave: pair lists, FP32 factorisation, refined solutions, alpha_K
-  bool kmark_fwd = false;   // record kev[0], kev[1] around the factor buckets (pass A, profiling)
+  // stage-1 forward of one wave: pair lists, refined solutions, alpha_K
+  bool kmark_fwd = false;   // record kev[0], kev[1] around the solve buckets (pass A, profiling)
   bool tally_lu = true;     // count LU-fallback systems in pass A only (pass C may recompute)
   auto stage1_forward = [&](int wv, const std::vector<int>& cuts, const std::vector<std::vector<Bucket>>& bk,
                             const int* order) -> int {
@@ -1015,7 +1020,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
       phase_launch[LMBD_PHASE_SCS] += c1 - c0;
     } else {
       if (kmark_fwd) cudaEventRecord(c->kev[0], s);
-      nvtxRangePushA("lmbd SCS factor buckets");
+      nvtxRangePushA("lmbd SCS solve buckets");
       Fork fk(c, s, (int)bk[wv].size());
       for (size_t i = 0; i < bk[wv].size(); ++i) {
         const Bucket& b = bk[wv][i];
@@ -1134,11 +1139,10 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
           launch_paper_force_seeds(w, dp, cc, cc + 1, max_ns, s);
         } else {
           launch_mbd_adj_series(w, dp, cc, cc + 1, s);
-          if (sliced_pair && tc05) {
-            if (!launch_pair_tc(w, dp, cc, cc + 1, max_ns, DIG_P, s)) return LMBD_ECUDA;
-          }
+          if (sliced_pair && tc05)
+            launch_pair_tc(w, dp, cc, cc + 1, max_ns, s);
           else if (sliced_pair)
-            launch_mbd_adj_pair_oz2(w, dp, cc, cc + 1, max_ns, DIG_P, s);
+            launch_mbd_adj_pair_oz2(w, dp, cc, cc + 1, max_ns, s);
           else if (sparse)
             launch_sp_adj_pair(w, dp, cc, cc + 1, max_pairs, s);
           else
@@ -1157,11 +1161,10 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
       } else {
         launch_mbd_adj_series(w, dp, c0, c1, s);
         mark(LMBD_PHASE_ADJ_PAIR);
-        if (sliced_pair && tc05) {
-          if (!launch_pair_tc(w, dp, c0, c1, max_ns, DIG_P, s)) return LMBD_ECUDA;
-        }
+        if (sliced_pair && tc05)
+          launch_pair_tc(w, dp, c0, c1, max_ns, s);
         else if (sliced_pair)
-          launch_mbd_adj_pair_oz2(w, dp, c0, c1, max_ns, DIG_P, s);
+          launch_mbd_adj_pair_oz2(w, dp, c0, c1, max_ns, s);
         else if (sparse)
           launch_sp_adj_pair(w, dp, c0, c1, max_pairs, s);
         else
@@ -1307,7 +1310,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
   if (*c->status_h & LMBD_FLAG_TIMEOUT) return LMBD_ETIMEOUT;
   // the block-sparse fill found other partners than its count: cannot happen for one site list
   if (*c->status_h & LMBD_FLAG_PATTERN) return LMBD_ECUDA;
-  if (*c->status_h & (LMBD_FLAG_NOT_SPD | LMBD_FLAG_NOT_CONVERGED)) return LMBD_NOT_SPD;
+  if (*c->status_h & LMBD_FLAG_NOT_SPD) return LMBD_NOT_SPD;
   if (*c->status_h & LMBD_FLAG_MODEL) return LMBD_EMODEL;
   if (split == 1 && one_wave && persist && !per_atom) {
     c->kept_valid = true;
@@ -1908,7 +1911,6 @@ int noalloc_central(const lmbd_species* species_params, int n_species, const lmb
   w.counts = cv.take<Counts>(N);
   w.off_k1 = cv.take<long long>(N + 1);
   w.off_s = cv.take<long long>(N + 1);
-  w.off_b = cv.take<long long>(N + 1);
   w.off_t = cv.take<long long>(N + 1);
   w.totals = cv.take<long long>(16);   // the offsets kernel writes 16 totals
   w.status = cv.take<int>(4);
@@ -1942,7 +1944,7 @@ int noalloc_central(const lmbd_species* species_params, int n_species, const lmb
   int launches = 0;
   launch_free_atom(w, dp, s);
   launch_neighbors(w, dp, g, s, &launches);
-  launch_offsets(w, dp, s);
+  launch_offsets(w, s);
   CK(cudaGetLastError());
   long long tot[16];
   int flags = 0;

@@ -13,7 +13,6 @@
 #define LMBD_FLAG_NOT_SPD 1
 #define LMBD_FLAG_CAPACITY 2
 #define LMBD_FLAG_COINCIDENT 4
-#define LMBD_FLAG_NOT_CONVERGED 8
 #define LMBD_FLAG_MODEL 16          // Lorentzian model not applicable: alpha~(0) < alpha~(omega_ref),
                                     // or a fitted phi without decaying term
 #define LMBD_FLAG_TIMEOUT 32        // a bounded device wait (tensor-core pipeline) ran out
@@ -111,7 +110,6 @@ struct Work {
   // per-centre offsets (exclusive prefix sums, N + 1 entries)
   long long* off_k1;           // sum n1
   long long* off_s;            // sum ns
-  long long* off_b;            // sum nq (3 n1)^2
   long long* off_t;            // sum (3 ns)^2
   long long* off_p;            // sum of SCS pairs per centre
   long long* off_a;            // sum of SCS adjacency entries per centre
@@ -249,24 +247,6 @@ __device__ __forceinline__ void fermi(double r, double s, double d, double& f, d
 
 // T_SR written as F(r) [A0(r) I + B0(r) r r^T] (Eq. T_SR with Eqs. g-func, h-func):
 // A0 = g / r^3, B0 = (h~ - 3 g) / r^5 with x = r/sigma, h~ = (4/sqrt(pi)) x^3 exp(-x^2).
-// Also returns the radial derivatives A0', B0'.
-__device__ __forceinline__ void tsr_radial(double r, double sigma, double& A0, double& B0,
-                                           double& dA0, double& dB0) {
-  const double two_over_sqrtpi = 1.1283791670955126;
-  double x = r / sigma;
-  double ex = exp(-x * x);
-  double g = erf(x) - two_over_sqrtpi * x * ex;
-  double ht = 2.0 * two_over_sqrtpi * x * x * x * ex;
-  double ir = 1.0 / r;
-  double ir2 = ir * ir;
-  double ir3 = ir2 * ir;
-  double ir4 = ir2 * ir2;
-  A0 = g * ir3;
-  B0 = (ht - 3.0 * g) * ir4 * ir;
-  dA0 = (ht - 3.0 * g) * ir4;
-  dB0 = (15.0 * g - 5.0 * ht - 2.0 * x * x * ht) * ir4 * ir2;
-}
-
 __device__ __forceinline__ void tsr_value(double r, double sigma, double& A0, double& B0) {
   const double two_over_sqrtpi = 1.1283791670955126;
   double x = r / sigma;
@@ -396,7 +376,7 @@ void launch_sites_refresh(const Work& w, const DevParams& p, const Grid& g, cuda
 void launch_skin_check(const Work& w, const double* ref_pos, const int* ref_spec, double half_skin2, int* flag,
                        cudaStream_t s);
 void launch_neighbors(const Work& w, const DevParams& p, const Grid& g, cudaStream_t s, int* launches);
-void launch_offsets(const Work& w, const DevParams& p, cudaStream_t s);
+void launch_offsets(const Work& w, cudaStream_t s);
 void launch_scs_count(const Work& w, const DevParams& p, int max_n12, cudaStream_t s);
 void launch_scs_fill(const Work& w, const DevParams& p, int c0, int c1, int max_n12, int max_n1, cudaStream_t s);
 void launch_pair_radial(const Work& w, const DevParams& p, cudaStream_t s);
@@ -446,17 +426,17 @@ void launch_chain_oz2(const Work& w, const DevParams& p, int m, int c0, int c1, 
 // W = D v_m digit planes for chain step m (one block per central atom)
 void launch_slice_w(const Work& w, const DevParams& p, int m, int c0, int c1, int digits, cudaStream_t s);
 // chain step on the fifth-generation tensor cores (tcgen05, TMEM accumulators), digits 5 or 6
-// (digits 5 or 6; returns false for another digit count or when the device cannot be queried)
+// (returns false for another digit count)
 bool launch_chain_tc(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, int digits, int st,
                      cudaStream_t s);
 size_t chain_tc_smem(int digits);
 // P and Q digit planes (blockIdx.y = 0: P, 1: Q)
-void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, int digits, cudaStream_t s);
-// adjoint pair matrix and its per-pair contraction on the tcgen05 tensor cores (digits 5 only;
-// returns false for another digit count)
-bool launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits, cudaStream_t s);
-void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, int digits,
-                             cudaStream_t s);
+void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s);
+// adjoint pair matrix and its per-pair contraction, 5 digits: tcgen05 tensor cores, warp-level products
+void launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
+void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
+// SMs of the current device
+int device_sms();
 
 // Raise the dynamic shared-memory limit of a kernel to at least `bytes` (never lowers it: the
 // limit is process-wide, and lowering it while another host thread launches the same kernel

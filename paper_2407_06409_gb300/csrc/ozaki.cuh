@@ -6,18 +6,20 @@
 // multiplication by using fast routines of matrix multiplication", and its tensor-core use by
 // Mukunoki et al.):
 //   * every row of A (column of B) is scaled by a power of two 2^e so that |a| < 2^e;
-//   * the scaled value is truncated to 7 S bits and split into S signed 7-bit digits,
-//       a = 2^e sum_k d_k 2^{-7k},  |d_k| <= 127  (exact in bf16);
+//   * the scaled value is rounded to 7 S bits and split into S signed 7-bit digits,
+//       a = 2^e sum_k d_k 2^{-7k},  |d_k| <= 127  (exact in bf16); rounding up to 2^e itself gives
+//     a first digit of 128 and zeros (FP64 P and Q, oz_digits, are truncated instead);
 //   * digit planes are multiplied on the tensor cores (tcgen05.mma, tc_sliced.cuh, or the
 //     warp-level mma.sync below) with FP32 accumulation; every product d_k d_l is an integer
-//     below 2^14, and the K dimension is accumulated in chunks of at most OZ_KCHUNK = 256
-//     terms, so one digit pair sums to less than 2^22;
+//     of at most 2^14, and the K dimension is accumulated in chunks of at most OZ_KCHUNK = 256
+//     terms, so one digit pair sums to at most 2^22;
 //   * products with the same digit order m = k + l share one FP32 accumulator: with at most
-//     four pairs per order below m = 6 every partial sum stays below 2^24 and is exact;
+//     four pairs per order below m = 4 every partial sum stays within 2^24 and is exact;
 //     higher orders can round, at a level below 2^-52 of the leading term.  Pairs with
-//     m > S - 1 are dropped; after each K chunk the orders are recombined exactly as 64-bit
-//     integers, Y += sum_m acc_m 2^{7 (S - 1 - m)}, and the result is scaled once in FP64:
-//       c = 2^{e_row + e_col - 7 (S + 1)} Y.
+//     m > S - 1 are dropped; after each K chunk the orders are added up,
+//       c = 2^{e_row + e_col - 14} sum_m acc_m 2^{-7 m}:
+//     on the tcgen05 path in float-float (one chunk exactly, chunks joined with an error of about
+//     2^-46), on the warp-level path as 64-bit integers, scaled once in FP64.
 // The result differs from the FP64 product by at most ~S 2^{-7S} sum |a||b| (normwise);
 // the digit count S is chosen per product from the accuracy its consumer needs.
 #pragma once
@@ -62,35 +64,12 @@ __device__ __forceinline__ int oz_biased_exp(double v) {
 // Scale exponent from the largest biased exponent of a row/column: |v| < 2^(ex - 1022).
 __device__ __forceinline__ int oz_scale_exp(int max_biased) { return max_biased == 0 ? -1022 : max_biased - 1022; }
 
-// K chunk over which one digit order is accumulated in FP32 before the exact integer
-// recombination (every partial sum of the low orders stays an integer below 2^24).
+// K chunk over which one digit order is accumulated in FP32 before the orders are added up (every
+// partial sum of the low orders stays an integer within 2^24).
 #define OZ_KCHUNK 256
 
-__device__ __forceinline__ unsigned short oz_bf16_bits(int d) {
-  __nv_bfloat16 h = __float2bfloat16_rn((float)d);
-  return *reinterpret_cast<unsigned short*>(&h);
-}
-
 // Signed 7-bit digits of v relative to 2^e (|v| < 2^e): v ~= 2^e sum_{k=1..S} d_k 2^{-7k},
-// truncated toward zero (integer operations only), stored as bf16 bits at dst[(k - 1) plane].
-// S is a compile-time constant so the digits stay in registers.
-template <int S>
-__device__ __forceinline__ void oz_store_digits(unsigned short* dst, long long plane, double v, int e) {
-  const long long bits = __double_as_longlong(v);
-  const int ex = (int)((bits >> 52) & 0x7ff);
-  unsigned long long U = 0;
-  if (ex != 0) {
-    const unsigned long long mant = (unsigned long long)(bits & 0xFFFFFFFFFFFFFLL) | (1ULL << 52);
-    const int sh = (ex - 1075) + 7 * S - e;
-    if (sh >= 0) U = mant << sh;
-    else if (sh > -64) U = mant >> (-sh);
-  }
-  const int sg = bits < 0 ? -1 : 1;
-#pragma unroll
-  for (int k = 0; k < S; ++k) dst[k * plane] = oz_bf16_bits(sg * (int)((U >> (7 * (S - 1 - k))) & 127ULL));
-}
-
-// The same digits as bf16 bits in d[0..S-1].
+// truncated toward zero (integer operations only), as bf16 bits in d[0..S-1].
 template <int S>
 __device__ __forceinline__ void oz_digits(double v, int e, unsigned (&d)[S]) {
   const long long bits = __double_as_longlong(v);
@@ -134,8 +113,6 @@ __device__ __forceinline__ void oz_mma(float* d, const uint32_t* a, const uint32
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-
-__device__ __forceinline__ uint32_t oz_ld32(const unsigned short* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
 // ---------------------------------------------------------------------------------------
 // shared-memory staged variant

@@ -1,33 +1,34 @@
-// Sliced FP64 products on the fifth-generation tensor cores: the block-wide main loop shared by
-// the Krylov-chain kernel (k_chain_tc.cu) and the adjoint pair-matrix kernel (k_pair_tc.cu).
+// Sliced FP64 products on the fifth-generation tensor cores: shapes, barriers, tear-down, image copies and
+// the block-wide main loop of the adjoint pair-matrix kernel (k_pair_tc.cu).  The Krylov-chain kernel
+// (k_chain_tc.cu) takes shapes and copies from here and runs the same stages from separate roles.
 //
 // One CTA of 256 threads owns a 128 x NB output tile.  A (128 rows) and B (NB rows) are S digit
-// planes of signed 7-bit integers stored as bf16 (ozaki.cuh), K-major, brought
-// in by the caller's copy function: tile images (tcs_image_copy), or boxes of 2-D tensor maps (inner
-// dimension K, one row per matrix row, 64-byte swizzle) in tcs_mainloop.  The loop
-//   * stages K slices of 32 of every plane of A and B into a three-deep ring of 64-byte-swizzled
-//     shared-memory tiles with bulk tensor copies (TMA, cp.async.bulk.tensor) issued by one
-//     thread; each slot has a "full" mbarrier counting the bytes in flight (K past the tensor's
-//     extent is zero-filled by the copy engine);
+// planes of signed 7-bit integers stored as bf16 (ozaki.cuh), K-major, in memory as images of the
+// shared-memory tiles.  The loop
+//   * stages K slices of 32 of every plane of A and B into a ring of NBUF 64-byte-swizzled
+//     shared-memory slots with bulk copies (cp.async.bulk) issued by one thread; each slot has a
+//     "full" mbarrier counting the bytes in flight;
 //   * keeps one FP32 accumulator per digit order g in tensor memory, NB columns each, order g
 //     at columns [g NB, g NB + NB).  The B planes of a slot are consecutive in shared memory, so
 //     planes l0 .. l0 + n - 1 form one taller B operand, and the product of A plane k with it,
 //     written at column (k + l0) NB, lands each pair (k, l) in the accumulator of order k + l:
 //     one tcgen05.mma (M = 128, N = n NB <= 256, K = 16, bf16 -> FP32) per A plane covers all
 //     its digit pairs with k + l <= S - 1;
-//   * the same thread issues each slot's MMAs once its copies have landed, commits them to the
-//     slot's "empty" mbarrier, and refills the slot of the previous stage (whose MMAs are done by
-//     then) with the stage three ahead, so copies and MMAs overlap;
+//   * the same thread issues each slot's MMAs once its copies have landed (to the next multiple of 16
+//     past K), commits them to the slot's "empty" mbarrier, and refills the slot of the previous
+//     stage (whose MMAs are done by then) with the stage NBUF ahead, so copies and MMAs overlap;
 //   * at the end of every K chunk of OZ_KCHUNK (every partial sum of the low digit orders is an
 //     integer below 2^24 and therefore exact in FP32) the thread commits an "accumulators"
 //     mbarrier and waits for it, a block barrier publishes the result, and all 256 threads hand
-//     the accumulators to `consume`, which reads them with tcgen05.ld and adds them up as
-//     integers; the next chunk restarts them.
-// Rows of a box past a plane's end read the next plane or centre: they only reach output rows
+//     the accumulators to `consume`, which reads them with tcgen05.ld and adds them up; the next
+//     chunk restarts them.
+// Rows of a slot past the tile's rows hold what was there before: they only reach output rows
 // (A) or columns (B) that the callers discard.  Every mbarrier wait of the loop is bounded (a
 // cycle budget, 2^32 by default); if one runs out the loop stops, and the teardown waits for the
 // block's copies and MMAs in flight (bounded by TCS_WAIT_CYCLES), frees tensor memory and sets
 // LMBD_FLAG_TIMEOUT.
+// Operands through 2-D tensor maps (tcs_mainloop, TcsTile, tc_encode_map) are for callers whose planes are
+// plain rows; the library's kernels have none left.
 #pragma once
 #include "lmbd_internal.cuh"
 #include "ozaki.cuh"

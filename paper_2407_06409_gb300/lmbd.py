@@ -388,7 +388,7 @@ def _make_energy_function():
 
         @staticmethod
         def forward(ctx, positions, model, cell, species, hirshfeld):
-            # the library keeps the forward state (factors, T_LR, Krylov blocks) for the backward
+            # the library keeps the forward state (SCS solutions, T_LR, Krylov blocks) for the backward
             e = model.energy_keep(positions.detach(), cell, species, hirshfeld)
             ctx.model = model
             ctx.save_for_backward(positions)
