@@ -260,7 +260,7 @@ bool launch_chain_tc(const Work& w, const DevParams& p, int m, int c0, int c1, i
   if (digits != 5 && digits != 6) return false;
   launch_slice_w(w, p, m, c0, c1, digits, s);
   const int tiles = (3 * max_ns + TCS_M - 1) / TCS_M;
-  const int items = (c1 - c0) * tiles, grid = std::min(items, device_sms());
+  const int items = (c1 - c0) * tiles, grid = std::min(items, w.sms);
   if (digits == 6) {
     raise_smem_limit((const void*)k_chain_tc<6>, TcsShape<6, CTC_NB>::kBytes);
     k_chain_tc<6><<<grid, CTC_THREADS, TcsShape<6, CTC_NB>::kBytes, s>>>(w, p, m, c0, items, tiles, st);

@@ -2521,17 +2521,13 @@ void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, 
   k_mbd_adj_pair_oz2<<<(c1 - c0) * tiles, 288, sm, s>>>(w, p, c0, tiles);
 }
 
-// FIT: the scale of fitted coefficients; the default series is compiled without it.
+// FIT: with the scale of fitted coefficients (zero for the others); the default path is compiled without it.
 template <int NM>
 static void run_adj_site_digits(const Work& w, const DevParams& p, int c0, int c1, int seg, cudaStream_t s) {
   const int n = c1 - c0;
-  if (w.trec_full) {
-    if (p.lanczos) k_adj_site_digits<NM, true, true><<<n, 256, 0, s>>>(w, p, c0, seg);
-    else k_adj_site_digits<NM, true, false><<<n, 256, 0, s>>>(w, p, c0, seg);
-  } else {
-    if (p.lanczos) k_adj_site_digits<NM, false, true><<<n, 256, 0, s>>>(w, p, c0, seg);
-    else k_adj_site_digits<NM, false, false><<<n, 256, 0, s>>>(w, p, c0, seg);
-  }
+  if (!w.trec_full) k_adj_site_digits<NM, false, true><<<n, 256, 0, s>>>(w, p, c0, seg);
+  else if (p.lanczos) k_adj_site_digits<NM, true, true><<<n, 256, 0, s>>>(w, p, c0, seg);
+  else k_adj_site_digits<NM, true, false><<<n, 256, 0, s>>>(w, p, c0, seg);
 }
 
 void launch_mbd_adj_series(const Work& w, const DevParams& p, int c0, int c1, cudaStream_t s) {

@@ -1550,7 +1550,7 @@ static void run_solve(const Work& w, const DevParams& p, const int* order, int c
 template <bool ADJ>
 static void run_solve_any(const Work& w, const DevParams& p, const int* order, int c0, int c1, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
-  const bool split = (long long)w.n_atoms * p.nqs <= 12LL * device_sms();
+  const bool split = (long long)w.n_atoms * p.nqs <= 12LL * w.sms;
   if (split) {
     if (max_n1 <= 32) run_solve<1, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
     else if (max_n1 <= 64) run_solve<2, 1, ADJ>(w, p, order, c0, c1, max_n1, s);
@@ -1570,30 +1570,30 @@ void launch_scs_adjoint(const Work& w, const DevParams& p, const int* order, int
 
 // Blocks per centre of the contraction: structures of fewer centres than fill the chip twice split
 // the frequencies (64-atom box, SCS adjoint phase 0.76 -> 0.57 ms, of which the solves 0.2).
-int scs_contract_split(int n_atoms, int nqs) {
-  const int want = (2 * device_sms() + n_atoms - 1) / (n_atoms > 0 ? n_atoms : 1);
+static int scs_contract_split(int n_atoms, int nqs, int sms) {
+  const int want = (2 * sms + n_atoms - 1) / (n_atoms > 0 ? n_atoms : 1);
   const int per = (nqs + want - 1) / want;
   return (nqs + per - 1) / per;
 }
 // Shared memory of its blocks: lambda and X of all a block's frequencies, or two blocks per SM; a centre
 // whose |K1| does not fit takes its frequencies in chunks.
-static size_t scs_contract_smem(int n_atoms, int max_n1, int nqs) {
-  const int split = scs_contract_split(n_atoms, nqs), per = (nqs + split - 1) / split;
+static size_t scs_contract_smem(int split, int max_n1, int nqs) {
+  const int per = (nqs + split - 1) / split;
   return std::min((size_t)144 * max_n1 * per, (size_t)112 * 1024);
 }
 // float2 of gradient scratch per pair: 3, and 14 sums when the frequencies go in chunks, per block
-int scs_contract_scratch(int n_atoms, int max_n1, int nqs) {
-  const int split = scs_contract_split(n_atoms, nqs), per = (nqs + split - 1) / split;
-  return split * (scs_contract_smem(n_atoms, max_n1, nqs) < (size_t)144 * max_n1 * per ? 3 + CON_W : 3);
+int scs_contract_scratch(int n_atoms, int max_n1, int nqs, int sms) {
+  const int split = scs_contract_split(n_atoms, nqs, sms), per = (nqs + split - 1) / split;
+  return split * (scs_contract_smem(split, max_n1, nqs) < (size_t)144 * max_n1 * per ? 3 + CON_W : 3);
 }
 
 void launch_scs_contract(const Work& w, const DevParams& p, int c0, int c1, int max_n1, cudaStream_t s) {
   if (c1 <= c0) return;
-  const int split = scs_contract_split(w.n_atoms, p.nqs);
-  const size_t sm = scs_contract_smem(w.n_atoms, max_n1, p.nqs);
+  const int split = scs_contract_split(w.n_atoms, p.nqs, w.sms);
+  const size_t sm = scs_contract_smem(split, max_n1, p.nqs);
   raise_smem_limit((const void*)k_scs_contract, sm);
   k_scs_contract<<<(c1 - c0) * split, 256, sm, s>>>(w, p, c0, split, (int)sm,
-                                                    scs_contract_scratch(w.n_atoms, max_n1, p.nqs));
+                                                    scs_contract_scratch(w.n_atoms, max_n1, p.nqs, w.sms));
 }
 
 // LU fallback launches: a fixed grid of lu_blocks persistent blocks (one dense slot each);

@@ -32,7 +32,7 @@ void raise_smem_limit(const void* func, size_t bytes) {
     cur = bytes;
 }
 
-int device_sms() {
+static int device_sms() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     cudaGetLastError();
@@ -682,6 +682,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
 
   Work w{};
   w.n_atoms = N;
+  w.sms = device_sms();
   w.pos = (const double*)pos;
   w.species = (const int*)spec;
   w.nu = (const double*)nu;
@@ -921,7 +922,7 @@ int run(Ctx* c, int N, const double* pos_in, const double* cell, const int* spec
                  sliced_pair, dp.nqs, tc05 ? (3 * max_ns + 31) / 32 * 32 : 0, sparse,
                  !sparse && (!sliced_chain || dp.lanczos || dp.logmode || dp.paper), sliced_chain && dp.lanczos, rec_pair,
                  !sparse && (!sliced_pair || dp.paper || nf > 32),
-                 scs_contract_scratch(N, max_n1, dp.nqs)};
+                 scs_contract_scratch(N, max_n1, dp.nqs, w.sms)};
   auto s1 = [&](int a, int b) { return L.stage1(o, a, b, nullptr, nullptr); };
   auto s1x = [&](int a, int b) { return forces ? L.scs_adjoint(o, a, b, nullptr, nullptr) : (size_t)0; };
   auto s2 = [&](int a, int b) { return L.stage2(o, a, b, nullptr, nullptr, nullptr); };

@@ -81,6 +81,7 @@ struct Counts {
 struct Work {
   int n_atoms;
   int site_cap;                // capacity of one centre's site list
+  int sms;                     // SMs of the device
   // inputs (device copies)
   const double* pos;           // N x 3 Angstrom
   const int* species;          // N
@@ -387,7 +388,7 @@ void launch_scs_lu_forward(const Work& w, const DevParams& p, int lu_blocks, int
 void launch_scs_lu_adjoint(const Work& w, const DevParams& p, int lu_blocks, int c0, int c1, int max_n1,
                            cudaStream_t s);
 void launch_scs_contract(const Work& w, const DevParams& p, int c0, int c1, int max_n1, cudaStream_t s);
-int scs_contract_scratch(int n_atoms, int max_n1, int nqs);   // float2 of gradient scratch per pair
+int scs_contract_scratch(int n_atoms, int max_n1, int nqs, int sms);   // float2 of gradient scratch per pair
 bool scs_capacity(int max_n1, int max_n12);
 void launch_mbd_prepare_sized(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
 void launch_mbd_chain_sized(const Work& w, const DevParams& p, int m, int c0, int c1, int max_ns, cudaStream_t s);
@@ -435,8 +436,6 @@ void launch_slice_pq(const Work& w, const DevParams& p, int c0, int c1, cudaStre
 // adjoint pair matrix and its per-pair contraction, 5 digits: tcgen05 tensor cores, warp-level products
 void launch_pair_tc(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
 void launch_mbd_adj_pair_oz2(const Work& w, const DevParams& p, int c0, int c1, int max_ns, cudaStream_t s);
-// SMs of the current device
-int device_sms();
 
 // Raise the dynamic shared-memory limit of a kernel to at least `bytes` (never lowers it: the
 // limit is process-wide, and lowering it while another host thread launches the same kernel

@@ -21,7 +21,6 @@
 #include "../paper_2407_06409_gb300/csrc/k_chain_tc.cu"
 
 // what the chain's launcher calls; this program launches the kernel itself
-int device_sms() { return 1; }
 void launch_slice_w(const Work&, const DevParams&, int, int, int, int, cudaStream_t) {}
 void raise_smem_limit(const void* f, size_t bytes) { cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); }
 
