@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(256, 2)
   const int erow = emax[0], ecol = emax[1];
   int scale = erow + ecol - 14;                    // the digits are 2^(er + ec - 14) sum acc_g 2^(-7 g)
   if (t0 == 0) scale = max(scale, emax[2]);
+  const int half = scale >> 1;                     // 2^scale in two exact factors: it can pass the FP64 range
   const int row = 32 * (warp & 3) + lane;
   if (row < 3 * PTC_SA) {
     const bool rv = 3 * s0 + row < 3 * ns;
@@ -203,11 +204,12 @@ __global__ void __launch_bounds__(256, 2)
   for (int e = tid; e < 2 * PTC_SA * PTC_GL; e += blockDim.x) gp[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   if (t0 == 0) {   // central column: the further term X0
+    const double d1 = oz_pow2(-half), d2 = oz_pow2(half - scale);
     for (int e = tid; e < 9 * PTC_SA; e += blockDim.x) {
       const int sl = e / 9, u = e % 9;
       if (s0 + sl >= ns) continue;
       float2& m = Ms[(3 * sl + u / 3) * PTC_LD + u % 3];
-      const ff v = ff_add(ff_make(m.x, m.y), ff_from_double(oz_ldexp(w.x0buf[(offs + s0 + sl) * 9 + u], -scale)));
+      const ff v = ff_add(ff_make(m.x, m.y), ff_from_double(w.x0buf[(offs + s0 + sl) * 9 + u] * d1 * d2));
       m = make_float2(v.hi, v.lo);
     }
     __syncthreads();
@@ -231,6 +233,7 @@ __global__ void __launch_bounds__(256, 2)
   __syncthreads();
   // deterministic per-site sums, one thread per (site, component): row sites get -g, column sites +g
   const float2* g2 = reinterpret_cast<const float2*>(gp);
+  const double u1 = oz_pow2(half), u2 = oz_pow2(scale - half);
   for (int e = tid; e < 4 * (PTC_SA + PTC_SB); e += blockDim.x) {
     const int d = e & 3, sd = e >> 2;
     const bool rs = sd < PTC_SA;
@@ -243,7 +246,7 @@ __global__ void __launch_bounds__(256, 2)
       const float2 v = g2[4 * (first + o * step) + d];
       s2[o & 1] = ff_add(s2[o & 1], ff_make(v.x, v.y));
     }
-    const double sum = oz_ldexp(ff_to_double(ff_add(s2[0], s2[1])), scale);
+    const double sum = ff_to_double(ff_add(s2[0], s2[1])) * u1 * u2;
     if (sum == 0.0) continue;
     if (d == 3) atomicAdd(&w.rbar[offs + ss], sum);
     else atomicAdd(w.gacc + 3 * w.site_atom[(long long)c * w.site_cap + ss] + d, rs ? -sum : sum);
