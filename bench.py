@@ -30,12 +30,17 @@ FP32_PEAK_TFLOPS = 80.5          # 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz
 # DRAM bytes (read + write) of the forward SCS solves (k_scs_solve) per atom: ncu on the
 # 512-atom box, profiles/ncu_all_kernels_box512.md; scaled to a launch by atoms / launches
 SCS_SOLVE_DRAM_BYTES_PER_ATOM = 0.314e6
+# conjugate-gradient steps of a forward SCS system, all refinement passes, three right-hand sides together:
+# mean over the benchmark box (12 frequencies and omega = 0), counted with a counter in a copy of the
+# kernel; 57 flops per step and ordered pair of sites for the three right-hand sides
+CG_STEPS_PER_SYSTEM, CG_FLOPS_PER_PAIR = 29.8, 57.0
+FLOAT_FLOAT = ("float-float (2^-46): SCS pair terms, refinement residuals of the FP32 conjugate gradients, SCS adjoint "
+               "contraction")
 PRECISION = ("chain products: 6-digit (energy blocks) / 5-digit (adjoint-only blocks) bf16 Ozaki slices "
-             "of the operands, exact recombination; adjoint pair product: 5-digit slices, float-float "
-             "operands and epilogue; SCS: FP32 conjugate gradients with iterative refinement to FP64 "
-             "accuracy (float-float residuals); everything else FP64")
-PRECISION_FP64 = ("chain and adjoint pair products in FP64; SCS: FP32 conjugate gradients with "
-                  "iterative refinement to FP64 accuracy (float-float residuals); everything else FP64")
+             "of the operands; adjoint pair product: 5-digit slices; digit orders added up in float-float; "
+             + FLOAT_FLOAT + ", T_LR pair records and blocks, series and pair sums of the adjoint; "
+             "the rest (distances, exponentials, erf, blends, traces, sums over pairs of atoms) FP64")
+PRECISION_FP64 = "chain and adjoint pair products in FP64; " + FLOAT_FLOAT + "; the rest FP64"
 WORKLOAD = ("periodic random box, 4096 atoms, 0.1 atoms/A^3, 4 species; r_SCS 5 A, MBD sphere 7 A "
             "(r_MBD,1 = r_MBD,2 = 7 A), 12 omega, n_max 6; energies + forces within 1e-10 rel. / "
             "1e-8 eV/A of the FP64 oracle (see precision)")
@@ -351,8 +356,8 @@ def run_ours(args, world, rank, local):
         # The forward SCS solves.  Method work (the dense linear algebra of the local screening
         # solves): per centre and SCS frequency a Cholesky factorisation, (3 n1)^3 / 3 flops, and
         # 12 (3 n1)^2 for the triangular solves with 3 right-hand sides (the count of the work
-        # estimate of the scope table; the kernel solves the same systems by conjugate gradients on
-        # their sparse pair lists).  It runs on the FP32 SIMT pipe, so the peak is that pipe's
+        # estimate of the scope table; the kernel solves the same systems by conjugate gradients with
+        # dense products over the sites of a system).  It runs on the FP32 SIMT pipe, so the peak is that pipe's
         # nominal rate from unit counts and the maximum clock.  Time: the kernel's own bucket
         # launches, fork to join (CUDA events around them in the library).
         nq = 2 if args.omega_ref > 0 else (args.fit_nodes + 2 if args.fit_nodes > 0 else 13)
@@ -363,23 +368,27 @@ def run_ours(args, world, rank, local):
         t_fac = kernel_ms["scs_factor"] / args.steps * 1e-3 if kernel_ms["scs_factor"] > 0 else avg_ms * 1e-3
         work = w_method / n_fac
         achieved = work / (t_fac / n_fac) / 1e12
-        # a second figure: the part of the kernel's instruction mix that the pair counts fix, the
-        # float-float right-hand side and residuals (the FP64-equivalent flop count of those sums, each
-        # float-float multiply-add about 20 FP32 operations, i.e. 10 per FP64 flop)
+        # a second figure, the kernel's own work: the float-float right-hand side and residuals (the
+        # FP64-equivalent flop count of those sums, each float-float multiply-add about 20 FP32
+        # operations, i.e. 10 per FP64 flop) and, at the counted frequencies, the conjugate-gradient steps
         pairs, adj = float(st_last["scs_pairs"]), float(st_last["scs_adjacency"])
         wff = nq * (60.0 * adj + 36.0 * (pairs - adj / 2.0) + 2.0 * pairs)
-        t_star = 10.0 * wff / (FP32_PEAK_TFLOPS * 1e12)
+        wcg = CG_FLOPS_PER_PAIR * CG_STEPS_PER_SYSTEM * nq * float(np.sum(n1 ** 2)) if nq == 13 else 0.0
+        t_star = (10.0 * wff + wcg) / (FP32_PEAK_TFLOPS * 1e12)
         roofline = {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP32_PEAK_TFLOPS,
                     "traffic": SCS_SOLVE_DRAM_BYTES_PER_ATOM * args.atoms / n_fac,
                     "kernel": kernel_names[dom], "launches_per_step": n_fac, "ms_per_step": t_fac * 1e3,
                     "work_per_step": w_method,
-                    "peak_note": "flops of a dense solve, sum_k nq [(3 n1)^3/3 + 12 (3 n1)^2], over the time of "
-                                 "the kernel, which solves by conjugate gradients on the sparse pair lists, against the FP32 SIMT pipe it runs on: 152 SMs x 128 lanes x 2 flops x "
-                                 "2.07 GHz = 80.5 TFLOP/s nominal (unit counts and maximum clock)",
-                    "composite": {"peak_note": "the float-float right-hand side and residuals alone, at 10 "
-                                               "FP32 operations per FP64-equivalent flop, on the FP32 pipe "
-                                               "(80.5 TFLOP/s)",
+                    "peak_note": "flops of direct dense solves, sum_k nq [(3 n1)^3/3 + 12 (3 n1)^2], over the time of "
+                                 "the kernel (conjugate gradients with dense products over a packed triangle of pair "
+                                 "couplings in shared memory), against the FP32 SIMT pipe it runs on: 152 SMs x "
+                                 "128 lanes x 2 flops x 2.07 GHz = 80.5 TFLOP/s nominal (unit counts and maximum clock)",
+                    "composite": {"peak_note": "the kernel's own operations on the same pipe: conjugate-gradient steps "
+                                               "(29.8 per system, counted once on this workload; left out for other "
+                                               "frequency sets) and the float-float right-hand side and residuals "
+                                               "at 10 FP32 operations per FP64-equivalent flop",
+                                  "work_conjugate_gradients": wcg,
                                   "work_float_float_fp64_equiv": wff, "t_star_ms": t_star * 1e3,
                                   "frac": t_star / t_fac}}
     elif dom in ("chain", "adj_pair"):
