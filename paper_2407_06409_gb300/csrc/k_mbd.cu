@@ -498,7 +498,7 @@ __device__ __forceinline__ void lf_block_sum(const double* v, double* red, doubl
 // their rounding errors and then added to the running sum, so the low words stay small (energies of the
 // fitted series, error against 64 bits: 3.7e-13 with FP64 products, 3.3e-13 now).  The recurrence itself stays in FP64: v and the vector that becomes the
 // next one lie in shared memory, column-major and touched only by the thread of their row.
-// 300 atoms (spheres of 143 sites), 12 frequencies, 12 steps: 25.8 -> 6.1 ms.
+// 300 atoms (spheres of 143 sites), 12 frequencies, 12 steps: 25.8 -> 6.0 ms.
 template <int QC>
 __global__ void __launch_bounds__(LF_THREADS) k_lanczos_fit(Work w, DevParams p, int c0, int q0, int qc, int L3) {
   extern __shared__ double lfs[];
@@ -2054,7 +2054,7 @@ __global__ void __launch_bounds__(256) k_slice_w(Work w, DevParams p, int m, int
 // FP32 pipe (2^-46, against the 2^-35 of the digits); the weights c_n of each frequency are scaled to unit
 // size (callers' weights may be of any magnitude, and fitted coefficients differ by 2^150 between
 // frequencies; see series_scale), the exponent goes to Q's rows and the sums.  FP64 P and Q
-// and their separate slicing took 5.2 + 1.75 ms per 4096-atom step; now 4.9 ms with the tile images that
+// and their separate slicing took 5.2 + 1.75 ms per 4096-atom step; now 4.2 ms with the tile images that
 // save the pair product 0.4 ms.
 // Five signed 7-bit digits of v relative to 2^e (s1 = 2^(35 - e)), rounded to nearest, as bf16 bits.
 __device__ __forceinline__ void pq_digits(ff v, float s1, unsigned (&d)[5]) {
