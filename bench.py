@@ -28,7 +28,7 @@ METRIC = "atoms/s for lMBD energy+forces on 1 GB300 (batched vs per-atom launch)
 FP64_PEAK_TFLOPS = 1.25          # nominal GB300 FP64 (DFMA and DMMA), profiling recipe table
 FP32_PEAK_TFLOPS = 80.5          # 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz (unit counts and clock)
 # DRAM bytes (read + write) of the forward SCS solves (k_scs_solve) per atom: ncu on the
-# 512-atom box, profiles/ncu_hot_kernels_box512.md; scaled to a launch by atoms / launches
+# 512-atom box; scaled to a launch by atoms / launches
 SCS_SOLVE_DRAM_BYTES_PER_ATOM = 0.314e6
 # conjugate-gradient steps of a forward SCS system, all refinement passes, three right-hand sides together:
 # mean over the benchmark box (12 frequencies and omega = 0), counted with a counter in a copy of the
